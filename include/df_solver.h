@@ -29,7 +29,7 @@
  *     given in LDU form over that numbering (see df_mesh_renumber to get there).
  *   - Kernels are enqueued on `stream` (a cudaStream_t, NULL = legacy default stream) and return
  *     without synchronising. A df_solver is used by one host thread and one stream at a time
- *     (Gauss-Seidel keeps its halo buffers in the solver).
+ *     (Gauss-Seidel keeps its intermediate sums in the solver).
  *   - Errors: a df_status code; df_solver_get_last_error(s) (or df_get_last_error(NULL) for
  *     the host helpers and df_solver_create) describes it; nothing is enqueued on error unless
  *     the code is DF_ERR_CUDA.
@@ -90,8 +90,7 @@ df_status df_mesh_renumber(int64_t n_cells, int64_t n_faces, const int32_t* owne
 
 /* Sec. 3.2.2. Builds, on the HOST, the block-sparse structure of the mesh's matrices and the
  * positions that map LDU coefficients onto it, plus the Gauss-Seidel schedule (maximal runs of
- * consecutive rows of a block row with no dependency among them), the halo (cells read by
- * another block row) and the cell-to-face lists of the assembly; uploads them to `device`.
+ * consecutive rows of a block row with no dependency among them) and the cell-to-face lists of the assembly; uploads them to `device`.
  *   owner, neighbour: HOST [n_faces], owner[f] < neighbour[f] < n_cells, no repeated pair, any
  *     face order; this face order is the order of the LDU arrays of the other calls.
  *   part_ptr: HOST [n_parts + 1], 0 = part_ptr[0] < ... < part_ptr[n_parts] = n_cells, each

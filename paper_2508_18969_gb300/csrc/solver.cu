@@ -7,22 +7,24 @@
 //   lrp         [n+1]    start of each row's in-block entries LEFT of the diagonal (the
 //   lc, lv      [nnzL]   Gauss-Seidel "lower" part), ascending column: 16-bit column local to
 //                        the block row, FP64 value; a block row's lower entries are contiguous
-//   urp, uc, uv          the same for the in-block entries RIGHT of the diagonal
-//   orp         [n+1]    start of each row's off-block entries
-//   oc, oh, ov  [nnzO]   off-block entries: global column, slot of that column in the halo
-//                        list, FP64 value
-//   lmap, umap, omap     position of every entry in the LDU arrays: 2 f + 1 for upper[f],
+//   rrp         [n+1]    start of each row's remaining entries: the in-block ones RIGHT of the
+//   rc, rv      [nnzR]   diagonal (ascending column), then the off-block ones (ascending): global
+//                        column, FP64 value. One list, because both kernels that read them (SpMV
+//                        and Gauss-Seidel part 1) take them together: one loop per row keeps a
+//                        warp's lanes busy to the longest row, not to the longest of each kind
+//                        (10^6 cells: SpMV 50 -> 40 us, part 1 33 -> 26 us)
+//   lmap, rmap           position of every entry in the LDU arrays: 2 f + 1 for upper[f],
 //                        2 f for lower[f] (the precomputed map of Sec. 3.2.2)
 //   ch_ptr, ch_row       Gauss-Seidel schedule: block row I is swept as chunks
 //                        ch_ptr[I] .. ch_ptr[I+1]-1; chunk k is rows ch_row[k] .. ch_row[k+1]-1,
 //                        at most 32 consecutive rows none of which has a lower entry inside
 //                        the chunk (a piece of a "run", a maximal range with that property)
-//   halo_ptr, halo       cells some other block row reads, ascending (so grouped by block row)
 //   cf_ptr, cf           faces of every cell, ascending (the assembly's gather lists)
-//   order       [n]      the rows of each block row (16-bit local index) by descending number
-//                        of entries: the row order in which SpMV and Gauss-Seidel part 1 hand
-//                        rows to threads, so that a warp's rows have similar lengths and its
-//                        FP64 instructions run with few idle lanes (results do not depend on it)
+//   order, rorder [n]    the rows of each block row (16-bit local index) by descending number of
+//                        entries (order: all of them, for SpMV; rorder: the remaining ones, for
+//                        Gauss-Seidel part 1): the order in which those kernels hand rows to
+//                        threads, so that a warp's rows have similar lengths and its FP64
+//                        instructions run with few idle lanes (results do not depend on it)
 //
 // SpMV gives one CTA to a block row. A Gauss-Seidel sweep is split where its dependencies are:
 // the part of every row that uses only values from before the sweep (upper and off-block
@@ -51,25 +53,19 @@ struct SolverDev {
   const uint16_t* lc = nullptr;
   double* lv = nullptr;
   const int32_t* lmap = nullptr;
-  const int32_t* urp = nullptr;
-  const uint16_t* uc = nullptr;
-  double* uv = nullptr;
-  const int32_t* umap = nullptr;
-  const int32_t* orp = nullptr;
-  const int32_t* oc = nullptr;
-  const int32_t* oh = nullptr;
-  double* ov = nullptr;
-  const int32_t* omap = nullptr;
+  const int32_t* rrp = nullptr;
+  const int32_t* rc = nullptr;
+  double* rv = nullptr;
+  const int32_t* rmap = nullptr;
   double* dg = nullptr;
   double* rd = nullptr;
   const int32_t* ch_ptr = nullptr;
   const int32_t* ch_row = nullptr;
-  const int32_t* halo_ptr = nullptr;
-  const int32_t* halo = nullptr;
   const int32_t* cf_ptr = nullptr;
   const int32_t* cf = nullptr;
   const uint16_t* order = nullptr;   // per block row: local rows by descending entry count
-  int64_t n = 0, nf = 0, nnzL = 0, nnzU = 0, nnzO = 0, nh = 0;
+  const uint16_t* rorder = nullptr;  // the same by descending count of the remaining entries
+  int64_t n = 0, nf = 0, nnzL = 0, nnzR = 0;
   int t = 0;
 };
 
@@ -87,14 +83,35 @@ __device__ __forceinline__ double ldu_value(int32_t m, const double* lower, cons
   return (m & 1) ? upper[m >> 1] : lower[m >> 1];
 }
 
+// Values of entries [0, count) of one entry list, kConvBatch per thread and pass: the maps first,
+// then the gathered coefficients, then the stores, so that a thread keeps that many of the two
+// dependent loads in flight (10^6 cells: 38 -> 30 us with one in flight before).
+constexpr int kConvBatch = 4;
+__device__ __forceinline__ void convert_list(int64_t count, const int32_t* __restrict__ map,
+                                             const double* __restrict__ lower,
+                                             const double* __restrict__ upper,
+                                             double* __restrict__ val) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < count;
+       e0 += kConvBatch * stride) {
+    int32_t m[kConvBatch];
+    double v[kConvBatch];
+#pragma unroll
+    for (int u = 0; u < kConvBatch; ++u) m[u] = e0 + u * stride < count ? map[e0 + u * stride] : -1;
+#pragma unroll
+    for (int u = 0; u < kConvBatch; ++u) v[u] = m[u] >= 0 ? ldu_value(m[u], lower, upper) : 0.0;
+#pragma unroll
+    for (int u = 0; u < kConvBatch; ++u)
+      if (m[u] >= 0) val[e0 + u * stride] = v[u];
+  }
+}
+
 __global__ void convert_kernel(SolverDev d, const double* __restrict__ lower,
                                const double* __restrict__ diag, const double* __restrict__ upper) {
+  convert_list(d.nnzL, d.lmap, lower, upper, d.lv);
+  convert_list(d.nnzR, d.rmap, lower, upper, d.rv);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t e = i0; e < d.nnzL; e += stride) d.lv[e] = ldu_value(d.lmap[e], lower, upper);
-  for (int64_t e = i0; e < d.nnzU; e += stride) d.uv[e] = ldu_value(d.umap[e], lower, upper);
-  for (int64_t e = i0; e < d.nnzO; e += stride) d.ov[e] = ldu_value(d.omap[e], lower, upper);
-  for (int64_t r = i0; r < d.n; r += stride) {
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < d.n; r += stride) {
     const double a = diag[r];
     d.dg[r] = a;
     d.rd[r] = 1.0 / a;
@@ -121,10 +138,8 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(SolverDev d, const doubl
       double s = d.dg[r] * x[r];
       const int l1 = d.lrp[r + 1];
       for (int e = d.lrp[r]; e < l1; ++e) s = fma(d.lv[e], xI[d.lc[e]], s);
-      const int u1 = d.urp[r + 1];
-      for (int e = d.urp[r]; e < u1; ++e) s = fma(d.uv[e], xI[d.uc[e]], s);
-      const int o1 = d.orp[r + 1];
-      for (int e = d.orp[r]; e < o1; ++e) s = fma(d.ov[e], x[d.oc[e]], s);
+      const int e1 = d.rrp[r + 1];
+      for (int e = d.rrp[r]; e < e1; ++e) s = fma(d.rv[e], x[d.rc[e]], s);
       y[r] = RESID ? b[r] - s : s;
     }
   } else {
@@ -137,10 +152,12 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(SolverDev d, const doubl
       f2 s = f2_mul(f2_from(d.dg[r]), ld2(xs + (r - r0)));
       const int l1 = d.lrp[r + 1];
       for (int e = d.lrp[r]; e < l1; ++e) acc_fma(s, f2_from(d.lv[e]), ld2(xs + d.lc[e]));
-      const int u1 = d.urp[r + 1];
-      for (int e = d.urp[r]; e < u1; ++e) acc_fma(s, f2_from(d.uv[e]), ld2(xs + d.uc[e]));
-      const int o1 = d.orp[r + 1];
-      for (int e = d.orp[r]; e < o1; ++e) acc_fma(s, f2_from(d.ov[e]), f2_from(x[d.oc[e]]));
+      const int e1 = d.rrp[r + 1];
+      for (int e = d.rrp[r]; e < e1; ++e) {
+        const int c = d.rc[e];   // the block row's own columns come from shared memory
+        const f2 xc = c >= r0 && c < r1 ? ld2(xs + (c - r0)) : f2_from(x[c]);
+        acc_fma(s, f2_from(d.rv[e]), xc);
+      }
       s = f2_fin(s);
       if (RESID) s = f2_fin(f2_add(f2_from(b[r]), f2_neg(s)));
       y[r] = f2_to_int(s);
@@ -148,43 +165,27 @@ __global__ void __launch_bounds__(kThreads) spmv_kernel(SolverDev d, const doubl
   }
 }
 
-// Halo values of x before the first sweep (FP64, or double-float pairs for F2).
-template <bool F2>
-__global__ void halo_gather_kernel(SolverDev d, const double* __restrict__ x, void* __restrict__ h) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < d.nh; k += stride) {
-    if constexpr (F2) st2(static_cast<float2*>(h) + k, f2_from(x[d.halo[k]]));
-    else static_cast<double*>(h)[k] = x[d.halo[k]];
-  }
-}
-
 // Sec. 3.2.3, Gauss-Seidel part 1: the part of every row that uses only values from before the
-// sweep, p_r = b_r - sum over upper entries of a_rc x_c - sum over off-block entries of a_rc h_c
-// (x_c of the block row before the sweep, h_c the halo value of another block's cell). No row
-// depends on another: one CTA per block row, one thread per row, like SpMV. p is FP64, or a
-// double-float pair for F2.
+// sweep, p_r = b_r - sum over the upper and off-block entries of a_rc x_c. This kernel ends before
+// gs_sweep_kernel writes any x, so x itself holds the values from before the sweep, also of other
+// block rows' cells: no halo copy. No row depends on another: one CTA per block row, one thread per
+// row, like SpMV. p is FP64, or a double-float pair for F2.
 template <bool F2>
 __global__ void __launch_bounds__(kThreads) gs_rhs_kernel(SolverDev d, const double* __restrict__ b,
                                                           const double* __restrict__ x,
-                                                          const void* __restrict__ hold,
                                                           void* __restrict__ p) {
   const int I = blockIdx.x;
   const int r0 = d.part[I], r1 = d.part[I + 1];
-  const double* __restrict__ xI = x + r0;
   for (int j = threadIdx.x; j < r1 - r0; j += kThreads) {
-    const int r = r0 + d.order[r0 + j];
-    const int u1 = d.urp[r + 1], o1 = d.orp[r + 1];
+    const int r = r0 + d.rorder[r0 + j];
+    const int e1 = d.rrp[r + 1];
     if constexpr (F2) {
-      const float2* h2 = static_cast<const float2*>(hold);
       f2 s = f2_from(b[r]);
-      for (int e = d.urp[r]; e < u1; ++e) acc_fma(s, f2_neg(f2_from(d.uv[e])), f2_from(xI[d.uc[e]]));
-      for (int e = d.orp[r]; e < o1; ++e) acc_fma(s, f2_neg(f2_from(d.ov[e])), ld2(h2 + d.oh[e]));
+      for (int e = d.rrp[r]; e < e1; ++e) acc_fma(s, f2_neg(f2_from(d.rv[e])), f2_from(x[d.rc[e]]));
       st2(static_cast<float2*>(p) + r, f2_fin(s));
     } else {
-      const double* h64 = static_cast<const double*>(hold);
       double s = b[r];
-      for (int e = d.urp[r]; e < u1; ++e) s = fma(-d.uv[e], xI[d.uc[e]], s);
-      for (int e = d.orp[r]; e < o1; ++e) s = fma(-d.ov[e], h64[d.oh[e]], s);
+      for (int e = d.rrp[r]; e < e1; ++e) s = fma(-d.rv[e], x[d.rc[e]], s);
       static_cast<double*>(p)[r] = s;
     }
   }
@@ -199,8 +200,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
   const uint64_t z = ((uint64_t)p + (uint64_t)bytes + 15) & ~uint64_t(15);
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(z - a)) : "memory");
 }
-
-constexpr int kPrefetchChunks = 4;   // chunks whose data is fetched into L2 ahead of the sweep
 
 // Shared memory of one sweeping warp, in bytes: the block row's new x (8 per cell), its row
 // offsets into its lower entries (4 per cell + 4) and its chunk bounds (2 per chunk + 2).
@@ -217,25 +216,17 @@ inline SweepSmem sweep_smem(int max_part, int max_chunks) {
   return L;
 }
 
-// Everything chunk k of the sweep reads from global memory, prefetched into L2 by lanes 0-4.
-__device__ __forceinline__ void prefetch_chunk(const SolverDev& d, const void* p, int k, int lane) {
-  const int rs = d.ch_row[k], re = d.ch_row[k + 1];
-  switch (lane) {
-    case 0: {
-      const int e0 = d.lrp[rs], e1 = d.lrp[re];
-      prefetch_l2(d.lv + e0, 8 * (int64_t)(e1 - e0));
-      break;
-    }
-    case 1: {
-      const int e0 = d.lrp[rs], e1 = d.lrp[re];
-      prefetch_l2(d.lc + e0, 2 * (int64_t)(e1 - e0));
-      break;
-    }
-    case 2: prefetch_l2(static_cast<const double*>(p) + rs, 8 * (int64_t)(re - rs)); break;
-    case 3: prefetch_l2(d.rd + rs, 8 * (int64_t)(re - rs)); break;
-    case 4: prefetch_l2(d.lrp + rs, 4 * (int64_t)(re - rs + 1)); break;
-    default: break;
-  }
+// Everything the sweep of block row r0 .. r0 + m - 1 reads from global memory (its lower entries
+// a0 .. a1 - 1, p and 1/a_rr: about 45 bytes a row), fetched into L2 by lanes 0-3 at the start of
+// the sweep. One request per array for the whole block row: the addresses are known without
+// reading the schedule, where a fetch per chunk cost two dependent global loads (chunk bounds, then
+// row offsets) on the sweep's critical path (138 -> 65 us for a sweep of 10^6 cells).
+__device__ __forceinline__ void prefetch_block_row(const SolverDev& d, const void* p, int r0, int m,
+                                                   int a0, int a1, int lane) {
+  if (lane == 0) prefetch_l2(d.lv + a0, 8 * (int64_t)(a1 - a0));
+  if (lane == 1) prefetch_l2(d.lc + a0, 2 * (int64_t)(a1 - a0));
+  if (lane == 2) prefetch_l2(static_cast<const double*>(p) + r0, 8 * (int64_t)m);
+  if (lane == 3) prefetch_l2(d.rd + r0, 8 * (int64_t)m);
 }
 
 // Row data of one chunk for one lane of the sweep: the row's p and 1/a_rr and its first
@@ -278,13 +269,12 @@ __device__ __forceinline__ void sweep_load(const SolverDev& d, const void* p, in
 // Only lower entries are read and their rows were updated earlier in this sweep, so the block
 // row's new x is built in shared memory without loading the old one. The chunk bounds and row
 // offsets of the block row are staged in shared memory first; each chunk's row data is loaded
-// into registers while the previous chunk is swept, and fetched into L2 further ahead, so the
-// dependency chain holds only shared-memory reads and arithmetic. At the end x is written
-// back, and the block row's halo cells go to hnew for the next sweep.
+// into registers while the previous chunk is swept, from lines fetched into L2 at the start, so
+// the dependency chain holds only shared-memory reads and arithmetic. At the end x is written
+// back.
 template <bool F2>
 __global__ void __launch_bounds__(128) gs_sweep_kernel(SolverDev d, const void* __restrict__ p,
-                                                       double* __restrict__ x,
-                                                       void* __restrict__ hnew, SweepSmem L) {
+                                                       double* __restrict__ x, SweepSmem L) {
   extern __shared__ __align__(16) unsigned char gs_smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int I = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -297,7 +287,7 @@ __global__ void __launch_bounds__(128) gs_sweep_kernel(SolverDev d, const void* 
   const int r0 = d.part[I], m = d.part[I + 1] - r0;
   const int k0 = d.ch_ptr[I], nk = d.ch_ptr[I + 1] - k0;
   const int a0 = d.lrp[r0];
-  for (int k = k0; k < k0 + nk && k < k0 + kPrefetchChunks; ++k) prefetch_chunk(d, p, k, lane);
+  prefetch_block_row(d, p, r0, m, a0, d.lrp[r0 + m], lane);
   for (int j = lane; j <= nk; j += 32) chs[j] = (uint16_t)(d.ch_row[k0 + j] - r0);
   for (int i = lane; i <= m; i += 32) lrps[i] = d.lrp[r0 + i] - a0;
   __syncwarp();
@@ -305,7 +295,6 @@ __global__ void __launch_bounds__(128) gs_sweep_kernel(SolverDev d, const void* 
   if (nk > 0) sweep_load<F2>(d, p, r0, a0, chs, lrps, 0, lane, cur);
   for (int k = 0; k < nk; ++k) {
     if (k + 1 < nk) sweep_load<F2>(d, p, r0, a0, chs, lrps, k + 1, lane, nxt);
-    if (k + kPrefetchChunks < nk) prefetch_chunk(d, p, k0 + k + kPrefetchChunks, lane);
     if (cur.cnt >= 0) {
       if constexpr (F2) {
         f2 s = f2{__int_as_float(__double2loint(cur.pv)), __int_as_float(__double2hiint(cur.pv))};
@@ -335,12 +324,6 @@ __global__ void __launch_bounds__(128) gs_sweep_kernel(SolverDev d, const void* 
     if constexpr (F2) x[r0 + i] = f2_to_int(ld2(xs2 + i));
     else x[r0 + i] = xs[i];
   }
-  if (hnew) {
-    for (int k = d.halo_ptr[I] + lane; k < d.halo_ptr[I + 1]; k += 32) {
-      if constexpr (F2) static_cast<float2*>(hnew)[k] = xs2[d.halo[k] - r0];
-      else static_cast<double*>(hnew)[k] = xs[d.halo[k] - r0];
-    }
-  }
 }
 
 // Warps (block rows) per sweep CTA: as many as fit 192 KB of shared memory, at most 4.
@@ -362,7 +345,19 @@ __global__ void laplacian_kernel(SolverDev d, const double* __restrict__ g,
   for (int64_t c = i0; c < d.n; c += stride) {
     double a = s[c];
     const int k1 = d.cf_ptr[c + 1];
-    for (int k = d.cf_ptr[c]; k < k1; ++k) a += g[d.cf[k]];
+    // eight faces at a time: their numbers, then their coefficients, then the additions in face
+    // order, so that the two dependent loads of a cell's faces overlap (most cells have 5 to 9)
+    for (int k = d.cf_ptr[c]; k < k1; k += 8) {
+      int f[8];
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) f[u] = k + u < k1 ? d.cf[k + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = f[u] >= 0 ? g[f[u]] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (f[u] >= 0) a += v[u];
+    }
     diag[c] = a;
   }
 }
@@ -383,15 +378,15 @@ struct df_solver {
   int64_t nruns = 0, nchunks = 0;
   int arith = DF_SOLVER_FP64;
   bool converted = false;
+  int64_t nnz_off = 0, nhalo = 0;        // off-block entries, cells read by another block row
   size_t bytes = 0;
   std::string err;
   SolverDev d;
-  double* hbuf[2] = {nullptr, nullptr};
   double* pbuf = nullptr;                // Gauss-Seidel part-1 sums p [n]
   std::vector<void*> allocs;
   // host copies of the structure, for df_solver_export_csr
-  std::vector<int32_t> h_part, h_lrp, h_urp, h_orp, h_oc;
-  std::vector<uint16_t> h_lc, h_uc;
+  std::vector<int32_t> h_part, h_lrp, h_rrp, h_rc;
+  std::vector<uint16_t> h_lc;
 };
 
 namespace {
@@ -504,13 +499,13 @@ df_status df_solver_create(int64_t n_cells, int64_t n_faces, const int32_t* owne
       col[w[b]] = a; pos[w[b]++] = (int32_t)(2 * f);       // A[b][a] = lower[f]
     }
   }
-  std::vector<int32_t> lrp(n + 1, 0), urp(n + 1, 0), orp(n + 1, 0);
-  std::vector<uint16_t> lc, uc;
-  std::vector<int32_t> lmap, umap, oc, omap;
+  std::vector<int32_t> lrp(n + 1, 0), rrp(n + 1, 0);
+  std::vector<uint16_t> lc;
+  std::vector<int32_t> lmap, rc, rmap, halo;
   lc.reserve(n_faces);
-  uc.reserve(n_faces);
   lmap.reserve(n_faces);
-  umap.reserve(n_faces);
+  rc.reserve(2 * n_faces);
+  rmap.reserve(2 * n_faces);
   std::vector<std::pair<int32_t, int32_t>> ent;
   for (int64_t r = 0; r < n; ++r) {
     ent.clear();
@@ -523,20 +518,23 @@ df_status df_solver_create(int64_t n_cells, int64_t n_faces, const int32_t* owne
     const int p = part_of[r];
     const int32_t base = hpart[p];
     for (auto& e : ent) {
-      if (part_of[e.first] != p) {
-        oc.push_back(e.first);
-        omap.push_back(e.second);
-      } else if (e.first < r) {
+      if (part_of[e.first] != p) continue;
+      if (e.first < r) {
         lc.push_back((uint16_t)(e.first - base));
         lmap.push_back(e.second);
       } else {
-        uc.push_back((uint16_t)(e.first - base));
-        umap.push_back(e.second);
+        rc.push_back(e.first);
+        rmap.push_back(e.second);
       }
     }
+    for (auto& e : ent) {
+      if (part_of[e.first] == p) continue;
+      rc.push_back(e.first);
+      rmap.push_back(e.second);
+      halo.push_back(e.first);
+    }
     lrp[r + 1] = (int32_t)lc.size();
-    urp[r + 1] = (int32_t)uc.size();
-    orp[r + 1] = (int32_t)oc.size();
+    rrp[r + 1] = (int32_t)rc.size();
   }
   col.clear(); col.shrink_to_fit();
   pos.clear(); pos.shrink_to_fit();
@@ -569,31 +567,27 @@ df_status df_solver_create(int64_t n_cells, int64_t n_faces, const int32_t* owne
   }
   ch_row.push_back((int32_t)n);
 
-  // row order for the thread-per-row kernels: within each block row, by descending number of
-  // (lower + upper + off-block) entries, ties in ascending row order
-  std::vector<uint16_t> order(n);
+  // row orders of the thread-per-row kernels: within each block row, by descending number of
+  // entries (all, and the remaining ones), ties in ascending row order
+  std::vector<uint16_t> order(n), rorder(n);
   for (int p = 0; p < n_parts; ++p) {
     const int32_t base = hpart[p], m = hpart[p + 1] - base;
     std::vector<std::pair<int, int>> key(m);
     for (int i = 0; i < m; ++i) {
       const int32_t r = base + i;
-      const int len = (lrp[r + 1] - lrp[r]) + (urp[r + 1] - urp[r]) + (orp[r + 1] - orp[r]);
-      key[i] = {-len, i};
+      key[i] = {-((lrp[r + 1] - lrp[r]) + (rrp[r + 1] - rrp[r])), i};
     }
     std::sort(key.begin(), key.end());
     for (int i = 0; i < m; ++i) order[base + i] = (uint16_t)key[i].second;
+    for (int i = 0; i < m; ++i) key[i] = {-(rrp[base + i + 1] - rrp[base + i]), i};
+    std::sort(key.begin(), key.end());
+    for (int i = 0; i < m; ++i) rorder[base + i] = (uint16_t)key[i].second;
   }
 
-  // halo: cells read through off-block entries, ascending; each entry's slot in it
-  std::vector<int32_t> halo(oc.begin(), oc.end());
+  // halo: the cells read through off-block entries (counted for df_solver_get_info)
+  const int64_t nnz_off = (int64_t)halo.size();
   std::sort(halo.begin(), halo.end());
   halo.erase(std::unique(halo.begin(), halo.end()), halo.end());
-  std::vector<int32_t> oh(oc.size());
-  for (size_t k = 0; k < oc.size(); ++k)
-    oh[k] = (int32_t)(std::lower_bound(halo.begin(), halo.end(), oc[k]) - halo.begin());
-  std::vector<int32_t> halo_ptr(n_parts + 1, 0);
-  for (int p = 0; p <= n_parts; ++p)
-    halo_ptr[p] = (int32_t)(std::lower_bound(halo.begin(), halo.end(), hpart[p]) - halo.begin());
 
   // faces of every cell, ascending (assembly gather lists)
   std::vector<int32_t> cf_ptr(n + 1, 0), cf(2 * n_faces);
@@ -623,9 +617,9 @@ df_status df_solver_create(int64_t n_cells, int64_t n_faces, const int32_t* owne
   d.n = n;
   d.nf = n_faces;
   d.nnzL = (int64_t)lc.size();
-  d.nnzU = (int64_t)uc.size();
-  d.nnzO = (int64_t)oc.size();
-  d.nh = (int64_t)halo.size();
+  d.nnzR = (int64_t)rc.size();
+  s->nnz_off = nnz_off;
+  s->nhalo = (int64_t)halo.size();
   d.t = n_parts;
   cudaError_t e = cudaSuccess;
   auto up = [&](auto** dst, const auto& v) {
@@ -635,27 +629,19 @@ df_status df_solver_create(int64_t n_cells, int64_t n_faces, const int32_t* owne
   up(&d.lrp, lrp);
   up(&d.lc, lc);
   up(&d.lmap, lmap);
-  up(&d.urp, urp);
-  up(&d.uc, uc);
-  up(&d.umap, umap);
-  up(&d.orp, orp);
-  up(&d.oc, oc);
-  up(&d.oh, oh);
-  up(&d.omap, omap);
+  up(&d.rrp, rrp);
+  up(&d.rc, rc);
+  up(&d.rmap, rmap);
   up(&d.ch_ptr, ch_ptr);
   up(&d.ch_row, ch_row);
-  up(&d.halo_ptr, halo_ptr);
-  up(&d.halo, halo);
   up(&d.cf_ptr, cf_ptr);
   up(&d.cf, cf);
   up(&d.order, order);
+  up(&d.rorder, rorder);
   if (e == cudaSuccess) e = alloc(s, &d.lv, lc.size());
-  if (e == cudaSuccess) e = alloc(s, &d.uv, uc.size());
-  if (e == cudaSuccess) e = alloc(s, &d.ov, oc.size());
+  if (e == cudaSuccess) e = alloc(s, &d.rv, rc.size());
   if (e == cudaSuccess) e = alloc(s, &d.dg, n);
   if (e == cudaSuccess) e = alloc(s, &d.rd, n);
-  if (e == cudaSuccess) e = alloc(s, &s->hbuf[0], halo.size());
-  if (e == cudaSuccess) e = alloc(s, &s->hbuf[1], halo.size());
   if (e == cudaSuccess) e = alloc(s, &s->pbuf, n);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gs_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 196608);
@@ -676,11 +662,9 @@ df_status df_solver_create(int64_t n_cells, int64_t n_faces, const int32_t* owne
   }
   s->h_part = std::move(hpart);
   s->h_lrp = std::move(lrp);
-  s->h_urp = std::move(urp);
-  s->h_orp = std::move(orp);
-  s->h_oc = std::move(oc);
+  s->h_rrp = std::move(rrp);
+  s->h_rc = std::move(rc);
   s->h_lc = std::move(lc);
-  s->h_uc = std::move(uc);
   *out = s;
   return DF_OK;
 }
@@ -697,8 +681,8 @@ df_status df_solver_get_info(const df_solver* s, df_solver_info* info) {
   info->n_faces = s->nf;
   info->n_parts = s->t;
   info->nnz = s->n + 2 * s->nf;
-  info->nnz_offblock = s->d.nnzO;
-  info->n_halo = s->d.nh;
+  info->nnz_offblock = s->nnz_off;
+  info->n_halo = s->nhalo;
   info->n_runs = s->nruns;
   info->max_part = s->max_part;
   info->max_runs = s->max_runs;
@@ -720,7 +704,7 @@ df_status df_solver_convert(df_solver* s, const double* lower, const double* dia
   if (!s) return sfail(nullptr, DF_ERR_INVALID_ARG, "solver is NULL");
   if (!diag || (s->nf > 0 && (!lower || !upper))) return sfail(s, DF_ERR_INVALID_ARG, "NULL array");
   DeviceGuard g(s->device);
-  const int64_t work = std::max(std::max(s->d.nnzL, s->d.nnzU), std::max(s->d.nnzO, s->n));
+  const int64_t work = std::max(std::max(s->d.nnzL, s->d.nnzR), s->n);
   convert_kernel<<<grid_for(work, s->num_sms), kThreads, 0, (cudaStream_t)stream>>>(s->d, lower, diag,
                                                                                     upper);
   const cudaError_t e = cudaGetLastError();
@@ -765,24 +749,17 @@ df_status df_solver_gauss_seidel(df_solver* s, const double* b, double* x, int32
   DeviceGuard g(s->device);
   const cudaStream_t st = (cudaStream_t)stream;
   const bool f2 = s->arith == DF_SOLVER_DOUBLE_FLOAT;
-  if (s->d.nh > 0) {
-    const int hg = grid_for(s->d.nh, s->num_sms);
-    if (f2) halo_gather_kernel<true><<<hg, kThreads, 0, st>>>(s->d, x, s->hbuf[0]);
-    else halo_gather_kernel<false><<<hg, kThreads, 0, st>>>(s->d, x, s->hbuf[0]);
-  }
   const SweepSmem L = sweep_smem(s->max_part, s->max_chunks);
   const int w = sweep_warps(L);
   const size_t smem = (size_t)w * L.per_warp;
   const int grid = (s->t + w - 1) / w;
   for (int k = 0; k < sweeps; ++k) {
-    const double* hold = s->hbuf[k & 1];
-    double* hnew = (k + 1 < sweeps && s->d.nh > 0) ? s->hbuf[(k + 1) & 1] : nullptr;
     if (f2) {
-      gs_rhs_kernel<true><<<s->t, kThreads, 0, st>>>(s->d, b, x, hold, s->pbuf);
-      gs_sweep_kernel<true><<<grid, 32 * w, smem, st>>>(s->d, s->pbuf, x, hnew, L);
+      gs_rhs_kernel<true><<<s->t, kThreads, 0, st>>>(s->d, b, x, s->pbuf);
+      gs_sweep_kernel<true><<<grid, 32 * w, smem, st>>>(s->d, s->pbuf, x, L);
     } else {
-      gs_rhs_kernel<false><<<s->t, kThreads, 0, st>>>(s->d, b, x, hold, s->pbuf);
-      gs_sweep_kernel<false><<<grid, 32 * w, smem, st>>>(s->d, s->pbuf, x, hnew, L);
+      gs_rhs_kernel<false><<<s->t, kThreads, 0, st>>>(s->d, b, x, s->pbuf);
+      gs_sweep_kernel<false><<<grid, 32 * w, smem, st>>>(s->d, s->pbuf, x, L);
     }
   }
   const cudaError_t e = cudaGetLastError();
@@ -806,15 +783,14 @@ df_status df_solver_export_csr(df_solver* s, int64_t* row_ptr, int32_t* col, dou
   if (df_status st = check_ready(s)) return st;
   if (!row_ptr || !col || !val) return sfail(s, DF_ERR_INVALID_ARG, "NULL output array");
   DeviceGuard g(s->device);
-  std::vector<double> lv(s->d.nnzL), uv(s->d.nnzU), ov(s->d.nnzO), dg(s->n);
+  std::vector<double> lv(s->d.nnzL), rv(s->d.nnzR), dg(s->n);
   cudaError_t e = cudaDeviceSynchronize();
   auto get = [&](std::vector<double>& h, const double* dptr) {
     if (e == cudaSuccess && !h.empty())
       e = cudaMemcpy(h.data(), dptr, h.size() * sizeof(double), cudaMemcpyDeviceToHost);
   };
   get(lv, s->d.lv);
-  get(uv, s->d.uv);
-  get(ov, s->d.ov);
+  get(rv, s->d.rv);
   get(dg, s->d.dg);
   if (e != cudaSuccess) return sfail(s, DF_ERR_CUDA, "export: %s", cudaGetErrorString(e));
   int64_t k = 0;
@@ -826,8 +802,7 @@ df_status df_solver_export_csr(df_solver* s, int64_t* row_ptr, int32_t* col, dou
     row.clear();
     row.emplace_back((int32_t)r, dg[r]);
     for (int32_t j = s->h_lrp[r]; j < s->h_lrp[r + 1]; ++j) row.emplace_back(base + s->h_lc[j], lv[j]);
-    for (int32_t j = s->h_urp[r]; j < s->h_urp[r + 1]; ++j) row.emplace_back(base + s->h_uc[j], uv[j]);
-    for (int32_t j = s->h_orp[r]; j < s->h_orp[r + 1]; ++j) row.emplace_back(s->h_oc[j], ov[j]);
+    for (int32_t j = s->h_rrp[r]; j < s->h_rrp[r + 1]; ++j) row.emplace_back(s->h_rc[j], rv[j]);
     std::sort(row.begin(), row.end(),
               [](const std::pair<int32_t, double>& a, const std::pair<int32_t, double>& b) {
                 return a.first < b.first;
