@@ -273,4 +273,40 @@ cudaError_t prepare_tc(const TcLayer& L);
 int tc_stages(int BN, int out_kind, bool pair = false);
 int tc_epi_warps_per_quarter();
 
+// ---- FP32 layers on the tensor cores (mlp_split.cu) ----
+// Operands are three BF16 planes of an FP32 matrix: plane p at base + p * plane elements, rows of ld
+// elements (ld a multiple of 8).
+struct SplitLayer {
+  CUtensorMap tmA;         // activations [3][rows][K], box {64, 128, 1}
+  CUtensorMap tmW[2];      // weights [3][N][K], a map per tiling (mlp_split.cu)
+  CUtensorMap tmO;         // output: BF16 planes or FP32, box {32, 32, 1}
+  CUtensorMap tmG;         // GELU'(z) FP32 (mode 1)
+  int N = 0, K = 0;
+  int tw[2] = {0, 0};      // tile width of each tiling
+  const void* A = nullptr;
+  int64_t lda = 0, a_plane = 0;
+  const void* W = nullptr;
+  int64_t ldw = 0, w_plane = 0;
+  int64_t o_plane = 0;
+  const float* bias = nullptr;   // [N], zero padded to 32
+  bool planes = true;      // output as planes (hidden layers) or FP32
+  bool gelu = true;
+  const float4* gtab = nullptr;  // tabulated GELU or NULL for the tanh form
+  int mode = 0;            // 0 plain, 1 also store GELU'(z) to g, 2 scale rows by g[row / ntan]
+  float* g = nullptr;
+  int64_t ldg = 0;
+  int ntan = 1;
+  int ksplit = 1;          // split-K partial products (FP32 output), as TcLayer
+  int64_t split_rows = 0;
+};
+// Encodes L's tensor maps (set the other fields first): A has a_rows rows per plane, the output
+// buffer o_rows rows of pitch ldo; G (mode 1: written, mode 2: read) has pitch L.ldg.
+bool split_encode(SplitLayer& L, int64_t a_rows, void* out, int64_t o_rows, int64_t ldo, float* G,
+                  char* err, size_t errlen);
+cudaError_t prepare_split(const SplitLayer& L);
+cudaError_t launch_split(const SplitLayer& L, const RowMap& rows, int num_sms, int* err, cudaStream_t st);
+// Planes of the valid rows of `in` (cols columns, zero padded to ldo).
+cudaError_t launch_split_rows(const RowMap& rows, int cols, const float* in, int64_t ldi, void* out,
+                              int64_t ldo, int64_t plane, int num_sms, cudaStream_t st);
+
 }  // namespace dfgb

@@ -133,7 +133,9 @@ void free_state(df_state* s) {
   for (auto p : s->W32) f(p);
   for (auto p : s->bias) f(p);
   for (auto p : s->Wlp) f(p);
+  for (auto p : s->Wsp) f(p);
   for (auto p : s->col_scale) f(p);
+  f(s->xs);
   f(s->x); f(s->act[0]); f(s->act[1]); f(s->O); f(s->h0); f(s->rho_row); f(s->rstat);
   f(s->idx); f(s->cscr); f(s->vjpJ); f(s->vjpT);
   for (int b = 0; b < 2; ++b) {
@@ -168,11 +170,18 @@ int prof_family(df_state* s, const char* name) {
   return (int)s->prof_names.size() - 1;
 }
 
-// The network layers a6-a7 on rows of the batch buffers: x -> act -> ... -> O.
-df_status run_mlp(df_state* s, const RowMap& rm, cudaStream_t st) {
+// The network layers a6-a7 on rows of the batch buffers: x -> act -> ... -> O. An FP32 network reads
+// its input rows from xin (pitch ldin), by default the state's own x.
+df_status run_mlp(df_state* s, const RowMap& rm, cudaStream_t st, const float* xin, int64_t ldin) {
   cudaError_t e = cudaSuccess;
   static const char* kLayer[8] = {"layer0", "layer1", "layer2", "layer3",
                                   "layer4", "layer5", "layer6", "layer7"};
+  if (s->precision == DF_FP32) {
+    ProfScope ps(s, "input_planes", st);
+    e = launch_split_rows(rm, s->K0, xin ? xin : (const float*)s->x, xin ? ldin : s->ldx, s->xs,
+                          s->ldxs, s->cap * s->ldxs, s->num_sms, st);
+    if (e != cudaSuccess) return cuda_fail(s, e, "input planes");
+  }
   int l0 = 0;
   if (s->fuse01) {
     ProfScope ps(s, "layer0+1", st);
@@ -181,19 +190,9 @@ df_status run_mlp(df_state* s, const RowMap& rm, cudaStream_t st) {
     l0 = 2;
   }
   for (int l = l0; l < s->L; ++l) {
-    const bool last = l == s->L - 1;
     ProfScope ps(s, kLayer[l], st);
-    if (s->precision == DF_FP32) {
-      const float* A = (l == 0) ? (const float*)s->x : (const float*)s->act[(l - 1) & 1];
-      const int64_t lda = (l == 0) ? s->ldx : s->act_ld[(l - 1) & 1];
-      float* Cout = last ? s->O : (float*)s->act[l & 1];
-      const int64_t ldc = last ? s->ldo : s->act_ld[l & 1];
-      e = launch_sgemm_bias_act(rm, s->widths[l + 1], s->Kp8[l], A, lda, s->W32[l], s->Kp8[l],
-                                s->bias[l], Cout, ldc, !last, s->num_sms, st, 0, nullptr, 0, 1,
-                                last ? nullptr : s->d_gtab);
-    } else {
-      e = launch_tc_gemm(s->tcl[l], rm, s->num_sms, s->d_err, st);
-    }
+    if (s->precision == DF_FP32) e = launch_split(s->spl[l], rm, s->num_sms, s->d_err, st);
+    else e = launch_tc_gemm(s->tcl[l], rm, s->num_sms, s->d_err, st);
     if (e != cudaSuccess) return cuda_fail(s, e, "network layer launch");
   }
   return DF_OK;
@@ -563,6 +562,12 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
       CK(cudaMemcpy(d, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice), "copy");
       s->W32.push_back(d);
       s->Kp8.push_back(kp);
+      const int64_t kp16 = round_up(Kl, 16);
+      void* pl = nullptr;
+      CK(cudaMalloc(&pl, sizeof(__nv_bfloat16) * 3 * (size_t)Nl * kp16), "weight planes");
+      s->Wsp.push_back(pl);
+      CK(launch_split_rows(RowMap{nullptr, nullptr, 0, Nl}, Kl, d, kp, pl, kp16, Nl * kp16, s->num_sms,
+                           nullptr), "weight planes");
     } else {
       const int kp = (int)round_up(Kl, 16);
       void* d = nullptr;
@@ -608,10 +613,17 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
   int64_t wmax[2] = {8, 8};
   for (int l = 0; l + 1 < L; ++l)
     wmax[l & 1] = std::max<int64_t>(wmax[l & 1], round_up(s->widths[l + 1], lp ? 16 : 8));
+  // (an FP32 network's input and activations are three BF16 planes, mlp_split.cu)
   for (int b = 0; b < 2; ++b) {
-    s->act_ld[b] = wmax[b];
-    CK(cudaMalloc(&s->act[b], eb * (size_t)s->cap * wmax[b]), "activations");
-    CK(cudaMemset(s->act[b], 0, eb * (size_t)s->cap * wmax[b]), "memset");
+    s->act_ld[b] = lp ? wmax[b] : round_up(wmax[b], 16);
+    const size_t bytes = (lp ? eb : 6) * (size_t)s->cap * s->act_ld[b];
+    CK(cudaMalloc(&s->act[b], bytes), "activations");
+    CK(cudaMemset(s->act[b], 0, bytes), "memset");
+  }
+  if (!lp) {
+    s->ldxs = round_up(s->K0, 16);
+    CK(cudaMalloc(&s->xs, 6 * (size_t)s->cap * s->ldxs), "input planes");
+    CK(cudaMemset(s->xs, 0, 6 * (size_t)s->cap * s->ldxs), "memset");
   }
   s->ldo = round_up(nout, 8);
   CK(dalloc(&s->O, (size_t)s->cap * s->ldo), "network output");
@@ -619,6 +631,34 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
   CK(dalloc(&s->rho_row, (size_t)s->cap), "rho");
   CK(dalloc(&s->rstat, (size_t)s->cap), "row status");
 
+  if (!lp) {
+    char emsg[256];
+    for (int l = 0; l < L; ++l) {
+      const bool last = l == L - 1;
+      SplitLayer S;
+      S.N = s->widths[l + 1];
+      S.K = s->widths[l];
+      S.A = l == 0 ? s->xs : s->act[(l - 1) & 1];
+      S.lda = l == 0 ? s->ldxs : s->act_ld[(l - 1) & 1];
+      S.a_plane = s->cap * S.lda;
+      S.W = s->Wsp[l];
+      S.ldw = round_up(S.K, 16);
+      S.w_plane = S.N * S.ldw;
+      S.bias = s->bias[l];
+      S.planes = S.gelu = !last;
+      S.gtab = last ? nullptr : s->d_gtab;
+      const int64_t ldo = last ? s->ldo : s->act_ld[l & 1];
+      S.o_plane = s->cap * ldo;
+      if (!split_encode(S, s->cap, last ? (void*)s->O : s->act[l & 1], s->cap, ldo, nullptr, emsg,
+                        sizeof emsg)) {
+        free_state(s);
+        delete s;
+        return fail(nullptr, DF_ERR_CUDA, "%s", emsg);
+      }
+      CK(prepare_split(S), "kernel attributes");
+      s->spl.push_back(S);
+    }
+  }
   if (lp) {
     char emsg[256];
     for (int l = 0; l < L; ++l) {
@@ -811,7 +851,7 @@ df_status run_step(df_state* s, int64_t n_cells, double dt, double* T, const dou
                          src ? s->rho_row : nullptr);
     }
     if (e != cudaSuccess) return cuda_fail(s, e, "eos_pre launch");
-    if ((rc = run_mlp(s, rm, st)) != DF_OK) return rc;
+    if ((rc = run_mlp(s, rm, st, nullptr, 0)) != DF_OK) return rc;
     {
       ProfScope ps(s, "eos_post", st);
       e = launch_eos_post(s->P, rm, s->O, s->ldo, s->h0, T, p, Y, ldY, s->rstat, cell_status, st,
@@ -1521,13 +1561,12 @@ df_status df_mlp_forward(df_state* s, int64_t n_rows, const float* x, float* O, 
   const float xs = s->precision == DF_FP8_E4M3 ? s->act_scale[0] : 1.0f;
   for (int64_t r0 = 0; r0 < n_rows; r0 += s->cap) {
     const int64_t rows = std::min<int64_t>(s->cap, n_rows - r0);
-    const int64_t total = rows * s->ldx;
-    const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)s->num_sms * 16);
-    cast_rows_kernel<<<g, 256, 0, st>>>(rows, s->K0, x + r0 * s->K0, s->K0, s->x, s->ldx, xk, xs);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(s, e, "input cast");
     const RowMap rm{nullptr, nullptr, 0, rows};
-    df_status rc = run_mlp(s, rm, st);
+    cudaError_t e = cudaSuccess;
+    if (s->precision != DF_FP32)   // an FP32 network splits its planes from the caller's rows
+      e = launch_cast_rows(rows, s->K0, x + r0 * s->K0, s->K0, s->x, s->ldx, xk, xs, s->num_sms, st);
+    if (e != cudaSuccess) return cuda_fail(s, e, "input cast");
+    df_status rc = run_mlp(s, rm, st, x + r0 * s->K0, s->K0);
     if (rc != DF_OK) return rc;
     e = cudaMemcpy2DAsync(O + r0 * s->nout, sizeof(float) * s->nout, s->O, sizeof(float) * s->ldo,
                           sizeof(float) * s->nout, (size_t)rows, cudaMemcpyDeviceToDevice, st);
@@ -1558,7 +1597,7 @@ df_status df_propnet_infer(df_state* s, int64_t n_cells, const double* h, const 
     }
     if (e != cudaSuccess) return cuda_fail(s, e, "property-network inputs");
     const RowMap rm{nullptr, nullptr, 0, rows};
-    df_status rc = run_mlp(s, rm, st);
+    df_status rc = run_mlp(s, rm, st, nullptr, 0);
     if (rc != DF_OK) return rc;
     {
       ProfScope ps(s, "prop_outputs", st);

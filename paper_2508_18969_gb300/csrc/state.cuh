@@ -82,6 +82,10 @@ struct df_state {
   int64_t* d_iters = nullptr;            // Newton iterations of the last step
   std::vector<float*> W32;               // FP32 weights, [N x Kp8] zero padded (SIMT)
   std::vector<int> Kp8;
+  std::vector<void*> Wsp;                // FP32 network: weights as BF16 planes [3][N][Kp16]
+  std::vector<SplitLayer> spl;           // FP32 network: its layers (mlp_split.cu)
+  void* xs = nullptr;                    // FP32 network: input rows as planes [3][cap][ldxs]
+  int64_t ldxs = 0;
   std::vector<float*> bias;
   std::vector<void*> Wlp;                // BF16 / FP8 weights [N x Kp16]
   std::vector<float*> col_scale;         // FP8 dequantisation scale per output channel

@@ -112,6 +112,10 @@ cudaError_t publish_all(df_state* s, cudaStream_t st) {
                                    bf16 ? nullptr : s->W32[l], s->Kp8[l],
                                    bf16 ? s->Wlp[l] : nullptr, s->Kp8[l], t->WT[l], t->ldt[l],
                                    bf16, st);
+    if (e == cudaSuccess && !bf16)   // the planes the inference layers read
+      e = launch_split_rows(RowMap{nullptr, nullptr, 0, s->widths[l + 1]}, s->widths[l], s->W32[l],
+                            s->Kp8[l], s->Wsp[l], round_up(s->widths[l], 16),
+                            s->widths[l + 1] * round_up(s->widths[l], 16), s->num_sms, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
