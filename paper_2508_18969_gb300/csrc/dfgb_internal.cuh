@@ -167,7 +167,7 @@ cudaError_t launch_loss_grad(int64_t B, int n, const float* O, int64_t ldo, cons
 // multiple of 64, ldi and ldo even. With colsum (and scratch of scratch_floats >= C floats),
 // also colsum[c] = sum_r in[r][c], FP32, in a fixed order.
 cudaError_t launch_transpose(int64_t R, int64_t C, const void* in, int64_t ldi, void* out,
-                             int64_t ldo, int64_t Rpad, bool bf16, int num_sms, cudaStream_t st,
+                             int64_t ldo, int64_t Rpad, int num_sms, cudaStream_t st,
                              float* colsum = nullptr, float* scratch = nullptr,
                              int64_t scratch_floats = 0);
 // out[i] = sum_{s < splits} part[s * stride + i] (fixed order), i < count.
@@ -175,9 +175,12 @@ cudaError_t launch_sum_splits(int splits, int64_t count, int64_t stride, const f
                               float* out, cudaStream_t st);
 cudaError_t launch_adam(int64_t count, float* w, float* m, float* v, const float* g, float lr,
                         float b1, float b2, float eps, float c1, float c2, cudaStream_t st);
-cudaError_t launch_publish(int N, int K, const float* Wm, int64_t ldm, float* W32, int64_t ld32,
-                           void* Wb, int64_t ldb, void* WT, int64_t ldt, bool WT_bf16,
-                           cudaStream_t st);
+// out[c] = sum of column c < C of `planes` (1 or 3) stacked BF16 matrices [R x ld], FP32, fixed order.
+cudaError_t launch_colsum(int64_t R, int64_t C, const void* in, int64_t ld, int planes, int64_t plane,
+                          float* out, int num_sms, float* scratch, int64_t scratch_floats,
+                          cudaStream_t st);
+cudaError_t launch_publish(int N, int K, const float* Wm, int64_t ldm, float* W32, int64_t ld32, void* Wb,
+                           int64_t ldb, void* WT, int64_t ldt, cudaStream_t st);
 
 // ---- launchers (compact.cu) ----
 constexpr int64_t kCompactChunk = 4096;   // cells per block of the compaction kernels
@@ -287,6 +290,9 @@ struct SplitLayer {
   int64_t lda = 0, a_plane = 0;
   const void* W = nullptr;
   int64_t ldw = 0, w_plane = 0;
+  // MN-major operands: bit 0, A holds its K reduction rows of M columns; bit 1, W its K rows of N columns
+  int tr = 0;
+  int M = 0;
   int64_t o_plane = 0;
   const float* bias = nullptr;   // [N], zero padded to 32
   bool planes = true;      // output as planes (hidden layers) or FP32

@@ -1,9 +1,9 @@
-// a6-a7 in plain FP32 on the CUDA cores (no tensor cores): the "plain FP32 step" the
-// tensor-core paths are measured against. Register-tiled SGEMM, 128x128 block tile, BK = 8,
-// 256 threads each owning an 8x8 sub-tile, double-buffered shared memory, persistent over
-// the tiles of the (device-counted) valid rows, with bias + tanh-GELU (Sec. 3.3.2) fused
-// into the epilogue. GELU uses the accurate tanhf here, since this path's error budget is
-// the FP32 one.
+// Network layers as chains of FP32 FMAs on the CUDA cores, for the FP32 passes whose results leave in
+// FP64 and are held to 1e-9 of earlier versions' values, which no other order of summation keeps: the
+// Jacobian of the step and property-network inference (every other FP32 pass runs on the tensor cores,
+// mlp_split.cu). Register-tiled SGEMM, 128x128 block tile, BK = 8, 256 threads each owning an 8x8
+// sub-tile, double-buffered shared memory, persistent over the tiles of the (device-counted) valid
+// rows, with bias + tanh-GELU (Sec. 3.3.2, the accurate tanhf) fused into the epilogue.
 #include "dfgb_internal.cuh"
 
 namespace dfgb {

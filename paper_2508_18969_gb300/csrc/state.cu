@@ -136,6 +136,7 @@ void free_state(df_state* s) {
   for (auto p : s->Wsp) f(p);
   for (auto p : s->col_scale) f(p);
   f(s->xs);
+  if (s->act32_own) { f(s->act32[0]); f(s->act32[1]); }
   f(s->x); f(s->act[0]); f(s->act[1]); f(s->O); f(s->h0); f(s->rho_row); f(s->rstat);
   f(s->idx); f(s->cscr); f(s->vjpJ); f(s->vjpT);
   for (int b = 0; b < 2; ++b) {
@@ -168,6 +169,26 @@ int prof_family(df_state* s, const char* name) {
   s->prof_launches.push_back(0);
   s->prof_ms.push_back(0.0);
   return (int)s->prof_names.size() - 1;
+}
+
+// The layers of an FP32 property network (df_propnet_infer) as chains of FP32 FMAs: its outputs leave in
+// FP64, and callers hold them to 1e-9 of the values of earlier versions, which a sum in another order
+// would not keep.
+static df_status run_propnet_fp32(df_state* s, const RowMap& rm, cudaStream_t st) {
+  static const char* kLayer[8] = {"layer0", "layer1", "layer2", "layer3",
+                                  "layer4", "layer5", "layer6", "layer7"};
+  for (int l = 0; l < s->L; ++l) {
+    const bool last = l == s->L - 1;
+    ProfScope ps(s, kLayer[l], st);
+    const float* A = l == 0 ? (const float*)s->x : s->act32[(l - 1) & 1];
+    const int64_t lda = l == 0 ? s->ldx : s->act32_ld[(l - 1) & 1];
+    const cudaError_t e = launch_sgemm_bias_act(
+        rm, s->widths[l + 1], s->Kp8[l], A, lda, s->W32[l], s->Kp8[l], s->bias[l],
+        last ? s->O : s->act32[l & 1], last ? s->ldo : s->act32_ld[l & 1], !last, s->num_sms, st, 0,
+        nullptr, 0, 1, last ? nullptr : s->d_gtab);
+    if (e != cudaSuccess) return cuda_fail(s, e, "network layer launch");
+  }
+  return DF_OK;
 }
 
 // The network layers a6-a7 on rows of the batch buffers: x -> act -> ... -> O. An FP32 network reads
@@ -618,12 +639,25 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
     s->act_ld[b] = lp ? wmax[b] : round_up(wmax[b], 16);
     const size_t bytes = (lp ? eb : 6) * (size_t)s->cap * s->act_ld[b];
     CK(cudaMalloc(&s->act[b], bytes), "activations");
-    CK(cudaMemset(s->act[b], 0, bytes), "memset");
+    if (lp) CK(cudaMemset(s->act[b], 0, bytes), "memset");   // (nothing reads the planes' pads)
+  }
+  // The FP32 activations of a property network share the planes' memory, unless a hidden width is not
+  // a multiple of 8: the FMA GEMM then reads pad columns (times zero weights), which must stay zero.
+  bool pads = false;
+  for (int l = 1; l < L; ++l) pads = pads || (s->widths[l] & 7);
+  for (int b = 0; !lp && netonly && b < 2; ++b) {
+    s->act32_ld[b] = wmax[b];
+    s->act32_own = pads;
+    if (!pads) {
+      s->act32[b] = (float*)s->act[b];
+      continue;
+    }
+    CK(dalloc(&s->act32[b], (size_t)s->cap * wmax[b]), "activations");
+    CK(cudaMemset(s->act32[b], 0, sizeof(float) * (size_t)s->cap * wmax[b]), "memset");
   }
   if (!lp) {
     s->ldxs = round_up(s->K0, 16);
     CK(cudaMalloc(&s->xs, 6 * (size_t)s->cap * s->ldxs), "input planes");
-    CK(cudaMemset(s->xs, 0, 6 * (size_t)s->cap * s->ldxs), "memset");
   }
   s->ldo = round_up(nout, 8);
   CK(dalloc(&s->O, (size_t)s->cap * s->ldo), "network output");
@@ -1597,7 +1631,7 @@ df_status df_propnet_infer(df_state* s, int64_t n_cells, const double* h, const 
     }
     if (e != cudaSuccess) return cuda_fail(s, e, "property-network inputs");
     const RowMap rm{nullptr, nullptr, 0, rows};
-    df_status rc = run_mlp(s, rm, st, nullptr, 0);
+    df_status rc = s->precision == DF_FP32 ? run_propnet_fp32(s, rm, st) : run_mlp(s, rm, st, nullptr, 0);
     if (rc != DF_OK) return rc;
     {
       ProfScope ps(s, "prop_outputs", st);

@@ -86,6 +86,9 @@ struct df_state {
   std::vector<SplitLayer> spl;           // FP32 network: its layers (mlp_split.cu)
   void* xs = nullptr;                    // FP32 network: input rows as planes [3][cap][ldxs]
   int64_t ldxs = 0;
+  float* act32[2] = {nullptr, nullptr};  // FP32 property network: activations of df_propnet_infer
+  int64_t act32_ld[2] = {0, 0};
+  bool act32_own = false;                // not in the planes' memory
   std::vector<float*> bias;
   std::vector<void*> Wlp;                // BF16 / FP8 weights [N x Kp16]
   std::vector<float*> col_scale;         // FP8 dequantisation scale per output channel

@@ -83,6 +83,17 @@ __device__ constexpr uint32_t idesc() {
          ((uint32_t)(MROWS >> 4) << 24);
 }
 
+// MN-major operands (the product's row or column index runs along memory): instruction-descriptor
+// bits, and the descriptor of a 128-byte-swizzled tile made of boxes of 64 columns x 64 rows (k) of
+// BF16, 128 bytes a row: 8-row groups 1024 B apart (stride byte offset), the next 64 columns one box
+// (leading byte offset) further.
+constexpr uint32_t kIdescMnA = 1u << 15, kIdescMnB = 1u << 16;
+constexpr int kMnBox = 64 * 128;
+__device__ __forceinline__ uint64_t desc_mn128(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(kMnBox >> 4) << 16) |
+         ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
 template <bool FP8>
 __device__ __forceinline__ void mma_issue(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t id,
                                           uint32_t accum) {

@@ -107,16 +107,6 @@ template <> struct Pair<__nv_bfloat16> {
   static __device__ __forceinline__ __nv_bfloat16 first(V v) { return __low2bfloat16(v); }
   static __device__ __forceinline__ __nv_bfloat16 second(V v) { return __high2bfloat16(v); }
 };
-template <> struct Pair<float> {
-  using V = float2;
-  static __device__ __forceinline__ float lo(V v) { return v.x; }
-  static __device__ __forceinline__ float hi(V v) { return v.y; }
-  static __device__ __forceinline__ V make(float a, float b) { return make_float2(a, b); }
-  static __device__ __forceinline__ V zero() { return make_float2(0.0f, 0.0f); }
-  static __device__ __forceinline__ float first(V v) { return v.x; }
-  static __device__ __forceinline__ float second(V v) { return v.y; }
-};
-
 constexpr int kTp = 64;   // transpose tile: 64 rows x 64 columns, 256 threads
 
 // out[c][r] = in[r][c] for c < C, r < Rpad (zero for R <= r < Rpad). Block (x, y) takes the
@@ -186,6 +176,57 @@ __global__ void __launch_bounds__(256, 6) transpose_kernel(int64_t R, int64_t C,
   }
 }
 
+// part[y * C + c] = sum over the rows y, y + gridDim.y, ... of column c of a matrix of NP BF16 planes
+// (value = sum of the planes), FP32, in a fixed order: the bias gradient. Block x takes 256 columns, a
+// warp one row at a time (512 contiguous bytes a plane), eight columns a lane.
+template <int NP>
+__global__ void __launch_bounds__(256) colsum_kernel(int64_t R, int64_t C,
+                                                     const __nv_bfloat16* __restrict__ in, int64_t ld,
+                                                     int64_t plane, float* __restrict__ part) {
+  __shared__ float red[8][256];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t c = (int64_t)blockIdx.x * 256 + 8 * lane;
+  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (c < ld) {   // ld is a multiple of 8: whole 16-byte groups inside the row
+    const int64_t step = (int64_t)gridDim.y * 8;
+    constexpr int U = NP == 1 ? 4 : 2;   // rows in flight
+    for (int64_t r0 = blockIdx.y * 8 + w; r0 < R; r0 += U * step) {
+      uint4 q[U][NP];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+          q[u][p] = r0 + u * step < R
+                        ? *reinterpret_cast<const uint4*>(in + p * plane + (r0 + u * step) * ld + c)
+                        : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int p = NP - 1; p >= 0; --p) {
+          const uint32_t x[4] = {q[u][p].x, q[u][p].y, q[u][p].z, q[u][p].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {   // BF16 is the upper half of FP32
+            v[2 * e] += __uint_as_float(x[e] << 16);
+            v[2 * e + 1] += __uint_as_float(x[e] & 0xFFFF0000u);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] += v[e];
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) red[w][8 * lane + e] = s[e];
+  __syncthreads();
+  const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (col < C) {
+    float t = 0.0f;
+    for (int k = 0; k < 8; ++k) t += red[k][threadIdx.x];
+    part[(int64_t)blockIdx.y * C + col] = t;
+  }
+}
+
 // out[i] = sum_{s < splits} part[s * stride + i], in order of s.
 __global__ void split_sum_kernel(int splits, int64_t count, int64_t stride,
                                  const float* __restrict__ part, float* __restrict__ out) {
@@ -226,22 +267,19 @@ __global__ void adam_kernel(int64_t count, float* __restrict__ w, float* __restr
   }
 }
 
-// Working copies of a master weight matrix Wm [N x ldm]: FP32 [N x ld32] (SIMT), BF16
-// [N x ldb] (tensor cores), and the transposed copy [K x ldt] (FP32 or BF16) for the input
-// gradient GEMM. Any destination may be NULL. Pads stay as allocated (zero).
+// Working copies of a master weight matrix Wm [N x ldm]: FP32 [N x ld32], or BF16 [N x ldb] and the
+// transposed BF16 copy [K x ldt] for the input gradient GEMM. Any destination may be NULL. Pads stay as
+// allocated (zero).
 __global__ void publish_kernel(int N, int K, const float* __restrict__ Wm, int64_t ldm, float* W32,
-                               int64_t ld32, __nv_bfloat16* Wb, int64_t ldb, void* WT, int64_t ldt,
-                               int WT_bf16) {
+                               int64_t ld32, __nv_bfloat16* Wb, int64_t ldb, __nv_bfloat16* WT,
+                               int64_t ldt) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * K;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int r = (int)(e / K), c = (int)(e % K);
     const float w = Wm[(int64_t)r * ldm + c];
     if (W32) W32[(int64_t)r * ld32 + c] = w;
     if (Wb) Wb[(int64_t)r * ldb + c] = __float2bfloat16_rn(w);
-    if (WT) {
-      if (WT_bf16) ((__nv_bfloat16*)WT)[(int64_t)c * ldt + r] = __float2bfloat16_rn(w);
-      else ((float*)WT)[(int64_t)c * ldt + r] = w;
-    }
+    if (WT) WT[(int64_t)c * ldt + r] = __float2bfloat16_rn(w);
   }
 }
 
@@ -278,8 +316,8 @@ cudaError_t launch_loss_grad(int64_t B, int n, const float* O, int64_t ldo, cons
 }
 
 cudaError_t launch_transpose(int64_t R, int64_t C, const void* in, int64_t ldi, void* out,
-                             int64_t ldo, int64_t Rpad, bool bf16, int num_sms, cudaStream_t st,
-                             float* colsum, float* scratch, int64_t scratch_floats) {
+                             int64_t ldo, int64_t Rpad, int num_sms, cudaStream_t st, float* colsum,
+                             float* scratch, int64_t scratch_floats) {
   if (C <= 0) return cudaSuccess;
   if (Rpad <= 0 || (Rpad % kTp) || (ldi & 1) || (ldo & 1)) {
     if (colsum && Rpad <= 0) return cudaMemsetAsync(colsum, 0, sizeof(float) * C, st);
@@ -296,14 +334,25 @@ cudaError_t launch_transpose(int64_t R, int64_t C, const void* in, int64_t ldi, 
   }
   const dim3 grid((unsigned)strips, (unsigned)groups);
   float* part = colsum ? scratch : nullptr;
-  if (bf16)
-    transpose_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
-        R, C, (const __nv_bfloat16*)in, ldi, (__nv_bfloat16*)out, ldo, Rpad, part);
-  else
-    transpose_kernel<float><<<grid, 256, 0, st>>>(R, C, (const float*)in, ldi, (float*)out, ldo,
-                                                  Rpad, part);
+  transpose_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
+      R, C, (const __nv_bfloat16*)in, ldi, (__nv_bfloat16*)out, ldo, Rpad, part);
   if (colsum)
     sum_parts_warp_kernel<<<(unsigned)((C + 7) / 8), 256, 0, st>>>((int)groups, (int)C, scratch, colsum);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_colsum(int64_t R, int64_t C, const void* in, int64_t ld, int planes, int64_t plane,
+                          float* out, int num_sms, float* scratch, int64_t scratch_floats,
+                          cudaStream_t st) {
+  if (C <= 0) return cudaSuccess;
+  if ((ld & 7) || scratch_floats < C) return cudaErrorInvalidValue;
+  const int64_t strips = (C + 255) / 256;
+  int64_t groups = std::max<int64_t>(1, std::min<int64_t>((R + 63) / 64, (4LL * std::max(num_sms, 1) + strips - 1) / strips));
+  groups = std::min<int64_t>(groups, scratch_floats / C);
+  const dim3 grid((unsigned)strips, (unsigned)groups);
+  if (planes == 1) colsum_kernel<1><<<grid, 256, 0, st>>>(R, C, (const __nv_bfloat16*)in, ld, plane, scratch);
+  else colsum_kernel<3><<<grid, 256, 0, st>>>(R, C, (const __nv_bfloat16*)in, ld, plane, scratch);
+  sum_parts_warp_kernel<<<(unsigned)((C + 7) / 8), 256, 0, st>>>((int)groups, (int)C, scratch, out);
   return cudaGetLastError();
 }
 
@@ -321,11 +370,10 @@ cudaError_t launch_adam(int64_t count, float* w, float* m, float* v, const float
   return cudaGetLastError();
 }
 
-cudaError_t launch_publish(int N, int K, const float* Wm, int64_t ldm, float* W32, int64_t ld32,
-                           void* Wb, int64_t ldb, void* WT, int64_t ldt, bool WT_bf16,
-                           cudaStream_t st) {
-  publish_kernel<<<blocks_for((int64_t)N * K), kThreads, 0, st>>>(
-      N, K, Wm, ldm, W32, ld32, (__nv_bfloat16*)Wb, ldb, WT, ldt, WT_bf16 ? 1 : 0);
+cudaError_t launch_publish(int N, int K, const float* Wm, int64_t ldm, float* W32, int64_t ld32, void* Wb,
+                           int64_t ldb, void* WT, int64_t ldt, cudaStream_t st) {
+  publish_kernel<<<blocks_for((int64_t)N * K), kThreads, 0, st>>>(N, K, Wm, ldm, W32, ld32, (__nv_bfloat16*)Wb,
+                                                                  ldb, (__nv_bfloat16*)WT, ldt);
   return cudaGetLastError();
 }
 

@@ -4,12 +4,12 @@
 // SIMT path, BF16 for the tensor-core path) the reaction step reads in place.
 //
 // Backward pass of layer l (Z_l = H_{l-1} W_l^T + b_l, H_l = GELU(Z_l), linear read-out):
-//   dW_l = dZ_l^T H_{l-1}   (GEMM over the batch: both operands transposed first, so the
-//                            batch becomes the contiguous reduction dimension)
+//   dW_l = dZ_l^T H_{l-1}   (GEMM over the batch, split-K; BF16: both operands transposed first, so
+//                            the batch becomes the contiguous reduction dimension; FP32: both read
+//                            along their columns by the tensor core)
 //   db_l = column sums of dZ_l
-//   dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})   (GEMM against the transposed weight copy, the
-//                                             GELU' factor applied in its epilogue)
-// Every step runs in the kernels of train.cu, mlp_simt.cu and mlp_tc.cu.
+//   dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})   (the GELU' factor applied in the GEMM's epilogue)
+// Every step runs in the kernels of train.cu, mlp_split.cu (FP32) and mlp_tc.cu (BF16).
 #include "state.cuh"
 #include "../../include/df_propnet.h"
 
@@ -23,7 +23,7 @@ struct Trn {
   std::vector<int64_t> ldw;              // row pitch of the [N_l x K_l] FP32 matrices
   std::vector<float*> Wm, mW, vW, dW;    // master weights, Adam moments, gradients
   std::vector<float*> mb, vb, db;        // bias moments and gradients (master = state bias)
-  std::vector<void*> WT;                 // transposed working weights [K_l x ldt_l]
+  std::vector<void*> WT;                 // BF16: transposed working weights [K_l x ldt_l]
   std::vector<int64_t> ldt;
   int64_t t = 0;                         // Adam steps taken
   int64_t host_wver = 0;                 // weight version of the state's host copies
@@ -35,9 +35,12 @@ struct Trn {
   int64_t B = 0, Bp = 0;                 // Bp = B rounded up to 64 (transposed length)
   int64_t ldT = 0;                       // pitch of the transposes: Bp + 64, so that rows of a
                                          // transpose are not a power of two apart in memory
-  void* x = nullptr;
+  void* x = nullptr;                     // input rows, BF16 or FP32
   int64_t ldx = 0;
-  std::vector<void*> H, G, dZ;           // hidden outputs, GELU'(Z), output gradients
+  void* xp = nullptr;                    // FP32: the input rows' planes
+  float* dZ32 = nullptr;                 // FP32: gradient of the network output before its split
+  std::vector<void*> H, G, dZ;           // hidden outputs, GELU'(Z), output gradients; an FP32 network
+                                         // holds H and dZ as three BF16 planes, G in FP32
   std::vector<int64_t> ldh, ldg, ldz;
   float* O = nullptr;
   float* Oh = nullptr;
@@ -49,7 +52,9 @@ struct Trn {
   int64_t lddx = 0;
   double* h0 = nullptr;
   int32_t* rstat = nullptr;
-  std::vector<TcLayer> fwd, dgrad, wgrad;  // tensor-core layers (BF16 states)
+  std::vector<TcLayer> fwd, dgrad, wgrad;  // BF16 states
+  std::vector<SplitLayer> sfwd, sdg, swg;  // FP32 states
+  int64_t wg_rows = -1;                  // batch rows the swg maps are encoded for
   int64_t rows = -1;                     // rows of the last training forward pass
 };
 
@@ -62,7 +67,7 @@ void free_trn(Trn* t) {
     for (float* p : *v) f(p);
   for (void* p : t->WT) f(p);
   f(t->loss); f(t->scratch); f(t->zero_bias);
-  f(t->x); f(t->O); f(t->Oh); f(t->ZT); f(t->HT); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
+  f(t->x); f(t->xp); f(t->dZ32); f(t->O); f(t->Oh); f(t->ZT); f(t->HT); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
   for (auto v : {&t->H, &t->G, &t->dZ})
     for (void* p : *v) f(p);
   delete t;
@@ -89,36 +94,37 @@ int wgrad_splits(int64_t tiles, int kblocks, int num_sms) {
 
 void free_batch(Trn* t) {
   auto f = [](void* p) { if (p) cudaFree(p); };
-  f(t->x); f(t->O); f(t->Oh); f(t->ZT); f(t->HT); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
+  f(t->x); f(t->xp); f(t->dZ32); f(t->O); f(t->Oh); f(t->ZT); f(t->HT); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
   for (auto v : {&t->H, &t->G, &t->dZ})
     for (void* p : *v) f(p);
-  t->x = t->ZT = t->HT = nullptr;
-  t->O = t->Oh = t->dX = t->dWp = nullptr;
+  t->x = t->xp = t->ZT = t->HT = nullptr;
+  t->O = t->Oh = t->dX = t->dWp = t->dZ32 = nullptr;
   t->h0 = nullptr;
   t->rstat = nullptr;
   t->H.clear(); t->G.clear(); t->dZ.clear();
   t->ldh.clear(); t->ldg.clear(); t->ldz.clear();
   t->fwd.clear(); t->dgrad.clear(); t->wgrad.clear();
+  t->sfwd.clear(); t->sdg.clear(); t->swg.clear();
+  t->wg_rows = -1;
   t->B = t->Bp = t->ldT = 0;
   t->rows = -1;
 }
 
-// Writes the working copies (state FP32 or BF16 weights, transposed copies) from the masters.
+// Writes the working copies (FP32 weights and their planes; BF16 weights and their transposes) from
+// the masters.
 cudaError_t publish_all(df_state* s, cudaStream_t st) {
   Trn* t = s->trn;
   const bool bf16 = s->precision == DF_BF16;
-  for (int l = 0; l < s->L; ++l) {
-    cudaError_t e = launch_publish(s->widths[l + 1], s->widths[l], t->Wm[l], t->ldw[l],
-                                   bf16 ? nullptr : s->W32[l], s->Kp8[l],
-                                   bf16 ? s->Wlp[l] : nullptr, s->Kp8[l], t->WT[l], t->ldt[l],
-                                   bf16, st);
-    if (e == cudaSuccess && !bf16)   // the planes the inference layers read
-      e = launch_split_rows(RowMap{nullptr, nullptr, 0, s->widths[l + 1]}, s->widths[l], s->W32[l],
-                            s->Kp8[l], s->Wsp[l], round_up(s->widths[l], 16),
-                            s->widths[l + 1] * round_up(s->widths[l], 16), s->num_sms, st);
-    if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  for (int l = 0; l < s->L && e == cudaSuccess; ++l) {
+    const int N = s->widths[l + 1], K = s->widths[l];
+    e = launch_publish(N, K, t->Wm[l], t->ldw[l], bf16 ? nullptr : s->W32[l], s->Kp8[l],
+                       bf16 ? s->Wlp[l] : nullptr, s->Kp8[l], t->WT[l], t->ldt[l], st);
+    if (e == cudaSuccess && !bf16)
+      e = launch_split_rows(RowMap{nullptr, nullptr, 0, N}, K, t->Wm[l], t->ldw[l], s->Wsp[l],
+                            round_up(K, 16), N * round_up(K, 16), s->num_sms, st);
   }
-  return cudaSuccess;
+  return e;
 }
 
 // Masters from the state's host weights, zero moments, transposed working copies.
@@ -128,8 +134,6 @@ df_status ensure_params(df_state* s) {
   Trn* t = new Trn();
   s->trn = t;
   const bool bf16 = s->precision == DF_BF16;
-  const size_t eb = bf16 ? 2 : 4;
-  const int64_t al = bf16 ? 16 : 8;
   cudaError_t e = cudaSuccess;
   auto zalloc = [&](void** p, size_t bytes) {
     if (e != cudaSuccess) return;
@@ -157,9 +161,9 @@ df_status ensure_params(df_state* s) {
     zalloc((void**)&db, sizeof(float) * N);
     t->Wm.push_back(Wm); t->mW.push_back(mW); t->vW.push_back(vW); t->dW.push_back(dW);
     t->mb.push_back(mb); t->vb.push_back(vb); t->db.push_back(db);
-    const int64_t ldt = round_up(N, al);
+    const int64_t ldt = round_up(N, 16);
     void* WT = nullptr;
-    zalloc(&WT, eb * K * ldt);
+    if (bf16) zalloc(&WT, 2 * K * ldt);
     t->WT.push_back(WT);
     t->ldt.push_back(ldt);
     if (e == cudaSuccess)
@@ -192,8 +196,8 @@ df_status ensure_batch(df_state* s, int64_t B) {
   B = round_up(B, 128);
   const int L = s->L, K0 = s->K0;
   const bool bf16 = s->precision == DF_BF16;
-  const size_t eb = bf16 ? 2 : 4;
-  const int64_t al = bf16 ? 16 : 8;
+  const size_t eb = bf16 ? 2 : 6, gb = bf16 ? 2 : 4;   // bytes of an activation and of a GELU'(Z)
+  const int64_t al = 16;
   const int64_t Bp = round_up(B, 64);
   const int64_t ldT = Bp + 64;
   auto zalloc = [&](void** p, size_t bytes) {
@@ -202,7 +206,8 @@ df_status ensure_batch(df_state* s, int64_t B) {
     if (e == cudaSuccess) e = cudaMemset(*p, 0, bytes ? bytes : 1);
   };
   t->ldx = round_up(K0, al);
-  zalloc(&t->x, eb * B * t->ldx);
+  zalloc(&t->x, gb * B * t->ldx);
+  if (!bf16) zalloc(&t->xp, eb * B * t->ldx);
   int64_t nmax = 8, kmax = 8;
   for (int l = 0; l < L; ++l) {
     const int N = s->widths[l + 1];
@@ -212,7 +217,7 @@ df_status ensure_batch(df_state* s, int64_t B) {
     const int64_t ldh = round_up(N, al), ldg = round_up(N, 32), ldz = round_up(N, al);
     if (l < L - 1) {
       zalloc(&H, eb * B * ldh);
-      zalloc(&G, eb * B * ldg);
+      zalloc(&G, gb * B * ldg);
     }
     zalloc(&dZ, eb * B * ldz);
     t->H.push_back(H); t->G.push_back(G); t->dZ.push_back(dZ);
@@ -221,16 +226,18 @@ df_status ensure_batch(df_state* s, int64_t B) {
   t->ldo = round_up(s->nout, 8);
   zalloc((void**)&t->O, sizeof(float) * B * t->ldo);
   zalloc((void**)&t->Oh, sizeof(float) * B * t->ldo);
-  zalloc(&t->ZT, eb * nmax * ldT);
-  zalloc(&t->HT, eb * kmax * ldT);
+  if (bf16) {
+    zalloc(&t->ZT, eb * nmax * ldT);
+    zalloc(&t->HT, eb * kmax * ldT);
+  } else {
+    zalloc((void**)&t->dZ32, sizeof(float) * B * t->ldz[L - 1]);
+  }
   t->lddx = round_up(K0, 4);
   zalloc((void**)&t->dX, sizeof(float) * B * t->lddx);
-  if (bf16) {
-    int64_t wmaxp = 0;
-    for (int l = 0; l < L; ++l)
-      wmaxp = std::max<int64_t>(wmaxp, round_up(s->widths[l + 1], 128) * t->ldw[l]);
-    zalloc((void**)&t->dWp, sizeof(float) * kMaxSplit * wmaxp);
-  }
+  int64_t wmaxp = 0;
+  for (int l = 0; l < L; ++l)
+    wmaxp = std::max<int64_t>(wmaxp, round_up(s->widths[l + 1], 128) * t->ldw[l]);
+  zalloc((void**)&t->dWp, sizeof(float) * kMaxSplit * wmaxp);
   zalloc((void**)&t->h0, sizeof(double) * B);
   zalloc((void**)&t->rstat, sizeof(int32_t) * B);
   if (e != cudaSuccess) {
@@ -240,6 +247,77 @@ df_status ensure_batch(df_state* s, int64_t B) {
   t->B = B;
   t->Bp = Bp;
   t->ldT = ldT;
+  if (!bf16) {
+    char emsg[256];
+    for (int l = 0; l < L; ++l) {
+      const bool last = l == L - 1;
+      const int N = s->widths[l + 1], K = s->widths[l];
+      // forward: hidden layers also store GELU'(Z); the read-out is linear, FP32
+      SplitLayer F;
+      F.N = N;
+      F.K = K;
+      F.A = l == 0 ? t->xp : t->H[l - 1];
+      F.lda = l == 0 ? t->ldx : t->ldh[l - 1];
+      F.a_plane = B * F.lda;
+      F.W = s->Wsp[l];
+      F.ldw = round_up(K, 16);
+      F.w_plane = N * F.ldw;
+      F.bias = s->bias[l];
+      F.planes = F.gelu = !last;
+      F.mode = last ? 0 : 1;
+      F.ldg = t->ldg[l];
+      F.o_plane = B * t->ldh[l];
+      bool ok = split_encode(F, B, last ? (void*)t->O : t->H[l], B, last ? t->ldo : t->ldh[l],
+                             (float*)t->G[l], emsg, sizeof emsg);
+      // input gradient dZ_l W_l with W_l read along its other dimension; layer 0's result is the FP32
+      // gradient of the network input, the others are scaled by GELU'(Z_{l-1})
+      SplitLayer D;
+      D.tr = 2;
+      D.N = K;
+      D.K = N;
+      D.A = t->dZ[l];
+      D.lda = t->ldz[l];
+      D.a_plane = B * D.lda;
+      D.W = s->Wsp[l];
+      D.ldw = round_up(K, 16);
+      D.w_plane = N * D.ldw;
+      D.bias = t->zero_bias;
+      D.gelu = false;
+      D.planes = l > 0;
+      D.mode = l > 0 ? 2 : 0;
+      D.ldg = l > 0 ? t->ldg[l - 1] : 0;
+      D.o_plane = l > 0 ? B * t->ldz[l - 1] : 0;
+      ok = ok && split_encode(D, B, l > 0 ? t->dZ[l - 1] : (void*)t->dX, B, l > 0 ? t->ldz[l - 1] : t->lddx,
+                              l > 0 ? (float*)t->G[l - 1] : nullptr, emsg, sizeof emsg);
+      // weight gradient dZ_l^T H_{l-1}, both read along their columns (maps encoded per batch size)
+      SplitLayer G;
+      G.tr = 3;
+      G.N = K;
+      G.M = N;
+      G.K = (int)B;
+      G.A = t->dZ[l];
+      G.lda = t->ldz[l];
+      G.a_plane = B * G.lda;
+      G.W = F.A;
+      G.ldw = F.lda;
+      G.w_plane = F.a_plane;
+      G.bias = t->zero_bias;
+      G.gelu = G.planes = false;
+      G.split_rows = round_up(N, 128);   // each split owns whole 128-row tiles
+      if (!ok) {
+        free_batch(t);
+        return fail(s, DF_ERR_CUDA, "%s", emsg);
+      }
+      t->sfwd.push_back(F);
+      t->sdg.push_back(D);
+      t->swg.push_back(G);
+      if ((e = prepare_split(F)) != cudaSuccess || (e = prepare_split(D)) != cudaSuccess ||
+          (e = prepare_split(G)) != cudaSuccess) {
+        free_batch(t);
+        return cuda_fail(s, e, "kernel attributes");
+      }
+    }
+  }
   if (bf16) {
     char emsg[256];
     bool ok = true;
@@ -346,22 +424,45 @@ cudaError_t forward(df_state* s, int64_t R, cudaStream_t st) {
   Trn* t = s->trn;
   const RowMap rows{nullptr, nullptr, 0, R};
   for (int l = 0; l < s->L; ++l) {
-    const bool last = l == s->L - 1;
-    cudaError_t e;
-    if (s->precision == DF_BF16) {
-      e = launch_tc_gemm(t->fwd[l], rows, s->num_sms, s->d_err, st);
-    } else {
-      const float* A = l == 0 ? (const float*)t->x : (const float*)t->H[l - 1];
-      const int64_t lda = l == 0 ? t->ldx : t->ldh[l - 1];
-      e = launch_sgemm_bias_act(rows, s->widths[l + 1], s->Kp8[l], A, lda, s->W32[l], s->Kp8[l],
-                                s->bias[l], last ? t->O : (float*)t->H[l],
-                                last ? t->ldo : t->ldh[l], !last, s->num_sms, st, last ? 0 : 1,
-                                last ? nullptr : (float*)t->G[l], last ? 0 : t->ldg[l], 1);
-    }
+    const cudaError_t e = s->precision == DF_BF16
+                              ? launch_tc_gemm(t->fwd[l], rows, s->num_sms, s->d_err, st)
+                              : launch_split(t->sfwd[l], rows, s->num_sms, s->d_err, st);
     if (e != cudaSuccess) return e;
   }
   t->rows = R;
   return cudaSuccess;
+}
+
+// The rows of the network input (FP32, pitch ldi) as the planes t->xp of an FP32 network.
+cudaError_t input_planes(df_state* s, int64_t R, const float* in, int64_t ldi, cudaStream_t st) {
+  Trn* t = s->trn;
+  return launch_split_rows(RowMap{nullptr, nullptr, 0, R}, s->K0, in, ldi, t->xp, t->ldx, t->B * t->ldx,
+                           s->num_sms, st);
+}
+
+// dZ_{L-1} of an FP32 network from the FP32 output gradient (pitch ldi).
+cudaError_t output_planes(df_state* s, int64_t R, const float* in, int64_t ldi, cudaStream_t st) {
+  Trn* t = s->trn;
+  const int64_t ld = t->ldz[s->L - 1];
+  return launch_split_rows(RowMap{nullptr, nullptr, 0, R}, s->nout, in, ldi, t->dZ[s->L - 1], ld, t->B * ld,
+                           s->num_sms, st);
+}
+
+// The FP32 weight-gradient maps for a batch of R rows: rows past R read as zero.
+bool encode_wgrad(df_state* s, int64_t R) {
+  Trn* t = s->trn;
+  if (t->wg_rows == R) return true;
+  char emsg[256];
+  for (int l = 0; l < s->L; ++l) {
+    SplitLayer& G = t->swg[l];
+    G.K = (int)R;
+    if (!split_encode(G, R, t->dWp, (int64_t)kMaxSplit * G.split_rows, t->ldw[l], nullptr, emsg, sizeof emsg)) {
+      t->wg_rows = -1;
+      return false;
+    }
+  }
+  t->wg_rows = R;
+  return true;
 }
 
 // Backward pass over R rows from dZ_{L-1} (already in t->dZ[L-1]); fills dW, db and, when
@@ -372,49 +473,44 @@ cudaError_t backward(df_state* s, int64_t R, bool want_dx, cudaStream_t st) {
   const int64_t Rp = round_up(R, 64);
   const RowMap rows{nullptr, nullptr, 0, R};
   cudaError_t e = cudaSuccess;
+  if (!bf16 && !encode_wgrad(s, R)) return cudaErrorInvalidValue;
   for (int l = s->L - 1; l >= 0 && e == cudaSuccess; --l) {
     const int N = s->widths[l + 1], K = s->widths[l];
-    const void* Hin = l == 0 ? t->x : t->H[l - 1];
-    const int64_t ldin = l == 0 ? t->ldx : t->ldh[l - 1];
-    // dZ_l^T, with db_l = column sums of dZ_l from the same pass
-    e = launch_transpose(R, N, t->dZ[l], t->ldz[l], t->ZT, t->ldT, Rp, bf16, s->num_sms, st,
-                         t->db[l], t->scratch, t->scratch_floats);
-    if (e == cudaSuccess)
-      e = launch_transpose(R, K, Hin, ldin, t->HT, t->ldT, Rp, bf16, s->num_sms, st);
     const RowMap wrows{nullptr, nullptr, 0, N};
-    if (e == cudaSuccess) {
-      if (bf16) {
-        TcLayer Wg = t->wgrad[l];
-        Wg.K = (int)Rp;
-        // work items: 128-row tiles, or 256-row tiles on the GPU's CTA pairs
-        const int64_t rows_per = Wg.pair ? 256 : 128;
-        const int64_t tiles = ((N + rows_per - 1) / rows_per) * ((K + Wg.BN - 1) / Wg.BN);
-        Wg.ksplit = wgrad_splits(tiles, (int)(Rp / 64), Wg.pair ? s->num_sms / 2 : s->num_sms);
-        // each split owns whole 128-row tiles (a tile's store covers all its rows)
-        Wg.split_rows = round_up(N, 128);
-        e = launch_tc_gemm(Wg, wrows, s->num_sms, s->d_err, st);
-        if (e == cudaSuccess)
-          e = launch_sum_splits(Wg.ksplit, (int64_t)N * t->ldw[l], Wg.split_rows * t->ldw[l],
-                                t->dWp, t->dW[l], st);
-      } else {
-        e = launch_sgemm_bias_act(wrows, K, (int)Rp, (const float*)t->ZT, t->ldT,
-                                  (const float*)t->HT, t->ldT, t->zero_bias, t->dW[l], t->ldw[l],
-                                  false, s->num_sms, st);
-      }
+    if (bf16) {
+      const void* Hin = l == 0 ? t->x : t->H[l - 1];
+      const int64_t ldin = l == 0 ? t->ldx : t->ldh[l - 1];
+      // dZ_l^T, with db_l = column sums of dZ_l from the same pass
+      e = launch_transpose(R, N, t->dZ[l], t->ldz[l], t->ZT, t->ldT, Rp, s->num_sms, st, t->db[l],
+                           t->scratch, t->scratch_floats);
+      if (e == cudaSuccess) e = launch_transpose(R, K, Hin, ldin, t->HT, t->ldT, Rp, s->num_sms, st);
+      if (e != cudaSuccess) break;
+      TcLayer Wg = t->wgrad[l];
+      Wg.K = (int)Rp;
+      // work items: 128-row tiles, or 256-row tiles on the GPU's CTA pairs
+      const int64_t rows_per = Wg.pair ? 256 : 128;
+      const int64_t tiles = ((N + rows_per - 1) / rows_per) * ((K + Wg.BN - 1) / Wg.BN);
+      Wg.ksplit = wgrad_splits(tiles, (int)(Rp / 64), Wg.pair ? s->num_sms / 2 : s->num_sms);
+      // each split owns whole 128-row tiles (a tile's store covers all its rows)
+      Wg.split_rows = round_up(N, 128);
+      e = launch_tc_gemm(Wg, wrows, s->num_sms, s->d_err, st);
+      if (e == cudaSuccess)
+        e = launch_sum_splits(Wg.ksplit, (int64_t)N * t->ldw[l], Wg.split_rows * t->ldw[l], t->dWp,
+                              t->dW[l], st);
+    } else {
+      SplitLayer G = t->swg[l];
+      e = launch_colsum(R, N, t->dZ[l], t->ldz[l], 3, t->B * t->ldz[l], t->db[l], s->num_sms, t->scratch,
+                        t->scratch_floats, st);
+      const int64_t tiles = ((N + 255) / 256) * ((K + G.tw[0] - 1) / G.tw[0]);
+      G.ksplit = wgrad_splits(tiles, (int)(Rp / 64), s->num_sms / 2);
+      if (e == cudaSuccess) e = launch_split(G, wrows, s->num_sms, s->d_err, st);
+      if (e == cudaSuccess)
+        e = launch_sum_splits(G.ksplit, (int64_t)N * t->ldw[l], G.split_rows * t->ldw[l], t->dWp,
+                              t->dW[l], st);
     }
     if (e != cudaSuccess || (l == 0 && !want_dx)) continue;
-    if (bf16) {
-      e = launch_tc_gemm(t->dgrad[l], rows, s->num_sms, s->d_err, st);
-    } else if (l > 0) {
-      e = launch_sgemm_bias_act(rows, K, (int)t->ldt[l], (const float*)t->dZ[l], t->ldz[l],
-                                (const float*)t->WT[l], t->ldt[l], t->zero_bias,
-                                (float*)t->dZ[l - 1], t->ldz[l - 1], false, s->num_sms, st, 2,
-                                (float*)t->G[l - 1], t->ldg[l - 1], 1);
-    } else {
-      e = launch_sgemm_bias_act(rows, K, (int)t->ldt[0], (const float*)t->dZ[0], t->ldz[0],
-                                (const float*)t->WT[0], t->ldt[0], t->zero_bias, t->dX, t->lddx,
-                                false, s->num_sms, st);
-    }
+    e = bf16 ? launch_tc_gemm(t->dgrad[l], rows, s->num_sms, s->d_err, st)
+             : launch_split(t->sdg[l], rows, s->num_sms, s->d_err, st);
   }
   return e;
 }
@@ -490,6 +586,7 @@ df_status df_train_step(df_state* s, int64_t batch, const double* T, const doubl
       ProfScope ps(s, "train_inputs", st);
       e = launch_eos_pre(s->P, cells, T, p, Y, ld, t->h0, nullptr, t->x, bf16 ? kXBF16 : kXF32,
                          t->ldx, 1.0f, t->rstat, st);
+      if (e == cudaSuccess && !bf16) e = input_planes(s, batch, (const float*)t->x, t->ldx, st);
       if (e == cudaSuccess) e = launch_train_targets(s->P, batch, Y, Y_target, ld, t->Oh, t->ldo, st);
     }
     if (e == cudaSuccess) {
@@ -497,8 +594,10 @@ df_status df_train_step(df_state* s, int64_t batch, const double* T, const doubl
       e = forward(s, batch, st);
     }
     if (e == cudaSuccess)
-      e = launch_loss_grad(batch, s->n, t->O, t->ldo, t->Oh, t->ldo, t->dZ[s->L - 1],
-                           t->ldz[s->L - 1], bf16, t->loss, t->scratch, st);
+      e = launch_loss_grad(batch, s->n, t->O, t->ldo, t->Oh, t->ldo,
+                           bf16 ? t->dZ[s->L - 1] : (void*)t->dZ32, t->ldz[s->L - 1], bf16, t->loss,
+                           t->scratch, st);
+    if (e == cudaSuccess && !bf16) e = output_planes(s, batch, t->dZ32, t->ldz[s->L - 1], st);
     if (e == cudaSuccess) {
       ProfScope ps(s, "train_backward", st);
       e = backward(s, batch, false, st);
@@ -535,6 +634,7 @@ df_status df_propnet_train_step(df_state* s, int64_t batch, const double* h, con
       ProfScope ps(s, "train_inputs", st);
       e = launch_prop_inputs(s->d_norm, s->n, s->lambda, batch, h, p, Y, ldY, t->x, t->ldx,
                              bf16 ? kXBF16 : kXF32, s->num_sms, st);
+      if (e == cudaSuccess && !bf16) e = input_planes(s, batch, (const float*)t->x, t->ldx, st);
       if (e == cudaSuccess)
         e = launch_prop_targets(s->d_norm, s->K0, s->nout, batch, target, ldt, t->Oh, t->ldo,
                                 s->num_sms, st);
@@ -544,8 +644,10 @@ df_status df_propnet_train_step(df_state* s, int64_t batch, const double* h, con
       e = forward(s, batch, st);
     }
     if (e == cudaSuccess)
-      e = launch_loss_grad(batch, s->nout, t->O, t->ldo, t->Oh, t->ldo, t->dZ[s->L - 1],
-                           t->ldz[s->L - 1], bf16, t->loss, t->scratch, st);
+      e = launch_loss_grad(batch, s->nout, t->O, t->ldo, t->Oh, t->ldo,
+                           bf16 ? t->dZ[s->L - 1] : (void*)t->dZ32, t->ldz[s->L - 1], bf16, t->loss,
+                           t->scratch, st);
+    if (e == cudaSuccess && !bf16) e = output_planes(s, batch, t->dZ32, t->ldz[s->L - 1], st);
     if (e == cudaSuccess) {
       ProfScope ps(s, "train_backward", st);
       e = backward(s, batch, false, st);
@@ -573,8 +675,9 @@ df_status df_mlp_forward_train(df_state* s, int64_t n_rows, const float* x, floa
     t->rows = 0;
     return DF_OK;
   }
-  cudaError_t e = launch_cast_rows(n_rows, s->K0, x, s->K0, t->x, t->ldx,
-                                   s->precision == DF_BF16 ? kXBF16 : kXF32, 1.0f, s->num_sms, st);
+  cudaError_t e = s->precision == DF_BF16
+                      ? launch_cast_rows(n_rows, s->K0, x, s->K0, t->x, t->ldx, kXBF16, 1.0f, s->num_sms, st)
+                      : input_planes(s, n_rows, x, s->K0, st);
   if (e == cudaSuccess) e = forward(s, n_rows, st);
   if (e == cudaSuccess)
     e = cudaMemcpy2DAsync(O, sizeof(float) * s->nout, t->O, sizeof(float) * t->ldo,
@@ -602,8 +705,10 @@ df_status df_mlp_backward(df_state* s, int64_t n_rows, const float* dO, float* d
     return e == cudaSuccess ? DF_OK : cuda_fail(s, e, "gradient reset");
   }
   const int L = s->L;
-  cudaError_t e = launch_cast_rows(n_rows, s->nout, dO, s->nout, t->dZ[L - 1], t->ldz[L - 1],
-                                   s->precision == DF_BF16 ? kXBF16 : kXF32, 1.0f, s->num_sms, st);
+  cudaError_t e = s->precision == DF_BF16
+                      ? launch_cast_rows(n_rows, s->nout, dO, s->nout, t->dZ[L - 1], t->ldz[L - 1], kXBF16,
+                                         1.0f, s->num_sms, st)
+                      : output_planes(s, n_rows, dO, s->nout, st);
   if (e == cudaSuccess) e = backward(s, n_rows, dX != nullptr, st);
   if (e == cudaSuccess && dX)
     e = cudaMemcpy2DAsync(dX, sizeof(float) * s->K0, t->dX, sizeof(float) * t->lddx,
