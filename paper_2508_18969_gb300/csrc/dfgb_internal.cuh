@@ -163,25 +163,38 @@ cudaError_t launch_prop_outputs(const double* norm, int K0, int m, int64_t rows,
 cudaError_t launch_loss_grad(int64_t B, int n, const float* O, int64_t ldo, const float* Oh,
                              int64_t ldh, void* dO, int64_t ldd, bool bf16, float* loss,
                              float* scratch, cudaStream_t st);
-// out [C x ldo] = in^T for in [R x ldi]; rows R..Rpad-1 of the transpose are zero. Rpad a
-// multiple of 64, ldi and ldo even. With colsum (and scratch of scratch_floats >= C floats),
-// also colsum[c] = sum_r in[r][c], FP32, in a fixed order.
-cudaError_t launch_transpose(int64_t R, int64_t C, const void* in, int64_t ldi, void* out,
-                             int64_t ldo, int64_t Rpad, int num_sms, cudaStream_t st,
-                             float* colsum = nullptr, float* scratch = nullptr,
-                             int64_t scratch_floats = 0);
 // out[i] = sum_{s < splits} part[s * stride + i] (fixed order), i < count.
 cudaError_t launch_sum_splits(int splits, int64_t count, int64_t stride, const float* part,
                               float* out, cudaStream_t st);
-cudaError_t launch_adam(int64_t count, float* w, float* m, float* v, const float* g, float lr,
-                        float b1, float b2, float eps, float c1, float c2, cudaStream_t st);
+// One Adam update of every layer and its working copies, in one launch. W, m, v, g are [N x ld] (ld a
+// multiple of 8, zero pads), b and its moments and gradient [N]. Wb: BF16 copy [N x ldb] (ldb >= ld) or
+// NULL; W32 (pitch ld) and Wp (three BF16 planes [N x ldp], ldp >= ld): an FP32 network's copies or NULL.
+struct AdamLayer {
+  float *W, *m, *v;
+  const float* g;
+  float *b, *mb, *vb;
+  const float* gb;
+  void* Wb;
+  int64_t ldb;
+  float* W32;
+  void* Wp;
+  int64_t ldp;
+  int64_t ld;
+  int N, K;        // K <= ld: the columns past K stay zero
+  int64_t first;   // first work item of the layer (set by launch_adam)
+};
+constexpr int kMaxLayers = 8;
+struct AdamArgs {
+  AdamLayer layer[kMaxLayers];
+  int L;
+  int64_t items;
+};
+cudaError_t launch_adam(AdamArgs a, float lr, float b1, float b2, float eps, float c1, float c2,
+                        int num_sms, cudaStream_t st);
 // out[c] = sum of column c < C of `planes` (1 or 3) stacked BF16 matrices [R x ld], FP32, fixed order.
 cudaError_t launch_colsum(int64_t R, int64_t C, const void* in, int64_t ld, int planes, int64_t plane,
                           float* out, int num_sms, float* scratch, int64_t scratch_floats,
                           cudaStream_t st);
-cudaError_t launch_publish(int N, int K, const float* Wm, int64_t ldm, float* W32, int64_t ld32, void* Wb,
-                           int64_t ldb, void* WT, int64_t ldt, cudaStream_t st);
-
 // ---- launchers (compact.cu) ----
 constexpr int64_t kCompactChunk = 4096;   // cells per block of the compaction kernels
 // Stable list of cells with T > T_react. Needs scratch of compact_scratch_words(n) int64.
@@ -240,6 +253,8 @@ struct TcLayer {
   int ksplit = 1;        // split-K (plain mode): split s covers k-blocks [s kbs, (s+1) kbs) and
   int64_t split_rows = 0;  // stores its partial product at output rows + s * split_rows
   bool pair = false;     // computed by CTA pairs (cta_group::2): 256-row tiles, tmB box BN/2
+  int tr = 0;            // MN-major operands (BF16), boxes {64, 64}: bit 0 A (K rows of output rows'
+                         // columns), bit 1 W (K rows of N columns)
   long long wait_budget = 0;  // clocks a pipeline wait may take before the kernel gives up
                               // (<= 0: the default, ~1 s)
 };

@@ -33,6 +33,7 @@
 // eight epilogue warps (two per TMEM lane quarter, each holding every other 32-column chunk of its 32
 // rows: up to 128 FP32 accumulators a thread). Waits are bounded and drains complete as in mlp_tc.cu.
 #include "dfgb_internal.cuh"
+#include "planes.cuh"
 #include "tc_ptx.cuh"
 
 #include <cuda_bf16.h>
@@ -56,7 +57,7 @@ enum { kSPlain = 0, kSStoreG = 1, kSRowG = 2 };
 // row or column index runs along memory (MN-major), so the backward pass needs no transposed copy of
 // the activations, output gradients or weights. 10,007 rows of 32-1600-800-400-30, forward and backward:
 // 7.95 -> 1.01 ms (the FMA GEMM ran a weight gradient on 4 to 91 blocks, 1.5 ms each, after transposes).
-enum { kTrA = 1, kTrW = 2 };
+constexpr int kTrA = 1, kTrW = 2;
 
 // The two tilings. Wide: 256-column tiles on CTA pairs, one epilogue group of up to 128 accumulators
 // a thread. Small: 64-column tiles on single CTAs, two groups.
@@ -118,24 +119,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t sr
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
                ::"l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(src)
                : "memory");
-}
-
-// The three BF16 planes of one FP32 value. Infinities and NaN stay in plane 0; a finite value that
-// would round to a BF16 infinity is truncated there instead (the remainder stays exact).
-__device__ __forceinline__ void split_one(float v, __nv_bfloat16& h0, __nv_bfloat16& h1,
-                                          __nv_bfloat16& h2) {
-  h0 = __float2bfloat16_rn(v);
-  float r = v - __bfloat162float(h0);
-  if (!(fabsf(r) <= 3.0e38f)) {
-    if (!isfinite(v)) {
-      h1 = h2 = __float2bfloat16_rn(0.0f);
-      return;
-    }
-    h0 = __ushort_as_bfloat16((unsigned short)(__float_as_uint(v) >> 16));
-    r = v - __bfloat162float(h0);
-  }
-  h1 = __float2bfloat16_rn(r);
-  h2 = __float2bfloat16_rn(r - __bfloat162float(h1));
 }
 
 // One element of A W^T over k in [k0, k1) as a chain of FP32 FMAs, from the planes.

@@ -280,7 +280,11 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t (&r)[32], const Tc
   }
 }
 
-template <bool FP8, int BN, int OUTK, int ACT, bool SCALE, int MODE, bool PAIR>
+// TR (training, BF16): operands read along their other dimension, as in mlp_split.cu. kTrA: A holds
+// its K reduction rows of M columns; kTrW: W its K rows of N columns.
+constexpr int kTrA = 1, kTrW = 2;
+
+template <bool FP8, int BN, int OUTK, int ACT, bool SCALE, int MODE, bool PAIR, int TR>
 __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)), 1) tc_gemm_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmG, TcArgs g) {
@@ -290,6 +294,7 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
   static_assert(BN % 32 == 0, "tile width must be a multiple of 32");
   // each CTA of a pair holds whole 8-row swizzle atoms of W
   static_assert(!PAIR || (BN / 2) % 8 == 0, "paired tile width must split into 8-row groups");
+  static_assert(TR == 0 || (!FP8 && ((TR & kTrW) == 0 || C::kBRows % 64 == 0)), "MN-major operands come in 64-column boxes");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;                                   // kStages x 16 KB
@@ -388,15 +393,23 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
         }
         const uint32_t dA = smem_u32(sA + s * BM * kRowBytes);
         const uint32_t dB = smem_u32(sB + s * C::kBRows * kRowBytes);
-        if constexpr (PAIR) {
-          const uint32_t full_leader = map_shared(full0 + 8 * s, 0);
-          if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * s, 2 * C::kStageBytes);
-          tma_load_2d_pair(dA, &tmA, full_leader, kb * kelems, m0);
-          tma_load_2d_pair(dB, &tmB, full_leader, kb * kelems, n0);
+        const uint32_t bar = PAIR ? map_shared(full0 + 8 * s, 0) : full0 + 8 * s;
+        if (!PAIR || rank == 0) mbar_arrive_expect_tx(full0 + 8 * s, (PAIR ? 2 : 1) * C::kStageBytes);
+        auto load = [&](uint32_t dst, const CUtensorMap* map, int x, int y) {
+          if constexpr (PAIR) tma_load_2d_pair(dst, map, bar, x, y);
+          else tma_load_2d(dst, map, bar, x, y);
+        };
+        if constexpr (TR & kTrA) {
+#pragma unroll
+          for (int i = 0; i < BM / 64; ++i) load(dA + i * kMnBox, &tmA, m0 + 64 * i, kb * kelems);
         } else {
-          mbar_arrive_expect_tx(full0 + 8 * s, C::kStageBytes);
-          tma_load_2d(dA, &tmA, full0 + 8 * s, kb * kelems, m0);
-          tma_load_2d(dB, &tmB, full0 + 8 * s, kb * kelems, n0);
+          load(dA, &tmA, kb * kelems, m0);
+        }
+        if constexpr (TR & kTrW) {
+#pragma unroll
+          for (int i = 0; i < C::kBRows / 64; ++i) load(dB + i * kMnBox, &tmB, n0 + 64 * i, kb * kelems);
+        } else {
+          load(dB, &tmB, kb * kelems, n0);
         }
       }
     }
@@ -426,7 +439,10 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
     }
   } else if (warp == 1 && lane == 0 && rank == 0) {
     // ---------------- MMA issuer ----------------
-    constexpr uint32_t id0 = idesc<FP8, 0, PAIR ? 2 * BM : BM>();
+    constexpr uint32_t id0 = idesc<FP8, 0, PAIR ? 2 * BM : BM>() | ((TR & kTrA) ? kIdescMnA : 0u) |
+                             ((TR & kTrW) ? kIdescMnB : 0u);
+    // descriptor step of one instruction: 32 bytes of a K-major row, or 16 rows of 128 bytes
+    constexpr uint32_t stepA = (TR & kTrA) ? 128 : 2, stepB = (TR & kTrW) ? 128 : 2;
     uint32_t it = 0, j = 0;
     bool ok = true;
     for (ItemWalk w(t_first, units_m32, tiles_n); w.split < g.ksplit && ok;
@@ -448,14 +464,15 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
           break;
         }
         tc_fence_after();
-        const uint64_t da = desc_sw128(smem_u32(sA + s * BM * kRowBytes));
-        const uint64_t db = desc_sw128(smem_u32(sB + s * C::kBRows * kRowBytes));
+        const uint32_t aA = smem_u32(sA + s * BM * kRowBytes), aB = smem_u32(sB + s * C::kBRows * kRowBytes);
+        const uint64_t da = (TR & kTrA) ? desc_mn128(aA) : desc_sw128(aA);
+        const uint64_t db = (TR & kTrW) ? desc_mn128(aB) : desc_sw128(aB);
 #pragma unroll
         for (int kk = 0; kk < kRowBytes / 32; ++kk) {  // 32 bytes of K per instruction
           if constexpr (PAIR)
-            mma_issue_pair<FP8>(dt, da + 2 * kk, db + 2 * kk, id, (kb != kb0 || kk) ? 1u : 0u);
+            mma_issue_pair<FP8>(dt, da + stepA * kk, db + stepB * kk, id, (kb != kb0 || kk) ? 1u : 0u);
           else
-            mma_issue<FP8>(dt, da + 2 * kk, db + 2 * kk, id, (kb != kb0 || kk) ? 1u : 0u);
+            mma_issue<FP8>(dt, da + stepA * kk, db + stepB * kk, id, (kb != kb0 || kk) ? 1u : 0u);
         }
         // frees the stage (in both CTAs of a pair) when these MMAs have read it
         if constexpr (PAIR) mma_commit_pair_both(empty0 + 8 * s);
@@ -572,7 +589,7 @@ EncodeTiledFn encode_fn() {
 }
 
 // Opts the kernel instance into its dynamic shared memory, once per device.
-template <bool FP8, int BN, int OUTK, int ACT, int MODE, bool PAIR>
+template <bool FP8, int BN, int OUTK, int ACT, int MODE, bool PAIR, int TR>
 cudaError_t tc_attr(int* max_clusters) {
   static bool attr_done[64] = {false};
   static int clusters[64] = {0};
@@ -582,7 +599,7 @@ cudaError_t tc_attr(int* max_clusters) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
     using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE)>;
-    auto kern = tc_gemm_kernel<FP8, BN, OUTK, ACT, FP8, MODE, PAIR>;
+    auto kern = tc_gemm_kernel<FP8, BN, OUTK, ACT, FP8, MODE, PAIR, TR>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (e != cudaSuccess) return e;
     if (PAIR) {
@@ -611,13 +628,13 @@ cudaError_t tc_attr(int* max_clusters) {
   return cudaSuccess;
 }
 
-template <bool FP8, int BN, int OUTK, int ACT, int MODE = kModePlain, bool PAIR = false>
+template <bool FP8, int BN, int OUTK, int ACT, int MODE = kModePlain, bool PAIR = false, int TR = 0>
 cudaError_t launch_bn(const TcLayer& L, const TcArgs& a, int num_sms, cudaStream_t st) {
   using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE)>;
   constexpr bool SCALE = FP8;
-  auto kern = tc_gemm_kernel<FP8, BN, OUTK, ACT, SCALE, MODE, PAIR>;
+  auto kern = tc_gemm_kernel<FP8, BN, OUTK, ACT, SCALE, MODE, PAIR, TR>;
   int max_clusters = 0;
-  cudaError_t e0 = tc_attr<FP8, BN, OUTK, ACT, MODE, PAIR>(&max_clusters);
+  cudaError_t e0 = tc_attr<FP8, BN, OUTK, ACT, MODE, PAIR, TR>(&max_clusters);
   if (e0 != cudaSuccess) return e0;
   if (num_sms <= 0) return cudaSuccess;  // attribute set-up only
   const CUtensorMap& tmG = L.mode == kModeStoreG ? L.tmG : L.tmO;
@@ -657,6 +674,34 @@ cudaError_t launch_bn(const TcLayer& L, const TcArgs& a, int num_sms, cudaStream
 template <bool FP8>
 cudaError_t launch_fmt(const TcLayer& L, const TcArgs& a, int num_sms, cudaStream_t st) {
   constexpr int HID = FP8 ? kXFP8 : kXBF16;
+  if (L.tr != 0) {
+    // training, BF16: the input gradient against W read along its columns (scaled by GELU', or FP32 for
+    // the network input), and the weight gradient with both operands read so (FP32, split-K)
+    if (FP8 || L.gelu || L.gtab) return cudaErrorInvalidValue;
+    constexpr int kBoth = kTrA | kTrW;
+    if (L.tr == kTrW && L.mode == kModeRowG && L.out_kind == kXBF16) {
+      if (L.pair) return L.BN == 256 ? launch_bn<false, 256, kXBF16, kActNone, kModeRowG, true, kTrW>(L, a, num_sms, st) : cudaErrorInvalidValue;
+      switch (L.BN) {
+        case 64: return launch_bn<false, 64, kXBF16, kActNone, kModeRowG, false, kTrW>(L, a, num_sms, st);
+        case 128: return launch_bn<false, 128, kXBF16, kActNone, kModeRowG, false, kTrW>(L, a, num_sms, st);
+        case 256: return launch_bn<false, 256, kXBF16, kActNone, kModeRowG, false, kTrW>(L, a, num_sms, st);
+        default: return cudaErrorInvalidValue;
+      }
+    }
+    if (L.mode != kModePlain || L.out_kind != kXF32) return cudaErrorInvalidValue;
+    if (L.tr == kTrW)
+      return !L.pair && L.BN == 64 ? launch_bn<false, 64, kXF32, kActNone, kModePlain, false, kTrW>(L, a, num_sms, st)
+                                   : cudaErrorInvalidValue;
+    if (L.tr != kBoth) return cudaErrorInvalidValue;
+    if (!L.pair)
+      return L.BN == 64 ? launch_bn<false, 64, kXF32, kActNone, kModePlain, false, kBoth>(L, a, num_sms, st)
+                        : cudaErrorInvalidValue;
+    switch (L.BN) {
+      case 128: return launch_bn<false, 128, kXF32, kActNone, kModePlain, true, kBoth>(L, a, num_sms, st);
+      case 256: return launch_bn<false, 256, kXF32, kActNone, kModePlain, true, kBoth>(L, a, num_sms, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   if (L.mode != kModePlain) {
     if (FP8 || L.out_kind != kXBF16) return cudaErrorInvalidValue;
     if (L.pair) {
@@ -697,16 +742,8 @@ cudaError_t launch_fmt(const TcLayer& L, const TcArgs& a, int num_sms, cudaStrea
     }
   }
   if (L.pair) {
-    // CTA pairs: hidden layers with more than one k-block, and the FP32 weight-gradient GEMMs
-    // (no activation, split-K over the batch) of training
-    if (!L.gelu) {
-      if (FP8 || L.gtab || L.out_kind != kXF32) return cudaErrorInvalidValue;
-      switch (L.BN) {
-        case 128: return launch_bn<false, 128, kXF32, kActNone, kModePlain, true>(L, a, num_sms, st);
-        case 256: return launch_bn<false, 256, kXF32, kActNone, kModePlain, true>(L, a, num_sms, st);
-        default: return cudaErrorInvalidValue;
-      }
-    }
+    // CTA pairs: hidden layers with more than one k-block
+    if (!L.gelu) return cudaErrorInvalidValue;
     if (L.gtab) {
       if (FP8 || L.out_kind != kXBF16) return cudaErrorInvalidValue;
       switch (L.BN) {

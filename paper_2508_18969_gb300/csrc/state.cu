@@ -48,7 +48,7 @@ df_status cuda_fail(df_state* s, cudaError_t e, const char* where) {
 //     stream faster per row), x1.25 when the tile leaves the TMA ring fewer than four stages.
 //     On the 1600 -> 800 layer of 2^20 rows this orders the measured times of single 160, 224
 //     and pair 160, 224, 256 tiles (2.15, 1.91, 1.82, 1.73, 1.75 ms) within 7 %.
-int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair) {
+int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair, bool mn) {
   static const int hid[] = {256, 224, 192, 160, 128, 64};
   static const int last[] = {64, 32};
   static const int paired[] = {256, 224, 160};
@@ -59,6 +59,7 @@ int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair) {
   int best = cand[nc - 1];
   double best_cost = 1e300;
   auto consider = [&](int bn, bool pair) {
+    if (mn && (pair ? bn != 256 : bn % 64 != 0 || bn == 192)) return;
     const double tiles = (double)((N + bn - 1) / bn);
     double cost;
     if (one_kblock) {

@@ -155,7 +155,8 @@ void free_trn(Trn* t);
 df_status sync_host_weights(df_state* s);
 // Tile of a tensor-core layer of N outputs and K inputs: its width, | DF_TILE_PAIR when CTA
 // pairs are allowed and cheaper.
-int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair);
+// With mn (W read along its columns) only the widths that whole 64-column boxes make up.
+int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair, bool mn = false);
 
 struct DeviceGuard {
   int prev = -1;

@@ -3,6 +3,7 @@
 // gradients dZ W, the latter scaled by GELU'(z) in its epilogue) run on the same tcgen05 /
 // SIMT kernels as the forward pass; these kernels prepare their operands.
 #include "dfgb_internal.cuh"
+#include "planes.cuh"
 
 #include <cuda_bf16.h>
 
@@ -96,86 +97,6 @@ __global__ void loss_grad_kernel(int64_t B, int n, const float* __restrict__ O, 
   }
 }
 
-// Two adjacent elements of a row: the unit of every global access of transpose_kernel.
-template <typename T> struct Pair;
-template <> struct Pair<__nv_bfloat16> {
-  using V = __nv_bfloat162;
-  static __device__ __forceinline__ float lo(V v) { return __low2float(v); }
-  static __device__ __forceinline__ float hi(V v) { return __high2float(v); }
-  static __device__ __forceinline__ V make(__nv_bfloat16 a, __nv_bfloat16 b) { return __halves2bfloat162(a, b); }
-  static __device__ __forceinline__ V zero() { return __float2bfloat162_rn(0.0f); }
-  static __device__ __forceinline__ __nv_bfloat16 first(V v) { return __low2bfloat16(v); }
-  static __device__ __forceinline__ __nv_bfloat16 second(V v) { return __high2bfloat16(v); }
-};
-constexpr int kTp = 64;   // transpose tile: 64 rows x 64 columns, 256 threads
-
-// out[c][r] = in[r][c] for c < C, r < Rpad (zero for R <= r < Rpad). Block (x, y) takes the
-// 64-column strip x and the row tiles y, y + gridDim.y, ...; every global access moves two
-// adjacent elements of a row, 128 (BF16) or 256 (FP32) contiguous bytes per warp. The loads of
-// the next tile are issued before the stores of the current one, so that each SM keeps enough
-// bytes in flight to cover the DRAM latency of this scattered pattern. With part, the block also
-// stores the FP32 column sums of its rows, part[y * C + c], summed in a fixed order (the bias
-// gradient of the dZ transpose).
-template <typename T>
-__global__ void __launch_bounds__(256, 6) transpose_kernel(int64_t R, int64_t C,
-                                                           const T* __restrict__ in, int64_t ldi,
-                                                           T* __restrict__ out, int64_t ldo,
-                                                           int64_t Rpad, float* __restrict__ part) {
-  using P = Pair<T>;
-  using V = typename P::V;
-  __shared__ T tile[kTp][kTp + 2];
-  __shared__ float red[8][kTp];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t c0 = (int64_t)blockIdx.x * kTp;
-  const int64_t c = c0 + 2 * lane;   // this thread's two columns c, c + 1 (load phase)
-  const bool col_ok = c < C, pad_hi = c + 1 >= C;
-  const int64_t ntiles = Rpad / kTp;
-  // c < C: both elements lie inside the row's pitch (ldi and c even); a pad is zeroed at use
-  const T* src = in + c;
-  V v[kTp / 8];
-  auto load = [&](int64_t tt) {
-#pragma unroll
-    for (int j = 0; j < kTp / 8; ++j) {
-      const int64_t r = tt * kTp + w + 8 * j;
-      v[j] = (r < R && col_ok) ? *reinterpret_cast<const V*>(src + r * ldi) : P::zero();
-    }
-  };
-  float s0 = 0.0f, s1 = 0.0f;
-  int64_t t = blockIdx.y;
-  if (t < ntiles) load(t);
-  for (; t < ntiles; t += gridDim.y) {
-#pragma unroll
-    for (int j = 0; j < kTp / 8; ++j) {
-      V x = v[j];
-      if (pad_hi) x = P::make(P::first(x), P::first(P::zero()));
-      s0 += P::lo(x);
-      s1 += P::hi(x);
-      tile[w + 8 * j][2 * lane] = P::first(x);
-      tile[w + 8 * j][2 * lane + 1] = P::second(x);
-    }
-    __syncthreads();
-    const int64_t r0 = t * kTp;
-    if (t + gridDim.y < ntiles) load(t + gridDim.y);
-#pragma unroll
-    for (int j = 0; j < kTp / 8; ++j) {
-      const int cl = w + 8 * j;
-      if (c0 + cl < C)
-        *reinterpret_cast<V*>(out + (c0 + cl) * ldo + r0 + 2 * lane) =
-            P::make(tile[2 * lane][cl], tile[2 * lane + 1][cl]);
-    }
-    __syncthreads();
-  }
-  if (!part) return;
-  red[w][2 * lane] = s0;
-  red[w][2 * lane + 1] = s1;
-  __syncthreads();
-  if (threadIdx.x < kTp && c0 + threadIdx.x < C) {
-    float s = 0.0f;
-    for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x];
-    part[(int64_t)blockIdx.y * C + c0 + threadIdx.x] = s;
-  }
-}
-
 // part[y * C + c] = sum over the rows y, y + gridDim.y, ... of column c of a matrix of NP BF16 planes
 // (value = sum of the planes), FP32, in a fixed order: the bias gradient. Block x takes 256 columns, a
 // warp one row at a time (512 contiguous bytes a plane), eight columns a lane.
@@ -251,35 +172,67 @@ __global__ void sum_parts_warp_kernel(int parts, int C, const float* __restrict_
   if (lane == 0) out[c] = s;
 }
 
-// Adam (Kingma & Ba 2015) on one parameter array: m, v moving averages of g and g^2, bias
-// corrections c1 = 1 - b1^t, c2 = 1 - b2^t, w -= lr (m / c1) / (sqrt(v / c2) + eps).
-__global__ void adam_kernel(int64_t count, float* __restrict__ w, float* __restrict__ m,
-                            float* __restrict__ v, const float* __restrict__ g, float lr, float b1,
-                            float b2, float eps, float c1, float c2) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = fmaf(b1, m[i], (1.0f - b1) * gi);
-    const float vi = fmaf(b2, v[i], (1.0f - b2) * gi * gi);
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// Adam (Kingma & Ba 2015) on one parameter: m, v moving averages of g and g^2, bias corrections
+// c1 = 1 - b1^t, c2 = 1 - b2^t, w -= lr (m / c1) / (sqrt(v / c2) + eps).
+struct AdamStep {
+  float lr, b1, b2, eps, c1, c2;
+  __device__ __forceinline__ void operator()(float& w, float& m, float& v, float g) const {
+    m = fmaf(b1, m, (1.0f - b1) * g);
+    v = fmaf(b2, v, (1.0f - b2) * g * g);
+    w -= lr * (m / c1) / (sqrtf(v / c2) + eps);
   }
-}
+};
 
-// Working copies of a master weight matrix Wm [N x ldm]: FP32 [N x ld32], or BF16 [N x ldb] and the
-// transposed BF16 copy [K x ldt] for the input gradient GEMM. Any destination may be NULL. Pads stay as
-// allocated (zero).
-__global__ void publish_kernel(int N, int K, const float* __restrict__ Wm, int64_t ldm, float* W32,
-                               int64_t ld32, __nv_bfloat16* Wb, int64_t ldb, __nv_bfloat16* WT,
-                               int64_t ldt) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)N * K;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e / K), c = (int)(e % K);
-    const float w = Wm[(int64_t)r * ldm + c];
-    if (W32) W32[(int64_t)r * ld32 + c] = w;
-    if (Wb) Wb[(int64_t)r * ldb + c] = __float2bfloat16_rn(w);
-    if (WT) WT[(int64_t)c * ldt + r] = __float2bfloat16_rn(w);
+// Every layer's update and its working copies in one launch (they were an update and a bias update per
+// layer, then a copy kernel per layer: twelve launches, 66 us of a step on the four-layer network). A work
+// item is four weights of a row (16-byte accesses) or four biases.
+__global__ void __launch_bounds__(kThreads) adam_kernel(const __grid_constant__ AdamArgs a, AdamStep step) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < a.items;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    int l = 0;
+    while (l + 1 < a.L && t >= a.layer[l + 1].first) ++l;
+    const AdamLayer& y = a.layer[l];
+    int64_t i = t - y.first;
+    const int64_t quads = y.N * y.ld / 4;
+    if (i >= quads) {   // biases
+      const int64_t c0 = 4 * (i - quads);
+      for (int64_t c = c0; c < c0 + 4 && c < y.N; ++c) step(y.b[c], y.mb[c], y.vb[c], y.gb[c]);
+      continue;
+    }
+    float4 w = reinterpret_cast<const float4*>(y.W)[i], m = reinterpret_cast<const float4*>(y.m)[i];
+    float4 v = reinterpret_cast<const float4*>(y.v)[i];
+    float4 g = reinterpret_cast<const float4*>(y.g)[i];
+    const int64_t per_row = y.ld / 4, r = i / per_row, c = 4 * (i - r * per_row);
+    if (c + 3 >= y.K) {   // pad columns hold another layer's sums
+      if (c >= y.K) g.x = 0.0f;
+      if (c + 1 >= y.K) g.y = 0.0f;
+      if (c + 2 >= y.K) g.z = 0.0f;
+      g.w = 0.0f;
+    }
+    step(w.x, m.x, v.x, g.x);
+    step(w.y, m.y, v.y, g.y);
+    step(w.z, m.z, v.z, g.z);
+    step(w.w, m.w, v.w, g.w);
+    reinterpret_cast<float4*>(y.W)[i] = w;
+    reinterpret_cast<float4*>(y.m)[i] = m;
+    reinterpret_cast<float4*>(y.v)[i] = v;
+    if (y.Wb) {
+      __align__(8) __nv_bfloat16 h[4] = {__float2bfloat16_rn(w.x), __float2bfloat16_rn(w.y),
+                                         __float2bfloat16_rn(w.z), __float2bfloat16_rn(w.w)};
+      *reinterpret_cast<uint2*>((__nv_bfloat16*)y.Wb + r * y.ldb + c) = *reinterpret_cast<const uint2*>(h);
+    }
+    if (y.W32) reinterpret_cast<float4*>(y.W32)[i] = w;
+    if (y.Wp) {
+      __align__(8) __nv_bfloat16 h[3][4];
+      split_one(w.x, h[0][0], h[1][0], h[2][0]);
+      split_one(w.y, h[0][1], h[1][1], h[2][1]);
+      split_one(w.z, h[0][2], h[1][2], h[2][2]);
+      split_one(w.w, h[0][3], h[1][3], h[2][3]);
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        *reinterpret_cast<uint2*>((__nv_bfloat16*)y.Wp + (p * (int64_t)y.N + r) * y.ldp + c) =
+            *reinterpret_cast<const uint2*>(h[p]);
+    }
   }
 }
 
@@ -304,7 +257,8 @@ cudaError_t launch_loss_grad(int64_t B, int n, const float* O, int64_t ldo, cons
                              float* scratch, cudaStream_t st) {
   if (B <= 0) return cudaMemsetAsync(loss, 0, sizeof(float), st);
   const float invB = 1.0f / (float)B;
-  const int g = blocks_for(B * ldd);
+  // few enough partial sums for the one warp that adds them (4096 took it 10 us)
+  const int g = std::min(blocks_for(B * ldd), 640);
   if (bf16)
     loss_grad_kernel<__nv_bfloat16><<<g, kThreads, 0, st>>>(B, n, O, ldo, Oh, ldh,
                                                             (__nv_bfloat16*)dO, ldd, invB, scratch);
@@ -312,32 +266,6 @@ cudaError_t launch_loss_grad(int64_t B, int n, const float* O, int64_t ldo, cons
     loss_grad_kernel<float><<<g, kThreads, 0, st>>>(B, n, O, ldo, Oh, ldh, (float*)dO, ldd, invB,
                                                     scratch);
   sum_parts_warp_kernel<<<1, 32, 0, st>>>(g, 1, scratch, loss);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_transpose(int64_t R, int64_t C, const void* in, int64_t ldi, void* out,
-                             int64_t ldo, int64_t Rpad, int num_sms, cudaStream_t st, float* colsum,
-                             float* scratch, int64_t scratch_floats) {
-  if (C <= 0) return cudaSuccess;
-  if (Rpad <= 0 || (Rpad % kTp) || (ldi & 1) || (ldo & 1)) {
-    if (colsum && Rpad <= 0) return cudaMemsetAsync(colsum, 0, sizeof(float) * C, st);
-    return Rpad <= 0 ? cudaSuccess : cudaErrorInvalidValue;
-  }
-  const int64_t strips = (C + kTp - 1) / kTp, ntiles = Rpad / kTp;
-  // about six blocks per SM (its resident count); with the sums, as many row groups as the
-  // scratch holds
-  int64_t groups = std::max<int64_t>(1, (6LL * std::max(num_sms, 1) + strips - 1) / strips);
-  groups = std::min(groups, ntiles);
-  if (colsum) {
-    if (!scratch || scratch_floats < C) return cudaErrorInvalidValue;
-    groups = std::min<int64_t>(groups, scratch_floats / C);
-  }
-  const dim3 grid((unsigned)strips, (unsigned)groups);
-  float* part = colsum ? scratch : nullptr;
-  transpose_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(
-      R, C, (const __nv_bfloat16*)in, ldi, (__nv_bfloat16*)out, ldo, Rpad, part);
-  if (colsum)
-    sum_parts_warp_kernel<<<(unsigned)((C + 7) / 8), 256, 0, st>>>((int)groups, (int)C, scratch, colsum);
   return cudaGetLastError();
 }
 
@@ -363,17 +291,16 @@ cudaError_t launch_sum_splits(int splits, int64_t count, int64_t stride, const f
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(int64_t count, float* w, float* m, float* v, const float* g, float lr,
-                        float b1, float b2, float eps, float c1, float c2, cudaStream_t st) {
-  if (count <= 0) return cudaSuccess;
-  adam_kernel<<<blocks_for(count), kThreads, 0, st>>>(count, w, m, v, g, lr, b1, b2, eps, c1, c2);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_publish(int N, int K, const float* Wm, int64_t ldm, float* W32, int64_t ld32, void* Wb,
-                           int64_t ldb, void* WT, int64_t ldt, cudaStream_t st) {
-  publish_kernel<<<blocks_for((int64_t)N * K), kThreads, 0, st>>>(N, K, Wm, ldm, W32, ld32, (__nv_bfloat16*)Wb,
-                                                                  ldb, (__nv_bfloat16*)WT, ldt);
+cudaError_t launch_adam(AdamArgs a, float lr, float b1, float b2, float eps, float c1, float c2,
+                        int num_sms, cudaStream_t st) {
+  int64_t t = 0;
+  for (int l = 0; l < a.L; ++l) {
+    a.layer[l].first = t;
+    t += a.layer[l].N * a.layer[l].ld / 4 + (a.layer[l].N + 3) / 4;
+  }
+  a.items = t;
+  const int64_t g = std::max<int64_t>(1, std::min<int64_t>((t + kThreads - 1) / kThreads, 8LL * num_sms));
+  adam_kernel<<<(unsigned)g, kThreads, 0, st>>>(a, AdamStep{lr, b1, b2, eps, c1, c2});
   return cudaGetLastError();
 }
 

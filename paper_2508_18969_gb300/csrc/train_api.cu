@@ -4,9 +4,8 @@
 // SIMT path, BF16 for the tensor-core path) the reaction step reads in place.
 //
 // Backward pass of layer l (Z_l = H_{l-1} W_l^T + b_l, H_l = GELU(Z_l), linear read-out):
-//   dW_l = dZ_l^T H_{l-1}   (GEMM over the batch, split-K; BF16: both operands transposed first, so
-//                            the batch becomes the contiguous reduction dimension; FP32: both read
-//                            along their columns by the tensor core)
+//   dW_l = dZ_l^T H_{l-1}   (GEMM over the batch, split-K, both operands read along their columns:
+//                            MN-major, no transposes)
 //   db_l = column sums of dZ_l
 //   dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})   (the GELU' factor applied in the GEMM's epilogue)
 // Every step runs in the kernels of train.cu, mlp_split.cu (FP32) and mlp_tc.cu (BF16).
@@ -23,8 +22,6 @@ struct Trn {
   std::vector<int64_t> ldw;              // row pitch of the [N_l x K_l] FP32 matrices
   std::vector<float*> Wm, mW, vW, dW;    // master weights, Adam moments, gradients
   std::vector<float*> mb, vb, db;        // bias moments and gradients (master = state bias)
-  std::vector<void*> WT;                 // BF16: transposed working weights [K_l x ldt_l]
-  std::vector<int64_t> ldt;
   int64_t t = 0;                         // Adam steps taken
   int64_t host_wver = 0;                 // weight version of the state's host copies
   float* loss = nullptr;                 // device loss of the last step
@@ -32,9 +29,7 @@ struct Trn {
   int64_t scratch_floats = 0;
   float* zero_bias = nullptr;
   // batch buffers for up to B rows
-  int64_t B = 0, Bp = 0;                 // Bp = B rounded up to 64 (transposed length)
-  int64_t ldT = 0;                       // pitch of the transposes: Bp + 64, so that rows of a
-                                         // transpose are not a power of two apart in memory
+  int64_t B = 0;
   void* x = nullptr;                     // input rows, BF16 or FP32
   int64_t ldx = 0;
   void* xp = nullptr;                    // FP32: the input rows' planes
@@ -45,8 +40,6 @@ struct Trn {
   float* O = nullptr;
   float* Oh = nullptr;
   int64_t ldo = 0;
-  void* ZT = nullptr;                    // dZ_l^T [N_l x Bp]
-  void* HT = nullptr;                    // H_{l-1}^T [K_l x Bp]
   float* dX = nullptr;                   // input gradient [B x lddx]
   float* dWp = nullptr;                  // split-K partial weight gradients [kMaxSplit x N x ldw]
   int64_t lddx = 0;
@@ -54,7 +47,7 @@ struct Trn {
   int32_t* rstat = nullptr;
   std::vector<TcLayer> fwd, dgrad, wgrad;  // BF16 states
   std::vector<SplitLayer> sfwd, sdg, swg;  // FP32 states
-  int64_t wg_rows = -1;                  // batch rows the swg maps are encoded for
+  int64_t wg_rows = -1;                  // batch rows the weight-gradient maps are encoded for
   int64_t rows = -1;                     // rows of the last training forward pass
 };
 
@@ -65,9 +58,8 @@ void free_trn(Trn* t) {
   auto f = [](void* p) { if (p) cudaFree(p); };
   for (auto v : {&t->Wm, &t->mW, &t->vW, &t->dW, &t->mb, &t->vb, &t->db})
     for (float* p : *v) f(p);
-  for (void* p : t->WT) f(p);
   f(t->loss); f(t->scratch); f(t->zero_bias);
-  f(t->x); f(t->xp); f(t->dZ32); f(t->O); f(t->Oh); f(t->ZT); f(t->HT); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
+  f(t->x); f(t->xp); f(t->dZ32); f(t->O); f(t->Oh); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
   for (auto v : {&t->H, &t->G, &t->dZ})
     for (void* p : *v) f(p);
   delete t;
@@ -94,10 +86,10 @@ int wgrad_splits(int64_t tiles, int kblocks, int num_sms) {
 
 void free_batch(Trn* t) {
   auto f = [](void* p) { if (p) cudaFree(p); };
-  f(t->x); f(t->xp); f(t->dZ32); f(t->O); f(t->Oh); f(t->ZT); f(t->HT); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
+  f(t->x); f(t->xp); f(t->dZ32); f(t->O); f(t->Oh); f(t->dX); f(t->dWp); f(t->h0); f(t->rstat);
   for (auto v : {&t->H, &t->G, &t->dZ})
     for (void* p : *v) f(p);
-  t->x = t->xp = t->ZT = t->HT = nullptr;
+  t->x = t->xp = nullptr;
   t->O = t->Oh = t->dX = t->dWp = t->dZ32 = nullptr;
   t->h0 = nullptr;
   t->rstat = nullptr;
@@ -106,20 +98,19 @@ void free_batch(Trn* t) {
   t->fwd.clear(); t->dgrad.clear(); t->wgrad.clear();
   t->sfwd.clear(); t->sdg.clear(); t->swg.clear();
   t->wg_rows = -1;
-  t->B = t->Bp = t->ldT = 0;
+  t->B = 0;
   t->rows = -1;
 }
 
-// Writes the working copies (FP32 weights and their planes; BF16 weights and their transposes) from
-// the masters.
+// Writes the working copies (FP32 weights and their planes, or BF16 weights) from the masters.
 cudaError_t publish_all(df_state* s, cudaStream_t st) {
   Trn* t = s->trn;
   const bool bf16 = s->precision == DF_BF16;
   cudaError_t e = cudaSuccess;
   for (int l = 0; l < s->L && e == cudaSuccess; ++l) {
     const int N = s->widths[l + 1], K = s->widths[l];
-    e = launch_publish(N, K, t->Wm[l], t->ldw[l], bf16 ? nullptr : s->W32[l], s->Kp8[l],
-                       bf16 ? s->Wlp[l] : nullptr, s->Kp8[l], t->WT[l], t->ldt[l], st);
+    e = launch_cast_rows(N, K, t->Wm[l], t->ldw[l], bf16 ? s->Wlp[l] : (void*)s->W32[l], s->Kp8[l],
+                         bf16 ? kXBF16 : kXF32, 1.0f, s->num_sms, st);
     if (e == cudaSuccess && !bf16)
       e = launch_split_rows(RowMap{nullptr, nullptr, 0, N}, K, t->Wm[l], t->ldw[l], s->Wsp[l],
                             round_up(K, 16), N * round_up(K, 16), s->num_sms, st);
@@ -127,7 +118,7 @@ cudaError_t publish_all(df_state* s, cudaStream_t st) {
   return e;
 }
 
-// Masters from the state's host weights, zero moments, transposed working copies.
+// Masters from the state's host weights, zero moments, working copies.
 df_status ensure_params(df_state* s) {
   if (s->trn) return DF_OK;
   if (!trains(s)) return fail(s, DF_ERR_UNSUPPORTED, "training needs a DF_FP32 or DF_BF16 state with DF_GELU_TANH");
@@ -161,11 +152,6 @@ df_status ensure_params(df_state* s) {
     zalloc((void**)&db, sizeof(float) * N);
     t->Wm.push_back(Wm); t->mW.push_back(mW); t->vW.push_back(vW); t->dW.push_back(dW);
     t->mb.push_back(mb); t->vb.push_back(vb); t->db.push_back(db);
-    const int64_t ldt = round_up(N, 16);
-    void* WT = nullptr;
-    if (bf16) zalloc(&WT, 2 * K * ldt);
-    t->WT.push_back(WT);
-    t->ldt.push_back(ldt);
     if (e == cudaSuccess)
       e = cudaMemcpy2D(Wm, sizeof(float) * ld, s->Wh[l].data(), sizeof(float) * K,
                        sizeof(float) * K, N, cudaMemcpyHostToDevice);
@@ -198,8 +184,6 @@ df_status ensure_batch(df_state* s, int64_t B) {
   const bool bf16 = s->precision == DF_BF16;
   const size_t eb = bf16 ? 2 : 6, gb = bf16 ? 2 : 4;   // bytes of an activation and of a GELU'(Z)
   const int64_t al = 16;
-  const int64_t Bp = round_up(B, 64);
-  const int64_t ldT = Bp + 64;
   auto zalloc = [&](void** p, size_t bytes) {
     if (e != cudaSuccess) return;
     e = cudaMalloc(p, bytes ? bytes : 1);
@@ -208,11 +192,8 @@ df_status ensure_batch(df_state* s, int64_t B) {
   t->ldx = round_up(K0, al);
   zalloc(&t->x, gb * B * t->ldx);
   if (!bf16) zalloc(&t->xp, eb * B * t->ldx);
-  int64_t nmax = 8, kmax = 8;
   for (int l = 0; l < L; ++l) {
     const int N = s->widths[l + 1];
-    nmax = std::max<int64_t>(nmax, N);
-    kmax = std::max<int64_t>(kmax, s->widths[l]);
     void *H = nullptr, *G = nullptr, *dZ = nullptr;
     const int64_t ldh = round_up(N, al), ldg = round_up(N, 32), ldz = round_up(N, al);
     if (l < L - 1) {
@@ -226,12 +207,7 @@ df_status ensure_batch(df_state* s, int64_t B) {
   t->ldo = round_up(s->nout, 8);
   zalloc((void**)&t->O, sizeof(float) * B * t->ldo);
   zalloc((void**)&t->Oh, sizeof(float) * B * t->ldo);
-  if (bf16) {
-    zalloc(&t->ZT, eb * nmax * ldT);
-    zalloc(&t->HT, eb * kmax * ldT);
-  } else {
-    zalloc((void**)&t->dZ32, sizeof(float) * B * t->ldz[L - 1]);
-  }
+  if (!bf16) zalloc((void**)&t->dZ32, sizeof(float) * B * t->ldz[L - 1]);
   t->lddx = round_up(K0, 4);
   zalloc((void**)&t->dX, sizeof(float) * B * t->lddx);
   int64_t wmaxp = 0;
@@ -245,8 +221,6 @@ df_status ensure_batch(df_state* s, int64_t B) {
     return cuda_fail(s, e, "training buffers");
   }
   t->B = B;
-  t->Bp = Bp;
-  t->ldT = ldT;
   if (!bf16) {
     char emsg[256];
     for (int l = 0; l < L; ++l) {
@@ -346,12 +320,13 @@ df_status ensure_batch(df_state* s, int64_t B) {
                   emsg, sizeof emsg) &&
            encode(&F.tmB, s->Wlp[l], K, N, s->Kp8[l], F.pair ? F.BN / 2 : F.BN, emsg, sizeof emsg) &&
            tc_encode_out(F, (uint64_t)B, emsg, sizeof emsg);
-      // input gradient: dZ_l [B x N] times W_l, i.e. against W_l^T [K x N]; layer 0's result
-      // is the FP32 gradient of the network input, the others are scaled by GELU'(Z_{l-1})
+      // input gradient: dZ_l [B x N] times W_l, read along its columns; layer 0's result is the
+      // FP32 gradient of the network input, the others are scaled by GELU'(Z_{l-1})
       TcLayer D{};
+      D.tr = 2;
       D.N = K;
       D.K = N;
-      const int dtile = pick_tile(K, N, l > 0, l > 0 ? kXBF16 : kXF32, true);
+      const int dtile = l > 0 ? pick_tile(K, N, true, kXBF16, true, true) : 64;
       D.BN = dtile & ~DF_TILE_PAIR;
       D.pair = (dtile & DF_TILE_PAIR) != 0;
       D.bias = t->zero_bias;
@@ -367,12 +342,14 @@ df_status ensure_batch(df_state* s, int64_t B) {
       D.ntan = 1;
       if (ok)
         ok = encode(&D.tmA, t->dZ[l], N, B, t->ldz[l], 128, emsg, sizeof emsg) &&
-             encode(&D.tmB, t->WT[l], N, K, t->ldt[l], D.pair ? D.BN / 2 : D.BN, emsg, sizeof emsg) &&
+             encode(&D.tmB, s->Wlp[l], K, N, s->Kp8[l], 64, emsg, sizeof emsg) &&
              tc_encode_out(D, (uint64_t)B, emsg, sizeof emsg);
-      // weight gradient: dZ_l^T [N x Bp] times (H_{l-1}^T [K x Bp])^T, FP32 out
+      // weight gradient: dZ_l^T H_{l-1}, both read along their columns, FP32 out (operand maps
+      // encoded per batch size, encode_wgrad)
       TcLayer Wg{};
+      Wg.tr = 3;
       Wg.N = K;
-      Wg.K = (int)Bp;
+      Wg.K = (int)B;
       // CTA pairs (256-row tiles, each CTA streaming half of the B tile) once dW has more
       // than one 128-row tile and 128 columns; the narrow cases on single CTAs
       Wg.pair = N > 128 && K >= 128;
@@ -380,7 +357,7 @@ df_status ensure_batch(df_state* s, int64_t B) {
         const int64_t c128 = (K + 127) / 128 * 192, c256 = (K + 255) / 256 * 256;
         Wg.BN = c256 <= c128 ? 256 : 128;
       } else {
-        Wg.BN = K <= 32 ? 32 : 64;
+        Wg.BN = 64;
       }
       Wg.bias = t->zero_bias;
       Wg.out = t->dWp;        // split-K partials, summed into dW afterwards
@@ -392,9 +369,7 @@ df_status ensure_batch(df_state* s, int64_t B) {
       Wg.mode = 0;
       Wg.ntan = 1;
       if (ok)
-        ok = encode(&Wg.tmA, t->ZT, Bp, N, ldT, 128, emsg, sizeof emsg) &&
-             encode(&Wg.tmB, t->HT, Bp, K, ldT, Wg.pair ? Wg.BN / 2 : Wg.BN, emsg, sizeof emsg) &&
-             tc_encode_out(Wg, (uint64_t)kMaxSplit * round_up(N, 128), emsg, sizeof emsg);
+        ok = tc_encode_out(Wg, (uint64_t)kMaxSplit * round_up(N, 128), emsg, sizeof emsg);
       if (!ok) break;
       t->fwd.push_back(F);
       t->dgrad.push_back(D);
@@ -448,17 +423,25 @@ cudaError_t output_planes(df_state* s, int64_t R, const float* in, int64_t ldi, 
                            s->num_sms, st);
 }
 
-// The FP32 weight-gradient maps for a batch of R rows: rows past R read as zero.
+// The weight-gradient GEMMs' operand maps for a batch of R rows: rows past R read as zero.
 bool encode_wgrad(df_state* s, int64_t R) {
   Trn* t = s->trn;
   if (t->wg_rows == R) return true;
+  t->wg_rows = -1;
   char emsg[256];
   for (int l = 0; l < s->L; ++l) {
-    SplitLayer& G = t->swg[l];
-    G.K = (int)R;
-    if (!split_encode(G, R, t->dWp, (int64_t)kMaxSplit * G.split_rows, t->ldw[l], nullptr, emsg, sizeof emsg)) {
-      t->wg_rows = -1;
-      return false;
+    if (s->precision == DF_BF16) {
+      TcLayer& G = t->wgrad[l];
+      G.K = (int)R;
+      if (!encode(&G.tmA, t->dZ[l], s->widths[l + 1], R, t->ldz[l], 64, emsg, sizeof emsg) ||
+          !encode(&G.tmB, l == 0 ? t->x : t->H[l - 1], s->widths[l], R, l == 0 ? t->ldx : t->ldh[l - 1], 64,
+                  emsg, sizeof emsg))
+        return false;
+    } else {
+      SplitLayer& G = t->swg[l];
+      G.K = (int)R;
+      if (!split_encode(G, R, t->dWp, (int64_t)kMaxSplit * G.split_rows, t->ldw[l], nullptr, emsg, sizeof emsg))
+        return false;
     }
   }
   t->wg_rows = R;
@@ -470,44 +453,34 @@ bool encode_wgrad(df_state* s, int64_t R) {
 cudaError_t backward(df_state* s, int64_t R, bool want_dx, cudaStream_t st) {
   Trn* t = s->trn;
   const bool bf16 = s->precision == DF_BF16;
-  const int64_t Rp = round_up(R, 64);
+  const int kblocks = (int)((R + 63) / 64);
   const RowMap rows{nullptr, nullptr, 0, R};
   cudaError_t e = cudaSuccess;
-  if (!bf16 && !encode_wgrad(s, R)) return cudaErrorInvalidValue;
+  if (!encode_wgrad(s, R)) return cudaErrorInvalidValue;
   for (int l = s->L - 1; l >= 0 && e == cudaSuccess; --l) {
     const int N = s->widths[l + 1], K = s->widths[l];
     const RowMap wrows{nullptr, nullptr, 0, N};
+    const int64_t split_rows = round_up(N, 128);   // each split owns whole 128-row tiles
+    int ksplit;
+    e = launch_colsum(R, N, t->dZ[l], t->ldz[l], bf16 ? 1 : 3, t->B * t->ldz[l], t->db[l], s->num_sms,
+                      t->scratch, t->scratch_floats, st);
+    if (e != cudaSuccess) break;
     if (bf16) {
-      const void* Hin = l == 0 ? t->x : t->H[l - 1];
-      const int64_t ldin = l == 0 ? t->ldx : t->ldh[l - 1];
-      // dZ_l^T, with db_l = column sums of dZ_l from the same pass
-      e = launch_transpose(R, N, t->dZ[l], t->ldz[l], t->ZT, t->ldT, Rp, s->num_sms, st, t->db[l],
-                           t->scratch, t->scratch_floats);
-      if (e == cudaSuccess) e = launch_transpose(R, K, Hin, ldin, t->HT, t->ldT, Rp, s->num_sms, st);
-      if (e != cudaSuccess) break;
       TcLayer Wg = t->wgrad[l];
-      Wg.K = (int)Rp;
       // work items: 128-row tiles, or 256-row tiles on the GPU's CTA pairs
       const int64_t rows_per = Wg.pair ? 256 : 128;
       const int64_t tiles = ((N + rows_per - 1) / rows_per) * ((K + Wg.BN - 1) / Wg.BN);
-      Wg.ksplit = wgrad_splits(tiles, (int)(Rp / 64), Wg.pair ? s->num_sms / 2 : s->num_sms);
-      // each split owns whole 128-row tiles (a tile's store covers all its rows)
-      Wg.split_rows = round_up(N, 128);
+      Wg.ksplit = ksplit = wgrad_splits(tiles, kblocks, Wg.pair ? s->num_sms / 2 : s->num_sms);
+      Wg.split_rows = split_rows;
       e = launch_tc_gemm(Wg, wrows, s->num_sms, s->d_err, st);
-      if (e == cudaSuccess)
-        e = launch_sum_splits(Wg.ksplit, (int64_t)N * t->ldw[l], Wg.split_rows * t->ldw[l], t->dWp,
-                              t->dW[l], st);
     } else {
       SplitLayer G = t->swg[l];
-      e = launch_colsum(R, N, t->dZ[l], t->ldz[l], 3, t->B * t->ldz[l], t->db[l], s->num_sms, t->scratch,
-                        t->scratch_floats, st);
       const int64_t tiles = ((N + 255) / 256) * ((K + G.tw[0] - 1) / G.tw[0]);
-      G.ksplit = wgrad_splits(tiles, (int)(Rp / 64), s->num_sms / 2);
-      if (e == cudaSuccess) e = launch_split(G, wrows, s->num_sms, s->d_err, st);
-      if (e == cudaSuccess)
-        e = launch_sum_splits(G.ksplit, (int64_t)N * t->ldw[l], G.split_rows * t->ldw[l], t->dWp,
-                              t->dW[l], st);
+      G.ksplit = ksplit = wgrad_splits(tiles, kblocks, s->num_sms / 2);
+      e = launch_split(G, wrows, s->num_sms, s->d_err, st);
     }
+    if (e == cudaSuccess)
+      e = launch_sum_splits(ksplit, (int64_t)N * t->ldw[l], split_rows * t->ldw[l], t->dWp, t->dW[l], st);
     if (e != cudaSuccess || (l == 0 && !want_dx)) continue;
     e = bf16 ? launch_tc_gemm(t->dgrad[l], rows, s->num_sms, s->d_err, st)
              : launch_split(t->sdg[l], rows, s->num_sms, s->d_err, st);
@@ -530,15 +503,25 @@ cudaError_t adam(df_state* s, const df_adam* hp, cudaStream_t st) {
   const float c2 = (float)(1.0 - std::pow(hp->beta2, (double)t->t));
   const float lr = (float)hp->lr, b1 = (float)hp->beta1, b2 = (float)hp->beta2,
               eps = (float)hp->eps;
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l < s->L && e == cudaSuccess; ++l) {
-    const int N = s->widths[l + 1];
-    e = launch_adam((int64_t)N * t->ldw[l], t->Wm[l], t->mW[l], t->vW[l], t->dW[l], lr, b1, b2, eps,
-                    c1, c2, st);
-    if (e == cudaSuccess)
-      e = launch_adam(N, s->bias[l], t->mb[l], t->vb[l], t->db[l], lr, b1, b2, eps, c1, c2, st);
+  AdamArgs a{};
+  a.L = s->L;
+  for (int l = 0; l < s->L; ++l) {
+    AdamLayer& y = a.layer[l];
+    y.W = t->Wm[l]; y.m = t->mW[l]; y.v = t->vW[l]; y.g = t->dW[l];
+    y.b = s->bias[l]; y.mb = t->mb[l]; y.vb = t->vb[l]; y.gb = t->db[l];
+    y.N = s->widths[l + 1];
+    y.K = s->widths[l];
+    y.ld = t->ldw[l];
+    if (s->precision == DF_BF16) {
+      y.Wb = s->Wlp[l];
+      y.ldb = s->Kp8[l];
+    } else {
+      y.W32 = s->W32[l];   // pitch Kp8 = ldw
+      y.Wp = s->Wsp[l];
+      y.ldp = round_up(s->widths[l], 16);
+    }
   }
-  if (e == cudaSuccess) e = publish_all(s, st);
+  const cudaError_t e = launch_adam(a, lr, b1, b2, eps, c1, c2, s->num_sms, st);
   s->wver += 1;
   return e;
 }
