@@ -36,7 +36,6 @@ constexpr double kInvR = 1.0 / kR;
 // SM holds 24 warps instead of 20 (eos_pre 0.71 -> 0.66 ms, eos_post 0.69 -> 0.66 ms on the
 // 2^20-cell step).
 constexpr int kThreads = 256;
-constexpr int kJacThreads = 64;  // the Jacobian's EoS kernel
 constexpr int kPreBlocks = 3;    // resident blocks per SM the register budget is sized for
 constexpr int kPostBlocks = 3;
 constexpr int kPropThreads = 128;  // the property and transport kernels
@@ -345,12 +344,6 @@ __device__ __forceinline__ double dlog_tab(double x, const double* lnt) {
   return fma(e, kLn2Hi, lnt[j] + fma(e, kLn2Lo, poly));
 }
 
-// 1/x from the FP32 reciprocal and one FP64 Newton step (relative error ~2^-46).
-__device__ __forceinline__ double drcp1(double x) {
-  const double r = f_to_d(__frcp_rn(d_to_f_trunc(x)));
-  return fma(r, fma(-x, r, 1.0), r);
-}
-
 // sqrt(x) for a positive normal x: t0 = x rsqrt_32(x), then one Newton step
 // t = t0 + (x - t0^2) r / 2 with the FP32 r = rsqrt_32(x) (relative error ~2^-44).
 __device__ __forceinline__ double dsqrt_pos(double x) {
@@ -477,15 +470,13 @@ __device__ __forceinline__ double g_dep(double Z, double A, double B, const doub
 //   Z^3 - (1 - B) Z^2 + (A - 3B^2 - 2B) Z - (AB - B^2 - B^3) = 0
 // above B with least departure Gibbs energy (ties within 1e-12 keep the larger root).
 // Seeds come from the FP32 closed form (Cardano for one real root, the trigonometric form
-// for three), each polished by FP64 Newton steps on the cubic: two, or with FAST one, plus a
-// second where the first moved the seed by more than 1e-6 relative (a poor seed).
+// for three), each polished by two FP64 Newton steps on the cubic.
 // The three-real-root case of select_Z: seeds from the trigonometric form, each polished, the
 // root above B with least departure Gibbs energy kept. Out of line: it is the rarer branch,
 // and keeping it out of the Newton loop's body keeps that loop's code small.
 __device__ __noinline__ double select_Z3(double A, double B, double c2, double c1, double c0,
                                          double P, double Q, const double* lnt, int& status);
 
-template <bool FAST>
 __device__ double select_Z(double A, double B, const double* lnt, int& status) {
   const double c2 = B - 1.0;
   const double c1 = A - 3.0 * B * B - 2.0 * B;
@@ -499,9 +490,7 @@ __device__ double select_Z(double A, double B, const double* lnt, int& status) {
     const float u = cbrtf(-0.5f * qf - copysignf(sq, qf));
     const float t = (u != 0.0f) ? u - pf / (3.0f * u) : 0.0f;
     const double Z0 = f_to_d(t) - c2 * (1.0 / 3.0);
-    double Z = cubic_step(Z0, c2, c1, c0);
-    if (!FAST || fabsf(d_to_f_trunc(Z - Z0)) > 1e-6f * fabsf(d_to_f_trunc(Z)))
-      Z = cubic_step(Z, c2, c1, c0);
+    const double Z = cubic_polish(Z0, c2, c1, c0);
     if (!(Z > B)) status |= kCellNoRoot;
     return Z;
   }
@@ -538,13 +527,10 @@ struct PRPoint {
   double Z, h_dep, cp_dep;  // molar departure enthalpy and its T-derivative at fixed p
 };
 
-// Real-fluid state at (T, p) of a composition (a2-a4), with the departure cp if asked. With
-// FAST (the T-from-h solve, whose cp only sets the chord slope) cp is evaluated in FP32 and
-// the cubic gets one polishing step.
-template <bool FAST>
+// Real-fluid state at (T, p) of a composition (a2-a4), with the departure cp if asked.
 __device__ PRPoint pr_point(const Mixture& m, double T, double p, bool want_cp, const double* lnt,
                             int& status) {
-  const double iT = FAST ? drcp1(T) : drcp(T);
+  const double iT = drcp(T);
   const double t = dsqrt_pos(T);
   const double it = t * iT;                       // 1 / sqrt(T)
   const double am = fma(-2.0 * m.A1, t, fma(m.A2, T, m.A0));
@@ -554,31 +540,15 @@ __device__ PRPoint pr_point(const Mixture& m, double T, double p, bool want_cp, 
   const double A = am * p * iRT * iRT;
   const double B = m.bm * p * iRT;
   PRPoint r;
-  r.Z = select_Z<FAST>(A, B, lnt, status);
+  r.Z = select_Z(A, B, lnt, status);
   const double Zp = r.Z + (1.0 + kSQ2) * B;
   const double Zm = r.Z + (1.0 - kSQ2) * B;
-  const double iZm = FAST ? drcp1(Zm) : drcp(Zm);
+  const double iZm = drcp(Zm);
   const double L = dlog_tab(Zp * iZm, lnt);
   const double tdam_am = fma(T, dam, -am);
   r.h_dep = fma(RT, r.Z - 1.0, tdam_am * m.kb * L);
   r.cp_dep = 0.0;
-  if (FAST && want_cp) {
-    // FP32: dA/dT = p (dam - 2 am / T) / (RT)^2 needs no division by am
-    const float Tf = d_to_f_trunc(T), iTf = __frcp_rn(Tf), itf = rsqrtf(Tf);
-    const float Z = d_to_f_trunc(r.Z), Af = d_to_f_trunc(A), Bf = d_to_f_trunc(B);
-    const float pf = d_to_f_trunc(p), iRTf = iTf * (float)kInvR;
-    const float d2am = 0.5f * d_to_f_trunc(m.A1) * itf * iTf;
-    const float dB = -Bf * iTf;
-    const float dA = pf * iRTf * iRTf * (d_to_f_trunc(dam) - 2.0f * d_to_f_trunc(am) * iTf);
-    const float FZ = fmaf(3.0f * Z, Z, -2.0f * (1.0f - Bf) * Z) + (Af - 3.0f * Bf * Bf - 2.0f * Bf);
-    const float FA = Z - Bf;
-    const float FB = Z * Z - (6.0f * Bf + 2.0f) * Z - (Af - 2.0f * Bf - 3.0f * Bf * Bf);
-    const float dZ = -(FA * dA + FB * dB) / FZ;
-    const float s2 = (float)kSQ2;
-    const float dL = (dZ + (1.0f + s2) * dB) / d_to_f_trunc(Zp) - (dZ + (1.0f - s2) * dB) / d_to_f_trunc(Zm);
-    r.cp_dep = f_to_d((float)kR * (Z - 1.0f) + (float)kR * Tf * dZ +
-                      d_to_f_trunc(m.kb) * (Tf * d2am * d_to_f_trunc(L) + d_to_f_trunc(tdam_am) * dL));
-  } else if (want_cp) {
+  if (want_cp) {
     const double d2am = 0.5 * m.A1 * it * iT;
     const double dB = -B * iT;
     const double dA = A * fma(dam, drcp(am), -2.0 * iT);
@@ -593,60 +563,11 @@ __device__ PRPoint pr_point(const Mixture& m, double T, double p, bool want_cp, 
   return r;
 }
 
-// a9: T from h(T, p, Y') = h0 for the composition of m, safeguarded Newton inside a bracket
-// that starts at [50, 5000] K and shrinks with the sign of h - h0. Adds flags to st and the
-// iteration count to iters; returns the last iterate.
-template <bool FAST>
-__device__ double solve_T(const Mixture& m, double pc, double h0c, double Told, const EosParams& P,
-                          const double* lnt, int& iters, int& st) {
-  double lo = kTLo, hi = kTHi;
-  double Tn = fmin(fmax(Told, lo), hi);
-  bool conv = false, need_cp = true;
-  double icp = 0.0;
-  const float tolf = (float)P.newton_tol;
-  for (int it = 0; it < P.newton_max_iter; ++it) {
-    ++iters;
-    int s2 = 0;
-    const PRPoint q = pr_point<FAST>(m, Tn, pc, need_cp, lnt, s2);
-    if (s2) {
-      st |= s2;
-      break;
-    }
-    const double f = h_ig(m, Tn) + q.h_dep * m.inv - h0c;
-    // Chord steps: the slope of the first iteration is reused while the iterates stay
-    // close (each step contracts the error by ~|1 - cp(T)/cp(T0)| ~ 1e-5 there); an FP32
-    // reciprocal of cp scales the step by 1 + O(1e-7) on top.
-    if (need_cp) icp = f_to_d(__frcp_rn(d_to_f_trunc(cp_ig(m, Tn) + q.cp_dep * m.inv)));
-    // Tn lies inside [lo, hi] (the start is clamped, later iterates are inside by
-    // construction), so the bracket update needs no min/max; the sign test reads the bit
-    if (__double2hiint(f) >= 0) hi = Tn; else lo = Tn;
-    const double step = -f * icp;
-    double Tx = Tn + step;
-    // a step within tolerance has converged (the test is a threshold, FP32 is enough); only
-    // a longer step that leaves the bracket (or is not finite) is replaced by bisection,
-    // after which the slope is evaluated afresh
-    const bool done = fabsf(d_to_f_trunc(step)) <= tolf * d_to_f_trunc(Tn);
-    need_cp = false;
-    if (!done && !(Tx > lo && Tx < hi)) {
-      Tx = 0.5 * (lo + hi);
-      need_cp = true;
-    }
-    Tn = Tx;
-    if (done) {
-      conv = true;
-      break;
-    }
-  }
-  if (!conv && st == 0) st |= kCellNotConverged;
-  if (!d_finite(Tn)) st |= kCellNonfinite;
-  return Tn;
-}
-
 // ---------------------------------------------------------------- double-float state
 // The real-fluid point of eos_pre and every Newton iteration of eos_post in double-float on
 // the FP32 pipes (~2^-46 relative per operation). On this GPU one FP64 instruction costs the
 // issue time of ~30 FP32 instructions (measured in the T-from-h kernel), and a double-float
-// operation takes 4 to 15. The steps are those of pr_point / solve_T above.
+// operation takes 4 to 15. The steps are those of pr_point above.
 
 // ln x for a positive normal double-float x from the double-float table lt (ln c_j, then
 // 1 / c_j): x = 2^e m, m in [1, 2); r = m / c_j - 1 (|r| < 2^-8) formed exactly to first order;
@@ -853,8 +774,13 @@ __device__ __forceinline__ float cp_ig_f(const MixDF& m, float T) {
                    2.0f * m.e[2].h), T, m.e[1].h);
 }
 
-// solve_T in double-float (a9): the same safeguarded chord-Newton iteration inside the bracket
-// [50, 5000] K, the residual h(T) - h0 and the iterates in double-float.
+// a9: T from h(T, p, Y') = h0 for the composition of m, safeguarded Newton inside a bracket that
+// starts at [50, 5000] K and shrinks with the sign of h - h0, the residual and the iterates in
+// double-float. Adds flags to st and the iteration count to iters; returns the last iterate. Chord
+// steps: the slope of the first iteration is reused while the iterates stay close (each step contracts
+// the error by ~|1 - cp(T)/cp(T0)| ~ 1e-5 there). A step within tolerance has converged; only a longer
+// step that leaves the bracket (or is not finite) is replaced by bisection, after which the slope is
+// evaluated afresh.
 __device__ f2 solve_T_df(const MixDF& m, f2 p, f2 h0, double Told, const EosParams& P,
                          const f2* lt, int& iters, int& st) {
   f2 lo = f2{(float)kTLo, 0.0f}, hi = f2{(float)kTHi, 0.0f};
@@ -873,7 +799,7 @@ __device__ f2 solve_T_df(const MixDF& m, f2 p, f2 h0, double Told, const EosPara
       break;
     }
     const f2 f = f2_sub(f2_fma(q.h_dep, m.inv, h_ig_df(m, Tn)), h0);
-    // chord steps with an FP32 reciprocal slope, as in solve_T
+    // an FP32 reciprocal slope scales the step by 1 + O(1e-7)
     if (need_cp) icp = __fdividef(1.0f, fmaf(q.cp_dep, m.inv.h, cp_ig_f(m, Tn.h)));
     if (__float_as_int(f.h) >= 0) hi = Tn; else lo = Tn;
     const f2 step = f2_mulf(f, -icp);
@@ -1213,7 +1139,7 @@ __global__ void __launch_bounds__(kPropThreads, kPropBlocks) props_kernel(EosPar
     Mixture m;
     mixture<kPropThreads>(ycol, n, c, m);
     int st = 0;
-    const PRPoint q = pr_point<false>(m, Tc, pc, cp != nullptr, c.lnt, st);
+    const PRPoint q = pr_point(m, Tc, pc, cp != nullptr, c.lnt, st);
     if (rho) rho[i] = pc / (m.inv * q.Z * kR * Tc);
     if (h) h[i] = h_ig(m, Tc) + q.h_dep * m.inv;
     if (cp) cp[i] = cp_ig(m, Tc) + q.cp_dep * m.inv;
@@ -1307,7 +1233,7 @@ __global__ void __launch_bounds__(kPropThreads, kPropBlocks) transport_kernel(Eo
       Mixture m;
       mixture<kPropThreads>(ycol, n, c, m);
       int st = 0;
-      const PRPoint q = pr_point<false>(m, Tk, pk, true, c.lnt, st);
+      const PRPoint q = pr_point(m, Tk, pk, true, c.lnt, st);
       const double rho = pk / (m.inv * q.Z * kR * Tk);            // kg/m^3
       const double cpm = cp_ig(m, Tk) + q.cp_dep * m.inv;           // J/(kg K)
       const double Wm = 1.0 / m.inv;
@@ -1354,81 +1280,114 @@ __global__ void __launch_bounds__(kPropThreads, kPropBlocks) transport_kernel(Eo
 
 // ---------------------------------------------------------------- Jacobian of the step
 
-// dh/dY_k of the mass-specific real-fluid enthalpy at fixed T, p (FP64), for the composition in
-// the per-thread column ycol (entry k at ycol[k * stride]). u_k = y_k sqrt(a_k), yr_k = y_k r_k,
-// v = K u, w = K yr use the columns ucol, rcol, vcol, wcol. With sigma = sum y, W = 1/sigma:
-//   a = W^2 u.Ku,  a' = -(W^2 / sqrt T) yr.Ku,  b = W sum y_k b_k,
-//   da/dy_k = 2 W^2 sqrt(a_k) v_k - 2 W a,  da'/dy_k = -2 W a' - (W^2 / sqrt T)(r_k v_k + sqrt(a_k) w_k),
-//   db/dy_k = W (b_k - b),  dZ from the implicit cubic, h = sum y_k h_k(T) + sigma h_dep,
+// b^m for an integer m >= 0 by squaring, in double-float.
+__device__ __forceinline__ f2 f2_ipow(f2 b, int m) {
+  f2 r = f2{1.0f, 0.0f};
+  for (; m; m >>= 1) {
+    if (m & 1) r = f2_mul(r, b);
+    if (m > 1) b = f2_mul(b, b);
+  }
+  return r;
+}
+
+// y^lambda for y > 0 and lambda = 1/m to within dl: r0 = FP32 power (relative error ~1e-6), then
+// r = r0 (1 + e)^(-1/m) with e = r0^m / y - 1 by its series to e^3 (|e| ~ 1e-5, truncation below
+// 1e-19), in double-float. Zero for y below the normal FP32 range.
+__device__ __forceinline__ f2 f2_root(f2 y, float lamf, int m, float dl) {
+  if (!(y.h > 1e-37f)) return f2{0.0f, 0.0f};
+  const float r0 = exp2f(lamf * log2f(y.h));
+  const f2 e = f2_addf(f2_mul(f2_ipow(f2{r0, 0.0f}, m), f2_rcp(y)), -1.0f);
+  const float im = 1.0f / (float)m;
+  // (1 + e)^(-1/m) - 1 = -e/m + (1/m)(1/m + 1) e^2 / 2 - (1/m)(1/m + 1)(1/m + 2) e^3 / 6
+  const float q = im * (im + 1.0f) * 0.5f * e.h * e.h * (1.0f - (im + 2.0f) * (1.0f / 3.0f) * e.h);
+  f2 c = f2_mul(e, f2_rcp(f2{-(float)m, 0.0f}));
+  c = f2_addf(c, dl != 0.0f ? q + dl * logf(y.h) : q);
+  return f2_add(f2{r0, 0.0f}, f2_mulf(c, r0));
+}
+
+// Real-fluid c_p of the state q = pr_point_df(m, T, p) and the coefficients of dh/dY_k at fixed T, p.
+// With u_k = y_k sqrt(a_k), yr_k = y_k r_k (y = Y / W), v = K u, w = K yr, sigma = sum y = 1 / W:
+//   a = W^2 u.v,  a' = -(W^2 / sqrt T) yr.v,  b = W sum y_k b_k,
+//   da/dy_k = 2 W^2 sqrt(a_k) v_k - 2 W a,  db/dy_k = W (b_k - b),
+//   da'/dy_k = -2 W a' - (W^2 / sqrt T)(r_k v_k + sqrt(a_k) w_k),
+//   dZ from the implicit cubic, h = sum y_k h_k(T) + sigma h_dep,
 //   dh/dY_k = (h_k(T) + h_dep + sigma dh_dep/dy_k) / W_k.
-__device__ void h_grad(const EosParams& P, int n, int64_t ystride, const double* ycol, double T,
-                       double p, int stride, double* ucol, double* rcol, int vstride,
-                       double* vcol, double* wcol, double* out, int out_stride, int& st) {
-  const double* spc = P.spc;
-  const double* K = P.Kmat;
-  const double t = sqrt(T);
-  double sig = 0.0, bs = 0.0;
-  for (int k = 0; k < n; ++k) {
-    const double* q = spc + k * kSpcStride;
-    const double y = ycol[k * ystride] * q[0];
-    sig += y;
-    bs += y * q[3];
-    ucol[k * stride] = y * (q[1] - q[2] * t);
-    rcol[k * stride] = y * q[2];
-  }
-  double G = 0.0, dGs = 0.0;
-  for (int k = 0; k < n; ++k) {
-    double v = 0.0, w = 0.0;
-    for (int j = 0; j < n; ++j) {
-      v = fma(K[k * n + j], ucol[j * stride], v);
-      w = fma(K[k * n + j], rcol[j * stride], w);
-    }
-    vcol[k * vstride] = v;
-    wcol[k * vstride] = w;
-    G = fma(ucol[k * stride], v, G);
-    dGs = fma(rcol[k * stride], v, dGs);
-  }
-  const double W = 1.0 / sig;
-  const double a = W * W * G;
-  const double da = -W * W * dGs / t;
-  const double b = W * bs;
-  const double RT = kR * T;
-  const double A = a * p / (RT * RT);
-  const double B = b * p / RT;
-  const double Z = select_Z<false>(A, B, P.lntab, st);
-  const double c1 = 1.0 + kSQ2, c2 = 1.0 - kSQ2;
-  const double Zp = Z + c1 * B, Zm = Z + c2 * B;
-  const double L = log(Zp / Zm);
-  const double kb = 1.0 / (2.0 * kSQ2 * b);
-  const double tda = T * da - a;
-  const double hdep = RT * (Z - 1.0) + tda * kb * L;
-  const double FZ = 3.0 * Z * Z - 2.0 * (1.0 - B) * Z + (A - 3.0 * B * B - 2.0 * B);
-  const double FA = Z - B;
-  const double FB = Z * Z - (6.0 * B + 2.0) * Z - (A - 2.0 * B - 3.0 * B * B);
-  for (int k = 0; k < n; ++k) {
-    const double* q = spc + k * kSpcStride;
-    const double sak = q[1] - q[2] * t;
-    const double vk = vcol[k * vstride], wk = wcol[k * vstride];
-    const double dak = 2.0 * W * W * sak * vk - 2.0 * W * a;
-    const double ddak = -2.0 * W * da - W * W * (q[2] * vk + sak * wk) / t;
-    const double dbk = W * (q[3] - b);
-    const double dAk = dak * p / (RT * RT);
-    const double dBk = dbk * p / RT;
-    const double dZk = -(FA * dAk + FB * dBk) / FZ;
-    const double dLk = (dZk + c1 * dBk) / Zp - (dZk + c2 * dBk) / Zm;
-    const double dkbk = -kb * dbk / b;
-    const double dhdep = RT * dZk + (T * ddak - dak) * kb * L + tda * (dkbk * L + kb * dLk);
-    const double hk = fma(fma(fma(fma(fma(q[9], T, q[8]), T, q[7]), T, q[6]), T, q[5]), T, q[4]);
-    out[k * out_stride] = q[0] * (hk + hdep + sig * dhdep);
-  }
+// h_dep depends on the composition through a, a' and b alone; with alpha, beta, gamma its derivatives,
+//   dh/dY_k = h_k/W_k + c0 / W_k + (c1 A_k - c2 R_k) v_k - c2 A_k w_k + c3 b_k / W_k,
+//   A_k = (s_k - r_k sqrt T) / W_k,  R_k = r_k / W_k,  c1 = 2 W alpha,  c2 = W beta / sqrt T,  c3 = gamma,
+//   c0 = h_dep - 2 a alpha - 2 a' beta - b gamma.
+struct HGrad {
+  f2 T, t, c0, c1, c2, c3;
+};
+
+__device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPointDF& q, const f2* lt, f2& cp,
+                                        HGrad& g) {
+  const f2 iT = f2_rcp(T), t = f2_sqrt_pos(T), it = f2_mul(t, iT);
+  const f2 am = f2_fma(m.A1, f2{-2.0f * t.h, -2.0f * t.l}, f2_fma(m.A2, T, m.A0));
+  const f2 dam = f2_fma(f2_neg(m.A1), it, m.A2);
+  const f2 RT = f2_mul(T, f2{kRh, kRl}), iRT = f2_mul(iT, f2{kIRh, kIRl});
+  const f2 pRT = f2_mul(p, iRT), pRT2 = f2_mul(pRT, iRT);
+  const f2 A = f2_mul(am, pRT2), B = f2_mul(m.bm, pRT), Z = q.Z;
+  const f2 c1s = f2{kSPh, kSPl}, c2s = f2{kSMh, kSMl};
+  const f2 iZp = f2_rcp(f2_fma(B, c1s, Z)), iZm = f2_rcp(f2_fma(B, c2s, Z));
+  const f2 L = f2_log_tab(f2_mul(f2_fma(B, c1s, Z), iZm), lt);
+  const f2 tda = f2_fma(T, dam, f2_neg(am));
+  const f2 kbL = f2_mul(m.kb, L);
+  // f_Z, f_A, f_B of the cubic: 3 Z^2 - 2 (1 - B) Z + A - 3 B^2 - 2 B, Z - B, Z^2 - (6 B + 2) Z - (A - 2 B - 3 B^2)
+  const f2 B3 = f2_mul(B, f2_addf(f2_mulf(B, 3.0f), 2.0f));
+  const f2 FZ = f2_add(f2_mul(Z, f2_add(f2_mulf(Z, 3.0f), f2_scale2(f2_addf(B, -1.0f)))), f2_sub(A, B3));
+  const f2 FA = f2_sub(Z, B);
+  const f2 FB = f2_add(f2_mul(Z, f2_sub(Z, f2_addf(f2_mulf(B, 6.0f), 2.0f))), f2_sub(B3, A));
+  const f2 iFZ = f2_rcp(FZ);
+  const f2 e1 = f2_sub(iZp, iZm), e2 = f2_sub(f2_mul(c1s, iZp), f2_mul(c2s, iZm));
+  const f2 tk = f2_mul(tda, m.kb);
+  // dh_dep = gz dZ + kb L d(T a' - a) + T a' terms; dZ = -(FA dA + FB dB) / FZ
+  const f2 gz = f2_fma(tk, e1, RT);
+  // c_p: d/dT at fixed composition, dA = A (a'/a - 2/T) = p (a' - 2 a / T) / (RT)^2, dB = -B / T
+  const f2 d2am = f2_mul(f2_mulf(m.A1, 0.5f), f2_mul(it, iT));
+  const f2 dA = f2_mul(pRT2, f2_sub(dam, f2_scale2(f2_mul(am, iT))));
+  const f2 dB = f2_neg(f2_mul(B, iT));
+  const f2 dZ = f2_neg(f2_mul(iFZ, f2_fma(FA, dA, f2_mul(FB, dB))));
+  const f2 dL = f2_fma(dZ, e1, f2_mul(dB, e2));
+  const f2 Rf = f2{kRh, kRl};
+  f2 cpd = f2_mul(Rf, f2_addf(Z, -1.0f));
+  cpd = f2_fma(RT, dZ, cpd);
+  cpd = f2_fma(f2_mul(T, d2am), kbL, cpd);
+  cpd = f2_fma(tk, dL, cpd);
+  f2 cpi = f2_mulf(m.e[5], 5.0f);
+  cpi = f2_fma(cpi, T, f2_mulf(m.e[4], 4.0f));
+  cpi = f2_fma(cpi, T, f2_mulf(m.e[3], 3.0f));
+  cpi = f2_fma(cpi, T, f2_scale2(m.e[2]));
+  cpi = f2_fma(cpi, T, m.e[1]);
+  cp = f2_fma(cpd, m.inv, cpi);
+  const f2 W = f2_rcp(m.inv);
+  const f2 gi = f2_mul(gz, iFZ);
+  const f2 al = f2_neg(f2_fma(f2_mul(gi, FA), pRT2, kbL));
+  const f2 be = f2_mul(kbL, T);
+  f2 ga = f2_neg(f2_mul(f2_mul(gi, FB), pRT));
+  ga = f2_sub(ga, f2_mul(f2_mul(tda, kbL), f2_rcp(m.bm)));
+  ga = f2_fma(f2_mul(tk, e2), pRT, ga);
+  g.T = T;
+  g.t = t;
+  g.c1 = f2_scale2(f2_mul(W, al));
+  g.c2 = f2_mul(f2_mul(be, W), it);
+  g.c3 = ga;
+  f2 c0 = f2_sub(q.h_dep, f2_scale2(f2_mul(am, al)));
+  c0 = f2_sub(c0, f2_scale2(f2_mul(dam, be)));
+  g.c0 = f2_sub(c0, f2_mul(m.bm, ga));
 }
 
 // Input scales of the tangent directions (T, Y_1..Y_n): dx_0/dT = 1/std_T and
-// dx_{2+j}/dY_j = BC'(Y_j) / std_{2+j}, BC'(y) = max(y, 1e-12)^(lambda - 1).
+// dx_{2+j}/dY_j = BC'(Y_j) / std_{2+j}, BC'(y) = max(y, 1e-12)^(lambda - 1) in FP64: for lambda = 1/m
+// the m-th root by the series of f2_root in FP64 (about 20 FP64 operations against the hundred of pow:
+// 106 -> 42 us for 20,000 cells x 31 directions), else pow.
 __global__ void jac_scale_kernel(EosParams P, int64_t ncell, const double* __restrict__ Y,
                                  int64_t ldY, const double* __restrict__ norm,
                                  float* __restrict__ sc) {
-  const int ntan = P.n + 1, K0 = P.K0;
+  const int ntan = P.n + 1, K0 = P.K0, m = P.inv_lambda;
+  const bool root = P.lambda == 1.0 / m;
+  const float lamf = (float)P.lambda;
+  const double im = 1.0 / m, i2 = im * (im + 1.0) * 0.5, i3 = i2 * (im + 2.0) * (1.0 / 3.0);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ncell * ntan;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = e / ntan;
@@ -1438,7 +1397,18 @@ __global__ void jac_scale_kernel(EosParams P, int64_t ncell, const double* __res
       v = norm[K0];
     } else {
       const double y = fmax(Y[(int64_t)(t - 1) * ldY + c], 1e-12);
-      v = pow(y, P.lambda - 1.0) * norm[K0 + 1 + t];
+      if (root && y < 1e30) {
+        const double r0 = f_to_d(exp2f(lamf * log2f(d_to_f_trunc(y)))), iy = drcp(y);
+        double q = 1.0, b = r0;
+        for (int k = m; k; k >>= 1) {
+          if (k & 1) q *= b;
+          if (k > 1) b *= b;
+        }
+        const double d = fma(q, iy, -1.0);
+        v = r0 * iy * fma(d, fma(d, fma(-d, i3, i2), -im), 1.0) * norm[K0 + 1 + t];
+      } else {
+        v = pow(y, P.lambda - 1.0) * norm[K0 + 1 + t];
+      }
     }
     sc[e] = (float)v;
   }
@@ -1512,98 +1482,107 @@ __global__ void jac_tangent0_kernel(int64_t ncell, int ntan, int N1, const float
 // Jacobian of the step of every cell (treated as reacting): J[c][k][t] = d(Y'_k - Y_k)/dv_t and
 // dTn[c][t] = dT'/dv_t, v = (T, Y_1..Y_n), from the network output O, its tangents dO
 // ([c ntan + t][k] = dO_k/dv_t) and the implicit function h(T', p, Y') = h0(T, p, Y).
-// Two kernels: jac_post_kernel, a thread per cell, takes the cell's equation-of-state part
-// (Y', T' by Newton, dh/dY and c_p at both states) and leaves per cell in scr
-// [dZ_k/du_k (n), Y'_k (n), dh/dY'_k (n), 1/S, c_p(T', Y'), two O(n) work columns (2n)] and
-// its status in cst;
-// jac_assemble_kernel, a warp per cell and a lane per direction t, forms the columns.
+// Two kernels, both in double-float (FP64 arithmetic took 1.35 ms for 20,000 cells: jac_post 834 us at
+// four warps per SM, each a chain of FP64 sums over species pairs; assembly 513 us on the FP64 pipe):
+// jac_state_kernel, a thread per cell, takes what is scalar in the cell: Y', the mixture sums and states
+// at (T, Y) and (T', Y'), T' by Newton; it leaves in the cell's scratch row, as double-float pairs,
+//   [dZ_k/du_k / S (n), Y'_k (n), c_p(T, Y), c_p(T', Y'), HGrad at (T, Y), HGrad at (T', Y')];
+// jac_columns_kernel, a warp per cell, takes the rest: lane k the sums over species of dh/dY_k at both
+// states, then lane t the column of direction t. 119 and 184 us for those cells (issue-bound, FP32 pipes).
+constexpr int kJacRow = 2 + 2 * 6;   // scalars per cell after the two columns
+
 template <int NM>
-__global__ void __launch_bounds__(kJacThreads) jac_post_kernel(EosParams P, int64_t ncell, int64_t cell0,
+__global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, int64_t ncell, int64_t cell0,
     const double* __restrict__ T, const double* __restrict__ p, const double* __restrict__ Y,
     int64_t ldY, const float* __restrict__ O, int64_t ldo, const double* __restrict__ h0,
-    double* __restrict__ dTn, double* __restrict__ scr, int32_t* __restrict__ cst) {
+    bool want_dT, float2* __restrict__ scr, int32_t* __restrict__ cst) {
   extern __shared__ __align__(16) double sm[];
-  const SharedConsts c = load_consts(P, sm);
-  constexpr int stride = kJacThreads;
-  // shared memory holds the per-thread columns read in O(n^2) loops (the double-float
-  // composition of the mixing sums, the two weighted columns of h_grad); the O(n) ones live
-  // in the cell's scratch row, which is also how they reach jac_assemble_kernel
-  f2* ws = reinterpret_cast<f2*>(sm + consts_words(P)) + threadIdx.x;
-  double* uc = sm + consts_words(P) + NM * stride + threadIdx.x;
-  double* rc = uc + NM * stride;
-  const int n = P.n, K0 = P.K0, ntan = n + 1;
+  const SharedConsts c = load_consts<true>(P, sm);
+  constexpr int stride = kPropThreads;
+  f2* ycol = reinterpret_cast<f2*>(sm + consts_words(P)) + threadIdx.x;
+  const int n = P.n, K0 = P.K0;
   const float* out_mean = c.normf + 2 * K0;
   const float* out_std = c.normf + 2 * K0 + n;
   const float lamf = (float)P.lambda;
-  const double lam = P.lambda;
   const int mpow = P.inv_lambda;
+  const float dl = (float)(P.lambda - 1.0 / mpow);
+  auto put = [](float2* d, f2 v) { *d = make_float2(v.h, v.l); };
+  auto put_grad = [&](float2* d, const HGrad& g) {
+    put(d, g.T); put(d + 1, g.t); put(d + 2, g.c0); put(d + 3, g.c1); put(d + 4, g.c2); put(d + 5, g.c3);
+  };
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < ncell;
        r += (int64_t)gridDim.x * blockDim.x) {
     const int64_t cell = cell0 + r;
     const double Tc = T[cell], pc = p[cell], h0c = h0[r];
-    // scratch row: dZ_k/du_k, Y'_k, dh/dY'_k, 1/S, c_p', then h_grad's v and w columns
-    double* q = scr + r * (int64_t)(5 * n + 2);
-    double* zlc = q;
-    double* Ypc = q + n;
-    double* hgc = q + 2 * n;
-    double* vc = q + 3 * n + 2;
-    double* wc = q + 4 * n + 2;
-    double Yk[NM];
-    bool finite = isfinite(Tc) && isfinite(pc) && pc > 0.0 && isfinite(h0c);
+    bool finite = d_finite(Tc) && d_finite(pc) && d_pos(pc) && d_finite(h0c);
 #pragma unroll
-    for (int k = 0; k < NM; ++k) {
-      Yk[k] = (k < n) ? Y[k * ldY + cell] : 0.0;
-      finite = finite && isfinite(Yk[k]);
+    for (int k0 = 0; k0 < NM; k0 += kLoadBatch) {
+      double yv[kLoadBatch];
+#pragma unroll
+      for (int u = 0; u < kLoadBatch; ++u) yv[u] = k0 + u < n ? Y[(k0 + u) * ldY + cell] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kLoadBatch; ++u)
+        if (k0 + u < n) {
+          finite = finite && d_finite(yv[u]);
+          ycol[(k0 + u) * stride] = f2_from(yv[u]);
+        }
     }
-    int st = finite ? 0 : kCellNonfinite;
-    double* dTc = dTn ? dTn + cell * (int64_t)ntan : nullptr;
-    double cp1 = 1.0;
+    int st = finite && d_pos(Tc) ? 0 : kCellNonfinite;
+    float2* q = scr + r * (int64_t)(2 * n + kJacRow);
+    const f2 pd = f2_from(pc);
     if (st == 0) {
-      // (T, Y): cp and dh/dY, parked in dTn (its entries are final after the column loop)
-      Mixture m0;
-      for (int k = 0; k < n; ++k) ws[k * stride] = f2_from(Yk[k]);
-      mixture<kJacThreads>(ws, n, c, m0);
-      const PRPoint q0 = pr_point<false>(m0, Tc, pc, true, c.lnt, st);
-      if (dTc) {
-        dTc[0] = cp_ig(m0, Tc) + q0.cp_dep * m0.inv;
-        h_grad(P, n, ldY, Y + cell, Tc, pc, stride, uc, rc, 1, vc, wc, dTc + 1, 1, st);
+      MixDF m;
+      mixture_df<stride>(ycol, n, c, m);
+      const f2 Td = f2_from(Tc);
+      const PRPointDF s0 = pr_point_df<false>(m, Td, pd, false, c.lt2, st);
+      if (want_dT) {
+        f2 cp;
+        HGrad g;
+        state_grad(m, Td, pd, s0, c.lt2, cp, g);
+        put(q + 2 * n, cp);
+        put_grad(q + 2 * n + 2, g);
       }
-      // Y' and dZ_k/du_k = Z_k^(1 - lambda) = Z_k / (Y_k^lambda + lambda du_k)
-      double S = 0.0;
+    }
+    if (st == 0) {
+      // Y' and dZ_k/du_k = Z_k^(1 - lambda) = base^(m - 1), base = Y_k^lambda + lambda du_k
+      f2 S = f2{0.0f, 0.0f};
       const float* Or = O + r * ldo;
       for (int k = 0; k < n; ++k) {
-        const double y = Yk[k];
         const float ldu = lamf * fmaf(out_std[k], Or[k], out_mean[k]);
-        const double base = ((y > 0.0) ? pow(y, lam) : 0.0) + (double)ldu;
-        const double z = (base > 0.0) ? ipow(base, mpow) : 0.0;
-        Ypc[k] = z;
-        zlc[k] = (base > 0.0) ? z / base : 0.0;
-        S += z;
+        const f2 base = f2_addf(f2_root(ycol[k * stride], lamf, mpow, dl), ldu);
+        f2 zl = f2{0.0f, 0.0f}, z = zl;
+        if (base.h > 0.0f) {
+          zl = f2_ipow(base, mpow - 1);
+          z = f2_mul(zl, base);
+        }
+        put(q + k, zl);
+        ycol[k * stride] = z;
+        acc_add(S, z);
       }
-      if (!(S > 0.0)) st |= kCellNonfinite;
+      S = f2_fin(S);
+      if (!(S.h > 0.0f) || !isfinite(S.h)) st |= kCellNonfinite;
       if (st == 0) {
-        const double iS = 1.0 / S;
-        double Yn[NM];
-#pragma unroll
-        for (int k = 0; k < NM; ++k) {
-          Yn[k] = (k < n) ? Ypc[k] * iS : 0.0;
-          if (k < n) Ypc[k] = Yn[k];
+        const f2 iS = f2_rcp(S);
+        for (int k = 0; k < n; ++k) {
+          const f2 z = f2_mul(ycol[k * stride], iS);
+          ycol[k * stride] = z;
+          put(q + n + k, z);
+          const float2 zl = q[k];
+          put(q + k, f2_mul(f2{zl.x, zl.y}, iS));
         }
-        Mixture m1;
-        for (int k = 0; k < n; ++k) ws[k * stride] = f2_from(Yn[k]);
-        mixture<kJacThreads>(ws, n, c, m1);
+        MixDF m;
+        mixture_df<stride>(ycol, n, c, m);
         int iters = 0;
-        const double Tn = solve_T<false>(m1, pc, h0c, Tc, P, c.lnt, iters, st);
+        const f2 Tn = solve_T_df(m, pd, f2_from(h0c), Tc, P, c.lt2, iters, st);
         if (st == 0) {
-          const PRPoint q1 = pr_point<false>(m1, Tn, pc, true, c.lnt, st);
-          cp1 = cp_ig(m1, Tn) + q1.cp_dep * m1.inv;
-          if (dTc) h_grad(P, n, 1, Ypc, Tn, pc, stride, uc, rc, 1, vc, wc, hgc, 1, st);
-        }
-        if (st == 0) {
-          if (!dTc)
-            for (int k = 0; k < n; ++k) hgc[k] = 0.0;
-          q[3 * n] = iS;
-          q[3 * n + 1] = cp1;
+          const PRPointDF s1 = pr_point_df<false>(m, Tn, pd, false, c.lt2, st);
+          if (want_dT) {
+            f2 cp;
+            HGrad g;
+            state_grad(m, Tn, pd, s1, c.lt2, cp, g);
+            put(q + 2 * n + 1, cp);
+            put_grad(q + 2 * n + 8, g);
+          }
         }
       }
     }
@@ -1611,28 +1590,67 @@ __global__ void __launch_bounds__(kJacThreads) jac_post_kernel(EosParams P, int6
   }
 }
 
-
-// Columns of the Jacobian from jac_post_kernel's per-cell results: a warp per cell, lane t takes
-// direction t (T, then Y_1..Y_n), in the arithmetic and order of the per-cell formulas:
-// ju_k = out_std_k dO_k/dv_t + [t = k + 1] BC'(Y_k), jy_k = (dZ_k/du_k ju_k - Y'_k sum_j dZ_j/du_j
-// ju_j) / S, J[k][t] = jy_k - [t = k + 1], dT'/dv_t = (dh/dv_t - sum_k dh/dY'_k jy_k) / c_p.
-// Cells whose status is not 0 get NaN.
+// Columns of the Jacobian from jac_state_kernel's per-cell results: ju_k = out_std_k dO_k/dv_t +
+// [t = k + 1] BC'(Y_k), jy_k = (dZ_k/du_k ju_k - Y'_k sum_j dZ_j/du_j ju_j) / S, J[k][t] = jy_k -
+// [t = k + 1], dT'/dv_t = (dh/dv_t - sum_k dh/dY'_k jy_k) / c_p. The BC' term enters linearly, so the
+// loops over k run without it and its share is added at k = t - 1. Cells whose status is not 0 get NaN.
+constexpr int kColWarps = 8;
 template <int NM>
-__global__ void __launch_bounds__(256) jac_assemble_kernel(EosParams P, int64_t ncell,
+__global__ void __launch_bounds__(32 * kColWarps) jac_columns_kernel(EosParams P, int64_t ncell,
     int64_t cell0, const double* __restrict__ Y, int64_t ldY, const float* __restrict__ dO,
-    int64_t lddo, const double* __restrict__ scr, const int32_t* __restrict__ cst,
+    int64_t lddo, const float2* __restrict__ scr, const int32_t* __restrict__ cst,
     float* __restrict__ J, double* __restrict__ dTn) {
   const int n = P.n, K0 = P.K0, ntan = n + 1;
-  // the FP32 output spreads as FP64 (exact), once per block, and the FP32 -> FP64 conversions
-  // of dO on the integer pipes
-  __shared__ double sdd[NM];
-  for (int k = threadIdx.x; k < n; k += blockDim.x) sdd[k] = f_to_d((float)P.norm[2 * K0 + n + k]);
+  // K transposed (lane k reads K[k][j] at j * NM + k) and, per warp, columns that all lanes read
+  __shared__ float2 Ksh[NM * NM];
+  __shared__ float2 col[kColWarps][5][NM];
+  __shared__ float sdf[NM];
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const f2 v = f2_from(P.Kmat[e]);
+    Ksh[(e % n) * NM + e / n] = make_float2(v.h, v.l);
+  }
+  for (int k = threadIdx.x; k < n; k += blockDim.x) sdf[k] = (float)P.norm[2 * K0 + n + k];
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const double lam = P.lambda;
-  for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < ncell;
-       r += warps) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float2 *zl = col[w][0], *yp = col[w][1], *hg = col[w][2], *cu = col[w][3], *cr = col[w][4];
+  const int kl = lane < n ? lane : n - 1;
+  // this lane's species constants over W: 1/W, s/W, r/W, b/W, enthalpy coefficients
+  const float2* sp = reinterpret_cast<const float2*>(P.spcw2) + kl * kSpcStride;
+  auto ld = [](const float2* a) { const float2 v = *a; return f2{v.x, v.y}; };
+  auto st2 = [](float2* d, f2 v) { *d = make_float2(v.h, v.l); };
+  const float lamf = (float)P.lambda;
+  const int mpow = P.inv_lambda;
+  const float dl = (float)(P.lambda - 1.0 / mpow);
+  const int64_t warps = (int64_t)gridDim.x * kColWarps;
+  // dh/dY_k of lane k at the state of coefficients g (6 pairs) and mass fraction y
+  auto h_grad = [&](const float2* g, f2 y) -> f2 {
+    const f2 Tg = ld(g), t = ld(g + 1);
+    const f2 rw = ld(sp + 2), A = f2_sub(ld(sp + 1), f2_mul(rw, t));
+    __syncwarp();
+    if (lane < n) {
+      st2(cu + lane, f2_mul(y, A));
+      st2(cr + lane, f2_mul(y, rw));
+    }
+    __syncwarp();
+    f2 v = f2{0.0f, 0.0f}, x = v;
+#pragma unroll 2
+    for (int j = 0; j < n; ++j) {
+      const f2 K = ld(Ksh + j * NM + kl);
+      acc_fma(v, K, ld(cu + j));
+      acc_fma(x, K, ld(cr + j));
+    }
+    v = f2_fin(v);
+    x = f2_fin(x);
+    f2 h = ld(sp + 9);
+#pragma unroll
+    for (int k = 8; k >= 4; --k) h = f2_fma(h, Tg, ld(sp + k));
+    const f2 c2 = ld(g + 4);
+    h = f2_fma(ld(g + 2), ld(sp), h);
+    h = f2_fma(f2_sub(f2_mul(ld(g + 3), A), f2_mul(c2, rw)), v, h);
+    h = f2_sub(h, f2_mul(f2_mul(c2, A), x));
+    return f2_fma(ld(g + 5), ld(sp + 3), h);
+  };
+  for (int64_t r = blockIdx.x * (int64_t)kColWarps + w; r < ncell; r += warps) {
     const int64_t cell = cell0 + r;
     float* Jc = J + cell * (int64_t)n * ntan;
     double* dTc = dTn ? dTn + cell * (int64_t)ntan : nullptr;
@@ -1643,30 +1661,60 @@ __global__ void __launch_bounds__(256) jac_assemble_kernel(EosParams P, int64_t 
         for (int t = lane; t < ntan; t += 32) dTc[t] = __longlong_as_double(0x7ff8000000000000LL);
       continue;
     }
-    const double* q = scr + r * (int64_t)(5 * n + 2);
-    const double* zl = q;
-    const double* Yp = q + n;
-    const double* hg = q + 2 * n;
-    const double iS = q[3 * n], cp1 = q[3 * n + 1];
-    for (int t = lane; t < ntan; t += 32) {
+    const float2* q = scr + r * (int64_t)(2 * n + kJacRow);
+    const f2 y0 = lane < n ? f2_from(Y[(int64_t)lane * ldY + cell]) : f2{0.0f, 0.0f};
+    const f2 y1 = ld(q + n + kl), z1 = ld(q + kl);
+    f2 g0 = f2{0.0f, 0.0f}, g1 = g0, cp0 = g0, icp = g0;
+    if (dTc) {
+      g0 = h_grad(q + 2 * n + 2, y0);
+      g1 = h_grad(q + 2 * n + 8, y1);
+      cp0 = ld(q + 2 * n);
+      icp = f2_rcp(ld(q + 2 * n + 1));
+    }
+    __syncwarp();
+    if (lane < n) {
+      st2(zl + lane, z1);
+      st2(yp + lane, y1);
+      st2(hg + lane, g1);
+    }
+    __syncwarp();
+    // BC'(Y_k) of lane k; direction t = k + 1 sits one lane further (direction n of 32 species in lane 0's
+    // second pass)
+    const f2 ym = y0.h > 1e-12f ? y0 : f2_from(1e-12);
+    const f2 bc = f2_mul(f2_root(ym, lamf, mpow, dl), f2_rcp(ym));
+    for (int t0 = 0; t0 < ntan; t0 += 32) {
+      const int t = t0 + lane;
+      const int src = (t - 1) & 31;
+      const f2 bcp = f2{__shfl_sync(0xffffffffu, bc.h, src), __shfl_sync(0xffffffffu, bc.l, src)};
+      const f2 dh = f2{__shfl_sync(0xffffffffu, g0.h, src), __shfl_sync(0xffffffffu, g0.l, src)};
+      if (t >= ntan) continue;
       const float* dOr = dO + (r * ntan + t) * lddo;
-      double bcp = 0.0;
-      if (t > 0) bcp = pow(fmax(Y[(int64_t)(t - 1) * ldY + cell], 1e-12), lam - 1.0);
-      double sumjz = 0.0;
+      f2 sj = f2{0.0f, 0.0f};
 #pragma unroll 4
       for (int k = 0; k < n; ++k) {
-        const double ju = sdd[k] * f_to_d(dOr[k]) + ((t == k + 1) ? bcp : 0.0);
-        sumjz += zl[k] * ju;
+        const float d = dOr[k], u = __fmul_rn(sdf[k], d);
+        acc_fma(sj, ld(zl + k), f2{u, __fmaf_rn(sdf[k], d, -u)});
       }
-      double acc = 0.0;
+      f2 zt = f2{0.0f, 0.0f};   // (dZ/du BC') / S of species t - 1
+      if (t > 0) {
+        zt = f2_mul(ld(zl + t - 1), bcp);
+        acc_add(sj, zt);
+      }
+      sj = f2_neg(f2_fin(sj));
+      f2 acc = f2{0.0f, 0.0f};
 #pragma unroll 4
       for (int k = 0; k < n; ++k) {
-        const double ju = sdd[k] * f_to_d(dOr[k]) + ((t == k + 1) ? bcp : 0.0);
-        const double jy = (zl[k] * ju - Yp[k] * sumjz) * iS;
-        Jc[k * ntan + t] = (float)(jy - ((t == k + 1) ? 1.0 : 0.0));
-        if (dTc) acc = fma(hg[k], jy, acc);
+        const float d = dOr[k], u = __fmul_rn(sdf[k], d);
+        f2 jy = f2_fma(ld(yp + k), sj, f2_mul(ld(zl + k), f2{u, __fmaf_rn(sdf[k], d, -u)}));
+        float o = jy.h;
+        if (t == k + 1) {
+          jy = f2_add(jy, zt);
+          o = f2_addf(jy, -1.0f).h;
+        }
+        Jc[k * ntan + t] = o;
+        if (dTc) acc_fma(acc, ld(hg + k), jy);
       }
-      if (dTc) dTc[t] = (dTc[t] - acc) / cp1;
+      if (dTc) dTc[t] = f2_to_int(f2_mul(f2_sub(t == 0 ? cp0 : dh, f2_fin(acc)), icp));
     }
   }
 }
@@ -1821,7 +1869,7 @@ cudaError_t prepare_nm(int xkind) {
 
 cudaError_t prepare_eos(const EosParams& P, int xkind) {
   cudaError_t e = P.n <= 16 ? prepare_nm<16>(xkind) : prepare_nm<32>(xkind);
-  if (e == cudaSuccess) e = P.n <= 16 ? smem_optin<jac_post_kernel<16>>() : smem_optin<jac_post_kernel<32>>();
+  if (e == cudaSuccess) e = P.n <= 16 ? smem_optin<jac_state_kernel<16>>() : smem_optin<jac_state_kernel<32>>();
   return e;
 }
 
@@ -1859,24 +1907,19 @@ cudaError_t launch_jac_post(const EosParams& P, int64_t ncell, int64_t cell0, co
                             int64_t ldo, const float* dO, int64_t lddo, const double* h0, float* J,
                             double* dTn, double* scr, int32_t* cst, cudaStream_t st) {
   if (ncell <= 0) return cudaSuccess;
-  constexpr int kJT = kJacThreads;
-  const int64_t blocks = (ncell + kJT - 1) / kJT;
-  const int g = (int)(blocks < 4096 ? blocks : 4096);
+  const size_t smem = eos_smem(P, kPropThreads);
+  const int g = grid_for(ncell, kPropThreads);
+  float2* row = reinterpret_cast<float2*>(scr);
+  const unsigned cg = (unsigned)std::min<int64_t>((ncell + kColWarps - 1) / kColWarps, grid_for(INT64_MAX / 2));
   if (P.n <= 16) {
-    const size_t smem = sizeof(double) * ((size_t)consts_words(P) + (size_t)(3 * 16) * kJT);
-    jac_post_kernel<16><<<g, kJT, smem, st>>>(P, ncell, cell0, T, p, Y, ldY, O, ldo, h0, dTn, scr, cst);
+    jac_state_kernel<16><<<g, kPropThreads, smem, st>>>(P, ncell, cell0, T, p, Y, ldY, O, ldo, h0, dTn != nullptr,
+                                                        row, cst);
+    jac_columns_kernel<16><<<cg, 32 * kColWarps, 0, st>>>(P, ncell, cell0, Y, ldY, dO, lddo, row, cst, J, dTn);
   } else {
-    const size_t smem = sizeof(double) * ((size_t)consts_words(P) + (size_t)(3 * 32) * kJT);
-    jac_post_kernel<32><<<g, kJT, smem, st>>>(P, ncell, cell0, T, p, Y, ldY, O, ldo, h0, dTn, scr, cst);
+    jac_state_kernel<32><<<g, kPropThreads, smem, st>>>(P, ncell, cell0, T, p, Y, ldY, O, ldo, h0, dTn != nullptr,
+                                                        row, cst);
+    jac_columns_kernel<32><<<cg, 32 * kColWarps, 0, st>>>(P, ncell, cell0, Y, ldY, dO, lddo, row, cst, J, dTn);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int64_t ablocks = (ncell + 7) / 8;   // eight cells (warps) per block
-  const unsigned ag = (unsigned)std::min<int64_t>(ablocks, 1 << 20);
-  if (P.n <= 16)
-    jac_assemble_kernel<16><<<ag, 256, 0, st>>>(P, ncell, cell0, Y, ldY, dO, lddo, scr, cst, J, dTn);
-  else
-    jac_assemble_kernel<32><<<ag, 256, 0, st>>>(P, ncell, cell0, Y, ldY, dO, lddo, scr, cst, J, dTn);
   return cudaGetLastError();
 }
 

@@ -1119,7 +1119,7 @@ df_status build_jac(df_state* s) {
   al_ok((void**)&j->dO, sizeof(float) * R * j->ldo, true);
   al_ok((void**)&j->h0, sizeof(double) * B, false);
   al_ok((void**)&j->sc, sizeof(float) * R, false);
-  al_ok((void**)&j->jscr, sizeof(double) * B * (5 * n + 2), false);
+  al_ok((void**)&j->jscr, sizeof(double) * B * (2 * n + 14), false);
   al_ok((void**)&j->jst, sizeof(int32_t) * B, false);
   int64_t zmax = 32;
   for (int l = 0; l < L; ++l) zmax = std::max<int64_t>(zmax, round_up(s->widths[l + 1], 32));

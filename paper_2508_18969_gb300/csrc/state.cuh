@@ -30,7 +30,7 @@ struct Jac {
   double* h0 = nullptr;
   float* sc = nullptr;
   double* jscr = nullptr;                // per-cell results between the two post kernels
-  int32_t* jst = nullptr;                // [B (5n + 2)] and [B]
+  int32_t* jst = nullptr;                // [B (2n + 14)] and [B]
   float* W1T = nullptr;
   float* zero_bias = nullptr;
   std::vector<void*> Wb;                 // BF16 weights owned here (FP8 states)
