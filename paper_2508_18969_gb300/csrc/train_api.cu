@@ -75,13 +75,23 @@ bool trains(const df_state* s) {
 
 constexpr int kMaxSplit = 16;   // split-K of the weight-gradient GEMMs
 
-// Splits of a weight-gradient GEMM over the batch: about two waves of tiles on the GPU, no
-// split empty (an empty split would store an uninitialised accumulator).
-int wgrad_splits(int64_t tiles, int kblocks, int num_sms) {
-  int S = (int)std::min<int64_t>(kMaxSplit, std::max<int64_t>(1, (2 * num_sms + tiles - 1) / tiles));
-  S = std::min(S, std::max(1, kblocks / 8));
-  while (S > 1 && (int64_t)(S - 1) * ((kblocks + S - 1) / S) >= kblocks) --S;
-  return S;
+// Splits of a weight-gradient GEMM over the batch, whose few tiles (4 x 7 on 76 CTA pairs for the 1600 ->
+// 800 layer) leave a last wave nearly empty for most counts: the one with the least time in waves of
+// tiles, a split counted as half a per cent for its partial sums; no split empty (an empty split would
+// store an uninitialised accumulator) or shorter than eight k-blocks.
+int wgrad_splits(int64_t tiles, int kblocks, int slots) {
+  int best = 1;
+  double cost = 1e30;
+  for (int S = 1; S <= std::min(kMaxSplit, std::max(1, kblocks / 8)); ++S) {
+    const int per = (kblocks + S - 1) / S;
+    if ((int64_t)(S - 1) * per >= kblocks) continue;
+    const double c = (double)((tiles * S + slots - 1) / slots) * per * (1.0 + 0.005 * S);
+    if (c < cost) {
+      cost = c;
+      best = S;
+    }
+  }
+  return best;
 }
 
 void free_batch(Trn* t) {
