@@ -243,6 +243,38 @@ __device__ __forceinline__ void acc_renorm(float& h, float& l) {
   h = t;
 }
 
+// The same on two independent values with the packed FP32x2 instructions (one issue for both; the
+// rounding of each half is that of the scalar instruction, so the results are the scalar ones bit for
+// bit). a - b as fma(b, -1, a): one rounding, like the subtraction.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+}
+__device__ __forceinline__ void acc_off_fma2(float2& h, float2& l, float2 ah, float2 al, float2 bh,
+                                             float2 bl) {
+  const float2 s = __ffma2_rn(ah, bh, h);
+  const float2 r = __ffma2_rn(ah, bh, sub2(h, s));
+  l = __fadd2_rn(l, r);
+  l = __ffma2_rn(ah, bl, l);
+  l = __ffma2_rn(al, bh, l);
+  h = s;
+}
+__device__ __forceinline__ void acc_renorm2(float2& h, float2& l) {
+  const float2 t = __fadd2_rn(h, l);
+  l = sub2(l, sub2(t, h));
+  h = t;
+}
+__device__ __forceinline__ void norm2(float2 a, float2 b, float2& h, float2& l) {
+  h = __fadd2_rn(a, b);
+  l = sub2(b, sub2(h, a));
+}
+__device__ __forceinline__ void mul2(float2 ah, float2 al, float2 bh, float2 bl, float2& h, float2& l) {
+  const float2 p = __fmul2_rn(ah, bh);
+  float2 e = __ffma2_rn(ah, bh, __fmul2_rn(p, make_float2(-1.0f, -1.0f)));
+  e = __ffma2_rn(ah, bl, e);
+  e = __ffma2_rn(al, bh, e);
+  norm2(p, e, h, l);
+}
+
 // Smallest power of two >= x for a finite x >= 0 (the smallest normal for subnormal x).
 __device__ __forceinline__ float pow2_up(float x) {
   return __uint_as_float((__float_as_uint(x) + 0x007FFFFFu) & 0xFF800000u);

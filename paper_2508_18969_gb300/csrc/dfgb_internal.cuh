@@ -59,15 +59,20 @@ struct EosParams {
   const double* spc;
   const double* Kmat;
   const double* norm;
-  // Double-float (hi, lo) tables of the mixing sums, with 1/W folded in:
-  //   spcw2[k][j]: j = 0 1/W_k, 1 s_k/W_k, 2 r_k/W_k, 3 b_k/W_k, 4..9 hc_j/W_k;
-  //   K4 = (Ks hi, Ks lo, Kr hi, Kr lo) for the pairs j > i, row by row (row i from entry
-  //   i n - i (i + 1) / 2), with Ks_ij = (1 - k_ij) s_j / W_j, Kr_ij = (1 - k_ij) r_j / W_j;
-  //   kcol[j] = max_i |Ks_ij|, kcol[n + j] = max_i |Kr_ij| (rounded up by 2^-10: bounds for the
-  //   pair sums' accumulator offsets).
+  // Double-float (hi, lo) tables of the mixing sums, with 1/W folded in. Columns of a species: 0 1/W,
+  // 1 s/W, 2 r/W, 3 b/W, 4..9 hc_j/W. Packed arithmetic takes two sums at a time, so the kernels' tables
+  // put the hi parts of a pair side by side, then their lo parts:
+  //   spcw2[k][j] (hi, lo): the plain table (Jacobian columns);
+  //   spc4[k][5] float4: the pairs (0, 3), (4, 5), (6, 7), (8, 9), (1, 2);
+  //   K4: rows i of Ks_ij = (1 - k_ij) s_j / W_j and Kr_ij = (1 - k_ij) r_j / W_j over the species pairs
+  //   q = (2q, 2q + 1) with 2q + 1 > i, float4 (Ks, Ks', Ks lo, Ks' lo) then the same of Kr, entries
+  //   j <= i zero; row i starts where row i - 1 ends;
+  //   qabs[k][3] float4: |columns 0, 3, 4, 5|, |6, 7, 8, 9|, (max_i |Ks_ik|, max_i |Kr_ik|, rounded up by
+  //   2^-10), the bounds of the accumulators' offsets; zero rows pad an odd n.
   const float* spcw2;    // [n * kSpcStride * 2]
-  const float* K4;       // [2 n (n - 1)] (+ 4 floats of padding)
-  const float* kcol;     // [2 * n]
+  const float* spc4;     // [n * 20]
+  const float* K4;       // [8 * pair_blocks(n)]
+  const float* qabs;     // [12 * (n + (n & 1))]
   // FP32 pair corrections of the T-from-h solve, (k_ij s_j / W_j, k_ij r_j / W_j) for the
   // pairs j > i, row by row (row i from pair i n - i (i + 1) / 2)
   const float* kf2;      // [n (n - 1)] (+ 2 floats of padding)
@@ -86,6 +91,13 @@ struct EosParams {
   int64_t* flagged;      // device count of cells flagged by eos_post (may be NULL)
   int64_t* newton_iters; // device sum of Newton iterations (may be NULL)
 };
+
+// Blocks of the pair table K4: row i holds ceil(n / 2) - (i + 1) / 2 species pairs.
+__host__ __device__ constexpr int pair_blocks(int n) {
+  int c = 0;
+  for (int i = 0; i < n; ++i) c += (n + 1) / 2 - (i + 1) / 2;
+  return c;
+}
 
 enum XKind { kXF32 = 0, kXBF16 = 1, kXFP8 = 2 };
 

@@ -68,79 +68,91 @@ struct MixSums {
 };
 
 struct SharedConsts {
-  const f2* spcw;      // [n * kSpcStride] double-float species constants over W
-  const float4* K4;    // pairs j > i, row by row: (Ks, Kr) double-float, (1 - k_ij) s_j / W_j,
-                       // (1 - k_ij) r_j / W_j
-  const float* kcol;   // [2 n] max_i |Ks_ij|, then max_i |Kr_ij| (rounded up)
+  const float4* spc4;  // [5 n] EosParams::spc4
+  const float4* K4;    // EosParams::K4
+  const float4* qabs;  // EosParams::qabs
   const float2* kf2;   // pairs j > i: (k_ij s_j / W_j, k_ij r_j / W_j) in FP32 (T-from-h only)
   const double* lnt;   // [256] log table (ln c_j, then 1 / c_j); FP64 kernels only
   const f2* lt2;       // the same table in double-float, in the same words; DF kernels only
-  const double* norm;  // [2 K0 + 2 n]
-  const float* normf;  // the same in FP32 (for the FP32 feature and increment arithmetic)
+  const float* normf;  // normalisation constants [2 K0 + 2 n] in FP32
   const float* smax;   // [kSpcStride] EosParams::spcmax (T-from-h kernel only)
 };
 
-// 8-byte words of shared memory the constants take: FP64 normalisation, then the
-// double-float tables (one f2 per word), then the FP32 normalisation.
+// 8-byte words of shared memory the constants take (an even number: 16-byte columns follow): the log
+// table, then the species, pair and bound tables, then the normalisation in FP32.
 __host__ __device__ inline int consts_words(const EosParams& P) {
-  return 256 + 2 * P.K0 + 2 * P.n + P.n * kSpcStride + P.n * (P.n - 1) + 2 + P.n + (P.K0 + P.n + 1);
+  return (256 + 10 * P.n + 4 * pair_blocks(P.n) + 6 * (P.n + (P.n & 1)) + (P.K0 + P.n) + 1) & ~1;
 }
 
 // DF: the first 256 words hold the double-float log table (the kernels that evaluate the state
 // in double-float) instead of the FP64 one.
 template <bool DF = false>
 __device__ SharedConsts load_consts(const EosParams& P, double* sm0) {
-  const int nspc = P.n * kSpcStride, nk = P.n * P.n, nn = 2 * P.K0 + 2 * P.n;
+  const int nspc = 20 * P.n, nk = 8 * pair_blocks(P.n), na = 12 * (P.n + (P.n & 1)), nn = 2 * P.K0 + 2 * P.n;
   if (DF) {
     float* t = reinterpret_cast<float*>(sm0);
     for (int i = threadIdx.x; i < 512; i += blockDim.x) t[i] = P.lntab2[i];
   } else {
     for (int i = threadIdx.x; i < 256; i += blockDim.x) sm0[i] = P.lntab[i];
   }
-  double* sm = sm0 + 256;
-  for (int i = threadIdx.x; i < nn; i += blockDim.x) sm[i] = P.norm[i];
-  // fs is 16-byte aligned (256 + nn doubles; nn is even) and so is the pair table after
-  // the 8 n kSpcStride bytes of the species table
-  float* fs = reinterpret_cast<float*>(sm + nn);
-  for (int i = threadIdx.x; i < 2 * nspc; i += blockDim.x) fs[i] = P.spcw2[i];
-  const int nk4 = 2 * P.n * (P.n - 1) + 4;   // the triangle's floats, padded to 16 bytes
-  for (int i = threadIdx.x; i < nk4; i += blockDim.x) fs[2 * nspc + i] = P.K4[i];
-  for (int i = threadIdx.x; i < 2 * P.n; i += blockDim.x) fs[2 * nspc + nk4 + i] = P.kcol[i];
-  float* nf = fs + 2 * nspc + nk4 + 2 * P.n;
+  // 16-byte aligned, like every table after it (their sizes are multiples of four floats)
+  float* fs = reinterpret_cast<float*>(sm0 + 256);
+  for (int i = threadIdx.x; i < nspc; i += blockDim.x) fs[i] = P.spc4[i];
+  for (int i = threadIdx.x; i < nk; i += blockDim.x) fs[nspc + i] = P.K4[i];
+  for (int i = threadIdx.x; i < na; i += blockDim.x) fs[nspc + nk + i] = P.qabs[i];
+  float* nf = fs + nspc + nk + na;
   for (int i = threadIdx.x; i < nn; i += blockDim.x) nf[i] = (float)P.norm[i];
   __syncthreads();
-  return SharedConsts{reinterpret_cast<const f2*>(fs),
-                      reinterpret_cast<const float4*>(fs + 2 * nspc), fs + 2 * nspc + nk4,
-                      nullptr, DF ? nullptr : sm0,
-                      DF ? reinterpret_cast<const f2*>(sm0) : nullptr, sm, nf};
+  return SharedConsts{reinterpret_cast<const float4*>(fs), reinterpret_cast<const float4*>(fs + nspc),
+                      reinterpret_cast<const float4*>(fs + nspc + nk), nullptr, DF ? nullptr : sm0,
+                      DF ? reinterpret_cast<const f2*>(sm0) : nullptr, nf, nullptr};
 }
 
-// The layout of the T-from-h kernel: double-float log table, FP64 normalisation, double-float
-// species table, the FP32 k_ij pair table, FP32 normalisation (no double-float pair tables).
+// A thread's column of mass fractions in shared memory for mixture_sums: species pairs (2q, 2q + 1) as
+// float4 (hi, hi', lo, lo'), entry q at y4[q * STRIDE] (STRIDE the block's threads); a zero pads an odd n.
+template <int STRIDE>
+struct PairCol {
+  float4* y4;
+  __device__ __forceinline__ float* at(int k) const {
+    return reinterpret_cast<float*>(y4 + (k >> 1) * STRIDE) + (k & 1);
+  }
+  __device__ __forceinline__ f2 get(int k) const {
+    const float* p = at(k);
+    return f2{p[0], p[2]};
+  }
+  __device__ __forceinline__ void set(int k, f2 v) const {
+    float* p = at(k);
+    p[0] = v.h;
+    p[2] = v.l;
+  }
+  __device__ __forceinline__ void set_pair(int q, f2 a, f2 b) const {
+    y4[q * STRIDE] = make_float4(a.h, b.h, a.l, b.l);
+  }
+};
+
+// The layout of the T-from-h kernel: double-float log table, species table, the FP32 k_ij pair table,
+// FP32 normalisation (no double-float pair tables).
 __host__ __device__ inline int consts_words_post(const EosParams& P) {
-  return 256 + 2 * P.K0 + 2 * P.n + P.n * kSpcStride + P.n * (P.n - 1) / 2 + 1 +
-         (P.K0 + P.n + 1) + kSpcStride / 2;
+  return 256 + 10 * P.n + P.n * (P.n - 1) / 2 + 1 + (P.K0 + P.n) + kSpcStride / 2;
 }
 
 __device__ SharedConsts load_consts_post(const EosParams& P, double* sm0) {
-  const int nspc = P.n * kSpcStride, nn = 2 * P.K0 + 2 * P.n;
+  const int nspc = 20 * P.n, nn = 2 * P.K0 + 2 * P.n;
   float* t = reinterpret_cast<float*>(sm0);
   for (int i = threadIdx.x; i < 512; i += blockDim.x) t[i] = P.lntab2[i];
-  double* sm = sm0 + 256;
-  for (int i = threadIdx.x; i < nn; i += blockDim.x) sm[i] = P.norm[i];
-  float* fs = reinterpret_cast<float*>(sm + nn);
-  for (int i = threadIdx.x; i < 2 * nspc; i += blockDim.x) fs[i] = P.spcw2[i];
-  float* ks = fs + 2 * nspc;   // 8-byte aligned (8 n kSpcStride bytes after fs)
+  float* fs = reinterpret_cast<float*>(sm0 + 256);
+  for (int i = threadIdx.x; i < nspc; i += blockDim.x) fs[i] = P.spc4[i];
+  float* ks = fs + nspc;   // 16-byte aligned
   const int nkf = P.n * (P.n - 1) + 2;
   for (int i = threadIdx.x; i < nkf; i += blockDim.x) ks[i] = P.kf2[i];
   float* nf = ks + nkf;
   for (int i = threadIdx.x; i < nn; i += blockDim.x) nf[i] = (float)P.norm[i];
-  float* mx = nf + nn + 2;   // the FP32 normalisation takes K0 + n + 1 words
+  float* mx = nf + nn;
   for (int i = threadIdx.x; i < kSpcStride; i += blockDim.x) mx[i] = P.spcmax[i];
   __syncthreads();
-  return SharedConsts{reinterpret_cast<const f2*>(fs), nullptr, nullptr,
+  return SharedConsts{reinterpret_cast<const float4*>(fs), nullptr, nullptr,
                       reinterpret_cast<const float2*>(ks), nullptr,
-                      reinterpret_cast<const f2*>(sm0), sm, nf, mx};
+                      reinterpret_cast<const f2*>(sm0), nf, mx};
 }
 
 // FP64 reciprocal: FP32 seed, two FP64 Newton steps (relative error ~1 ulp).
@@ -153,135 +165,128 @@ __device__ __forceinline__ double drcp(double x) {
 }
 
 // Mixture coefficients of one composition (a1, a2 and the ideal-gas part of a4), all sums in
-// double-float. ycol is this thread's column of mass fractions (entry k at ycol[k * STRIDE], STRIDE
-// the block's threads).
+// double-float, two at a time with the packed FP32x2 instructions and 16-byte loads of species pairs.
+// The FP32 pipe takes a packed instruction in the time of two, so the gain is the loads, the broadcasts
+// and the issue slots: eos_pre 617 -> 599 us, eos_post 644 -> 616 us on 2^20 cells of 30 species, the
+// property kernel 211 -> 195 us on 2^18.
 // Symmetric quadratic forms with K_ii = 1, ys_i = Y_i s_i / W_i, yr_i = Y_i r_i / W_i:
 //   F0 = sum_ij K_ij ys_i ys_j = sum_i ys_i (ys_i + 2 P_i),  P_i = sum_{j>i} Ks_ij Y_j,
 //   F1 = sum_ij K_ij ys_i yr_j = sum_i ys_i (yr_i + Q_i) + yr_i P_i,  Q_i = sum_{j>i} Kr_ij Y_j,
 //   F2 = sum_ij K_ij yr_i yr_j = sum_i yr_i (yr_i + 2 Q_i).
-// The O(n^2) sums P_i and Q_i use offset accumulators (acc_off_fma) with one offset for all
-// rows: B = sum_j |Y_j| max_l |Ks_lj| (summed rounding up) bounds every partial sum of every
-// P_i (likewise for Q_i), and the offset is the power of two above B, or above 4 B when some
-// Y_j is negative. A row's error is then a few units of 2^-48 B rather than of its own suffix
-// bound, which the forms F weigh by ys_i <= B: the forms stay within ~2^-42 B^2, far inside the
-// 1e-10 the state is held to, for 16 fewer operations per row than per-row offsets.
-// Species i's terms of the O(n) sums (species-table columns 0 and 3..9) and its weighted mass
-// fractions ys_i = Y_i s_i / W_i, yr_i = Y_i r_i / W_i.
-__device__ __forceinline__ void species_row(const SharedConsts& c, int i, f2 y, float (&hq)[8],
-                                            float (&lq)[8], f2& ys, f2& yr) {
-  const float4* q4 = reinterpret_cast<const float4*>(c.spcw + i * kSpcStride);
-  const float4 a = q4[0], b = q4[1], d = q4[2], e = q4[3], g = q4[4];
-  acc_off_fma(hq[0], lq[0], y, f2{a.x, a.y});
-  acc_off_fma(hq[1], lq[1], y, f2{b.z, b.w});
-  acc_off_fma(hq[2], lq[2], y, f2{d.x, d.y});
-  acc_off_fma(hq[3], lq[3], y, f2{d.z, d.w});
-  acc_off_fma(hq[4], lq[4], y, f2{e.x, e.y});
-  acc_off_fma(hq[5], lq[5], y, f2{e.z, e.w});
-  acc_off_fma(hq[6], lq[6], y, f2{g.x, g.y});
-  acc_off_fma(hq[7], lq[7], y, f2{g.z, g.w});
-  ys = f2_mul(y, f2{a.z, a.w});
-  yr = f2_mul(y, f2{b.x, b.y});
-}
-
-// Species i's terms of the three forms: F0 += ys ys + ys (2 P), F1 += ys yr + ys Q + yr P,
-// F2 += yr yr + yr (2 Q).
-__device__ __forceinline__ void forms_row(f2 ys, f2 yr, f2 P, f2 Q, float& F0h, float& F0l,
-                                          float& F1h, float& F1l, float& F2h, float& F2l) {
-  acc_off_fma(F0h, F0l, ys, ys);
-  acc_off_fma(F0h, F0l, ys, f2_scale2(P));
-  acc_off_fma(F1h, F1l, ys, yr);
-  acc_off_fma(F1h, F1l, ys, Q);
-  acc_off_fma(F1h, F1l, yr, P);
-  acc_off_fma(F2h, F2l, yr, yr);
-  acc_off_fma(F2h, F2l, yr, f2_scale2(Q));
-}
-
+// The O(n^2) sums P_i and Q_i use offset accumulators (acc_off_fma), one for the even and one for the
+// odd species j, with one offset for all rows: B = sum_j |Y_j| max_l |Ks_lj| (summed rounding up) bounds
+// every partial sum of every P_i (likewise for Q_i), and the offset is the power of two above B, or above
+// 4 B when some Y_j is negative. The two accumulators' sums less their offsets are multiples of the same
+// 2^-23 (2^-24) of the offset and bounded by it, so their sum is exact. A row's error is then a few units
+// of 2^-48 B rather than of its own suffix bound, which the forms F weigh by ys_i <= B: the forms stay
+// within ~2^-42 B^2, far inside the 1e-10 the state is held to, for 16 fewer operations per row than
+// per-row offsets.
 template <int STRIDE>
-__device__ void mixture_sums(const f2* ycol, int n, const SharedConsts& c, MixSums& ms) {
-  constexpr int stride = STRIDE;   // threads per block: the column's entries are that far apart
+__device__ void mixture_sums(const PairCol<STRIDE> ycol, int n, const SharedConsts& c, MixSums& ms) {
+  const float4* y4 = ycol.y4;
+  const int nq = (n + 1) >> 1;
   // The O(n) sums (1/W, b/W and the six enthalpy coefficients, species-table columns 0 and 3..9)
   // take offset accumulators too, with bounds Bq = sum_j |Y_j| |q_j| from the same pass.
-  float Bs = 0.f, Br = 0.f, Bq[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) Bq[k] = 0.f;
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 Bsr = zero, Bq[4] = {zero, zero, zero, zero};
   unsigned neg = 0u;
 #pragma unroll 2
-  for (int j = 0; j < n; ++j) {
-    const float yh = ycol[j * stride].h, y = fabsf(yh);
-    neg |= __float_as_uint(yh);
-    const float4* q4 = reinterpret_cast<const float4*>(c.spcw + j * kSpcStride);
-    const float4 a = q4[0], b = q4[1], d = q4[2], e = q4[3], g = q4[4];
-    Bs = __fmaf_ru(y, c.kcol[j], Bs);
-    Br = __fmaf_ru(y, c.kcol[n + j], Br);
-    Bq[0] = __fmaf_ru(y, fabsf(a.x), Bq[0]);
-    Bq[1] = __fmaf_ru(y, fabsf(b.z), Bq[1]);
-    Bq[2] = __fmaf_ru(y, fabsf(d.x), Bq[2]);
-    Bq[3] = __fmaf_ru(y, fabsf(d.z), Bq[3]);
-    Bq[4] = __fmaf_ru(y, fabsf(e.x), Bq[4]);
-    Bq[5] = __fmaf_ru(y, fabsf(e.z), Bq[5]);
-    Bq[6] = __fmaf_ru(y, fabsf(g.x), Bq[6]);
-    Bq[7] = __fmaf_ru(y, fabsf(g.z), Bq[7]);
+  for (int q = 0; q < nq; ++q) {
+    const float4 v = y4[q * STRIDE];
+    neg |= __float_as_uint(v.x) | __float_as_uint(v.y);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const float y = fabsf(o ? v.y : v.x);
+      const float2 yy = make_float2(y, y);
+      const float4* t = c.qabs + 3 * (2 * q + o);
+      const float4 a = t[0], b = t[1], k = t[2];
+      Bsr = __ffma2_ru(yy, make_float2(k.x, k.y), Bsr);
+      Bq[0] = __ffma2_ru(yy, make_float2(a.x, a.y), Bq[0]);
+      Bq[1] = __ffma2_ru(yy, make_float2(a.z, a.w), Bq[1]);
+      Bq[2] = __ffma2_ru(yy, make_float2(b.x, b.y), Bq[2]);
+      Bq[3] = __ffma2_ru(yy, make_float2(b.z, b.w), Bq[3]);
+    }
   }
-  // the bounds are rounded up throughout; |Y_j| <= |hi| (1 + 2^-23) is inside kcol's margin,
+  const float Bs = Bsr.x, Br = Bsr.y;
+  // the bounds are rounded up throughout; |Y_j| <= |hi| (1 + 2^-23) is inside the column maxima's margin,
   // and the 2^-10 margin of the O(n) offsets covers the low parts of Y and of the table. The
   // terms are non-negative for Y >= 0 except in the enthalpy columns, whose coefficients have
   // either sign: those take the offset for terms of both signs.
   const float sgf = (neg >> 31) ? 4.0f : 1.0f;
-  float sq[8], hq[8], lq[8];
+  float2 sq[4], hq[4], lq[4];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    sq[k] = pow2_up(__fmul_ru((k < 2 ? sgf : 4.0f) * Bq[k], 1.0009765625f));
+  for (int k = 0; k < 4; ++k) {
+    const float f = k == 0 ? sgf : 4.0f;
+    sq[k] = make_float2(pow2_up(__fmul_ru(f * Bq[k].x, 1.0009765625f)), pow2_up(__fmul_ru(f * Bq[k].y, 1.0009765625f)));
     hq[k] = sq[k];
-    lq[k] = 0.f;
+    lq[k] = zero;
   }
   // The forms themselves: F0 += ys_i ys_i + ys_i (2 P_i), F1 += ys_i yr_i + ys_i Q_i + yr_i P_i,
-  // F2 += yr_i yr_i + yr_i (2 Q_i), each into an offset accumulator. The absolute values of the
-  // terms of F0 sum to sum_ij |K_ij| |ys_i| |ys_j| <= S_s Bs <= Bs^2, since S_s = sum_i |ys_i|
-  // <= Bs (K_jj = 1) and sum_j |K_ij| |ys_j| <= Bs for every i; likewise Bs Br bounds F1 and
+  // F2 += yr_i yr_i + yr_i (2 Q_i), each into an offset accumulator (F0 and F2 as a pair). The absolute
+  // values of the terms of F0 sum to sum_ij |K_ij| |ys_i| |ys_j| <= S_s Bs <= Bs^2, since S_s = sum_i
+  // |ys_i| <= Bs (K_jj = 1) and sum_j |K_ij| |ys_j| <= Bs for every i; likewise Bs Br bounds F1 and
   // Br^2 bounds F2.
-  const float sF0 = pow2_up(__fmul_ru(sgf, __fmul_ru(Bs, Bs)));
+  const float2 sF02 = make_float2(pow2_up(__fmul_ru(sgf, __fmul_ru(Bs, Bs))), pow2_up(__fmul_ru(sgf, __fmul_ru(Br, Br))));
   const float sF1 = pow2_up(__fmul_ru(sgf, __fmul_ru(Bs, Br)));
-  const float sF2 = pow2_up(__fmul_ru(sgf, __fmul_ru(Br, Br)));
-  float F0h = sF0, F0l = 0.f, F1h = sF1, F1l = 0.f, F2h = sF2, F2l = 0.f;
+  float2 F02h = sF02, F02l = zero;
+  float F1h = sF1, F1l = 0.f;
   const float sgs = pow2_up(sgf * Bs), sgr = pow2_up(sgf * Br);   // the rows' common offsets
+  const float4* kp = c.K4;
 #pragma unroll 1
   for (int i = 0; i < n; ++i) {
-    const f2 y = ycol[i * stride];
-    f2 ys, yr;
-    species_row(c, i, y, hq, lq, ys, yr);
-    float ph = sgs, pl = 0.f, qh = sgr, ql = 0.f;
-    const float4* Kr4 = c.K4 + (i * n - i * (i + 1) / 2) - (i + 1);   // Kr4[j], j > i
-#pragma unroll 4
-    for (int j = i + 1; j < n; ++j) {
-      const f2 yj = ycol[j * stride];
-      const float4 k = Kr4[j];
-      acc_off_fma(ph, pl, f2{k.x, k.y}, yj);
-      acc_off_fma(qh, ql, f2{k.z, k.w}, yj);
+    const float4 v = y4[(i >> 1) * STRIDE];
+    const float yh = (i & 1) ? v.y : v.x, yl = (i & 1) ? v.w : v.z;
+    const float2 yh2 = make_float2(yh, yh), yl2 = make_float2(yl, yl);
+    // the O(n) sums and ys_i = Y_i s_i / W_i, yr_i = Y_i r_i / W_i as a pair
+    const float4* t = c.spc4 + 5 * i;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 a = t[k];
+      acc_off_fma2(hq[k], lq[k], yh2, yl2, make_float2(a.x, a.y), make_float2(a.z, a.w));
     }
-    forms_row(ys, yr, f2_norm(__fsub_rn(ph, sgs), pl), f2_norm(__fsub_rn(qh, sgr), ql),
-              F0h, F0l, F1h, F1l, F2h, F2l);
+    const float4 sr = t[4];
+    float2 ysh, ysl;   // (ys, yr)
+    mul2(yh2, yl2, make_float2(sr.x, sr.y), make_float2(sr.z, sr.w), ysh, ysl);
+    float2 ph = make_float2(sgs, sgs), pl = zero, qh = make_float2(sgr, sgr), ql = zero;
+#pragma unroll 4
+    for (int q = (i + 1) >> 1; q < nq; ++q, kp += 2) {
+      const float4 yj = y4[q * STRIDE], a = kp[0], b = kp[1];
+      const float2 jh = make_float2(yj.x, yj.y), jl = make_float2(yj.z, yj.w);
+      acc_off_fma2(ph, pl, make_float2(a.x, a.y), make_float2(a.z, a.w), jh, jl);
+      acc_off_fma2(qh, ql, make_float2(b.x, b.y), make_float2(b.z, b.w), jh, jl);
+    }
+    float2 PQh, PQl;   // (P, Q)
+    norm2(make_float2(__fadd_rn(__fsub_rn(ph.x, sgs), __fsub_rn(ph.y, sgs)),
+                      __fadd_rn(__fsub_rn(qh.x, sgr), __fsub_rn(qh.y, sgr))),
+          make_float2(__fadd_rn(pl.x, pl.y), __fadd_rn(ql.x, ql.y)), PQh, PQl);
+    acc_off_fma2(F02h, F02l, ysh, ysl, ysh, ysl);
+    acc_off_fma2(F02h, F02l, ysh, ysl, __fadd2_rn(PQh, PQh), __fadd2_rn(PQl, PQl));
+    const f2 ys = f2{ysh.x, ysl.x}, yr = f2{ysh.y, ysl.y};
+    acc_off_fma(F1h, F1l, ys, yr);
+    acc_off_fma(F1h, F1l, ys, f2{PQh.y, PQl.y});
+    acc_off_fma(F1h, F1l, yr, f2{PQh.x, PQl.x});
     if ((i & 3) == 3) {  // every fourth species: keep the low parts small
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc_renorm(hq[k], lq[k]);
-      acc_renorm(F0h, F0l);
+      for (int k = 0; k < 4; ++k) acc_renorm2(hq[k], lq[k]);
+      acc_renorm2(F02h, F02l);
       acc_renorm(F1h, F1l);
-      acc_renorm(F2h, F2l);
     }
   }
-  const f2 F0 = f2_norm(__fsub_rn(F0h, sF0), F0l);
-  const f2 F1 = f2_norm(__fsub_rn(F1h, sF1), F1l);
-  const f2 F2 = f2_norm(__fsub_rn(F2h, sF2), F2l);
-  ms.inv = f2_norm(__fsub_rn(hq[0], sq[0]), lq[0]);
-  ms.bs = f2_norm(__fsub_rn(hq[1], sq[1]), lq[1]);
+  auto fin = [](float h, float sig, float l) { return f2_norm(__fsub_rn(h, sig), l); };
+  ms.F0 = fin(F02h.x, sF02.x, F02l.x);
+  ms.F1 = fin(F1h, sF1, F1l);
+  ms.F2 = fin(F02h.y, sF02.y, F02l.y);
+  ms.inv = fin(hq[0].x, sq[0].x, lq[0].x);
+  ms.bs = fin(hq[0].y, sq[0].y, lq[0].y);
 #pragma unroll
-  for (int k = 0; k < 6; ++k) ms.e[k] = f2_norm(__fsub_rn(hq[k + 2], sq[k + 2]), lq[k + 2]);
-  ms.F0 = F0;
-  ms.F1 = F1;
-  ms.F2 = F2;
+  for (int k = 0; k < 3; ++k) {
+    ms.e[2 * k] = fin(hq[k + 1].x, sq[k + 1].x, lq[k + 1].x);
+    ms.e[2 * k + 1] = fin(hq[k + 1].y, sq[k + 1].y, lq[k + 1].y);
+  }
 }
 
 template <int STRIDE>
-__device__ void mixture(const f2* ycol, int n, const SharedConsts& c, Mixture& m) {
+__device__ void mixture(const PairCol<STRIDE> ycol, int n, const SharedConsts& c, Mixture& m) {
   MixSums s;
   mixture_sums<STRIDE>(ycol, n, c, s);
   const double invd = f2_to(s.inv);
@@ -322,7 +327,7 @@ __device__ __forceinline__ void mix_df_final(const MixSums& s, MixDF& m) {
 }
 
 template <int STRIDE>
-__device__ void mixture_df(const f2* ycol, int n, const SharedConsts& c, MixDF& m) {
+__device__ void mixture_df(const PairCol<STRIDE> ycol, int n, const SharedConsts& c, MixDF& m) {
   MixSums s;
   mixture_sums<STRIDE>(ycol, n, c, s);
   mix_df_final(s, m);
@@ -358,21 +363,6 @@ __device__ __forceinline__ double dsqrt_pos(double x) {
 // corrections (k <= 0.1 of the squares) summed in FP32,
 //   F0 = S_s^2 - 2 sum_i ys_i Pk_i,  F1 = S_s S_r - sum_i (ys_i Qk_i + yr_i Pk_i),
 //   F2 = S_r^2 - 2 sum_i yr_i Qk_i,  Pk_i = sum_{j>i} k_ij ys_j,  Qk_i = sum_{j>i} k_ij yr_j.
-// Species i's terms of mixture_post's ten O(n) sums; q1, q2 return s_i / W_i and r_i / W_i.
-__device__ __forceinline__ void species_row_post(const SharedConsts& c, int i, f2 y,
-                                                 float (&hq)[kSpcStride], float (&lq)[kSpcStride],
-                                                 float& q1, float& q2) {
-  const float4* q4 = reinterpret_cast<const float4*>(c.spcw + i * kSpcStride);
-#pragma unroll
-  for (int k = 0; k < kSpcStride / 2; ++k) {
-    const float4 a = q4[k];
-    acc_off_fma(hq[2 * k], lq[2 * k], y, f2{a.x, a.y});
-    acc_off_fma(hq[2 * k + 1], lq[2 * k + 1], y, f2{a.z, a.w});
-    if (k == 0) q1 = a.z;
-    if (k == 1) q2 = a.x;
-  }
-}
-
 template <int STRIDE>
 __device__ void mixture_post(const f2* ycol, int n, const SharedConsts& c, MixDF& m) {
   constexpr int stride = STRIDE;
@@ -387,24 +377,32 @@ __device__ void mixture_post(const f2* ycol, int n, const SharedConsts& c, MixDF
     neg |= __float_as_uint(yh);
     S = __fadd_ru(S, fabsf(yh));
   }
-  float Bq[kSpcStride];
-#pragma unroll
-  for (int k = 0; k < kSpcStride; ++k) Bq[k] = __fmul_ru(S, c.smax[k]);
   // columns 0..3 (1/W, s/W, r/W, b/W) are non-negative; the enthalpy columns have either sign
   const float sgf = (neg >> 31) ? 4.0f : 1.0f;
-  float sq[kSpcStride], hq[kSpcStride], lq[kSpcStride];
+  auto sigma = [&](int col) {
+    return pow2_up(__fmul_ru((col < 4 ? sgf : 4.0f) * __fmul_ru(S, c.smax[col]), 1.0009765625f));
+  };
+  // the sums two at a time (packed), in the order of the species table's pairs
+  constexpr int colA[5] = {0, 4, 6, 8, 1}, colB[5] = {3, 5, 7, 9, 2};
+  float2 sq[5], hq[5], lq[5];
 #pragma unroll
-  for (int k = 0; k < kSpcStride; ++k) {
-    sq[k] = pow2_up(__fmul_ru((k < 4 ? sgf : 4.0f) * Bq[k], 1.0009765625f));
+  for (int k = 0; k < 5; ++k) {
+    sq[k] = make_float2(sigma(colA[k]), sigma(colB[k]));
     hq[k] = sq[k];
-    lq[k] = 0.f;
+    lq[k] = make_float2(0.f, 0.f);
   }
   float C0 = 0.f, C1 = 0.f, C2 = 0.f;
 #pragma unroll 1
   for (int i = 0; i < n; ++i) {
     const f2 y = ycol[i * stride];
-    float q1h, q2h;
-    species_row_post(c, i, y, hq, lq, q1h, q2h);
+    const float2 yh2 = make_float2(y.h, y.h), yl2 = make_float2(y.l, y.l);
+    const float4* t = c.spc4 + 5 * i;
+    float4 a;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      a = t[k];
+      acc_off_fma2(hq[k], lq[k], yh2, yl2, make_float2(a.x, a.y), make_float2(a.z, a.w));
+    }
     float Pk = 0.f, Qk = 0.f;
     const float2* R = c.kf2 + (i * n - i * (i + 1) / 2) - (i + 1);   // R[j], j > i
 #pragma unroll 4
@@ -416,16 +414,19 @@ __device__ void mixture_post(const f2* ycol, int n, const SharedConsts& c, MixDF
     }
     if ((i & 3) == 3) {  // every fourth species: keep the low parts small
 #pragma unroll
-      for (int k = 0; k < kSpcStride; ++k) acc_renorm(hq[k], lq[k]);
+      for (int k = 0; k < 5; ++k) acc_renorm2(hq[k], lq[k]);
     }
-    const float ysi = y.h * q1h, yri = y.h * q2h;
+    const float ysi = y.h * a.x, yri = y.h * a.y;   // s/W and r/W: the last pair
     C0 = fmaf(ysi, Pk, C0);
     C1 = fmaf(ysi, Qk, fmaf(yri, Pk, C1));
     C2 = fmaf(yri, Qk, C2);
   }
   f2 r[kSpcStride];
 #pragma unroll
-  for (int k = 0; k < kSpcStride; ++k) r[k] = f2_norm(__fsub_rn(hq[k], sq[k]), lq[k]);
+  for (int k = 0; k < 5; ++k) {
+    r[colA[k]] = f2_norm(__fsub_rn(hq[k].x, sq[k].x), lq[k].x);
+    r[colB[k]] = f2_norm(__fsub_rn(hq[k].y, sq[k].y), lq[k].y);
+  }
   const f2 inv = r[0], Ss = r[1], Sr = r[2], bs = r[3];
   const f2 Wm = f2_rcp(inv);
   const f2 W2 = f2_mul(Wm, Wm);
@@ -866,7 +867,7 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) eos_pre_kernel(EosParams
     int64_t ldx, float x_scale, int32_t* __restrict__ status, double* __restrict__ rho) {
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts<true>(P, sm);
-  f2* ycol = reinterpret_cast<f2*>(sm + consts_words(P)) + threadIdx.x;
+  const PairCol<kThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
   const int64_t nrow = valid_rows(rows);
   const int n = P.n, K0 = P.K0;
   const float lam = (float)P.lambda;
@@ -899,12 +900,12 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) eos_pre_kernel(EosParams
         if (k < n) {
           const double yd = yv[u];
           finite = finite && d_finite(yd);
-          ycol[k * kThreads] = f2_from(yd);
           if (xr && !xvec) {
             const float y = fmaxf(d_to_f_trunc(yd), 0.0f);
             const float bc = (y > 0.0f) ? (boxcox_pow<XT>(y, lam) - 1.0f) * ilam : -ilam;
             xr[2 + k] = to_x<XT>((bc - mf[2 + k]) * isf[2 + k], x_scale);
           }
+          if ((u & 1) == 0) ycol.set_pair(k >> 1, f2_from(yd), f2_from(yv[u + 1]));
         }
       }
     }
@@ -941,7 +942,7 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) eos_pre_kernel(EosParams
 #pragma unroll
         for (int k = 0; k < NM; ++k) {
           if (k < n) {
-            const float y = fmaxf(ycol[k * kThreads].h, 0.0f);
+            const float y = fmaxf(*ycol.at(k), 0.0f);
             const float bc = (y > 0.0f) ? (boxcox_pow<XT>(y, lam) - 1.0f) * ilam : -ilam;
             x_put(w, 2 + k, to_x<XT>((bc - mf[2 + k]) * isf[2 + k], x_scale));
           }
@@ -1130,12 +1131,13 @@ __global__ void __launch_bounds__(kPropThreads, kPropBlocks) props_kernel(EosPar
     int64_t ldY, double* rho, double* h, double* cp, double* Zo) {
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts(P, sm);
-  f2* ycol = reinterpret_cast<f2*>(sm + consts_words(P)) + threadIdx.x;
+  const PairCol<kPropThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
   const int n = P.n;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncell;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double Tc = T[i], pc = p[i];
-    for (int k = 0; k < n; ++k) ycol[k * kPropThreads] = f2_from(Y[k * ldY + i]);
+    for (int k = 0; k < n; k += 2)
+      ycol.set_pair(k >> 1, f2_from(Y[k * ldY + i]), k + 1 < n ? f2_from(Y[(k + 1) * ldY + i]) : f2{0.f, 0.f});
     Mixture m;
     mixture<kPropThreads>(ycol, n, c, m);
     int st = 0;
@@ -1215,18 +1217,17 @@ __global__ void __launch_bounds__(kPropThreads, kPropBlocks) transport_kernel(Eo
     int64_t ldY, double* mu, double* lam, double* alpha) {
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts(P, sm);
-  f2* ycol = reinterpret_cast<f2*>(sm + consts_words(P)) + threadIdx.x;
+  const PairCol<kPropThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
   const int n = P.n, nn = P.n * P.n;
-  constexpr int stride = kPropThreads;
   const float* __restrict__ tp = P.tpair;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncell;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double Tk = T[i], pk = p[i];
     bool finite = d_finite(Tk) && d_finite(pk) && d_pos(pk) && d_pos(Tk);
-    for (int k = 0; k < n; ++k) {
-      const double yk = Y[k * ldY + i];
-      finite = finite && d_finite(yk);
-      ycol[k * stride] = f2_from(yk);
+    for (int k = 0; k < n; k += 2) {
+      const double ya = Y[k * ldY + i], yb = k + 1 < n ? Y[(k + 1) * ldY + i] : 0.0;
+      finite = finite && d_finite(ya) && d_finite(yb);
+      ycol.set_pair(k >> 1, f2_from(ya), f2_from(yb));
     }
     double m_out = __longlong_as_double(0x7ff8000000000000LL), l_out = m_out, a_out = m_out;
     if (finite) {
@@ -1239,17 +1240,17 @@ __global__ void __launch_bounds__(kPropThreads, kPropBlocks) transport_kernel(Eo
       const double Wm = 1.0 / m.inv;
       // mole fractions x_k = (Y_k / W_k) W_mix, kept in the column's high words
       const float Wmf = (float)Wm;
-      for (int k = 0; k < n; ++k) ycol[k * stride].h = ycol[k * stride].h * c.spcw[k * kSpcStride].h * Wmf;
+      for (int k = 0; k < n; ++k) *ycol.at(k) = *ycol.at(k) * c.spc4[5 * k].x * Wmf;
       // Chung's mixing sums, symmetric: sum_ij x_i x_j A_ij = sum_i x_i (A_ii x_i + 2 sum_{j>i} A_ij x_j)
       double S[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
       for (int a = 0; a < n; ++a) {
-        const float xa = ycol[a * stride].h;
+        const float xa = *ycol.at(a);
         float R4[4];
 #pragma unroll
         for (int qq = 0; qq < 4; ++qq) R4[qq] = 0.5f * __ldg(tp + qq * nn + a * n + a) * xa;
         for (int b = a + 1; b < n; ++b) {
-          const float xb = ycol[b * stride].h;
+          const float xb = *ycol.at(b);
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq) R4[qq] = fmaf(__ldg(tp + qq * nn + a * n + b), xb, R4[qq]);
         }
@@ -1499,7 +1500,7 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts<true>(P, sm);
   constexpr int stride = kPropThreads;
-  f2* ycol = reinterpret_cast<f2*>(sm + consts_words(P)) + threadIdx.x;
+  const PairCol<stride> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
   const int n = P.n, K0 = P.K0;
   const float* out_mean = c.normf + 2 * K0;
   const float* out_std = c.normf + 2 * K0 + n;
@@ -1524,7 +1525,7 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       for (int u = 0; u < kLoadBatch; ++u)
         if (k0 + u < n) {
           finite = finite && d_finite(yv[u]);
-          ycol[(k0 + u) * stride] = f2_from(yv[u]);
+          if ((u & 1) == 0) ycol.set_pair((k0 + u) >> 1, f2_from(yv[u]), f2_from(yv[u + 1]));
         }
     }
     int st = finite && d_pos(Tc) ? 0 : kCellNonfinite;
@@ -1549,14 +1550,14 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       const float* Or = O + r * ldo;
       for (int k = 0; k < n; ++k) {
         const float ldu = lamf * fmaf(out_std[k], Or[k], out_mean[k]);
-        const f2 base = f2_addf(f2_root(ycol[k * stride], lamf, mpow, dl), ldu);
+        const f2 base = f2_addf(f2_root(ycol.get(k), lamf, mpow, dl), ldu);
         f2 zl = f2{0.0f, 0.0f}, z = zl;
         if (base.h > 0.0f) {
           zl = f2_ipow(base, mpow - 1);
           z = f2_mul(zl, base);
         }
         put(q + k, zl);
-        ycol[k * stride] = z;
+        ycol.set(k, z);
         acc_add(S, z);
       }
       S = f2_fin(S);
@@ -1564,8 +1565,8 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       if (st == 0) {
         const f2 iS = f2_rcp(S);
         for (int k = 0; k < n; ++k) {
-          const f2 z = f2_mul(ycol[k * stride], iS);
-          ycol[k * stride] = z;
+          const f2 z = f2_mul(ycol.get(k), iS);
+          ycol.set(k, z);
           put(q + n + k, z);
           const float2 zl = q[k];
           put(q + k, f2_mul(f2{zl.x, zl.y}, iS));
@@ -1720,9 +1721,9 @@ __global__ void __launch_bounds__(32 * kColWarps) jac_columns_kernel(EosParams P
 }
 
 // Dynamic shared memory of an EoS block of `threads` threads: constants and the per-thread
-// double-float column of mass fractions (n words per thread).
+// double-float column of mass fractions (n words per thread, rounded up to whole pairs).
 size_t eos_smem(const EosParams& P, int threads = kThreads) {
-  return sizeof(double) * ((size_t)consts_words(P) + (size_t)P.n * threads);
+  return sizeof(double) * ((size_t)consts_words(P) + (size_t)(P.n + (P.n & 1)) * threads);
 }
 
 size_t eos_smem_post(const EosParams& P) {

@@ -130,7 +130,7 @@ void free_state(df_state* s) {
   s->jac = nullptr;
   free_trn(s->trn);
   s->trn = nullptr;
-  f(s->d_spc); f(s->d_K); f(s->d_norm); f(s->d_spc2); f(s->d_K4); f(s->d_kcol); f(s->d_kf2); f(s->d_lntab); f(s->d_lntab2); f(s->d_tsp); f(s->d_tpair); f(s->d_gtab); f(s->d_err); f(s->d_count); f(s->d_flagged); f(s->d_iters);
+  f(s->d_spc); f(s->d_K); f(s->d_norm); f(s->d_spc2); f(s->d_K4); f(s->d_spc4); f(s->d_qabs); f(s->d_kf2); f(s->d_lntab); f(s->d_lntab2); f(s->d_tsp); f(s->d_tpair); f(s->d_gtab); f(s->d_err); f(s->d_count); f(s->d_flagged); f(s->d_iters);
   for (auto p : s->W32) f(p);
   for (auto p : s->bias) f(p);
   for (auto p : s->Wlp) f(p);
@@ -410,32 +410,47 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
       Kr[(size_t)i * n + j] = K[(size_t)i * n + j] * q[2] * q[0];
     }
   const std::vector<float> spcw2 = split(spcw), Ks2 = split(Ks), Kr2 = split(Kr);
-  // the pair tables interleaved per (i, j): (Ks hi, Ks lo, Kr hi, Kr lo), one 16-byte load,
-  // the strict upper triangle j > i only, row by row (row i starts at i n - i (i + 1) / 2);
-  // then the column maxima max_i |Ks_ij| and max_i |Kr_ij|, rounded up, for the accumulator
-  // offsets of the pair sums
-  std::vector<float> K4((size_t)2 * n * (n - 1) + 4), kcol((size_t)2 * n, 0.0f);
-  for (int i = 0, t = 0; i < n; ++i)
-    for (int j = i + 1; j < n; ++j, ++t) {
-      const size_t o = (size_t)i * n + j;
-      K4[4 * (size_t)t] = Ks2[2 * o];
-      K4[4 * (size_t)t + 1] = Ks2[2 * o + 1];
-      K4[4 * (size_t)t + 2] = Kr2[2 * o];
-      K4[4 * (size_t)t + 3] = Kr2[2 * o + 1];
+  // the kernels' packed tables (layouts at EosParams)
+  const int nq = (n + 1) / 2;
+  std::vector<float> spc4((size_t)n * 20), K4((size_t)8 * pair_blocks(n)), qabs((size_t)12 * 2 * nq, 0.0f);
+  for (int k = 0; k < n; ++k) {
+    static const int first[5] = {0, 4, 6, 8, 1}, second[5] = {3, 5, 7, 9, 2};
+    for (int u = 0; u < 5; ++u) {
+      const float* row = &spcw2[2 * (size_t)k * kSpcStride];
+      float* o = &spc4[20 * (size_t)k + 4 * u];
+      o[0] = row[2 * first[u]];
+      o[1] = row[2 * second[u]];
+      o[2] = row[2 * first[u] + 1];
+      o[3] = row[2 * second[u] + 1];
     }
+  }
+  for (int i = 0, t = 0; i < n; ++i)
+    for (int q = (i + 1) / 2; q < nq; ++q, ++t)
+      for (int o = 0; o < 2; ++o) {
+        const int j = 2 * q + o;
+        if (j <= i || j >= n) continue;
+        const size_t e = (size_t)i * n + j;
+        float* d = &K4[8 * (size_t)t];
+        d[o] = Ks2[2 * e];
+        d[2 + o] = Ks2[2 * e + 1];
+        d[4 + o] = Kr2[2 * e];
+        d[6 + o] = Kr2[2 * e + 1];
+      }
   // (a negative entry, k_ij > 1, makes terms of both signs even for Y >= 0: the maxima are
   // scaled by four, which is what the offset needs for terms of both signs)
   bool kneg = false;
   for (size_t o = 0; o < (size_t)n * n; ++o) kneg = kneg || Ks[o] < 0.0 || Kr[o] < 0.0;
   for (int j = 0; j < n; ++j) {
+    static const int cols[8] = {0, 3, 4, 5, 6, 7, 8, 9};
+    for (int u = 0; u < 8; ++u) qabs[12 * (size_t)j + u] = std::fabs(spcw2[2 * ((size_t)j * kSpcStride + cols[u])]);
     double ms = 0.0, mr = 0.0;
     for (int i = 0; i < n; ++i) {
       ms = std::max(ms, std::fabs(Ks[(size_t)i * n + j]));
       mr = std::max(mr, std::fabs(Kr[(size_t)i * n + j]));
     }
     const double f = (kneg ? 4.0 : 1.0) * (1.0 + 1.0 / 1024.0);
-    kcol[j] = (float)(ms * f);
-    kcol[n + j] = (float)(mr * f);
+    qabs[12 * (size_t)j + 8] = (float)(ms * f);
+    qabs[12 * (size_t)j + 9] = (float)(mr * f);
   }
   // FP32 pair corrections of the T-from-h solve, interleaved (k_ij s_j / W_j, k_ij r_j / W_j)
   // for the pairs j > i, row by row (row i from pair i n - i (i + 1) / 2)
@@ -507,10 +522,12 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
   CK(cudaMemcpy(s->d_kf2, kf2.data(), sizeof(float) * kf2.size(), cudaMemcpyHostToDevice), "copy");
   CK(dalloc(&s->d_spc2, spcw2.size()), "constants");
   CK(dalloc(&s->d_K4, K4.size()), "constants");
-  CK(dalloc(&s->d_kcol, kcol.size()), "constants");
+  CK(dalloc(&s->d_spc4, spc4.size()), "constants");
+  CK(dalloc(&s->d_qabs, qabs.size()), "constants");
   CK(cudaMemcpy(s->d_spc2, spcw2.data(), sizeof(float) * spcw2.size(), cudaMemcpyHostToDevice), "copy");
   CK(cudaMemcpy(s->d_K4, K4.data(), sizeof(float) * K4.size(), cudaMemcpyHostToDevice), "copy");
-  CK(cudaMemcpy(s->d_kcol, kcol.data(), sizeof(float) * kcol.size(), cudaMemcpyHostToDevice), "copy");
+  CK(cudaMemcpy(s->d_spc4, spc4.data(), sizeof(float) * spc4.size(), cudaMemcpyHostToDevice), "copy");
+  CK(cudaMemcpy(s->d_qabs, qabs.data(), sizeof(float) * qabs.size(), cudaMemcpyHostToDevice), "copy");
   CK(dalloc(&s->d_err, 1), "error word");
   CK(cudaMemset(s->d_err, 0, sizeof(int)), "memset");
   CK(dalloc(&s->d_count, 1), "counters");
@@ -540,7 +557,8 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
   P.norm = s->d_norm;
   P.spcw2 = s->d_spc2;
   P.K4 = s->d_K4;
-  P.kcol = s->d_kcol;
+  P.spc4 = s->d_spc4;
+  P.qabs = s->d_qabs;
   P.kf2 = s->d_kf2;
   for (int j = 0; j < kSpcStride; ++j) {
     float mx = 0.0f;

@@ -56,7 +56,8 @@ struct df_state {
   double* d_norm = nullptr;
   float* d_spc2 = nullptr;               // double-float mixing-sum tables (EosParams)
   float* d_K4 = nullptr;
-  float* d_kcol = nullptr;
+  float* d_spc4 = nullptr;
+  float* d_qabs = nullptr;
   float* d_kf2 = nullptr;                // FP32 k_ij pair table (EosParams)
   double* d_lntab = nullptr;             // log table (EosParams)
   float* d_lntab2 = nullptr;             // the log table in double-float pairs
