@@ -1125,27 +1125,117 @@ __global__ void __launch_bounds__(kThreads, kPostBlocks) eos_post_kernel(EosPara
   }
 }
 
+// Real-fluid c_p of the state q = pr_point_df(m, T, p) and the coefficients of dh/dY_k at fixed T, p.
+// With u_k = y_k sqrt(a_k), yr_k = y_k r_k (y = Y / W), v = K u, w = K yr, sigma = sum y = 1 / W:
+//   a = W^2 u.v,  a' = -(W^2 / sqrt T) yr.v,  b = W sum y_k b_k,
+//   da/dy_k = 2 W^2 sqrt(a_k) v_k - 2 W a,  db/dy_k = W (b_k - b),
+//   da'/dy_k = -2 W a' - (W^2 / sqrt T)(r_k v_k + sqrt(a_k) w_k),
+//   dZ from the implicit cubic, h = sum y_k h_k(T) + sigma h_dep,
+//   dh/dY_k = (h_k(T) + h_dep + sigma dh_dep/dy_k) / W_k.
+// h_dep depends on the composition through a, a' and b alone; with alpha, beta, gamma its derivatives,
+//   dh/dY_k = h_k/W_k + c0 / W_k + (c1 A_k - c2 R_k) v_k - c2 A_k w_k + c3 b_k / W_k,
+//   A_k = (s_k - r_k sqrt T) / W_k,  R_k = r_k / W_k,  c1 = 2 W alpha,  c2 = W beta / sqrt T,  c3 = gamma,
+//   c0 = h_dep - 2 a alpha - 2 a' beta - b gamma.
+struct HGrad {
+  f2 T, t, c0, c1, c2, c3;
+};
+
+template <bool GRAD>
+__device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPointDF& q, const f2* lt, f2& cp,
+                                        HGrad& g) {
+  const f2 iT = f2_rcp(T), t = f2_sqrt_pos(T), it = f2_mul(t, iT);
+  const f2 am = f2_fma(m.A1, f2{-2.0f * t.h, -2.0f * t.l}, f2_fma(m.A2, T, m.A0));
+  const f2 dam = f2_fma(f2_neg(m.A1), it, m.A2);
+  const f2 RT = f2_mul(T, f2{kRh, kRl}), iRT = f2_mul(iT, f2{kIRh, kIRl});
+  const f2 pRT = f2_mul(p, iRT), pRT2 = f2_mul(pRT, iRT);
+  const f2 A = f2_mul(am, pRT2), B = f2_mul(m.bm, pRT), Z = q.Z;
+  const f2 c1s = f2{kSPh, kSPl}, c2s = f2{kSMh, kSMl};
+  const f2 iZp = f2_rcp(f2_fma(B, c1s, Z)), iZm = f2_rcp(f2_fma(B, c2s, Z));
+  const f2 L = f2_log_tab(f2_mul(f2_fma(B, c1s, Z), iZm), lt);
+  const f2 tda = f2_fma(T, dam, f2_neg(am));
+  const f2 kbL = f2_mul(m.kb, L);
+  // f_Z, f_A, f_B of the cubic: 3 Z^2 - 2 (1 - B) Z + A - 3 B^2 - 2 B, Z - B, Z^2 - (6 B + 2) Z - (A - 2 B - 3 B^2)
+  const f2 B3 = f2_mul(B, f2_addf(f2_mulf(B, 3.0f), 2.0f));
+  const f2 FZ = f2_add(f2_mul(Z, f2_add(f2_mulf(Z, 3.0f), f2_scale2(f2_addf(B, -1.0f)))), f2_sub(A, B3));
+  const f2 FA = f2_sub(Z, B);
+  const f2 FB = f2_add(f2_mul(Z, f2_sub(Z, f2_addf(f2_mulf(B, 6.0f), 2.0f))), f2_sub(B3, A));
+  const f2 iFZ = f2_rcp(FZ);
+  const f2 e1 = f2_sub(iZp, iZm), e2 = f2_sub(f2_mul(c1s, iZp), f2_mul(c2s, iZm));
+  const f2 tk = f2_mul(tda, m.kb);
+  // dh_dep = gz dZ + kb L d(T a' - a) + T a' terms; dZ = -(FA dA + FB dB) / FZ
+  const f2 gz = f2_fma(tk, e1, RT);
+  // c_p: d/dT at fixed composition, dA = A (a'/a - 2/T) = p (a' - 2 a / T) / (RT)^2, dB = -B / T
+  const f2 d2am = f2_mul(f2_mulf(m.A1, 0.5f), f2_mul(it, iT));
+  const f2 dA = f2_mul(pRT2, f2_sub(dam, f2_scale2(f2_mul(am, iT))));
+  const f2 dB = f2_neg(f2_mul(B, iT));
+  const f2 dZ = f2_neg(f2_mul(iFZ, f2_fma(FA, dA, f2_mul(FB, dB))));
+  const f2 dL = f2_fma(dZ, e1, f2_mul(dB, e2));
+  const f2 Rf = f2{kRh, kRl};
+  f2 cpd = f2_mul(Rf, f2_addf(Z, -1.0f));
+  cpd = f2_fma(RT, dZ, cpd);
+  cpd = f2_fma(f2_mul(T, d2am), kbL, cpd);
+  cpd = f2_fma(tk, dL, cpd);
+  f2 cpi = f2_mulf(m.e[5], 5.0f);
+  cpi = f2_fma(cpi, T, f2_mulf(m.e[4], 4.0f));
+  cpi = f2_fma(cpi, T, f2_mulf(m.e[3], 3.0f));
+  cpi = f2_fma(cpi, T, f2_scale2(m.e[2]));
+  cpi = f2_fma(cpi, T, m.e[1]);
+  cp = f2_fma(cpd, m.inv, cpi);
+  if constexpr (!GRAD) return;
+  const f2 W = f2_rcp(m.inv);
+  const f2 gi = f2_mul(gz, iFZ);
+  const f2 al = f2_neg(f2_fma(f2_mul(gi, FA), pRT2, kbL));
+  const f2 be = f2_mul(kbL, T);
+  f2 ga = f2_neg(f2_mul(f2_mul(gi, FB), pRT));
+  ga = f2_sub(ga, f2_mul(f2_mul(tda, kbL), f2_rcp(m.bm)));
+  ga = f2_fma(f2_mul(tk, e2), pRT, ga);
+  g.T = T;
+  g.t = t;
+  g.c1 = f2_scale2(f2_mul(W, al));
+  g.c2 = f2_mul(f2_mul(be, W), it);
+  g.c3 = ga;
+  f2 c0 = f2_sub(q.h_dep, f2_scale2(f2_mul(am, al)));
+  c0 = f2_sub(c0, f2_scale2(f2_mul(dam, be)));
+  g.c0 = f2_sub(c0, f2_mul(m.bm, ga));
+}
+
+// Density, enthalpy, c_p and compressibility of every cell (outputs may be NULL), in double-float like
+// eos_pre (with the state in FP64 its pipe was busy half of the time and a thread loaded its mass
+// fractions two at a time: 195 -> 152 us for 2^18 cells of 30 species; errors against FP64 as before,
+// 1.7e-13 in density and 1.4e-13 in c_p: the mixing sums, double-float all along, set them).
 template <int NM>
-__global__ void __launch_bounds__(kPropThreads, kPropBlocks) props_kernel(EosParams P, int64_t ncell,
+__global__ void __launch_bounds__(kThreads, kPreBlocks) props_kernel(EosParams P, int64_t ncell,
     const double* __restrict__ T, const double* __restrict__ p, const double* __restrict__ Y,
     int64_t ldY, double* rho, double* h, double* cp, double* Zo) {
   extern __shared__ __align__(16) double sm[];
-  const SharedConsts c = load_consts(P, sm);
-  const PairCol<kPropThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
+  const SharedConsts c = load_consts<true>(P, sm);
+  const PairCol<kThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
   const int n = P.n;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncell;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double Tc = T[i], pc = p[i];
-    for (int k = 0; k < n; k += 2)
-      ycol.set_pair(k >> 1, f2_from(Y[k * ldY + i]), k + 1 < n ? f2_from(Y[(k + 1) * ldY + i]) : f2{0.f, 0.f});
-    Mixture m;
-    mixture<kPropThreads>(ycol, n, c, m);
+    const f2 Td = f2_from(T[i]), pd = f2_from(p[i]);
+#pragma unroll
+    for (int k0 = 0; k0 < NM; k0 += kLoadBatch) {
+      double yv[kLoadBatch];
+#pragma unroll
+      for (int u = 0; u < kLoadBatch; ++u) yv[u] = k0 + u < n ? Y[(k0 + u) * ldY + i] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kLoadBatch; u += 2)
+        if (k0 + u < n) ycol.set_pair((k0 + u) >> 1, f2_from(yv[u]), f2_from(yv[u + 1]));
+    }
+    MixDF m;
+    mixture_df<kThreads>(ycol, n, c, m);
     int st = 0;
-    const PRPoint q = pr_point(m, Tc, pc, cp != nullptr, c.lnt, st);
-    if (rho) rho[i] = pc / (m.inv * q.Z * kR * Tc);
-    if (h) h[i] = h_ig(m, Tc) + q.h_dep * m.inv;
-    if (cp) cp[i] = cp_ig(m, Tc) + q.cp_dep * m.inv;
-    if (Zo) Zo[i] = q.Z;
+    const PRPointDF q = pr_point_df<false>(m, Td, pd, false, c.lt2, st);
+    if (rho) rho[i] = f2_to_int(f2_mul(pd, f2_rcp(f2_mul(f2_mul(m.inv, q.Z), f2_mul(Td, f2{kRh, kRl})))));
+    if (h) h[i] = f2_to_int(f2_fma(q.h_dep, m.inv, h_ig_df(m, Td)));
+    if (cp) {
+      f2 cpv;
+      HGrad g;
+      state_grad<false>(m, Td, pd, q, c.lt2, cpv, g);
+      cp[i] = f2_to_int(cpv);
+    }
+    if (Zo) Zo[i] = f2_to_int(q.Z);
   }
 }
 
@@ -1304,78 +1394,6 @@ __device__ __forceinline__ f2 f2_root(f2 y, float lamf, int m, float dl) {
   f2 c = f2_mul(e, f2_rcp(f2{-(float)m, 0.0f}));
   c = f2_addf(c, dl != 0.0f ? q + dl * logf(y.h) : q);
   return f2_add(f2{r0, 0.0f}, f2_mulf(c, r0));
-}
-
-// Real-fluid c_p of the state q = pr_point_df(m, T, p) and the coefficients of dh/dY_k at fixed T, p.
-// With u_k = y_k sqrt(a_k), yr_k = y_k r_k (y = Y / W), v = K u, w = K yr, sigma = sum y = 1 / W:
-//   a = W^2 u.v,  a' = -(W^2 / sqrt T) yr.v,  b = W sum y_k b_k,
-//   da/dy_k = 2 W^2 sqrt(a_k) v_k - 2 W a,  db/dy_k = W (b_k - b),
-//   da'/dy_k = -2 W a' - (W^2 / sqrt T)(r_k v_k + sqrt(a_k) w_k),
-//   dZ from the implicit cubic, h = sum y_k h_k(T) + sigma h_dep,
-//   dh/dY_k = (h_k(T) + h_dep + sigma dh_dep/dy_k) / W_k.
-// h_dep depends on the composition through a, a' and b alone; with alpha, beta, gamma its derivatives,
-//   dh/dY_k = h_k/W_k + c0 / W_k + (c1 A_k - c2 R_k) v_k - c2 A_k w_k + c3 b_k / W_k,
-//   A_k = (s_k - r_k sqrt T) / W_k,  R_k = r_k / W_k,  c1 = 2 W alpha,  c2 = W beta / sqrt T,  c3 = gamma,
-//   c0 = h_dep - 2 a alpha - 2 a' beta - b gamma.
-struct HGrad {
-  f2 T, t, c0, c1, c2, c3;
-};
-
-__device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPointDF& q, const f2* lt, f2& cp,
-                                        HGrad& g) {
-  const f2 iT = f2_rcp(T), t = f2_sqrt_pos(T), it = f2_mul(t, iT);
-  const f2 am = f2_fma(m.A1, f2{-2.0f * t.h, -2.0f * t.l}, f2_fma(m.A2, T, m.A0));
-  const f2 dam = f2_fma(f2_neg(m.A1), it, m.A2);
-  const f2 RT = f2_mul(T, f2{kRh, kRl}), iRT = f2_mul(iT, f2{kIRh, kIRl});
-  const f2 pRT = f2_mul(p, iRT), pRT2 = f2_mul(pRT, iRT);
-  const f2 A = f2_mul(am, pRT2), B = f2_mul(m.bm, pRT), Z = q.Z;
-  const f2 c1s = f2{kSPh, kSPl}, c2s = f2{kSMh, kSMl};
-  const f2 iZp = f2_rcp(f2_fma(B, c1s, Z)), iZm = f2_rcp(f2_fma(B, c2s, Z));
-  const f2 L = f2_log_tab(f2_mul(f2_fma(B, c1s, Z), iZm), lt);
-  const f2 tda = f2_fma(T, dam, f2_neg(am));
-  const f2 kbL = f2_mul(m.kb, L);
-  // f_Z, f_A, f_B of the cubic: 3 Z^2 - 2 (1 - B) Z + A - 3 B^2 - 2 B, Z - B, Z^2 - (6 B + 2) Z - (A - 2 B - 3 B^2)
-  const f2 B3 = f2_mul(B, f2_addf(f2_mulf(B, 3.0f), 2.0f));
-  const f2 FZ = f2_add(f2_mul(Z, f2_add(f2_mulf(Z, 3.0f), f2_scale2(f2_addf(B, -1.0f)))), f2_sub(A, B3));
-  const f2 FA = f2_sub(Z, B);
-  const f2 FB = f2_add(f2_mul(Z, f2_sub(Z, f2_addf(f2_mulf(B, 6.0f), 2.0f))), f2_sub(B3, A));
-  const f2 iFZ = f2_rcp(FZ);
-  const f2 e1 = f2_sub(iZp, iZm), e2 = f2_sub(f2_mul(c1s, iZp), f2_mul(c2s, iZm));
-  const f2 tk = f2_mul(tda, m.kb);
-  // dh_dep = gz dZ + kb L d(T a' - a) + T a' terms; dZ = -(FA dA + FB dB) / FZ
-  const f2 gz = f2_fma(tk, e1, RT);
-  // c_p: d/dT at fixed composition, dA = A (a'/a - 2/T) = p (a' - 2 a / T) / (RT)^2, dB = -B / T
-  const f2 d2am = f2_mul(f2_mulf(m.A1, 0.5f), f2_mul(it, iT));
-  const f2 dA = f2_mul(pRT2, f2_sub(dam, f2_scale2(f2_mul(am, iT))));
-  const f2 dB = f2_neg(f2_mul(B, iT));
-  const f2 dZ = f2_neg(f2_mul(iFZ, f2_fma(FA, dA, f2_mul(FB, dB))));
-  const f2 dL = f2_fma(dZ, e1, f2_mul(dB, e2));
-  const f2 Rf = f2{kRh, kRl};
-  f2 cpd = f2_mul(Rf, f2_addf(Z, -1.0f));
-  cpd = f2_fma(RT, dZ, cpd);
-  cpd = f2_fma(f2_mul(T, d2am), kbL, cpd);
-  cpd = f2_fma(tk, dL, cpd);
-  f2 cpi = f2_mulf(m.e[5], 5.0f);
-  cpi = f2_fma(cpi, T, f2_mulf(m.e[4], 4.0f));
-  cpi = f2_fma(cpi, T, f2_mulf(m.e[3], 3.0f));
-  cpi = f2_fma(cpi, T, f2_scale2(m.e[2]));
-  cpi = f2_fma(cpi, T, m.e[1]);
-  cp = f2_fma(cpd, m.inv, cpi);
-  const f2 W = f2_rcp(m.inv);
-  const f2 gi = f2_mul(gz, iFZ);
-  const f2 al = f2_neg(f2_fma(f2_mul(gi, FA), pRT2, kbL));
-  const f2 be = f2_mul(kbL, T);
-  f2 ga = f2_neg(f2_mul(f2_mul(gi, FB), pRT));
-  ga = f2_sub(ga, f2_mul(f2_mul(tda, kbL), f2_rcp(m.bm)));
-  ga = f2_fma(f2_mul(tk, e2), pRT, ga);
-  g.T = T;
-  g.t = t;
-  g.c1 = f2_scale2(f2_mul(W, al));
-  g.c2 = f2_mul(f2_mul(be, W), it);
-  g.c3 = ga;
-  f2 c0 = f2_sub(q.h_dep, f2_scale2(f2_mul(am, al)));
-  c0 = f2_sub(c0, f2_scale2(f2_mul(dam, be)));
-  g.c0 = f2_sub(c0, f2_mul(m.bm, ga));
 }
 
 // Input scales of the tangent directions (T, Y_1..Y_n): dx_0/dT = 1/std_T and
@@ -1539,7 +1557,7 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       if (want_dT) {
         f2 cp;
         HGrad g;
-        state_grad(m, Td, pd, s0, c.lt2, cp, g);
+        state_grad<true>(m, Td, pd, s0, c.lt2, cp, g);
         put(q + 2 * n, cp);
         put_grad(q + 2 * n + 2, g);
       }
@@ -1580,7 +1598,7 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
           if (want_dT) {
             f2 cp;
             HGrad g;
-            state_grad(m, Tn, pd, s1, c.lt2, cp, g);
+            state_grad<true>(m, Tn, pd, s1, c.lt2, cp, g);
             put(q + 2 * n + 1, cp);
             put_grad(q + 2 * n + 8, g);
           }
@@ -1839,7 +1857,7 @@ cudaError_t props_nm(const EosParams& P, int64_t n, const double* T, const doubl
                      cudaStream_t st) {
   cudaError_t e = smem_optin<props_kernel<NM>>();
   if (e != cudaSuccess) return e;
-  props_kernel<NM><<<grid_for(n, kPropThreads), kPropThreads, eos_smem(P, kPropThreads), st>>>(
+  props_kernel<NM><<<grid_resident<props_kernel<NM>>(n, eos_smem(P)), kThreads, eos_smem(P), st>>>(
       P, n, T, p, Y, ldY, rho, h, cp, Z);
   return cudaGetLastError();
 }
