@@ -191,13 +191,13 @@ _EOS_OTHER = (("// -------------------------------------------------------------
               ("cudaError_t launch_jac_scale(", "cudaError_t launch_eos_post("),
               ("cudaError_t launch_transport(", "}  // namespace dfgb"))
 MEASURED_TRAFFIC = {
-    ("layer0", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c22bd239ff26b709", 3157.2),
-    ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c22bd239ff26b709", 4751.2),
-    ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c22bd239ff26b709", 2340.1),
-    ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c22bd239ff26b709", 1062.8),
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "c12e4383ce9da4a2", 292.1,
+    ("layer0", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 3157.3),
+    ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 4757.1),
+    ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 2346.0),
+    ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 1068.1),
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21", 293.3,
                                         _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "c12e4383ce9da4a2", 578.5,
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21", 582.5,
                                          _EOS_OTHER),
     # one block Gauss-Seidel sweep (gs_rhs_kernel + gs_sweep_kernel), per cell, FP64, 512 cells
     # per block row (profiles/solver_kernels_mesh-2m.md)
@@ -411,14 +411,14 @@ def measure_peaks_live(torch, dev):
 # MEASURED_TRAFFIC).
 MEASURED_PIPES = {
     # profiles/eos_kernels_layer1d-30sp-512k_bf16.md (full capture, 512K rows, first step)
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "c12e4383ce9da4a2",
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21",
                                         {"binding": "issue (FP32 double-float arithmetic)",
-                                         "fma_pipe": 0.484, "alu_pipe": 0.197, "fp64_pipe": 0.012,
-                                         "issue_active": 0.740, "warps_per_sm": 20.9}, _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "c12e4383ce9da4a2",
+                                         "fma_pipe": 0.526, "alu_pipe": 0.308, "fp64_pipe": 0.013,
+                                         "issue_active": 0.615, "warps_per_sm": 21.1}, _EOS_OTHER),
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21",
                                          {"binding": "issue (FP32 double-float arithmetic)",
-                                          "fma_pipe": 0.323, "alu_pipe": 0.527, "fp64_pipe": 0.037,
-                                          "issue_active": 0.722, "warps_per_sm": 22.3}, _EOS_OTHER),
+                                          "fma_pipe": 0.334, "alu_pipe": 0.557, "fp64_pipe": 0.037,
+                                          "issue_active": 0.712, "warps_per_sm": 22.2}, _EOS_OTHER),
 }
 
 

@@ -209,10 +209,11 @@ cudaError_t launch_colsum(int64_t R, int64_t C, const void* in, int64_t ld, int 
                           cudaStream_t st);
 // ---- launchers (compact.cu) ----
 constexpr int64_t kCompactChunk = 4096;   // cells per block of the compaction kernels
-// Stable list of cells with T > T_react. Needs scratch of compact_scratch_words(n) int64.
+// Stable list of cells with T > T_react; clears *zero0 and *zero1 (may be NULL). Needs scratch of compact_scratch_words(n) int64.
 int64_t compact_scratch_words(int64_t n);
 cudaError_t launch_compact(int64_t n, double T_react, const double* T, int32_t* idx,
-                           int64_t* count, int32_t* status, int64_t* scratch, cudaStream_t st);
+                           int64_t* count, int32_t* status, int64_t* scratch, cudaStream_t st,
+                           int64_t* zero0 = nullptr, int64_t* zero1 = nullptr);
 
 // ---- launchers (mlp_simt.cu) ----
 // C[r, c] = act(sum_k A[r, k] W[c, k] + bias[c]) for valid rows r < rows(map), c < N.

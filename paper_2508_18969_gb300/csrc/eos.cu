@@ -22,6 +22,7 @@
 //   * the Box-Cox features that feed the network are FP32 (they are quantised anyway).
 #include "dfgb_internal.cuh"
 #include "ddfloat.cuh"
+#include "pdl.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
@@ -868,6 +869,7 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) eos_pre_kernel(EosParams
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts<true>(P, sm);
   const PairCol<kThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
+  pdl_begin();   // the constants above do not change; the cells and rows do
   const int64_t nrow = valid_rows(rows);
   const int n = P.n, K0 = P.K0;
   const float lam = (float)P.lambda;
@@ -1012,6 +1014,7 @@ __global__ void __launch_bounds__(kThreads, kPostBlocks) eos_post_kernel(EosPara
   const SharedConsts c = load_consts_post(P, sm);
   f2* ycol = reinterpret_cast<f2*>(sm + consts_words_post(P)) + threadIdx.x;
   constexpr int stride = kThreads;
+  pdl_begin();
   const int64_t nrow = valid_rows(rows);
   const int n = P.n, K0 = P.K0;
   const float* out_mean = c.normf + 2 * K0;
@@ -1807,10 +1810,8 @@ cudaError_t pre_launch(const EosParams& P, const RowMap& rows, const double* T, 
                        float xs, int32_t* status, cudaStream_t st, double* rho) {
   cudaError_t e = smem_optin<eos_pre_kernel<NM, XT>>();
   if (e != cudaSuccess) return e;
-  eos_pre_kernel<NM, XT><<<grid_resident<eos_pre_kernel<NM, XT>>(rows.nmax, eos_smem(P)), kThreads,
-                           eos_smem(P), st>>>(
-      P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, rho);
-  return cudaGetLastError();
+  return pdl_launch(eos_pre_kernel<NM, XT>, grid_resident<eos_pre_kernel<NM, XT>>(rows.nmax, eos_smem(P)), kThreads,
+                    eos_smem(P), st, 1, P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, rho);
 }
 
 template <int NM>
@@ -1834,10 +1835,8 @@ cudaError_t post_nm(const EosParams& P, const RowMap& rows, const float* O, int6
                     const Source& src) {
   cudaError_t e = smem_optin<eos_post_kernel<NM>>();
   if (e != cudaSuccess) return e;
-  eos_post_kernel<NM><<<grid_resident<eos_post_kernel<NM>>(rows.nmax, eos_smem_post(P)), kThreads,
-                        eos_smem_post(P), st>>>(
-      P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, src);
-  return cudaGetLastError();
+  return pdl_launch(eos_post_kernel<NM>, grid_resident<eos_post_kernel<NM>>(rows.nmax, eos_smem_post(P)), kThreads,
+                    eos_smem_post(P), st, 1, P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, src);
 }
 
 template <int NM>

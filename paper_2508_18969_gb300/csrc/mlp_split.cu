@@ -33,6 +33,7 @@
 // eight epilogue warps (two per TMEM lane quarter, each holding every other 32-column chunk of its 32
 // rows: up to 128 FP32 accumulators a thread). Waits are bounded and drains complete as in mlp_tc.cu.
 #include "dfgb_internal.cuh"
+#include "pdl.cuh"
 #include "planes.cuh"
 #include "tc_ptx.cuh"
 
@@ -344,6 +345,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
   volatile int* abort = &abort_sh;
+  pdl_begin();
 
   const int64_t M = valid_rows(g.rows);
   const int64_t tiles_m = (M + BM - 1) / BM;
@@ -669,23 +671,10 @@ cudaError_t split_go(const SplitLayer& L, SplitArgs a, int num_sms, cudaStream_t
   if (items > 0x7FFFFFFF) return cudaErrorInvalidValue;
   if constexpr (C::kPair) {
     const int64_t nc = std::max<int64_t>(1, std::min<int64_t>(items, std::min(max_clusters, num_sms / 2)));
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * nc), 1, 1);
-    cfg.blockDim = dim3(C::kThreads, 1, 1);
-    cfg.dynamicSmemBytes = C::kSmem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, L.tmA, L.tmW[CFG], L.tmO, L.tmG, a);
+    return pdl_launch(kern, (unsigned)(2 * nc), C::kThreads, C::kSmem, st, 2, L.tmA, L.tmW[CFG], L.tmO, L.tmG, a);
   } else {
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, num_sms));
-    kern<<<grid, C::kThreads, C::kSmem, st>>>(L.tmA, L.tmW[CFG], L.tmO, L.tmG, a);
-    return cudaGetLastError();
+    return pdl_launch(kern, grid, C::kThreads, C::kSmem, st, 1, L.tmA, L.tmW[CFG], L.tmO, L.tmG, a);
   }
 }
 
@@ -716,6 +705,7 @@ cudaError_t split_pick(const SplitLayer& L, const SplitArgs& a, int num_sms, cud
 // (16 bytes of each plane) per thread.
 __global__ void split_rows_kernel(RowMap rm, int cols, const float* __restrict__ in, int64_t ldi,
                                   __nv_bfloat16* __restrict__ out, int64_t ldo, int64_t plane) {
+  pdl_begin();
   const int64_t rows = valid_rows(rm);
   const int groups = (int)(ldo >> 3);
   const int64_t total = rows * groups;
@@ -817,8 +807,7 @@ cudaError_t launch_split_rows(const RowMap& rows, int cols, const float* in, int
   if (ldo & 7) return cudaErrorInvalidValue;
   const int64_t total = rows.nmax * (ldo >> 3);
   const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, (int64_t)num_sms * 16));
-  split_rows_kernel<<<g, 256, 0, st>>>(rows, cols, in, ldi, (__nv_bfloat16*)out, ldo, plane);
-  return cudaGetLastError();
+  return pdl_launch(split_rows_kernel, g, 256, 0, st, 1, rows, cols, in, ldi, (__nv_bfloat16*)out, ldo, plane);
 }
 
 }  // namespace dfgb

@@ -22,6 +22,7 @@
 // is a launch argument (default ~1 s); the drains on the way out always allow the full ~1 s,
 // so copies and MMAs in flight land before the CTA frees its tensor memory and exits.
 #include "dfgb_internal.cuh"
+#include "pdl.cuh"
 #include "tc_ptx.cuh"
 
 #include <cuda_bf16.h>
@@ -354,6 +355,7 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
   volatile int* abort = &abort_sh;
+  pdl_begin();
 
   const int64_t M = valid_rows(g.rows);
   const int64_t tiles_m = (M + BM - 1) / BM;
@@ -647,24 +649,11 @@ cudaError_t launch_bn(const TcLayer& L, const TcArgs& a, int num_sms, cudaStream
     const int64_t units = items;
     const int64_t cap = std::min<int64_t>(max_clusters, num_sms / 2);
     const int64_t nc = std::max<int64_t>(1, std::min<int64_t>(units, cap));
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * nc), 1, 1);
-    cfg.blockDim = dim3(C::kThreads, 1, 1);
-    cfg.dynamicSmemBytes = C::kSmemBytes;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, L.tmA, L.tmB, L.tmO, tmG, a);
+    return pdl_launch(kern, (unsigned)(2 * nc), C::kThreads, C::kSmemBytes, st, 2, L.tmA, L.tmB, L.tmO, tmG, a);
   } else {
     const int64_t tiles = items;
     const unsigned grid = (unsigned)(tiles < num_sms ? (tiles > 0 ? tiles : 1) : num_sms);
-    kern<<<grid, C::kThreads, C::kSmemBytes, st>>>(L.tmA, L.tmB, L.tmO, tmG, a);
-    return cudaGetLastError();
+    return pdl_launch(kern, grid, C::kThreads, C::kSmemBytes, st, 1, L.tmA, L.tmB, L.tmO, tmG, a);
   }
 }
 

@@ -1,6 +1,7 @@
 // C ABI of libdfgb (include/df.h): state creation, the fused reaction step and the stage
 // entry points. Host code only orchestrates; every step of the path runs in the kernels
 // of eos.cu, compact.cu, mlp_simt.cu and mlp_tc.cu.
+#include "pdl.cuh"
 #include "state.cuh"
 #include "../../include/df_propnet.h"
 
@@ -85,6 +86,7 @@ int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair, bool mn)
 
 __global__ void cast_rows_kernel(int64_t rows, int K, const float* __restrict__ in,
                                  int64_t ldi, void* out, int64_t ldo, int kind, float scale) {
+  pdl_begin();
   const int64_t total = rows * ldo;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -102,8 +104,7 @@ cudaError_t launch_cast_rows(int64_t rows, int K, const float* in, int64_t ldi, 
   const int64_t total = rows * ldo;
   if (total <= 0) return cudaSuccess;
   const unsigned g = (unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms * 16);
-  cast_rows_kernel<<<g, 256, 0, st>>>(rows, K, in, ldi, out, ldo, kind, scale);
-  return cudaGetLastError();
+  return pdl_launch(cast_rows_kernel, g, 256, 0, st, 1, rows, K, in, ldi, out, ldo, kind, scale);
 }
 
 int xkind_of(int precision) {
@@ -885,13 +886,10 @@ df_status run_step(df_state* s, int64_t n_cells, double dt, double* T, const dou
   DeviceGuard guard(s->device);
   if ((rc = ensure_compact(s, n_cells)) != DF_OK) return rc;
   cudaError_t e = cudaSuccess;
-  if (!keep_counters) {
-    e = cudaMemsetAsync(s->d_flagged, 0, sizeof(int64_t), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_iters, 0, sizeof(int64_t), st);
-  }
-  if (e == cudaSuccess) {
+  {
     ProfScope ps(s, "compact", st);
-    e = launch_compact(n_cells, s->T_react, T, s->idx, s->d_count, cell_status, s->cscr, st);
+    e = launch_compact(n_cells, s->T_react, T, s->idx, s->d_count, cell_status, s->cscr, st,
+                       keep_counters ? nullptr : s->d_flagged, keep_counters ? nullptr : s->d_iters);
   }
   if (e != cudaSuccess) return cuda_fail(s, e, "reacting-cell compaction");
   const int xk = xkind_of(s->precision);
