@@ -195,9 +195,9 @@ MEASURED_TRAFFIC = {
     ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 4757.1),
     ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 2346.0),
     ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "46a8f9170ef14963", 1068.1),
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21", 293.3,
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342", 293.3,
                                         _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21", 582.5,
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342", 582.5,
                                          _EOS_OTHER),
     # one block Gauss-Seidel sweep (gs_rhs_kernel + gs_sweep_kernel), per cell, FP64, 512 cells
     # per block row (profiles/solver_kernels_mesh-2m.md)
@@ -411,11 +411,11 @@ def measure_peaks_live(torch, dev):
 # MEASURED_TRAFFIC).
 MEASURED_PIPES = {
     # profiles/eos_kernels_layer1d-30sp-512k_bf16.md (full capture, 512K rows, first step)
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21",
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342",
                                         {"binding": "issue (FP32 double-float arithmetic)",
                                          "fma_pipe": 0.526, "alu_pipe": 0.308, "fp64_pipe": 0.013,
                                          "issue_active": 0.615, "warps_per_sm": 21.1}, _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "adf15f6574976c21",
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342",
                                          {"binding": "issue (FP32 double-float arithmetic)",
                                           "fma_pipe": 0.334, "alu_pipe": 0.557, "fp64_pipe": 0.037,
                                           "issue_active": 0.712, "warps_per_sm": 22.2}, _EOS_OTHER),

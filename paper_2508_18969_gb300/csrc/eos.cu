@@ -24,6 +24,8 @@
 #include "ddfloat.cuh"
 #include "pdl.cuh"
 
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -39,6 +41,10 @@ constexpr double kInvR = 1.0 / kR;
 constexpr int kThreads = 256;
 constexpr int kPreBlocks = 3;    // resident blocks per SM the register budget is sized for
 constexpr int kPostBlocks = 3;
+// Launches that one wave of smaller blocks holds run blocks of 64 threads without a register cap instead:
+// four times the blocks, so that no SM is idle while another has eight warps, and room for the compiler
+// to overlap a thread's chains (rule in small_blocks).
+constexpr int kSmallThreads = 64;
 constexpr int kPropThreads = 128;  // the property and transport kernels
 constexpr int kPropBlocks = 5;
 constexpr int kCellNotConverged = 1;
@@ -85,22 +91,27 @@ __host__ __device__ inline int consts_words(const EosParams& P) {
   return (256 + 10 * P.n + 4 * pair_blocks(P.n) + 6 * (P.n + (P.n & 1)) + (P.K0 + P.n) + 1) & ~1;
 }
 
+// Copies `floats` floats (a multiple of four, both 16-byte aligned).
+__device__ __forceinline__ void copy_table(float* dst, const float* src, int floats) {
+  for (int i = threadIdx.x; i < floats / 4; i += blockDim.x)
+    reinterpret_cast<float4*>(dst)[i] = __ldg(reinterpret_cast<const float4*>(src) + i);
+}
+
 // DF: the first 256 words hold the double-float log table (the kernels that evaluate the state
 // in double-float) instead of the FP64 one.
 template <bool DF = false>
 __device__ SharedConsts load_consts(const EosParams& P, double* sm0) {
   const int nspc = 20 * P.n, nk = 8 * pair_blocks(P.n), na = 12 * (P.n + (P.n & 1)), nn = 2 * P.K0 + 2 * P.n;
   if (DF) {
-    float* t = reinterpret_cast<float*>(sm0);
-    for (int i = threadIdx.x; i < 512; i += blockDim.x) t[i] = P.lntab2[i];
+    copy_table(reinterpret_cast<float*>(sm0), P.lntab2, 512);
   } else {
     for (int i = threadIdx.x; i < 256; i += blockDim.x) sm0[i] = P.lntab[i];
   }
   // 16-byte aligned, like every table after it (their sizes are multiples of four floats)
   float* fs = reinterpret_cast<float*>(sm0 + 256);
-  for (int i = threadIdx.x; i < nspc; i += blockDim.x) fs[i] = P.spc4[i];
-  for (int i = threadIdx.x; i < nk; i += blockDim.x) fs[nspc + i] = P.K4[i];
-  for (int i = threadIdx.x; i < na; i += blockDim.x) fs[nspc + nk + i] = P.qabs[i];
+  copy_table(fs, P.spc4, nspc);
+  copy_table(fs + nspc, P.K4, nk);
+  copy_table(fs + nspc + nk, P.qabs, na);
   float* nf = fs + nspc + nk + na;
   for (int i = threadIdx.x; i < nn; i += blockDim.x) nf[i] = (float)P.norm[i];
   __syncthreads();
@@ -139,10 +150,9 @@ __host__ __device__ inline int consts_words_post(const EosParams& P) {
 
 __device__ SharedConsts load_consts_post(const EosParams& P, double* sm0) {
   const int nspc = 20 * P.n, nn = 2 * P.K0 + 2 * P.n;
-  float* t = reinterpret_cast<float*>(sm0);
-  for (int i = threadIdx.x; i < 512; i += blockDim.x) t[i] = P.lntab2[i];
+  copy_table(reinterpret_cast<float*>(sm0), P.lntab2, 512);
   float* fs = reinterpret_cast<float*>(sm0 + 256);
-  for (int i = threadIdx.x; i < nspc; i += blockDim.x) fs[i] = P.spc4[i];
+  copy_table(fs, P.spc4, nspc);
   float* ks = fs + nspc;   // 16-byte aligned
   const int nkf = P.n * (P.n - 1) + 2;
   for (int i = threadIdx.x; i < nkf; i += blockDim.x) ks[i] = P.kf2[i];
@@ -861,14 +871,14 @@ __device__ __forceinline__ float boxcox_pow(float y, float lam) {
 constexpr int kLoadBatch = 16;
 
 // a1-a5 for the valid rows of a batch.
-template <int NM, typename XT>
-__global__ void __launch_bounds__(kThreads, kPreBlocks) eos_pre_kernel(EosParams P, RowMap rows,
+template <int NM, typename XT, int TH>
+__global__ void __launch_bounds__(TH, TH == kThreads ? kPreBlocks : 1) eos_pre_kernel(EosParams P, RowMap rows,
     const double* __restrict__ T, const double* __restrict__ p, const double* __restrict__ Y,
     int64_t ldY, double* __restrict__ h0, double* __restrict__ Zout, XT* __restrict__ x,
     int64_t ldx, float x_scale, int32_t* __restrict__ status, double* __restrict__ rho) {
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts<true>(P, sm);
-  const PairCol<kThreads> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
+  const PairCol<TH> ycol{reinterpret_cast<float4*>(sm + consts_words(P)) + threadIdx.x};
   pdl_begin();   // the constants above do not change; the cells and rows do
   const int64_t nrow = valid_rows(rows);
   const int n = P.n, K0 = P.K0;
@@ -922,7 +932,7 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) eos_pre_kernel(EosParams
     double h = __longlong_as_double(0x7ff8000000000000LL), Z = h;
     if (finite) {
       MixDF m;
-      mixture_df<kThreads>(ycol, n, c, m);
+      mixture_df<TH>(ycol, n, c, m);
       const f2 Td = f2_from(Tc), pd = f2_from(pc);
       const PRPointDF q = pr_point_df<false>(m, Td, pd, false, c.lt2, st);
       Z = f2_to_int(q.Z);
@@ -1005,15 +1015,15 @@ __device__ __forceinline__ f2 yprime_small(double y, float lamf, float ldu, int 
 // a8-a10 for the valid rows of a batch. Y' lives in this thread's shared-memory column (double-
 // float) from the increment to the write-back, which happens only once the Newton solve for T
 // has succeeded.
-template <int NM>
-__global__ void __launch_bounds__(kThreads, kPostBlocks) eos_post_kernel(EosParams P, RowMap rows,
+template <int NM, int TH>
+__global__ void __launch_bounds__(TH, TH == kThreads ? kPostBlocks : 1) eos_post_kernel(EosParams P, RowMap rows,
     const float* __restrict__ O, int64_t ldo, const double* __restrict__ h0,
     double* __restrict__ T, const double* __restrict__ p, double* __restrict__ Y, int64_t ldY,
     const int32_t* __restrict__ pre_status, int32_t* __restrict__ cell_status, Source src) {
   extern __shared__ __align__(16) double sm[];
   const SharedConsts c = load_consts_post(P, sm);
   f2* ycol = reinterpret_cast<f2*>(sm + consts_words_post(P)) + threadIdx.x;
-  constexpr int stride = kThreads;
+  constexpr int stride = TH;
   pdl_begin();
   const int64_t nrow = valid_rows(rows);
   const int n = P.n, K0 = P.K0;
@@ -1100,7 +1110,7 @@ __global__ void __launch_bounds__(kThreads, kPostBlocks) eos_post_kernel(EosPara
       const f2 iS = f2_rcp(S);
       for (int k = 0; k < n; ++k) ycol[k * stride] = f2_mul(ycol[k * stride], iS);
       MixDF m;
-      mixture_post<kThreads>(ycol, n, c, m);
+      mixture_post<TH>(ycol, n, c, m);
       Tn = f2_to_int(solve_T_df(m, f2_from(pc), f2_from(h0c), Told, P, c.lt2, iters, st));
     }
     if (st == 0 && src.omega) {
@@ -1747,8 +1757,8 @@ size_t eos_smem(const EosParams& P, int threads = kThreads) {
   return sizeof(double) * ((size_t)consts_words(P) + (size_t)(P.n + (P.n & 1)) * threads);
 }
 
-size_t eos_smem_post(const EosParams& P) {
-  return sizeof(double) * ((size_t)consts_words_post(P) + (size_t)P.n * kThreads);
+size_t eos_smem_post(const EosParams& P, int threads) {
+  return sizeof(double) * ((size_t)consts_words_post(P) + (size_t)P.n * threads);
 }
 
 // Opts a kernel into more than 48 KB of dynamic shared memory, once per device.
@@ -1771,27 +1781,30 @@ cudaError_t smem_optin() {
   return cudaSuccess;
 }
 
-// Grid of a grid-stride kernel: one wave of the blocks that fit on the device at once (the
-// occupancy of Kern at kThreads threads and smem bytes), fewer when there is less work.
+// Blocks of Kern (threads threads, smem bytes) that fit on the device at once.
 template <auto Kern>
-int grid_resident(int64_t nmax, size_t smem) {
+int64_t resident_blocks(size_t smem, int threads) {
   static int per_sm[64] = {0};
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int nb = (dev >= 0 && dev < 64) ? per_sm[dev] : 0;
   if (nb <= 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kern, kThreads, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kern, threads, smem) != cudaSuccess ||
         nb <= 0) {
       cudaGetLastError();
       nb = 4;
     }
     if (dev >= 0 && dev < 64) per_sm[dev] = nb;
   }
-  int64_t need = (nmax + kThreads - 1) / kThreads;
-  const int64_t cap = (int64_t)sms * nb;
-  if (need < 1) need = 1;
-  return (int)(need < cap ? need : cap);
+  return (int64_t)sms * nb;
+}
+
+// Grid of a grid-stride kernel: one wave of its resident blocks, fewer when there is less work.
+template <auto Kern>
+int grid_resident(int64_t nmax, size_t smem, int threads = kThreads) {
+  const int64_t need = std::max<int64_t>(1, (nmax + threads - 1) / threads);
+  return (int)std::min(need, resident_blocks<Kern>(smem, threads));
 }
 
 int grid_for(int64_t nmax, int threads = kThreads) {
@@ -1804,14 +1817,34 @@ int grid_for(int64_t nmax, int threads = kThreads) {
   return (int)(need < cap ? need : cap);
 }
 
-template <int NM, typename XT>
+// Whether an eos_pre or eos_post launch of at most nmax rows takes small blocks: while one wave of them
+// holds the rows (a second one would cost more than the large blocks' fuller SMs save). Step of 20,011
+// cells of 30 species 218 -> 192 us, of 50,021 cells 336 -> 285 us, of 4,096 cells of 9 species 82.6 ->
+// 77.7 us; at 77,003 cells, beyond the wave, small blocks took 427 us against 408.
+template <auto Kern>
+bool small_blocks(int64_t nmax, size_t smem) {
+  return nmax <= resident_blocks<Kern>(smem, kSmallThreads) * kSmallThreads;
+}
+
+template <int NM, typename XT, int TH>
 cudaError_t pre_launch(const EosParams& P, const RowMap& rows, const double* T, const double* p,
                        const double* Y, int64_t ldY, double* h0, double* Z, XT* x, int64_t ldx,
                        float xs, int32_t* status, cudaStream_t st, double* rho) {
-  cudaError_t e = smem_optin<eos_pre_kernel<NM, XT>>();
+  constexpr auto kern = eos_pre_kernel<NM, XT, TH>;
+  cudaError_t e = smem_optin<kern>();
   if (e != cudaSuccess) return e;
-  return pdl_launch(eos_pre_kernel<NM, XT>, grid_resident<eos_pre_kernel<NM, XT>>(rows.nmax, eos_smem(P)), kThreads,
-                    eos_smem(P), st, 1, P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, rho);
+  const size_t smem = eos_smem(P, TH);
+  return pdl_launch(kern, grid_resident<kern>(rows.nmax, smem, TH), TH, smem, st, 1, P, rows, T, p, Y, ldY, h0, Z, x,
+                    ldx, xs, status, rho);
+}
+
+template <int NM, typename XT>
+cudaError_t pre_th(const EosParams& P, const RowMap& rows, const double* T, const double* p,
+                   const double* Y, int64_t ldY, double* h0, double* Z, XT* x, int64_t ldx,
+                   float xs, int32_t* status, cudaStream_t st, double* rho) {
+  return small_blocks<eos_pre_kernel<NM, XT, kSmallThreads>>(rows.nmax, eos_smem(P, kSmallThreads))
+             ? pre_launch<NM, XT, kSmallThreads>(P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, st, rho)
+             : pre_launch<NM, XT, kThreads>(P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, st, rho);
 }
 
 template <int NM>
@@ -1820,12 +1853,25 @@ cudaError_t pre_nm(const EosParams& P, const RowMap& rows, const double* T, cons
                    int64_t ldx, float xs, int32_t* status, cudaStream_t st, double* rho) {
   switch (xkind) {
     case kXBF16:
-      return pre_launch<NM>(P, rows, T, p, Y, ldY, h0, Z, (__nv_bfloat16*)x, ldx, xs, status, st, rho);
+      return pre_th<NM>(P, rows, T, p, Y, ldY, h0, Z, (__nv_bfloat16*)x, ldx, xs, status, st, rho);
     case kXFP8:
-      return pre_launch<NM>(P, rows, T, p, Y, ldY, h0, Z, (__nv_fp8_e4m3*)x, ldx, xs, status, st, rho);
+      return pre_th<NM>(P, rows, T, p, Y, ldY, h0, Z, (__nv_fp8_e4m3*)x, ldx, xs, status, st, rho);
     default:
-      return pre_launch<NM>(P, rows, T, p, Y, ldY, h0, Z, (float*)x, ldx, xs, status, st, rho);
+      return pre_th<NM>(P, rows, T, p, Y, ldY, h0, Z, (float*)x, ldx, xs, status, st, rho);
   }
+}
+
+template <int NM, int TH>
+cudaError_t post_launch(const EosParams& P, const RowMap& rows, const float* O, int64_t ldo,
+                        const double* h0, double* T, const double* p, double* Y, int64_t ldY,
+                        const int32_t* pre_status, int32_t* cell_status, cudaStream_t st,
+                        const Source& src) {
+  constexpr auto kern = eos_post_kernel<NM, TH>;
+  cudaError_t e = smem_optin<kern>();
+  if (e != cudaSuccess) return e;
+  const size_t smem = eos_smem_post(P, TH);
+  return pdl_launch(kern, grid_resident<kern>(rows.nmax, smem, TH), TH, smem, st, 1, P, rows, O, ldo, h0, T, p, Y,
+                    ldY, pre_status, cell_status, src);
 }
 
 template <int NM>
@@ -1833,10 +1879,9 @@ cudaError_t post_nm(const EosParams& P, const RowMap& rows, const float* O, int6
                     const double* h0, double* T, const double* p, double* Y, int64_t ldY,
                     const int32_t* pre_status, int32_t* cell_status, cudaStream_t st,
                     const Source& src) {
-  cudaError_t e = smem_optin<eos_post_kernel<NM>>();
-  if (e != cudaSuccess) return e;
-  return pdl_launch(eos_post_kernel<NM>, grid_resident<eos_post_kernel<NM>>(rows.nmax, eos_smem_post(P)), kThreads,
-                    eos_smem_post(P), st, 1, P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, src);
+  return small_blocks<eos_post_kernel<NM, kSmallThreads>>(rows.nmax, eos_smem_post(P, kSmallThreads))
+             ? post_launch<NM, kSmallThreads>(P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, st, src)
+             : post_launch<NM, kThreads>(P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, st, src);
 }
 
 template <int NM>
@@ -1873,13 +1918,19 @@ cudaError_t launch_eos_pre(const EosParams& P, const RowMap& rows, const double*
   return pre_nm<32>(P, rows, T, p, Y, ldY, h0, Z, x, xkind, ldx, x_scale, status, st, rho);
 }
 
+template <int NM, int TH>
+cudaError_t prepare_step(int xkind) {
+  cudaError_t e = xkind == kXBF16  ? smem_optin<eos_pre_kernel<NM, __nv_bfloat16, TH>>()
+                  : xkind == kXFP8 ? smem_optin<eos_pre_kernel<NM, __nv_fp8_e4m3, TH>>()
+                                   : smem_optin<eos_pre_kernel<NM, float, TH>>();
+  if (e == cudaSuccess) e = smem_optin<eos_pre_kernel<NM, float, TH>>();  // stage entry point
+  return e == cudaSuccess ? smem_optin<eos_post_kernel<NM, TH>>() : e;
+}
+
 template <int NM>
 cudaError_t prepare_nm(int xkind) {
-  cudaError_t e = xkind == kXBF16  ? smem_optin<eos_pre_kernel<NM, __nv_bfloat16>>()
-                  : xkind == kXFP8 ? smem_optin<eos_pre_kernel<NM, __nv_fp8_e4m3>>()
-                                   : smem_optin<eos_pre_kernel<NM, float>>();
-  if (e == cudaSuccess) e = smem_optin<eos_pre_kernel<NM, float>>();  // stage entry point
-  if (e == cudaSuccess) e = smem_optin<eos_post_kernel<NM>>();
+  cudaError_t e = prepare_step<NM, kThreads>(xkind);
+  if (e == cudaSuccess) e = prepare_step<NM, kSmallThreads>(xkind);
   if (e == cudaSuccess) e = smem_optin<props_kernel<NM>>();
   if (e == cudaSuccess) e = smem_optin<transport_kernel<NM>>();
   return e;
@@ -1983,10 +2034,10 @@ int64_t eos_wave_cells(const EosParams& P, int xkind) {
     return (int64_t)sms * nb * kThreads;
   };
   if (P.n <= 16)
-    return xkind == kXBF16 ? wave(eos_pre_kernel<16, __nv_bfloat16>)
-           : xkind == kXFP8 ? wave(eos_pre_kernel<16, __nv_fp8_e4m3>) : wave(eos_pre_kernel<16, float>);
-  return xkind == kXBF16 ? wave(eos_pre_kernel<32, __nv_bfloat16>)
-         : xkind == kXFP8 ? wave(eos_pre_kernel<32, __nv_fp8_e4m3>) : wave(eos_pre_kernel<32, float>);
+    return xkind == kXBF16 ? wave(eos_pre_kernel<16, __nv_bfloat16, kThreads>)
+           : xkind == kXFP8 ? wave(eos_pre_kernel<16, __nv_fp8_e4m3, kThreads>) : wave(eos_pre_kernel<16, float, kThreads>);
+  return xkind == kXBF16 ? wave(eos_pre_kernel<32, __nv_bfloat16, kThreads>)
+         : xkind == kXFP8 ? wave(eos_pre_kernel<32, __nv_fp8_e4m3, kThreads>) : wave(eos_pre_kernel<32, float, kThreads>);
 }
 
 }  // namespace dfgb
