@@ -610,7 +610,7 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
       CK(launch_split_rows(RowMap{nullptr, nullptr, 0, Nl}, Kl, d, kp, pl, kp16, Nl * kp16, s->num_sms,
                            nullptr), "weight planes");
     } else {
-      const int kp = (int)round_up(Kl, 16);
+      const int kp = (int)lp_pitch(Kl, eb);
       void* d = nullptr;
       CK(cudaMalloc(&d, eb * (size_t)Nl * kp), "weights");
       float* cs = nullptr;
@@ -653,7 +653,7 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
   CK(cudaMalloc(&s->x, eb * (size_t)s->cap * s->ldx), "network input");
   int64_t wmax[2] = {8, 8};
   for (int l = 0; l + 1 < L; ++l)
-    wmax[l & 1] = std::max<int64_t>(wmax[l & 1], round_up(s->widths[l + 1], lp ? 16 : 8));
+    wmax[l & 1] = std::max(wmax[l & 1], lp ? lp_pitch(s->widths[l + 1], eb) : round_up(s->widths[l + 1], 8));
   // (an FP32 network's input and activations are three BF16 planes, mlp_split.cu)
   for (int b = 0; b < 2; ++b) {
     s->act_ld[b] = lp ? wmax[b] : round_up(wmax[b], 16);
