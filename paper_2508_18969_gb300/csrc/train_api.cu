@@ -673,8 +673,7 @@ df_status df_mlp_forward_train(df_state* s, int64_t n_rows, const float* x, floa
                       : input_planes(s, n_rows, x, s->K0, st);
   if (e == cudaSuccess) e = forward(s, n_rows, st);
   if (e == cudaSuccess)
-    e = cudaMemcpy2DAsync(O, sizeof(float) * s->nout, t->O, sizeof(float) * t->ldo,
-                          sizeof(float) * s->nout, (size_t)n_rows, cudaMemcpyDeviceToDevice, st);
+    e = launch_cast_rows(n_rows, s->nout, t->O, t->ldo, O, s->nout, kXF32, 1.0f, s->num_sms, st);
   return e == cudaSuccess ? DF_OK : cuda_fail(s, e, "training forward pass");
 }
 
@@ -704,8 +703,7 @@ df_status df_mlp_backward(df_state* s, int64_t n_rows, const float* dO, float* d
                       : output_planes(s, n_rows, dO, s->nout, st);
   if (e == cudaSuccess) e = backward(s, n_rows, dX != nullptr, st);
   if (e == cudaSuccess && dX)
-    e = cudaMemcpy2DAsync(dX, sizeof(float) * s->K0, t->dX, sizeof(float) * t->lddx,
-                          sizeof(float) * s->K0, (size_t)n_rows, cudaMemcpyDeviceToDevice, st);
+    e = launch_cast_rows(n_rows, s->K0, t->dX, t->lddx, dX, s->K0, kXF32, 1.0f, s->num_sms, st);
   return e == cudaSuccess ? DF_OK : cuda_fail(s, e, "training backward pass");
 }
 
