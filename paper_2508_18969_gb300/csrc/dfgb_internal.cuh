@@ -266,6 +266,8 @@ struct TcLayer {
   int ksplit = 1;        // split-K (plain mode): split s covers k-blocks [s kbs, (s+1) kbs) and
   int64_t split_rows = 0;  // stores its partial product at output rows + s * split_rows
   bool pair = false;     // computed by CTA pairs (cta_group::2): 256-row tiles, tmB box BN/2
+  int BN2 = 0;           // narrower pair tile of short launches (launch_tc_gemm), 0: none
+  CUtensorMap tmB2;      // its weight map
   int tr = 0;            // MN-major operands (BF16), boxes {64, 64}: bit 0 A (K rows of output rows'
                          // columns), bit 1 W (K rows of N columns)
   long long wait_budget = 0;  // clocks a pipeline wait may take before the kernel gives up

@@ -1203,7 +1203,13 @@ int tc_epi_warps_per_quarter() { return epi_per_quarter(false, kActTanh); }
 
 cudaError_t prepare_tc(const TcLayer& L) {
   TcArgs a{};
-  return L.elem_bytes == 1 ? launch_fmt<true>(L, a, 0, nullptr) : launch_fmt<false>(L, a, 0, nullptr);
+  cudaError_t e = L.elem_bytes == 1 ? launch_fmt<true>(L, a, 0, nullptr) : launch_fmt<false>(L, a, 0, nullptr);
+  if (e == cudaSuccess && L.pair && L.BN2 > 0) {
+    TcLayer S = L;
+    S.BN = L.BN2;
+    e = L.elem_bytes == 1 ? launch_fmt<true>(S, a, 0, nullptr) : launch_fmt<false>(S, a, 0, nullptr);
+  }
+  return e;
 }
 
 cudaError_t launch_tc_gemm(const TcLayer& L, const RowMap& rows, int num_sms, int* err,
@@ -1230,6 +1236,24 @@ cudaError_t launch_tc_gemm(const TcLayer& L, const RowMap& rows, int num_sms, in
   a.budget = L.wait_budget > 0 ? L.wait_budget : kWaitBudget;
   // a short budget needs a short suspend hint, or one try_wait could outlast it
   a.suspend = a.budget < kWaitBudget ? 32u : kSuspendNs;
+  // The narrower pair tile where the launch is so short that its waves of tiles cost less: a wave takes
+  // the larger of its MMAs' and its loads' time (0.97 and 1 per column and loaded row, as in pick_tile).
+  // Each element's sum is the same either way. Four BF16 layers 32-1600-800-400-30 on 500, 1500, 3001, 6000
+  // and 12,000 rows: 34.7, 34.4, 38.0, 48.5, 63.1 us with 224 columns, 32.8, 32.9, 36.1, 46.2, 61.5 so; from
+  // 16,000 rows on the rule keeps the layer's own tile.
+  if (L.pair && L.BN2 > 0) {
+    const int64_t units = (rows.nmax + 2 * BM - 1) / (2 * BM), slots = std::max(1, num_sms / 2);
+    auto cost = [&](int bn) {
+      const int64_t items = units * ((L.N + bn - 1) / bn) * a.ksplit;
+      return (double)((items + slots - 1) / slots) * std::max(0.97 * bn, 128.0 + bn / 2);
+    };
+    if (cost(L.BN2) < cost(L.BN)) {
+      TcLayer S = L;
+      S.BN = L.BN2;
+      S.tmB = L.tmB2;
+      return L.elem_bytes == 1 ? launch_fmt<true>(S, a, num_sms, st) : launch_fmt<false>(S, a, num_sms, st);
+    }
+  }
   return L.elem_bytes == 1 ? launch_fmt<true>(L, a, num_sms, st)
                            : launch_fmt<false>(L, a, num_sms, st);
 }

@@ -49,6 +49,8 @@ df_status cuda_fail(df_state* s, cudaError_t e, const char* where) {
 //     stream faster per row), x1.25 when the tile leaves the TMA ring fewer than four stages.
 //     On the 1600 -> 800 layer of 2^20 rows this orders the measured times of single 160, 224
 //     and pair 160, 224, 256 tiles (2.15, 1.91, 1.82, 1.73, 1.75 ms) within 7 %.
+constexpr int kShortTile = 160;   // pair tile of launches too short for the layer's own (launch_tc_gemm)
+
 int pick_tile(int N, int K, bool hidden, int out_kind, bool allow_pair, bool mn) {
   static const int hid[] = {256, 224, 192, 160, 128, 64};
   static const int last[] = {64, 32};
@@ -727,6 +729,7 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
       const int tile = pick_tile(T.N, T.K, !last, last ? kXF32 : xk, true);
       T.BN = tile & ~DF_TILE_PAIR;
       T.pair = (tile & DF_TILE_PAIR) != 0;
+      T.BN2 = T.pair && T.BN > kShortTile ? kShortTile : 0;
       if (const char* env = getenv("DFGB_BN")) {  // hidden-layer tile-width override (sweeps)
         const int v = atoi(env);
         if (!last && (v == 64 || v == 128 || v == 160 || v == 192 || v == 224 || v == 256)) {
@@ -751,6 +754,8 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
           !tc_encode_2d(&T.tmB, s->Wlp[l], (int)eb, (uint64_t)T.K, (uint64_t)T.N,
                         (uint64_t)s->Kp8[l] * eb, boxk, (uint32_t)(T.pair ? T.BN / 2 : T.BN),
                         emsg, sizeof emsg) ||
+          (T.BN2 > 0 && !tc_encode_2d(&T.tmB2, s->Wlp[l], (int)eb, (uint64_t)T.K, (uint64_t)T.N,
+                                      (uint64_t)s->Kp8[l] * eb, boxk, (uint32_t)T.BN2 / 2, emsg, sizeof emsg)) ||
           !tc_encode_out(T, (uint64_t)s->cap, emsg, sizeof emsg)) {
         free_state(s);
         delete s;
@@ -1441,6 +1446,7 @@ df_status retile(df_state* s, int l, int tile) {
     return fail(s, DF_ERR_CUDA, "%s", emsg);
   T.BN = bn;
   T.pair = pair;
+  T.BN2 = 0;   // the tile asked for runs whatever the rows
   cudaError_t e = prepare_tc(T);
   return e == cudaSuccess ? DF_OK : cuda_fail(s, e, "kernel attributes");
 }
