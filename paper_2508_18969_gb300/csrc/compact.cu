@@ -1,12 +1,15 @@
-// a0: stable compaction of the reacting cells (T > T_react) into an ascending index list. No inter-block
-// waiting. Up to 16,384 cells take one launch of one block, whose loads are then one memory latency.
-// More take two: per-chunk counts (warp ballot + popc), then a scatter in which each block adds up the
-// counts of the chunks before its own and ranks each reacting cell inside its chunk with ballot/popc
-// prefix sums; beyond 2^23 cells a one-block scan between them takes those sums over. Both chunk passes
-// load all of a thread's cells before testing any, so a chunk costs one memory latency. Cells are visited
-// in the same order by the count and the scatter pass, so the list is in ascending cell order. The first
-// launch also clears the caller's counters. (Two memsets and three launches before: about 14 us less of a
-// step on 4,096 or 20,000 cells.)
+// a0: stable compaction of the reacting cells (T > T_react) into an ascending index list. Up to 32,768 cells
+// take one launch, whose loads are one memory latency: one block up to 16,384 cells, beyond that one cluster
+// of eight blocks, which read one another's counts from shared memory (step of 20,011 and 30,011 cells of 9
+// species 118.4 -> 113.1 and 135.2 -> 129.8 us, of 30 species 192.4 -> 191.6 us; with 16 cells a thread and
+// up to 131,072 cells the cluster was 4 us slower than two launches, and so was one block on 20,000).
+// More take two launches, with no inter-block waiting: per-chunk counts (warp ballot + popc), then a scatter
+// in which each block adds up the counts of the chunks before its own and ranks each reacting cell inside its
+// chunk with ballot/popc prefix sums; beyond 2^23 cells a one-block scan between them takes those sums over.
+// Both chunk passes load all of a thread's cells before testing any, so a chunk costs one memory latency.
+// Cells are visited in the same order by the count and the scatter pass, so the list is in ascending cell
+// order. The first launch also clears the caller's counters. (Two memsets and three launches before: about
+// 14 us less of a step on 4,096 or 20,000 cells.)
 #include "dfgb_internal.cuh"
 #include "pdl.cuh"
 
@@ -18,25 +21,41 @@ constexpr int kItems = 16;                         // cells per thread per chunk
 constexpr int kChunk = kCompactChunk;              // 4096 cells per block
 constexpr int kWarps = kThreads / 32;
 constexpr int kCellNonfinite = 4;
+constexpr int64_t kOneLaunch = 8 * 4096;           // cells of the largest one-launch compaction
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p of the block of that rank in the cluster (p in shared memory, at the same place in every block).
+__device__ __forceinline__ int peer_int(const int* p, int rank) {
+  uint32_t a;
+  int v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
 
 __device__ __forceinline__ bool reacts(double t, double thr) { return t > thr; }
 
-// One block of 1024 threads, ITEMS cells each.
-template <int ITEMS>
+// One cluster of CL blocks of 1024 threads, ITEMS cells each: a block lists its own range of cells and
+// reads the counts of the blocks before it from their shared memory.
+template <int ITEMS, int CL>
 __global__ void __launch_bounds__(1024) compact_one_kernel(int n, double thr, const double* __restrict__ T,
     int32_t* __restrict__ status, int32_t* __restrict__ idx, int64_t* __restrict__ count,
     int64_t* __restrict__ zero0, int64_t* __restrict__ zero1) {
   __shared__ int tot[ITEMS][32];   // reacting cells per (pass j, warp), then their exclusive prefix
   __shared__ int row[32];
+  __shared__ int total;            // this block's reacting cells
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int rank = CL > 1 ? (int)blockIdx.x : 0, base = rank * (ITEMS * 1024);
   pdl_begin();
   double v[ITEMS];
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) v[j] = j * 1024 + t < n ? T[j * 1024 + t] : 0.0;
+  for (int j = 0; j < ITEMS; ++j) v[j] = base + j * 1024 + t < n ? T[base + j * 1024 + t] : 0.0;
   unsigned m[ITEMS];
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
-    const int i = j * 1024 + t;
+    const int i = base + j * 1024 + t;
     m[j] = __ballot_sync(0xffffffffu, i < n && reacts(v[j], thr));
     if (status && i < n) status[i] = isfinite(v[j]) ? 0 : kCellNonfinite;
     if (lane == 0) tot[j][warp] = __popc(m[j]);
@@ -55,12 +74,22 @@ __global__ void __launch_bounds__(1024) compact_one_kernel(int n, double thr, co
   __syncthreads();
   const unsigned below = (1u << lane) - 1u;
   int run = 0;
+  if constexpr (CL > 1) {
+    if (t == 0) {
+      int s = 0;
+      for (int j = 0; j < ITEMS; ++j) s += row[j];
+      total = s;
+    }
+    cluster_barrier();
+    for (int r = 0; r < rank; ++r) run += peer_int(&total, r);
+  }
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
-    if ((m[j] >> lane) & 1u) idx[run + tot[j][warp] + __popc(m[j] & below)] = j * 1024 + t;
+    if ((m[j] >> lane) & 1u) idx[run + tot[j][warp] + __popc(m[j] & below)] = base + j * 1024 + t;
     run += row[j];
   }
-  if (t == 0) {
+  if constexpr (CL > 1) cluster_barrier();   // no block leaves while another may read its total
+  if (t == 0 && (CL == 1 || rank == CL - 1)) {
     *count = run;
     if (zero0) *zero0 = 0;
     if (zero1) *zero1 = 0;
@@ -200,11 +229,12 @@ cudaError_t launch_compact(int64_t n, double T_react, const double* T, int32_t* 
     if (e == cudaSuccess && zero1) e = cudaMemsetAsync(zero1, 0, sizeof(int64_t), st);
     return e;
   }
-  if (n <= 16384) {   // (with 32 cells a thread, one block was slower than two launches on 20,000)
-    auto one = [&](auto kern) {
-      return pdl_launch(kern, 1, 1024, 0, st, 1, (int)n, T_react, T, status, idx, count, zero0, zero1);
+  if (n <= kOneLaunch) {
+    auto one = [&](auto kern, unsigned blocks) {
+      return pdl_launch(kern, blocks, 1024, 0, st, blocks, (int)n, T_react, T, status, idx, count, zero0, zero1);
     };
-    return n <= 4096 ? one(compact_one_kernel<4>) : one(compact_one_kernel<16>);
+    return n <= 4096    ? one(compact_one_kernel<4, 1>, 1)
+           : n <= 16384 ? one(compact_one_kernel<16, 1>, 1) : one(compact_one_kernel<4, 8>, 8);
   }
   const int64_t nb = (n + kChunk - 1) / kChunk;
   int64_t* counts = scratch;
