@@ -57,7 +57,9 @@ typedef int32_t df_status;
 /* Arithmetic of the network layers (a5-a7). The equation of state, Box-Cox, renormalisation
  * and Newton steps are FP64 in every mode (Sec. 3.3.1 keeps all non-network work double). */
 typedef enum {
-  DF_FP32 = 0,      /* SIMT FP32 GEMMs, accurate tanh: the plain FP32 step */
+  DF_FP32 = 0,      /* FP32 layers: tcgen05 GEMMs on three exact BF16 planes per operand (six
+                       products, FP32 sums renewed every 64 terms), or chains of FP32 FMAs for the
+                       Jacobian and df_propnet_infer; accurate GELU: the plain FP32 step */
   DF_BF16 = 1,      /* tcgen05 BF16 GEMMs, FP32 accumulation, BF16 activations */
   DF_FP8_E4M3 = 2   /* tcgen05 FP8 e4m3 GEMMs, FP32 accumulation; weights e4m3(W/s_c) with
                        per-output-channel s_c = max|W_c|/448, activations e4m3(32 v) */
@@ -101,7 +103,7 @@ typedef struct {
 
 /* Hidden-layer activation of the network (a6). Both are the tanh form of Sec. 3.3.2:
  *   DF_GELU_TANH   0.5 x (1 + tanh(c (x + 0.044715 x^3))), c = sqrt(2/pi), with the hardware
- *                  tanh approximation on tensor-core paths and tanhf on the FP32 path;
+ *                  tanh approximation in BF16 and FP8 networks and to FP32 accuracy in FP32 ones;
  *   DF_GELU_TABLE  the paper's tabulation: 0 for x <= -3, x for x >= 3, and in between the
  *                  second-order expansion about the table node at or below x (nodes every 0.01,
  *                  value, slope and half curvature in FP32). FP32 and BF16 networks, inference
@@ -335,7 +337,7 @@ void df_graph_destroy(df_graph* g);
  * ones are appended. Synchronises `stream`. A no-op for DF_FP32 states. The tiling changes
  * neither the arithmetic nor its order, so results are bit-identical before and after; call
  * it before capturing graphs (a graph keeps the launch parameters it recorded).
- * df_get_tiles reports the tile of each layer (0 for SIMT layers) in bn[0..max_layers): its
+ * df_get_tiles reports the tile of each layer (0 for the layers of DF_FP32 states) in bn[0..max_layers): its
  * width, | DF_TILE_PAIR when the layer runs on CTA pairs (two CTAs of a cluster share one
  * 256-row tile through cta_group::2 MMAs, each holding half of the tile's weight rows), and
  * the number of layers in *n_layers.
@@ -354,7 +356,7 @@ df_status df_get_tiles(df_state* s, int32_t* bn, int32_t max_layers, int32_t* n_
  * df_get_step_summary reports DF_ERR_TIMEOUT once. A budget of a few hundred clocks makes
  * waits give up on purpose, which is how the timeout path is tested without a fault. Applies
  * to launches made after the call (a captured graph keeps the budget it was captured with).
- * DF_ERR_UNSUPPORTED for DF_FP32 states (no tensor-core layers). Paper: no counterpart
+ * DF_ERR_UNSUPPORTED for DF_FP32 states (their layers keep the default budget). Paper: no counterpart
  * (failure handling). */
 df_status df_set_wait_limit(df_state* s, int64_t clocks);
 

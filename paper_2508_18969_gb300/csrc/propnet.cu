@@ -1,7 +1,8 @@
 // Kernels of the real-fluid property network (PRNet-style surrogate, Sec. 2): the network reads
 // a cell's conserved enthalpy, pressure and composition and yields its properties (here the
 // density and the temperature). Input rows, normalised training targets and de-normalised
-// outputs; the network layers themselves are the tcgen05 / SIMT GEMMs of the reaction step.
+// outputs; the network layers themselves are the tcgen05 GEMMs of the reaction step (FP32
+// inference: mlp_simt.cu).
 //
 // Normalisation (the layout of the state's norm array, K0 = n + 2 inputs, m outputs):
 //   norm[c] = input mean, norm[K0 + c] = 1 / input spread        (c < K0)

@@ -1,6 +1,7 @@
 // C ABI of libdfgb (include/df.h): state creation, the fused reaction step and the stage
 // entry points. Host code only orchestrates; every step of the path runs in the kernels
-// of eos.cu, compact.cu, mlp_simt.cu and mlp_tc.cu.
+// of eos.cu, compact.cu, mlp_split.cu (FP32 networks) and mlp_tc.cu (BF16 and FP8); mlp_simt.cu holds the
+// FP32 layers of the Jacobian and of property-network inference.
 #include "pdl.cuh"
 #include "state.cuh"
 #include "../../include/df_propnet.h"
@@ -1465,7 +1466,7 @@ extern "C" {
 df_status df_autotune(df_state* s, int64_t n_rows, const char* cache_path, void* stream) {
   if (!s) return fail(nullptr, DF_ERR_INVALID_ARG, "state is NULL");
   if (n_rows < 0) return fail(s, DF_ERR_INVALID_ARG, "n_rows < 0");
-  if (s->precision == DF_FP32) return DF_OK;  // the SIMT layers have a single tiling
+  if (s->precision == DF_FP32) return DF_OK;  // an FP32 layer picks its tiling per launch
   DeviceGuard guard(s->device);
   cudaStream_t st = (cudaStream_t)stream;
   cudaDeviceProp prop;

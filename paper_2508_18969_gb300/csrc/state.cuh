@@ -14,7 +14,7 @@ struct Trn;   // training context (train_api.cu)
 
 struct Jac {
   int64_t B = 0;                         // cells per Jacobian batch
-  bool bf16 = false;                     // BF16 tensor-core passes (else FP32 SIMT)
+  bool bf16 = false;                     // BF16 tensor-core passes (else FP32, mlp_simt.cu)
   size_t eb = 4;
   void* x = nullptr;
   int64_t ldx = 0;

@@ -1,7 +1,7 @@
 // Training of the chemistry network: targets, loss, the element-wise parts of the backward
 // pass and the Adam update. The GEMMs of the backward pass (weight gradients dZ^T H and input
-// gradients dZ W, the latter scaled by GELU'(z) in its epilogue) run on the same tcgen05 /
-// SIMT kernels as the forward pass; these kernels prepare their operands.
+// gradients dZ W, the latter scaled by GELU'(z) in its epilogue) run on the same tcgen05
+// kernels as the forward pass (mlp_tc.cu, mlp_split.cu).
 #include "dfgb_internal.cuh"
 #include "planes.cuh"
 

@@ -1,7 +1,7 @@
 // C ABI of network training (include/df.h, "training"): the loss of the normalised network
 // outputs against targets from a stiff integration, its gradients by a layer-by-layer
-// backward pass and Adam updates of FP32 master weights, whose working copies (FP32 for the
-// SIMT path, BF16 for the tensor-core path) the reaction step reads in place.
+// backward pass and Adam updates of FP32 master weights, whose working copies (FP32 and
+// three BF16 planes for an FP32 state, BF16 otherwise) the reaction step reads in place.
 //
 // Backward pass of layer l (Z_l = H_{l-1} W_l^T + b_l, H_l = GELU(Z_l), linear read-out):
 //   dW_l = dZ_l^T H_{l-1}   (GEMM over the batch, split-K, both operands read along their columns:
