@@ -191,10 +191,10 @@ _EOS_OTHER = (("// -------------------------------------------------------------
               ("cudaError_t launch_jac_scale(", "cudaError_t launch_eos_post("),
               ("cudaError_t launch_transport(", "}  // namespace dfgb"))
 MEASURED_TRAFFIC = {
-    ("layer0", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "573644641909b36e", 3157.3),
-    ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "573644641909b36e", 4757.1),
-    ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "573644641909b36e", 2346.0),
-    ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "573644641909b36e", 1068.1),
+    ("layer0", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 3157.3),
+    ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 4757.1),
+    ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 2346.0),
+    ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 1068.1),
     ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342", 293.3,
                                         _EOS_OTHER),
     ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342", 582.5,

@@ -73,9 +73,11 @@ constexpr int kActNone = 0, kActTanh = 1, kActTable = 2;
 // three, each loading the next chunk while it stores the current one. Measured on 2^20 rows of
 // the 32 -> 1600 layer: 0.83 ms with three per quarter (192-wide tiles), 0.61 ms with four
 // (256-wide), 0.60 ms with five (160-wide, one chunk per warp); on the CTA-pair 1600 -> 800
-// layer four were 2 % slower than three.
-__host__ __device__ constexpr int epi_per_quarter(bool pair, int act, int mode = 0) {
-  return !pair && act != kActNone && mode != kModeStoreG ? 5 : 3;
+// layer four were 2 % slower than three. FP8 pair tiles, whose MMAs take half the time, take four (with the
+// turns below, FP8 step of 2^22 cells 4713 -> 4689 us).
+__host__ __device__ constexpr int epi_per_quarter(bool pair, int act, int mode = 0, bool fp8 = false) {
+  if (pair) return fp8 ? 4 : 3;
+  return act != kActNone && mode != kModeStoreG ? 5 : 3;
 }
 
 // tanh-form GELU (Sec. 3.3.2), 0.5 x (1 + tanh(c (x + a x^3))), evaluated as
@@ -286,10 +288,10 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t (&r)[32], const Tc
 constexpr int kTrA = 1, kTrW = 2;
 
 template <bool FP8, int BN, int OUTK, int ACT, bool SCALE, int MODE, bool PAIR, int TR>
-__global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)), 1) tc_gemm_kernel(
+__global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE, FP8)), 1) tc_gemm_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmG, TcArgs g) {
-  using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE)>;
+  using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE, FP8)>;
   constexpr int kEpiWarps = C::kEpiWarps;
   // a 32-column epilogue chunk is stored as one TMA box, so chunks must not straddle tiles
   static_assert(BN % 32 == 0, "tile width must be a multiple of 32");
@@ -494,10 +496,10 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
   } else if (warp >= 2) {
     // ---------------- epilogue ----------------
     const int q = warp & 3;                   // TMEM lane quarter this warp may access
-    const int slot = (warp - 2) >> 2;         // which of the quarter's interleaved chunks
+    const int slot = (warp - 2) >> 2;         // which of the quarter's interleaved chunks (of the first tile)
     constexpr int kChunkStride = 32 * C::kEpq;
     uint8_t* stg = sOut + (warp - 2) * C::kStageOut;
-    int buf = 0;
+    int buf = 0, turn = slot;
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmO) : "memory");
     }
@@ -513,12 +515,15 @@ __global__ void __launch_bounds__(threads_for(epi_per_quarter(PAIR, ACT, MODE)),
       const int64_t m0 = mt + q * 32 + w.split * g.split_rows;
       const int n0 = w.nt(tiles_n) * BN;
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + a * C::kAccStride;
-      // chunks c = 32 slot + kChunkStride i; with three warps per quarter TMEM loads run one
+      // chunks c = 32 turn + kChunkStride i (turn moves on with each tile where the chunks do not divide
+      // evenly, or one warp would have the most of them in every tile: Adam step on 65,536 states 1102 ->
+      // 1092 us); with three warps per quarter TMEM loads run one
       // chunk ahead of the math, except in kModeStoreG, whose two stores per chunk leave no
       // registers for a second chunk in flight; with five, the quarter's other warps cover the
       // load. The odd CTA of a pair whose m tile lies past the rows stores nothing.
       uint32_t r0[32], r1[32];
-      int c0 = (PAIR && mt >= M) ? BN : 32 * slot;
+      int c0 = (PAIR && mt >= M) ? BN : 32 * turn;
+      if constexpr (BN % kChunkStride != 0) turn = turn + 1 < C::kEpq ? turn + 1 : 0;
       if constexpr (MODE == kModeStoreG || C::kEpq >= 4) {
         for (; c0 < BN; c0 += kChunkStride) {
           tmem_ld32(tbase + c0, r0);
@@ -600,7 +605,7 @@ cudaError_t tc_attr(int* max_clusters) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE)>;
+    using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE, FP8)>;
     auto kern = tc_gemm_kernel<FP8, BN, OUTK, ACT, FP8, MODE, PAIR, TR>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (e != cudaSuccess) return e;
@@ -632,7 +637,7 @@ cudaError_t tc_attr(int* max_clusters) {
 
 template <bool FP8, int BN, int OUTK, int ACT, int MODE = kModePlain, bool PAIR = false, int TR = 0>
 cudaError_t launch_bn(const TcLayer& L, const TcArgs& a, int num_sms, cudaStream_t st) {
-  using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE)>;
+  using C = Cfg<BN, OUTK, PAIR, epi_per_quarter(PAIR, ACT, MODE, FP8)>;
   constexpr bool SCALE = FP8;
   auto kern = tc_gemm_kernel<FP8, BN, OUTK, ACT, SCALE, MODE, PAIR, TR>;
   int max_clusters = 0;
