@@ -792,6 +792,9 @@ static df_status create_state(const df_mech_desc* mech, const df_mlp_desc* mlp,
   CK(prepare_eos(s->P, xk), "kernel attributes");
   for (const TcLayer& T : s->tcl) CK(prepare_tc(T), "kernel attributes");
   if (s->fuse01) CK(prepare_f01(), "kernel attributes");
+  // the weight planes and the zeroed buffers above are work of the legacy stream, which a caller's
+  // non-blocking stream does not wait for
+  CK(cudaStreamSynchronize(nullptr), "state set-up");
 #undef CK
   *out = s;
   return DF_OK;
