@@ -237,6 +237,8 @@ df_status ensure_batch(df_state* s, int64_t B) {
   zalloc((void**)&t->dWp, sizeof(float) * kMaxSplit * wmaxp);
   zalloc((void**)&t->h0, sizeof(double) * B);
   zalloc((void**)&t->rstat, sizeof(int32_t) * B);
+  // the buffers are zeroed on the legacy stream, which a caller's non-blocking stream does not wait for
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     free_batch(t);
     return cuda_fail(s, e, "training buffers");

@@ -33,3 +33,25 @@ def test_first_call_on_a_non_blocking_stream(df, prec):
         assert torch.equal(first, st.mlp_forward(x))
         torch.cuda.synchronize()
         st.close()
+
+
+@pytest.mark.parametrize("prec", ["DF_FP32", "DF_BF16"])
+def test_first_training_call_on_a_non_blocking_stream(df, prec):
+    mech = synth.mechanism.make_mechanism(9, 1, 3)
+    net = synth.network.make_network([11, 64, 4096, 9], 9, seed=1)
+    x, dO = torch.randn(20011, 11, device="cuda"), torch.randn(20011, 9, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    st = df.State(mech, net, precision=getattr(df, prec), batch_cells=128)
+    st.mlp_forward_train(x[:1])          # masters and moments; the batch buffers grow below
+    out = []
+    for _ in range(2):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            out.append([st.mlp_forward_train(x), st.mlp_backward(dO)])
+        torch.cuda.synchronize()
+        out[-1] += [t for l in range(3) for t in st.params(l, df._lib.DF_PARAM_GRADS, widths=net.widths)]
+        torch.cuda.synchronize()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    st.close()
