@@ -156,7 +156,10 @@ df_status df_chem_step_host(df_state* s, int64_t n_cells, double dt, double* T, 
  * and Z of every cell. Any output pointer may be NULL and is then not written.
  * Paper: Sec. 2 (supercritical mixture properties from the Peng-Robinson EoS; the equations are
  * Peng & Robinson 1976 with van der Waals one-fluid mixing, which the paper names but does not
- * print). Evaluated explicitly in FP64, as Sec. 3.3.1 keeps all non-network work double. */
+ * print). The sums over species and the departure functions are double-float (pairs of FP32 numbers: about
+ * 48 bits, FP32's exponent range), the cubic, its root and the density FP64: about 1e-13 relative to the
+ * terms on ordinary states, and that divided by the cubic's slope at the root near critical points and
+ * where two roots merge. Next to a saturation line the root of least Gibbs energy is told for p >= 1 kPa. */
 df_status df_real_fluid_props(df_state* s, int64_t n_cells, const double* T, const double* p,
                               const double* Y, int64_t ldY, double* rho, double* h, double* cp,
                               double* Z, void* stream);

@@ -473,6 +473,13 @@ __device__ __forceinline__ double cubic_polish(double Z, double c2, double c1, d
   return cubic_step(cubic_step(Z, c2, c1, c0), c2, c1, c0);
 }
 
+// Departure Gibbs energy in FP32 (for choosing among the three roots when the choice is clear).
+__device__ __forceinline__ float g_dep_f(float Z, float A, float B) {
+  const float s2 = 1.41421356f;
+  return Z - 1.0f - __logf(Z - B) -
+         __fdividef(A, 2.0f * s2 * B) * __logf(__fdividef(Z + (1.0f + s2) * B, Z + (1.0f - s2) * B));
+}
+
 __device__ __forceinline__ double g_dep(double Z, double A, double B, const double* lnt) {
   return Z - 1.0 - dlog_tab(Z - B, lnt) -
          A * drcp(2.0 * kSQ2 * B) * dlog_tab((Z + (1.0 + kSQ2) * B) * drcp(Z + (1.0 - kSQ2) * B), lnt);
@@ -516,6 +523,34 @@ __device__ __noinline__ double select_Z3(double A, double B, double c2, double c
   float cphi = (pf < 0.0f) ? (3.0f * d_to_f_trunc(Q) / (2.0f * pf)) * sqrtf(-3.0f / pf) : 0.0f;
   cphi = fminf(fmaxf(cphi, -1.0f), 1.0f);
   const float phi = acosf(cphi) * (1.0f / 3.0f);
+  // A root whose Gibbs energy is clearly the least by the FP32 seeds is the only one polished (2^18 states
+  // of which a third have three roots: 211 -> 180 us). The roots are stationary points of the Gibbs energy,
+  // so a seed's error (1e-6; 1e-4 next to a double root) enters squared over Z - B: 5e-3 is far enough from
+  // B, and 1e-3 more than the FP32 energies' own error.
+  {
+    const float Bf = d_to_f_trunc(B), Af = d_to_f_trunc(A), c23 = d_to_f_trunc(c2) * (1.0f / 3.0f);
+    float tbest = 0.0f, g1 = __int_as_float(0x7f800000), g2 = g1;
+    bool clear = true;
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k) {
+      const float tk = m * cosf(phi - 2.0943951023931955f * (float)k);
+      const float zk = tk - c23;
+      if (fabsf(zk - Bf) < 5e-3f) clear = false;
+      if (zk > Bf) {
+        const float g = g_dep_f(zk, Af, Bf);
+        if (!(g == g)) clear = false;
+        if (g < g1) {
+          g2 = g1;
+          g1 = g;
+          tbest = tk;
+        } else if (g < g2) {
+          g2 = g;
+        }
+      }
+    }
+    if (clear && g1 < g2 - 1e-3f)
+      return cubic_polish(cubic_polish(f_to_d(tbest) - c2 * (1.0 / 3.0), c2, c1, c0), c2, c1, c0);
+  }
   double best = __longlong_as_double(0x7ff8000000000000LL);
   double gbest = __longlong_as_double(0x7ff0000000000000LL);
 #pragma unroll
@@ -629,13 +664,6 @@ __device__ __forceinline__ f2 g_dep_df(f2 Z, f2 A, f2 B, const f2* lt) {
   const f2 L = f2_log_tab(f2_mul(Zp, f2_rcp(Zm)), lt);
   const f2 a = f2_mul(A, f2_rcp(f2_mul(B, f2{kS2h, kS2l})));
   return f2_sub(f2_sub(f2_addf(Z, -1.0f), f2_log_tab(f2_sub(Z, B), lt)), f2_mul(a, L));
-}
-
-// Departure Gibbs energy in FP32 (for choosing among the three roots when the choice is clear).
-__device__ __forceinline__ float g_dep_f(float Z, float A, float B) {
-  const float s2 = 1.41421356f;
-  return Z - 1.0f - __logf(Z - B) -
-         __fdividef(A, 2.0f * s2 * B) * __logf(__fdividef(Z + (1.0f + s2) * B, Z + (1.0f - s2) * B));
 }
 
 // Three real roots (select_Z3 in double-float). Out of line, as there. The roots above B are
@@ -1138,7 +1166,27 @@ __global__ void __launch_bounds__(TH, TH == kThreads ? kPostBlocks : 1) eos_post
   }
 }
 
+// Compressibility, the cubic's slope there and the density from the mixing sums in FP64, for the properties:
+// near the critical point and where roots merge the slope goes to zero and a root is off by the error of
+// the cubic's coefficients divided by it; a liquid's root at low pressure lies within 1e-4 of B, so that
+// only FP64 tells which root has the least Gibbs energy; a dilute gas's Z is 1 less a small number.
+struct Root64 {
+  double Z, slope, rho;
+};
+__device__ __forceinline__ Root64 root64(const MixSums& s, double T, double p, const double* lnt, int& status) {
+  const double Wm = drcp(f2_to(s.inv)), W2 = Wm * Wm, iT = drcp(T), t = dsqrt_pos(T);
+  const double am = W2 * fma(-2.0 * f2_to(s.F1), t, fma(f2_to(s.F2), T, f2_to(s.F0)));
+  const double iRT = iT * kInvR, pRT = p * iRT;
+  const double A = am * pRT * iRT, B = Wm * f2_to(s.bs) * pRT;
+  Root64 r;
+  r.Z = select_Z(A, B, lnt, status);
+  r.slope = fma(3.0 * r.Z, r.Z, -2.0 * (1.0 - B) * r.Z) + (A - 3.0 * B * B - 2.0 * B);
+  r.rho = pRT * Wm * drcp(r.Z);
+  return r;
+}
+
 // Real-fluid c_p of the state q = pr_point_df(m, T, p) and the coefficients of dh/dY_k at fixed T, p.
+// (Without GRAD: c_p and the departure enthalpy at the root q.Z, where the cubic's slope is given.)
 // With u_k = y_k sqrt(a_k), yr_k = y_k r_k (y = Y / W), v = K u, w = K yr, sigma = sum y = 1 / W:
 //   a = W^2 u.v,  a' = -(W^2 / sqrt T) yr.v,  b = W sum y_k b_k,
 //   da/dy_k = 2 W^2 sqrt(a_k) v_k - 2 W a,  db/dy_k = W (b_k - b),
@@ -1154,7 +1202,7 @@ struct HGrad {
 };
 
 template <bool GRAD>
-__device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPointDF& q, const f2* lt, f2& cp,
+__device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, PRPointDF& q, f2 slope, const f2* lt, f2& cp,
                                         HGrad& g) {
   const f2 iT = f2_rcp(T), t = f2_sqrt_pos(T), it = f2_mul(t, iT);
   const f2 am = f2_fma(m.A1, f2{-2.0f * t.h, -2.0f * t.l}, f2_fma(m.A2, T, m.A0));
@@ -1169,7 +1217,7 @@ __device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPoin
   const f2 kbL = f2_mul(m.kb, L);
   // f_Z, f_A, f_B of the cubic: 3 Z^2 - 2 (1 - B) Z + A - 3 B^2 - 2 B, Z - B, Z^2 - (6 B + 2) Z - (A - 2 B - 3 B^2)
   const f2 B3 = f2_mul(B, f2_addf(f2_mulf(B, 3.0f), 2.0f));
-  const f2 FZ = f2_add(f2_mul(Z, f2_add(f2_mulf(Z, 3.0f), f2_scale2(f2_addf(B, -1.0f)))), f2_sub(A, B3));
+  const f2 FZ = GRAD ? f2_add(f2_mul(Z, f2_add(f2_mulf(Z, 3.0f), f2_scale2(f2_addf(B, -1.0f)))), f2_sub(A, B3)) : slope;
   const f2 FA = f2_sub(Z, B);
   const f2 FB = f2_add(f2_mul(Z, f2_sub(Z, f2_addf(f2_mulf(B, 6.0f), 2.0f))), f2_sub(B3, A));
   const f2 iFZ = f2_rcp(FZ);
@@ -1194,7 +1242,10 @@ __device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPoin
   cpi = f2_fma(cpi, T, f2_scale2(m.e[2]));
   cpi = f2_fma(cpi, T, m.e[1]);
   cp = f2_fma(cpd, m.inv, cpi);
-  if constexpr (!GRAD) return;
+  if constexpr (!GRAD) {
+    q.h_dep = f2_fma(RT, f2_addf(Z, -1.0f), f2_mul(tk, L));
+    return;
+  }
   const f2 W = f2_rcp(m.inv);
   const f2 gi = f2_mul(gz, iFZ);
   const f2 al = f2_neg(f2_fma(f2_mul(gi, FA), pRT2, kbL));
@@ -1212,10 +1263,13 @@ __device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, const PRPoin
   g.c0 = f2_sub(c0, f2_mul(m.bm, ga));
 }
 
-// Density, enthalpy, c_p and compressibility of every cell (outputs may be NULL), in double-float like
-// eos_pre (with the state in FP64 its pipe was busy half of the time and a thread loaded its mass
-// fractions two at a time: 195 -> 152 us for 2^18 cells of 30 species; errors against FP64 as before,
-// 1.7e-13 in density and 1.4e-13 in c_p: the mixing sums, double-float all along, set them).
+// Density, enthalpy, c_p and compressibility of every cell (outputs may be NULL): the mixing sums in
+// double-float, the cubic, its root and the density in FP64 (Root64), the departure enthalpy and c_p in
+// double-float. 2^18 cells of 30 species: 195 us with all of the state in FP64 (its pipe busy half of the
+// time) and mass fractions loaded two at a time, 165 us so. With the cubic in double-float as well it was
+// 147 us, but took the other phase's root next to saturation lines below 20 kPa, and its roots near
+// critical points were twice as far off. Errors against FP64 on ordinary states: 1.7e-13 in density and
+// 1.4e-13 in c_p, set by the mixing sums.
 template <int NM>
 __global__ void __launch_bounds__(kThreads, kPreBlocks) props_kernel(EosParams P, int64_t ncell,
     const double* __restrict__ T, const double* __restrict__ p, const double* __restrict__ Y,
@@ -1236,19 +1290,22 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) props_kernel(EosParams P
       for (int u = 0; u < kLoadBatch; u += 2)
         if (k0 + u < n) ycol.set_pair((k0 + u) >> 1, f2_from(yv[u]), f2_from(yv[u + 1]));
     }
-    MixDF m;
-    mixture_df<kThreads>(ycol, n, c, m);
+    MixSums ms;
+    mixture_sums<kThreads>(ycol, n, c, ms);
     int st = 0;
-    const PRPointDF q = pr_point_df<false>(m, Td, pd, false, c.lt2, st);
-    if (rho) rho[i] = f2_to_int(f2_mul(pd, f2_rcp(f2_mul(f2_mul(m.inv, q.Z), f2_mul(Td, f2{kRh, kRl})))));
+    const Root64 z = root64(ms, T[i], p[i], P.lntab, st);
+    if (rho) rho[i] = z.rho;
+    if (Zo) Zo[i] = z.Z;
+    if (!h && !cp) continue;
+    MixDF m;
+    mix_df_final(ms, m);
+    PRPointDF q;
+    q.Z = f2_from(z.Z);
+    f2 cpv;
+    HGrad g;
+    state_grad<false>(m, Td, pd, q, f2_from(z.slope), c.lt2, cpv, g);
     if (h) h[i] = f2_to_int(f2_fma(q.h_dep, m.inv, h_ig_df(m, Td)));
-    if (cp) {
-      f2 cpv;
-      HGrad g;
-      state_grad<false>(m, Td, pd, q, c.lt2, cpv, g);
-      cp[i] = f2_to_int(cpv);
-    }
-    if (Zo) Zo[i] = f2_to_int(q.Z);
+    if (cp) cp[i] = f2_to_int(cpv);
   }
 }
 
@@ -1597,11 +1654,11 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       MixDF m;
       mixture_df<stride>(ycol, n, c, m);
       const f2 Td = f2_from(Tc);
-      const PRPointDF s0 = pr_point_df<false>(m, Td, pd, false, c.lt2, st);
+      PRPointDF s0 = pr_point_df<false>(m, Td, pd, false, c.lt2, st);
       if (want_dT) {
         f2 cp;
         HGrad g;
-        state_grad<true>(m, Td, pd, s0, c.lt2, cp, g);
+        state_grad<true>(m, Td, pd, s0, f2{0.0f, 0.0f}, c.lt2, cp, g);
         put(q + 2 * n, cp);
         put_grad(q + 2 * n + 2, g);
       }
@@ -1638,11 +1695,11 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
         int iters = 0;
         const f2 Tn = solve_T_df(m, pd, f2_from(h0c), Tc, P, c.lt2, iters, st);
         if (st == 0) {
-          const PRPointDF s1 = pr_point_df<false>(m, Tn, pd, false, c.lt2, st);
+          PRPointDF s1 = pr_point_df<false>(m, Tn, pd, false, c.lt2, st);
           if (want_dT) {
             f2 cp;
             HGrad g;
-            state_grad<true>(m, Tn, pd, s1, c.lt2, cp, g);
+            state_grad<true>(m, Tn, pd, s1, f2{0.0f, 0.0f}, c.lt2, cp, g);
             put(q + 2 * n + 1, cp);
             put_grad(q + 2 * n + 8, g);
           }
