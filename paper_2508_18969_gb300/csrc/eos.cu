@@ -668,8 +668,8 @@ __device__ __forceinline__ f2 g_dep_df(f2 Z, f2 A, f2 B, const f2* lt) {
 
 // Three real roots (select_Z3 in double-float). Out of line, as there. The roots above B are
 // first ranked by their FP32 seeds and FP32 departure Gibbs energies; when one root is lower
-// by more than 1e-4 (FP32 errors are ~1e-6 there) and no seed lies within 1e-5 of B, only
-// that root is polished. Otherwise every root is polished and compared in double-float.
+// by more than 1e-3 and no seed lies within 5e-3 of B (why these: select_Z3), only that root is
+// polished. Otherwise every root is polished and compared in double-float.
 __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23, float Pf,
                                         float Qf, const f2* lt, int& status) {
   const float m = (Pf < 0.0f) ? 2.0f * sqrtf(-Pf / 3.0f) : 0.0f;
@@ -683,7 +683,7 @@ __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23,
     for (int k = 0; k < 3; ++k) {
       const float tk = m * cosf(phi - 2.0943951023931955f * (float)k);
       const float zk = tk - c23.h;
-      if (fabsf(zk - B.h) <= 1e-5f * fabsf(B.h)) clear = false;
+      if (fabsf(zk - B.h) < 5e-3f) clear = false;
       if (zk > B.h) {
         const float g = g_dep_f(zk, A.h, B.h);
         if (!(g == g)) clear = false;
@@ -696,7 +696,7 @@ __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23,
         }
       }
     }
-    if (clear && g1 < g2 - 1e-4f) {
+    if (clear && g1 < g2 - 1e-3f) {
       f2 Z = f2_sub(f2{tbest, 0.0f}, c23);
 #pragma unroll 1
       for (int q = 0; q < 4; ++q) Z = cubic_step_df(Z, c2, c1, c0);

@@ -1,6 +1,7 @@
 """Real-fluid properties where the cubic is delicate: on either side of a saturation line (which of two roots
 has the least Gibbs energy), near the critical points and next to merging roots, and in the dilute limit,
-with trace species down to 1e-60.
+with trace species down to 1e-60; the compressibility that the reaction step starts from, and the derivatives
+of T' of a step that changes nothing.
 
 Bounds. The mixing sums are good to 2^-42 of their terms, so the cubic's value at a root is off by at most
 2^-41 of its terms' absolute sum S, the root by that over |f'(Z)|, and c_p, whose departure part goes with
@@ -119,3 +120,32 @@ def test_properties(kind):
     curve = np.abs(6 * Zo - 2 * (1 - B)) + 2 * (1 + B)
     dep = np.abs(s["cp"]) + o.R / s["W_mix"] * 10
     assert np.max(np.abs(cp - s["cp"]) / (dep * (2.0 ** -39 + 2 * curve * dZ / slope + 2 * dZ / (Zo - B)))) <= 1.0
+
+
+def test_step_and_jacobian_next_to_saturation():
+    """eos_pre's root is the one of least Gibbs energy: the other phase's Z is a factor off. With a network that
+    changes nothing (du = 0), h(T', p, Y) = h(T, p, Y) and h, homogeneous of degree 1 in Y, give dT'/dT = 1 and
+    dT'/dY_j = h / c_p; double-float errors of the root, by its slope, and of h's cancelling terms stay far
+    below the bound, which a state of the other phase misses by its heat of evaporation."""
+    import torch
+    import __graft_entry__ as g
+    g.build()
+    import paper_2508_18969_gb300 as df
+    T, p, Y = _states("saturation")
+    net = synth.network.make_network([11, 32, 9], 9, seed=1)
+    for W, b in zip(net.W, net.b):
+        W[:], b[:] = 0, 0
+    net.out_mean[:] = 0
+    dev = [torch.tensor(a, device="cuda") for a in (T, p, Y)]
+    s = o.state(MECH, T, p, Y)
+    st = df.State(MECH, net, T_react=0.0, batch_cells=512)
+    _, Z, _, status = (t.cpu().numpy() for t in st.eos_pre(*dev))
+    assert not status.any()
+    np.testing.assert_allclose(Z, s["Z"], rtol=1e-6)
+    _, dT = (t.cpu().numpy() for t in st.chem_jacobian(*dev))
+    st.close()
+    np.testing.assert_allclose(dT[:, 0], 1.0, rtol=1e-6)
+    scale = np.sum(np.abs(Y * species_h_molar(MECH.nasa, T)) / MECH.W[:, None], axis=0) + np.abs(s["h_dep"] / s["W_mix"])
+    j = Y.argmax(0)   # (Box-Cox slopes are floored for trace species)
+    off = np.abs(dT[np.arange(len(T)), 1 + j] - s["h"] / s["cp"]) * np.abs(s["cp"]) / scale
+    assert off.max() <= 1e-6, off.max()
