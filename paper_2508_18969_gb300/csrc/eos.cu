@@ -1451,11 +1451,10 @@ __device__ __forceinline__ f2 f2_ipow(f2 b, int m) {
   return r;
 }
 
-// y^lambda for y > 0 and lambda = 1/m to within dl: r0 = FP32 power (relative error ~1e-6), then
-// r = r0 (1 + e)^(-1/m) with e = r0^m / y - 1 by its series to e^3 (|e| ~ 1e-5, truncation below
-// 1e-19), in double-float. Zero for y below the normal FP32 range.
+// y^lambda for a normal FP32 y > 0 and lambda = 1/m to within dl: r0 = FP32 power (relative error
+// ~1e-6), then r = r0 (1 + e)^(-1/m) with e = r0^m / y - 1 by its series to e^3 (|e| ~ 1e-5,
+// truncation below 1e-19), in double-float.
 __device__ __forceinline__ f2 f2_root(f2 y, float lamf, int m, float dl) {
-  if (!(y.h > 1e-37f)) return f2{0.0f, 0.0f};
   const float r0 = exp2f(lamf * log2f(y.h));
   const f2 e = f2_addf(f2_mul(f2_ipow(f2{r0, 0.0f}, m), f2_rcp(y)), -1.0f);
   const float im = 1.0f / (float)m;
@@ -1464,6 +1463,13 @@ __device__ __forceinline__ f2 f2_root(f2 y, float lamf, int m, float dl) {
   f2 c = f2_mul(e, f2_rcp(f2{-(float)m, 0.0f}));
   c = f2_addf(c, dl != 0.0f ? q + dl * logf(y.h) : q);
   return f2_add(f2{r0, 0.0f}, f2_mulf(c, r0));
+}
+
+// y^lambda for any finite y (zero for y <= 0), in FP64. Out of line: for mass fractions whose low
+// part, or themselves, fall out of FP32's range. The root brings them back into it (1e-300 to 1e-30
+// for lambda = 0.1, to 2e-5 for 1/64), so they count as much as any other.
+__device__ __noinline__ f2 root_small(double y, double lam) {
+  return y > 0.0 ? f2_from(pow(y, lam)) : f2{0.0f, 0.0f};
 }
 
 // Input scales of the tangent directions (T, Y_1..Y_n): dx_0/dT = 1/std_T and
@@ -1669,7 +1675,9 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       const float* Or = O + r * ldo;
       for (int k = 0; k < n; ++k) {
         const float ldu = lamf * fmaf(out_std[k], Or[k], out_mean[k]);
-        const f2 base = f2_addf(f2_root(ycol.get(k), lamf, mpow, dl), ldu);
+        const f2 yk = ycol.get(k);
+        const f2 root = yk.h >= 1e-30f ? f2_root(yk, lamf, mpow, dl) : root_small(Y[k * ldY + cell], P.lambda);
+        const f2 base = f2_addf(root, ldu);
         f2 zl = f2{0.0f, 0.0f}, z = zl;
         if (base.h > 0.0f) {
           zl = f2_ipow(base, mpow - 1);
