@@ -323,7 +323,8 @@ struct SplitLayer {
   // MN-major operands: bit 0, A holds its K reduction rows of M columns; bit 1, W its K rows of N columns
   int tr = 0;
   int M = 0;
-  int64_t o_plane = 0;
+  void* out = nullptr;     // set by split_encode, like its pitch
+  int64_t ldo = 0, o_plane = 0;
   const float* bias = nullptr;   // [N], zero padded to 32
   bool planes = true;      // output as planes (hidden layers) or FP32
   bool gelu = true;

@@ -27,7 +27,12 @@
 //
 // Results that are not finite: products of an infinite operand with the other's planes would give
 // NaN (inf x 0) where FP32 arithmetic gives an infinity, and a sum near the end of the FP32 range
-// may overflow in another order. Such an element is recomputed as a chain of FP32 FMAs over k.
+// may overflow in another order. A CTA that met such a sum goes over its tiles once more when its
+// pipeline has ended (redo_nonfinite): elements whose result is not finite are recomputed as chains of
+// FP32 FMAs over k, in blocks through shared memory. Nothing waits for that pass inside the kernel, so
+// its length cannot run out a pipeline wait: one infinite gradient row, which touches every weight of a
+// layer, makes a backward pass of 65,536 rows 14.8 ms instead of 2.8, of 262,145 rows 74 instead of 10.7.
+// (As a chain per element in the epilogue it held up the other roles for as long, past their limit.)
 //
 // Warp roles (one CTA per SM): warp 0 TMA producer, warp 1 tensor memory and MMAs, then groups of
 // eight epilogue warps (two per TMEM lane quarter, each holding every other 32-column chunk of its 32
@@ -51,6 +56,7 @@ constexpr int kPlanes = 3;
 constexpr int kRing = 2;                        // stages per plane
 constexpr int kStgBytes = 4096;                 // staging per epilogue warp: 32 x 32 FP32
 constexpr int kABytes = BM * kRowBytes;         // one A plane of a stage
+constexpr int kBadWords = 64;                   // bits of marked m units, by m unit modulo their number
 
 enum { kSActNone = 0, kSActTanh = 1, kSActTable = 2 };
 enum { kSPlain = 0, kSStoreG = 1, kSRowG = 2 };
@@ -77,7 +83,7 @@ struct SCfg {
   static constexpr int kTmemCols = 2 * kGroups * kBN;    // two accumulators per group
   static constexpr int kSmem = kPlanes * kRing * kSlot + kEpiWarps * kStgBytes + 1024 + 512;
 };
-static_assert(SCfg<kWide>::kSmem <= kSmemLimit && SCfg<kSmall>::kSmem <= kSmemLimit, "stages must fit");
+static_assert(std::max(SCfg<kWide>::kSmem, SCfg<kSmall>::kSmem) + 4 * kBadWords + 64 <= kSmemLimit, "stages must fit");
 
 struct SplitArgs {
   RowMap rows;
@@ -93,6 +99,8 @@ struct SplitArgs {
   // the planes, for elements recomputed in FP32: entry (r, k) of A at r a_rs + k a_ks, likewise W
   const __nv_bfloat16 *A, *W;
   int64_t a_rs, a_ks, a_plane, w_rs, w_ks, w_plane;
+  void* out;               // and the output they go to
+  int64_t ldo, o_plane;
   int* err;
   long long budget;
   uint32_t suspend;
@@ -120,21 +128,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t sr
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
                ::"l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(src)
                : "memory");
-}
-
-// One element of A W^T over k in [k0, k1) as a chain of FP32 FMAs, from the planes.
-__device__ __noinline__ float dot_fp32(const SplitArgs& g, int64_t row, int col, int k0, int k1) {
-  const __nv_bfloat16* a = g.A + row * g.a_rs + k0 * g.a_ks;
-  const __nv_bfloat16* w = g.W + col * g.w_rs + k0 * g.w_ks;
-  float s = 0.0f;
-  for (int k = k0; k < k1 && s == s; ++k, a += g.a_ks, w += g.w_ks) {   // a NaN stays a NaN
-    const float av = __bfloat162float(a[0]) +
-                     (__bfloat162float(a[g.a_plane]) + __bfloat162float(a[2 * g.a_plane]));
-    const float wv = __bfloat162float(w[0]) +
-                     (__bfloat162float(w[g.w_plane]) + __bfloat162float(w[2 * g.w_plane]));
-    s = fmaf(av, wv, s);
-  }
-  return s;
 }
 
 // tanh-form GELU, 0.5 z (1 + tanh u) = z / (1 + exp(-2 u)), u = c (z + a z^3): one exponential and
@@ -196,14 +189,11 @@ __device__ __forceinline__ void store_f32(const float (&v)[32], const CUtensorMa
 template <bool PLANES, int ACT, int MODE>
 __device__ __forceinline__ void split_chunk(float (&v)[32], const SplitArgs& g, const CUtensorMap* tmO,
                                             const CUtensorMap* tmG, int64_t M, int64_t mrow, int64_t m0,
-                                            int col0, int k0, int k1, uint8_t* stg, int& buf, int lane) {
+                                            int col0, uint32_t mu, uint32_t* bad, uint8_t* stg, int& buf,
+                                            int lane) {
   const int64_t row = mrow + lane;          // row of A
   const bool row_ok = row < M;
-  if (any_nonfinite(v, 1.0f) && row_ok) {   // rare
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (!(fabsf(v[i]) <= 3.402823466e38f) && col0 + i < g.N) v[i] = dot_fp32(g, row, col0 + i, k0, k1);
-  }
+  if (any_nonfinite(v, 1.0f) && row_ok) atomicOr(bad + (mu >> 5) % kBadWords, 1u << (mu & 31));   // rare
   if constexpr (MODE == kSRowG) {
     const float4* gr = reinterpret_cast<const float4*>(g.G + ((row_ok ? row : M - 1) / g.ntan) * g.ldg + col0);
 #pragma unroll
@@ -287,10 +277,118 @@ __device__ __forceinline__ void split_chunk(float (&v)[32], const SplitArgs& g, 
   }
 }
 
+// Recomputes the non-finite results of the 128 x 32 outputs at rows m0 (of A; o0 of the output) and
+// columns col0 as chains of FP32 FMAs over k in [k0, k1), ascending, and stores those elements. All
+// threads of the block; the first 256 hold 4 x 4 elements each. Blocks of 32 k of both operands, summed
+// from their planes, go through shared memory; the loop ends once every such element is NaN, which is
+// the first block for the rows of a cell that is not finite.
+constexpr int kRedoK = 32;
+constexpr int kRedoA = BM + 4, kRedoW = 32 + 4;   // pitches
+template <bool PLANES, int ACT, int MODE>
+__device__ void redo_nonfinite(const SplitArgs& g, float* sm, int64_t M, int64_t m0, int64_t o0,
+                                            int col0, int k0, int k1) {
+  const int t = threadIdx.x, ty = t >> 3, tx = t & 7;
+  unsigned todo = 0;   // bit 4 i + j: element (4 ty + i, 4 tx + j)
+  if (t < 256) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int64_t r = m0 + 4 * ty + (e >> 2);
+      const int c = col0 + 4 * tx + (e & 3);
+      if (r >= M || c >= g.N) continue;
+      const int64_t o = (r - m0 + o0) * g.ldo + c;
+      const float v = PLANES ? __bfloat162float(((const __nv_bfloat16*)g.out)[o]) : ((const float*)g.out)[o];
+      if (!isfinite(v)) todo |= 1u << e;
+    }
+  }
+  if (!__syncthreads_or(todo != 0)) return;
+  float *sA = sm, *sW = sm + kRedoK * kRedoA;
+  float acc[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) acc[e] = 0.0f;
+  auto value = [](const __nv_bfloat16* p, int64_t plane) {
+    return __bfloat162float(__ldg(p)) + (__bfloat162float(__ldg(p + plane)) + __bfloat162float(__ldg(p + 2 * plane)));
+  };
+  // the operand's contiguous index runs along the threads
+  const bool ka = g.a_ks == 1, kw = g.w_ks == 1;
+  for (int kb = k0; kb < k1; kb += kRedoK) {
+    for (int i = t; i < BM * kRedoK; i += blockDim.x) {
+      const int r = ka ? i / kRedoK : i % BM, k = ka ? i % kRedoK : i / BM;
+      const bool in = m0 + r < M && kb + k < k1;
+      sA[k * kRedoA + r] = in ? value(g.A + (m0 + r) * g.a_rs + (kb + k) * g.a_ks, g.a_plane) : 0.0f;
+    }
+    for (int i = t; i < 32 * kRedoK; i += blockDim.x) {
+      const int c = kw ? i / kRedoK : i % 32, k = kw ? i % kRedoK : i / 32;
+      const bool in = col0 + c < g.N && kb + k < k1;
+      sW[k * kRedoW + c] = in ? value(g.W + (col0 + c) * g.w_rs + (kb + k) * g.w_ks, g.w_plane) : 0.0f;
+    }
+    __syncthreads();
+    bool more = false;
+    if (todo) {
+      const int nk = min(kRedoK, k1 - kb);
+      for (int k = 0; k < nk; ++k) {
+        const float4 a = *reinterpret_cast<const float4*>(sA + k * kRedoA + 4 * ty);
+        const float4 w = *reinterpret_cast<const float4*>(sW + k * kRedoW + 4 * tx);
+        const float av[4] = {a.x, a.y, a.z, a.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = fmaf(av[e >> 2], wv[e & 3], acc[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < 16; ++e) more = more || (((todo >> e) & 1u) && acc[e] == acc[e]);
+    }
+    if (!__syncthreads_or(more)) break;
+  }
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    if (!((todo >> e) & 1u)) continue;
+    const int64_t r = m0 + 4 * ty + (e >> 2), ro = r - m0 + o0;
+    const int c = col0 + 4 * tx + (e & 3);
+    float v = acc[e];
+    if constexpr (MODE == kSRowG) {
+      v *= g.G[(r / g.ntan) * g.ldg + c];
+    } else {
+      v += g.bias[c];
+      if constexpr (MODE == kSStoreG) g.G[ro * g.ldg + c] = gelu_grad_exp(v, gelu_exp(v));
+      if constexpr (ACT == kSActTanh) v = __fdividef(v, 1.0f + gelu_exp(v));
+      else if constexpr (ACT == kSActTable) v = gelu_from_table(v, g.gtab);
+    }
+    if constexpr (PLANES) {
+      __nv_bfloat16* o = (__nv_bfloat16*)g.out + ro * g.ldo + c;
+      split_one(v, o[0], o[g.o_plane], o[2 * g.o_plane]);
+    } else {
+      ((float*)g.out)[ro * g.ldo + c] = v;
+    }
+  }
+}
+
+// redo_nonfinite over this CTA's tiles whose m unit is marked in `bad`. Out of line, with everything formed anew: what it needs
+// must not take registers from the epilogue.
+template <int CFG, bool PLANES, int ACT, int MODE>
+__device__ __noinline__ void redo_tiles(const SplitArgs& g, const WalkStep& step, const uint32_t* bad) {
+  constexpr bool PAIR = SCfg<CFG>::kPair;
+  extern __shared__ uint8_t smem_raw[];
+  float* sm = (float*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  asm volatile("fence.proxy.async;" ::: "memory");
+  const int64_t M = valid_rows(g.rows), tiles_m = (M + BM - 1) / BM;
+  const uint32_t units_m = (uint32_t)(PAIR ? (tiles_m + 1) / 2 : tiles_m);
+  const int tiles_n = (g.N + g.tw - 1) / g.tw;
+  const int kbs = ((g.K + 63) / 64 + g.ksplit - 1) / g.ksplit;
+  for (ItemWalk w(PAIR ? blockIdx.x >> 1 : blockIdx.x, units_m, tiles_n); w.split < g.ksplit;
+       w.next(step, units_m, tiles_n)) {
+    if (!((bad[(w.mu >> 5) % kBadWords] >> (w.mu & 31)) & 1u)) continue;
+    const int k0 = w.split * kbs * 64, k1 = min(g.K, k0 + kbs * 64), n0 = w.nt(tiles_n) * g.tw;
+    const int64_t m0 = (PAIR ? w.mu * 2 + cluster_rank() : (int64_t)w.mu) * BM;
+    for (int c = n0; c < n0 + g.tw && c < g.N && m0 < M; c += 32) {
+      redo_nonfinite<PLANES, ACT, MODE>(g, sm, M, m0, m0 + w.split * g.split_rows, c, k0, k1);
+      __syncthreads();
+    }
+  }
+}
+
 template <int CFG, bool PLANES, int ACT, int MODE, int TR>
 __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-    const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmG, SplitArgs g) {
+    const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmG,
+    const __grid_constant__ SplitArgs g) {
   using C = SCfg<CFG>;
   constexpr bool PAIR = C::kPair;
   extern __shared__ uint8_t smem_raw[];
@@ -299,6 +397,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
   uint64_t* bars = (uint64_t*)(sOut + C::kEpiWarps * kStgBytes);
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
+  __shared__ uint32_t bad_sh[kBadWords];   // m units with sums that are not finite
   __shared__ WalkStep walk_sh;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -328,6 +427,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  for (int i = threadIdx.x; i < kBadWords; i += C::kThreads) bad_sh[i] = 0;
   if (warp == 1) {
     if constexpr (PAIR) {
       asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -559,8 +659,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
       for (int c = 0; c < C::kChunks; ++c) {
         const int col0 = nt * g.tw + 32 * (slot + 2 * c);
         if (32 * (slot + 2 * c) < width && col0 < g.N)
-          split_chunk<PLANES, ACT, MODE>(acc[c], g, &tmO, &tmG, M, mrow, m0, col0, kb0 * 64,
-                                         min(g.K, kb1 * 64), stg, buf, lane);
+          split_chunk<PLANES, ACT, MODE>(acc[c], g, &tmO, &tmG, M, mrow, m0, col0, w.mu, bad_sh, stg, buf, lane);
       }
     }
     if (lane == 0) bulk_wait_all();
@@ -578,6 +677,9 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                    "r"((uint32_t)C::kTmemCols) : "memory");
   }
+  // the stores above have completed, and so have all copies into and MMA reads of shared memory
+  if (__syncthreads_or(threadIdx.x < kBadWords && bad_sh[threadIdx.x % kBadWords]) && !abort_sh)
+    redo_tiles<CFG, PLANES, ACT, MODE>(g, walk_sh, bad_sh);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -734,6 +836,8 @@ bool split_encode(SplitLayer& L, int64_t a_rows, void* out, int64_t o_rows, int6
   const CUtensorMapSwizzle s128 = CU_TENSOR_MAP_SWIZZLE_128B, s64 = CU_TENSOR_MAP_SWIZZLE_64B;
   static const int most[2] = {SCfg<kWide>::kBN, SCfg<kSmall>::kBN};
   L.g = G;
+  L.out = out;
+  L.ldo = ldo;
   if (L.tr & kTrA) {   // columns 0..M-1 of the L.K rows; rows past them read as zero
     if (!encode_3d(&L.tmA, L.A, 2, L.M, L.K, kPlanes, L.lda, L.a_plane, 64, 64, s128, err, errlen)) return false;
   } else if (!encode_3d(&L.tmA, L.A, 2, L.K, a_rows, kPlanes, L.lda, L.a_plane, 64, BM, s128, err, errlen)) {
@@ -785,6 +889,9 @@ cudaError_t launch_split(const SplitLayer& L, const RowMap& rows, int num_sms, i
   a.w_rs = (L.tr & kTrW) ? 1 : L.ldw;
   a.w_ks = (L.tr & kTrW) ? L.ldw : 1;
   a.w_plane = L.w_plane;
+  a.out = L.out;
+  a.ldo = L.ldo;
+  a.o_plane = L.o_plane;
   a.err = err;
   a.budget = kWaitBudget;
   a.suspend = kSuspendNs;
