@@ -480,6 +480,9 @@ __device__ __forceinline__ float g_dep_f(float Z, float A, float B) {
          __fdividef(A, 2.0f * s2 * B) * __logf(__fdividef(Z + (1.0f + s2) * B, Z + (1.0f - s2) * B));
 }
 
+// The distance from B beyond which the Gibbs energy at an FP32 seed ranks its root (why: select_Z3).
+__device__ __forceinline__ float seed_distance(float cphi) { return fabsf(cphi) > 0.9999f ? 5e-3f : 3e-4f; }
+
 __device__ __forceinline__ double g_dep(double Z, double A, double B, const double* lnt) {
   return Z - 1.0 - dlog_tab(Z - B, lnt) -
          A * drcp(2.0 * kSQ2 * B) * dlog_tab((Z + (1.0 + kSQ2) * B) * drcp(Z + (1.0 - kSQ2) * B), lnt);
@@ -525,8 +528,8 @@ __device__ __noinline__ double select_Z3(double A, double B, double c2, double c
   const float phi = acosf(cphi) * (1.0f / 3.0f);
   // A root whose Gibbs energy is clearly the least by the FP32 seeds is the only one polished (2^18 states
   // of which a third have three roots: 211 -> 180 us). The roots are stationary points of the Gibbs energy,
-  // so a seed's error (1e-6; 1e-4 next to a double root) enters squared over Z - B: 5e-3 is far enough from
-  // B, and 1e-3 more than the FP32 energies' own error.
+  // so a seed's error enters squared over Z - B. It is below 1e-5 for |cos phi| <= 0.9999 and 1e-4 next to
+  // a double root: 3e-4 and 5e-3 are far enough from B for a margin of 1e-3.
   {
     const float Bf = d_to_f_trunc(B), Af = d_to_f_trunc(A), c23 = d_to_f_trunc(c2) * (1.0f / 3.0f);
     float tbest = 0.0f, g1 = __int_as_float(0x7f800000), g2 = g1;
@@ -535,7 +538,7 @@ __device__ __noinline__ double select_Z3(double A, double B, double c2, double c
     for (int k = 0; k < 3; ++k) {
       const float tk = m * cosf(phi - 2.0943951023931955f * (float)k);
       const float zk = tk - c23;
-      if (fabsf(zk - Bf) < 5e-3f) clear = false;
+      if (fabsf(zk - Bf) < seed_distance(cphi)) clear = false;
       if (zk > Bf) {
         const float g = g_dep_f(zk, Af, Bf);
         if (!(g == g)) clear = false;
@@ -668,8 +671,7 @@ __device__ __forceinline__ f2 g_dep_df(f2 Z, f2 A, f2 B, const f2* lt) {
 
 // Three real roots (select_Z3 in double-float). Out of line, as there. The roots above B are
 // first ranked by their FP32 seeds and FP32 departure Gibbs energies; when one root is lower
-// by more than 1e-3 and no seed lies within 5e-3 of B (why these: select_Z3), only that root is
-// polished. Otherwise every root is polished and compared in double-float.
+// by more than 1e-3 and no seed is too close to B (why: select_Z3), only that root is polished. Otherwise every root is polished and compared in double-float.
 __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23, float Pf,
                                         float Qf, const f2* lt, int& status) {
   const float m = (Pf < 0.0f) ? 2.0f * sqrtf(-Pf / 3.0f) : 0.0f;
@@ -683,7 +685,7 @@ __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23,
     for (int k = 0; k < 3; ++k) {
       const float tk = m * cosf(phi - 2.0943951023931955f * (float)k);
       const float zk = tk - c23.h;
-      if (fabsf(zk - B.h) < 5e-3f) clear = false;
+      if (fabsf(zk - B.h) < seed_distance(cphi)) clear = false;
       if (zk > B.h) {
         const float g = g_dep_f(zk, A.h, B.h);
         if (!(g == g)) clear = false;
