@@ -480,8 +480,12 @@ __device__ __forceinline__ float g_dep_f(float Z, float A, float B) {
          __fdividef(A, 2.0f * s2 * B) * __logf(__fdividef(Z + (1.0f + s2) * B, Z + (1.0f - s2) * B));
 }
 
-// The distance from B beyond which the Gibbs energy at an FP32 seed ranks its root (why: select_Z3).
-__device__ __forceinline__ float seed_distance(float cphi) { return fabsf(cphi) > 0.9999f ? 5e-3f : 3e-4f; }
+// The distance from B beyond which the Gibbs energy at an FP32 seed ranks its root: a hundred times the
+// seed's error (3e-7, and 2e-7 over the sine of phi, which goes to 0 at a double root). The roots are
+// stationary points of the Gibbs energy, so that error enters as (error / (Z - B))^2 / 2 = 5e-5.
+__device__ __forceinline__ float seed_distance(float cphi) {
+  return fmaf(2e-5f, rsqrtf(fmaxf(fmaf(-cphi, cphi, 1.0f), 1e-6f)), 3e-5f);
+}
 
 __device__ __forceinline__ double g_dep(double Z, double A, double B, const double* lnt) {
   return Z - 1.0 - dlog_tab(Z - B, lnt) -
@@ -527,9 +531,8 @@ __device__ __noinline__ double select_Z3(double A, double B, double c2, double c
   cphi = fminf(fmaxf(cphi, -1.0f), 1.0f);
   const float phi = acosf(cphi) * (1.0f / 3.0f);
   // A root whose Gibbs energy is clearly the least by the FP32 seeds is the only one polished (2^18 states
-  // of which a third have three roots: 211 -> 180 us). The roots are stationary points of the Gibbs energy,
-  // so a seed's error enters squared over Z - B. It is below 1e-5 for |cos phi| <= 0.9999 and 1e-4 next to
-  // a double root: 3e-4 and 5e-3 are far enough from B for a margin of 1e-3.
+  // of which a third have three roots: 211 -> 180 us): by more than 1e-4, which covers the seeds' error
+  // (seed_distance) and the FP32 energies' own (2e-5).
   {
     const float Bf = d_to_f_trunc(B), Af = d_to_f_trunc(A), c23 = d_to_f_trunc(c2) * (1.0f / 3.0f);
     float tbest = 0.0f, g1 = __int_as_float(0x7f800000), g2 = g1;
@@ -551,7 +554,7 @@ __device__ __noinline__ double select_Z3(double A, double B, double c2, double c
         }
       }
     }
-    if (clear && g1 < g2 - 1e-3f)
+    if (clear && g1 < g2 - 1e-4f)
       return cubic_polish(cubic_polish(f_to_d(tbest) - c2 * (1.0 / 3.0), c2, c1, c0), c2, c1, c0);
   }
   double best = __longlong_as_double(0x7ff8000000000000LL);
@@ -671,7 +674,7 @@ __device__ __forceinline__ f2 g_dep_df(f2 Z, f2 A, f2 B, const f2* lt) {
 
 // Three real roots (select_Z3 in double-float). Out of line, as there. The roots above B are
 // first ranked by their FP32 seeds and FP32 departure Gibbs energies; when one root is lower
-// by more than 1e-3 and no seed is too close to B (why: select_Z3), only that root is polished. Otherwise every root is polished and compared in double-float.
+// by more than 1e-4 and no seed is too close to B (as in select_Z3), only that root is polished. Otherwise every root is polished and compared in double-float.
 __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23, float Pf,
                                         float Qf, const f2* lt, int& status) {
   const float m = (Pf < 0.0f) ? 2.0f * sqrtf(-Pf / 3.0f) : 0.0f;
@@ -698,7 +701,7 @@ __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23,
         }
       }
     }
-    if (clear && g1 < g2 - 1e-3f) {
+    if (clear && g1 < g2 - 1e-4f) {
       f2 Z = f2_sub(f2{tbest, 0.0f}, c23);
 #pragma unroll 1
       for (int q = 0; q < 4; ++q) Z = cubic_step_df(Z, c2, c1, c0);

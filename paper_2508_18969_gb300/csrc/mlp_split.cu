@@ -31,7 +31,7 @@
 // pipeline has ended (redo_nonfinite): elements whose result is not finite are recomputed as chains of
 // FP32 FMAs over k, in blocks through shared memory. Nothing waits for that pass inside the kernel, so
 // its length cannot run out a pipeline wait: one infinite gradient row, which touches every weight of a
-// layer, makes a backward pass of 65,536 rows 14.8 ms instead of 2.8, of 262,145 rows 74 instead of 10.7.
+// layer, makes a backward pass of 65,536 rows 16 ms instead of 2.8, of 262,145 rows 77 instead of 10.6.
 // (As a chain per element in the epilogue it held up the other roles for as long, past their limit.)
 //
 // Warp roles (one CTA per SM): warp 0 TMA producer, warp 1 tensor memory and MMAs, then groups of
@@ -186,6 +186,8 @@ __device__ __forceinline__ void store_f32(const float (&v)[32], const CUtensorMa
 
 // One 32-column chunk of the epilogue on this thread's row: bias and activation (or the row-group
 // scale), then the three planes, or the FP32 values, through the warp's staging buffer and out by TMA.
+// A sum that is not finite leaves a result that is not (the activations and the scale keep it so), or
+// one to be looked at because it is large: either marks the m unit mu in `bad`.
 template <bool PLANES, int ACT, int MODE>
 __device__ __forceinline__ void split_chunk(float (&v)[32], const SplitArgs& g, const CUtensorMap* tmO,
                                             const CUtensorMap* tmG, int64_t M, int64_t mrow, int64_t m0,
@@ -193,7 +195,6 @@ __device__ __forceinline__ void split_chunk(float (&v)[32], const SplitArgs& g, 
                                             int lane) {
   const int64_t row = mrow + lane;          // row of A
   const bool row_ok = row < M;
-  if (any_nonfinite(v, 1.0f) && row_ok) atomicOr(bad + (mu >> 5) % kBadWords, 1u << (mu & 31));   // rare
   if constexpr (MODE == kSRowG) {
     const float4* gr = reinterpret_cast<const float4*>(g.G + ((row_ok ? row : M - 1) / g.ntan) * g.ldg + col0);
 #pragma unroll
@@ -225,11 +226,15 @@ __device__ __forceinline__ void split_chunk(float (&v)[32], const SplitArgs& g, 
       for (int i = 0; i < 32; ++i) v[i] = gelu_from_table(v[i], g.gtab);
     }
   }
+  const bool big = any_nonfinite(v, PLANES ? 4.0f : 1.0f);   // not finite, or too large for plain rounding (rare)
+  if (big && row_ok) {
+    atomicOr(bad + (mu >> 5) % kBadWords, 1u << (mu & 31));
+    bad[kBadWords] = 1;
+  }
   if constexpr (PLANES) {
     // the planes one after the other through two staging halves of 32 rows x 64 bytes (64-byte
     // swizzle); plane p + 1 is formed from what plane p leaves
     const int sw = swz<64>(lane);
-    const bool big = any_nonfinite(v, 4.0f);   // not finite, or too large for plain rounding (rare)
 #pragma unroll
     for (int p = 0; p < kPlanes; ++p) {
       uint32_t w[16];
@@ -290,7 +295,7 @@ __device__ void redo_nonfinite(const SplitArgs& g, float* sm, int64_t M, int64_t
   const int t = threadIdx.x, ty = t >> 3, tx = t & 7;
   unsigned todo = 0;   // bit 4 i + j: element (4 ty + i, 4 tx + j)
   if (t < 256) {
-#pragma unroll
+#pragma unroll 1
     for (int e = 0; e < 16; ++e) {
       const int64_t r = m0 + 4 * ty + (e >> 2);
       const int c = col0 + 4 * tx + (e & 3);
@@ -311,11 +316,13 @@ __device__ void redo_nonfinite(const SplitArgs& g, float* sm, int64_t M, int64_t
   // the operand's contiguous index runs along the threads
   const bool ka = g.a_ks == 1, kw = g.w_ks == 1;
   for (int kb = k0; kb < k1; kb += kRedoK) {
+#pragma unroll 1
     for (int i = t; i < BM * kRedoK; i += blockDim.x) {
       const int r = ka ? i / kRedoK : i % BM, k = ka ? i % kRedoK : i / BM;
       const bool in = m0 + r < M && kb + k < k1;
       sA[k * kRedoA + r] = in ? value(g.A + (m0 + r) * g.a_rs + (kb + k) * g.a_ks, g.a_plane) : 0.0f;
     }
+#pragma unroll 1
     for (int i = t; i < 32 * kRedoK; i += blockDim.x) {
       const int c = kw ? i / kRedoK : i % 32, k = kw ? i % kRedoK : i / 32;
       const bool in = col0 + c < g.N && kb + k < k1;
@@ -325,6 +332,7 @@ __device__ void redo_nonfinite(const SplitArgs& g, float* sm, int64_t M, int64_t
     bool more = false;
     if (todo) {
       const int nk = min(kRedoK, k1 - kb);
+#pragma unroll 1
       for (int k = 0; k < nk; ++k) {
         const float4 a = *reinterpret_cast<const float4*>(sA + k * kRedoA + 4 * ty);
         const float4 w = *reinterpret_cast<const float4*>(sW + k * kRedoW + 4 * tx);
@@ -337,12 +345,18 @@ __device__ void redo_nonfinite(const SplitArgs& g, float* sm, int64_t M, int64_t
     }
     if (!__syncthreads_or(more)) break;
   }
+  // the sums go through this thread's slots of shared memory, so that the stores are one loop body (the
+  // code of all sixteen made every launch 0.5 us longer, used or not)
+  float* mine = sW + kRedoK * kRedoW + t;
+  if (!todo) return;
 #pragma unroll
+  for (int e = 0; e < 16; ++e) mine[256 * e] = acc[e];
+#pragma unroll 1
   for (int e = 0; e < 16; ++e) {
     if (!((todo >> e) & 1u)) continue;
     const int64_t r = m0 + 4 * ty + (e >> 2), ro = r - m0 + o0;
     const int c = col0 + 4 * tx + (e & 3);
-    float v = acc[e];
+    float v = mine[256 * e];
     if constexpr (MODE == kSRowG) {
       v *= g.G[(r / g.ntan) * g.ldg + c];
     } else {
@@ -397,7 +411,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
   uint64_t* bars = (uint64_t*)(sOut + C::kEpiWarps * kStgBytes);
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
-  __shared__ uint32_t bad_sh[kBadWords];   // m units with sums that are not finite
+  __shared__ uint32_t bad_sh[kBadWords + 1];   // m units with sums that are not finite; whether any is
   __shared__ WalkStep walk_sh;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -427,7 +441,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  for (int i = threadIdx.x; i < kBadWords; i += C::kThreads) bad_sh[i] = 0;
+  for (int i = threadIdx.x; i <= kBadWords; i += C::kThreads) bad_sh[i] = 0;
   if (warp == 1) {
     if constexpr (PAIR) {
       asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -678,8 +692,7 @@ __global__ void __launch_bounds__(SCfg<CFG>::kThreads, 1) split_gemm_kernel(
                    "r"((uint32_t)C::kTmemCols) : "memory");
   }
   // the stores above have completed, and so have all copies into and MMA reads of shared memory
-  if (__syncthreads_or(threadIdx.x < kBadWords && bad_sh[threadIdx.x % kBadWords]) && !abort_sh)
-    redo_tiles<CFG, PLANES, ACT, MODE>(g, walk_sh, bad_sh);
+  if (bad_sh[kBadWords] && !abort_sh) redo_tiles<CFG, PLANES, ACT, MODE>(g, walk_sh, bad_sh);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
