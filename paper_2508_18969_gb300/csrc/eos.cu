@@ -25,6 +25,7 @@
 #include "pdl.cuh"
 
 #include <algorithm>
+#include <atomic>
 
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
@@ -1882,30 +1883,31 @@ cudaError_t smem_optin() {
   return cudaSuccess;
 }
 
-// Blocks of Kern (threads threads, smem bytes) that fit on the device at once.
+// Blocks of Kern (threads threads, smem bytes) that fit on the device at once. Kept per device and
+// species count, which fixes an instance's shared memory: it is what the block's size is chosen by.
 template <auto Kern>
-int64_t resident_blocks(size_t smem, int threads) {
-  static int per_sm[64] = {0};
+int64_t resident_blocks(int n, size_t smem, int threads) {
+  static std::atomic<int> per_sm[64][kMaxSpecies + 1];
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int nb = (dev >= 0 && dev < 64) ? per_sm[dev] : 0;
+  int nb = (dev >= 0 && dev < 64) ? per_sm[dev][n].load(std::memory_order_relaxed) : 0;
   if (nb <= 0) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kern, threads, smem) != cudaSuccess ||
         nb <= 0) {
       cudaGetLastError();
       nb = 4;
     }
-    if (dev >= 0 && dev < 64) per_sm[dev] = nb;
+    if (dev >= 0 && dev < 64) per_sm[dev][n].store(nb, std::memory_order_relaxed);
   }
   return (int64_t)sms * nb;
 }
 
 // Grid of a grid-stride kernel: one wave of its resident blocks, fewer when there is less work.
 template <auto Kern>
-int grid_resident(int64_t nmax, size_t smem, int threads = kThreads) {
+int grid_resident(int n, int64_t nmax, size_t smem, int threads = kThreads) {
   const int64_t need = std::max<int64_t>(1, (nmax + threads - 1) / threads);
-  return (int)std::min(need, resident_blocks<Kern>(smem, threads));
+  return (int)std::min(need, resident_blocks<Kern>(n, smem, threads));
 }
 
 int grid_for(int64_t nmax, int threads = kThreads) {
@@ -1923,8 +1925,8 @@ int grid_for(int64_t nmax, int threads = kThreads) {
 // cells of 30 species 218 -> 192 us, of 50,021 cells 336 -> 285 us, of 4,096 cells of 9 species 82.6 ->
 // 77.7 us; at 77,003 cells, beyond the wave, small blocks took 427 us against 408.
 template <auto Kern>
-bool small_blocks(int64_t nmax, size_t smem) {
-  return nmax <= resident_blocks<Kern>(smem, kSmallThreads) * kSmallThreads;
+bool small_blocks(int n, int64_t nmax, size_t smem) {
+  return nmax <= resident_blocks<Kern>(n, smem, kSmallThreads) * kSmallThreads;
 }
 
 template <int NM, typename XT, int TH>
@@ -1935,7 +1937,7 @@ cudaError_t pre_launch(const EosParams& P, const RowMap& rows, const double* T, 
   cudaError_t e = smem_optin<kern>();
   if (e != cudaSuccess) return e;
   const size_t smem = eos_smem(P, TH);
-  return pdl_launch(kern, grid_resident<kern>(rows.nmax, smem, TH), TH, smem, st, 1, P, rows, T, p, Y, ldY, h0, Z, x,
+  return pdl_launch(kern, grid_resident<kern>(P.n, rows.nmax, smem, TH), TH, smem, st, 1, P, rows, T, p, Y, ldY, h0, Z, x,
                     ldx, xs, status, rho);
 }
 
@@ -1943,7 +1945,7 @@ template <int NM, typename XT>
 cudaError_t pre_th(const EosParams& P, const RowMap& rows, const double* T, const double* p,
                    const double* Y, int64_t ldY, double* h0, double* Z, XT* x, int64_t ldx,
                    float xs, int32_t* status, cudaStream_t st, double* rho) {
-  return small_blocks<eos_pre_kernel<NM, XT, kSmallThreads>>(rows.nmax, eos_smem(P, kSmallThreads))
+  return small_blocks<eos_pre_kernel<NM, XT, kSmallThreads>>(P.n, rows.nmax, eos_smem(P, kSmallThreads))
              ? pre_launch<NM, XT, kSmallThreads>(P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, st, rho)
              : pre_launch<NM, XT, kThreads>(P, rows, T, p, Y, ldY, h0, Z, x, ldx, xs, status, st, rho);
 }
@@ -1971,7 +1973,7 @@ cudaError_t post_launch(const EosParams& P, const RowMap& rows, const float* O, 
   cudaError_t e = smem_optin<kern>();
   if (e != cudaSuccess) return e;
   const size_t smem = eos_smem_post(P, TH);
-  return pdl_launch(kern, grid_resident<kern>(rows.nmax, smem, TH), TH, smem, st, 1, P, rows, O, ldo, h0, T, p, Y,
+  return pdl_launch(kern, grid_resident<kern>(P.n, rows.nmax, smem, TH), TH, smem, st, 1, P, rows, O, ldo, h0, T, p, Y,
                     ldY, pre_status, cell_status, src);
 }
 
@@ -1980,7 +1982,7 @@ cudaError_t post_nm(const EosParams& P, const RowMap& rows, const float* O, int6
                     const double* h0, double* T, const double* p, double* Y, int64_t ldY,
                     const int32_t* pre_status, int32_t* cell_status, cudaStream_t st,
                     const Source& src) {
-  return small_blocks<eos_post_kernel<NM, kSmallThreads>>(rows.nmax, eos_smem_post(P, kSmallThreads))
+  return small_blocks<eos_post_kernel<NM, kSmallThreads>>(P.n, rows.nmax, eos_smem_post(P, kSmallThreads))
              ? post_launch<NM, kSmallThreads>(P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, st, src)
              : post_launch<NM, kThreads>(P, rows, O, ldo, h0, T, p, Y, ldY, pre_status, cell_status, st, src);
 }
@@ -2002,7 +2004,7 @@ cudaError_t props_nm(const EosParams& P, int64_t n, const double* T, const doubl
                      cudaStream_t st) {
   cudaError_t e = smem_optin<props_kernel<NM>>();
   if (e != cudaSuccess) return e;
-  props_kernel<NM><<<grid_resident<props_kernel<NM>>(n, eos_smem(P)), kThreads, eos_smem(P), st>>>(
+  props_kernel<NM><<<grid_resident<props_kernel<NM>>(P.n, n, eos_smem(P)), kThreads, eos_smem(P), st>>>(
       P, n, T, p, Y, ldY, rho, h, cp, Z);
   return cudaGetLastError();
 }
