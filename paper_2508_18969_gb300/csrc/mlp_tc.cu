@@ -1186,7 +1186,8 @@ int tc_stages(int BN, int out_kind, bool pair) {
     constexpr int B = decltype(bn)::value;
     if (pair)
       return out_kind == kXF32 ? Cfg<B, kXF32, true>::kStages
-             : out_kind == kXBF16 ? Cfg<B, kXBF16, true>::kStages : Cfg<B, kXFP8, true>::kStages;
+             : out_kind == kXBF16 ? Cfg<B, kXBF16, true, epi_per_quarter(true, kActTanh)>::kStages
+                                  : Cfg<B, kXFP8, true, epi_per_quarter(true, kActTanh, kModePlain, true)>::kStages;
     // single CTAs: FP32 out is the read-out (no activation), the others hidden layers
     return out_kind == kXF32 ? Cfg<B, kXF32>::kStages
            : out_kind == kXBF16 ? Cfg<B, kXBF16, false, epi_per_quarter(false, kActTanh)>::kStages
