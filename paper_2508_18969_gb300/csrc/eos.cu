@@ -1471,11 +1471,14 @@ __device__ __forceinline__ f2 f2_root(f2 y, float lamf, int m, float dl) {
   return f2_add(f2{r0, 0.0f}, f2_mulf(c, r0));
 }
 
-// y^lambda for any finite y (zero for y <= 0), in FP64. Out of line: for mass fractions whose low
-// part, or themselves, fall out of FP32's range. The root brings them back into it (1e-300 to 1e-30
-// for lambda = 0.1, to 2e-5 for 1/64), so they count as much as any other.
-__device__ __noinline__ f2 root_small(double y, double lam) {
-  return y > 0.0 ? f2_from(pow(y, lam)) : f2{0.0f, 0.0f};
+// y^lambda for 0 < y < 1e-30, whose double-float low part, or itself, falls out of FP32's range: the root
+// of y 2^(sm), which lies in it, times 2^-s. (Such species count as much as any other: the root of 1e-300
+// is 1e-30 for lambda = 0.1 and 2e-5 for 1/64.)
+__device__ __forceinline__ f2 root_small(double y, float lamf, int m, float dl) {
+  const int s = (m - 71 - max((__double2hiint(y) >> 20) - 1023, -1023)) / m;   // y 2^(sm) >= 2^-70 (normal y)
+  if (s > 120) return f2{0.0f, 0.0f};
+  const f2 r = f2_root(f2_from(y * __hiloint2double((1023 + s * m) << 20, 0)), lamf, m, dl);
+  return f2_mulf(r, __int_as_float((127 - s) << 23) * fmaf(-0.6931472f * dl, (float)(s * m), 1.0f));
 }
 
 // Input scales of the tangent directions (T, Y_1..Y_n): dx_0/dT = 1/std_T and
@@ -1682,7 +1685,13 @@ __global__ void __launch_bounds__(kPropThreads) jac_state_kernel(EosParams P, in
       for (int k = 0; k < n; ++k) {
         const float ldu = lamf * fmaf(out_std[k], Or[k], out_mean[k]);
         const f2 yk = ycol.get(k);
-        const f2 root = yk.h >= 1e-30f ? f2_root(yk, lamf, mpow, dl) : root_small(Y[k * ldY + cell], P.lambda);
+        f2 root = f2{0.0f, 0.0f};
+        if (yk.h >= 1e-30f) {
+          root = f2_root(yk, lamf, mpow, dl);
+        } else if (yk.h >= 0.0f) {
+          const double y = Y[k * ldY + cell];
+          if (y > 0.0) root = root_small(y, lamf, mpow, dl);
+        }
         const f2 base = f2_addf(root, ldu);
         f2 zl = f2{0.0f, 0.0f}, z = zl;
         if (base.h > 0.0f) {
