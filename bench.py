@@ -191,13 +191,13 @@ _EOS_OTHER = (("// -------------------------------------------------------------
               ("cudaError_t launch_jac_scale(", "cudaError_t launch_eos_post("),
               ("cudaError_t launch_transport(", "}  // namespace dfgb"))
 MEASURED_TRAFFIC = {
-    ("layer0", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 3157.3),
-    ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 4757.1),
-    ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 2346.0),
-    ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "8ceea90e82c7f2ee", 1068.1),
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342", 293.3,
+    ("layer0", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 3158.2),
+    ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 4757.3),
+    ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 2348.9),
+    ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 1067.6),
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88", 293.2,
                                         _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342", 582.5,
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88", 582.0,
                                          _EOS_OTHER),
     # one block Gauss-Seidel sweep (gs_rhs_kernel + gs_sweep_kernel), per cell, FP64, 512 cells
     # per block row (profiles/solver_kernels_mesh-2m.md)
@@ -411,14 +411,14 @@ def measure_peaks_live(torch, dev):
 # MEASURED_TRAFFIC).
 MEASURED_PIPES = {
     # profiles/eos_kernels_layer1d-30sp-512k_bf16.md (full capture, 512K rows, first step)
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342",
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88",
                                         {"binding": "issue (FP32 double-float arithmetic)",
-                                         "fma_pipe": 0.526, "alu_pipe": 0.308, "fp64_pipe": 0.013,
-                                         "issue_active": 0.615, "warps_per_sm": 21.1}, _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "d32a97b9bde42342",
+                                         "fma_pipe": 0.524, "alu_pipe": 0.308, "fp64_pipe": 0.013,
+                                         "issue_active": 0.612, "warps_per_sm": 21.1}, _EOS_OTHER),
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88",
                                          {"binding": "issue (FP32 double-float arithmetic)",
-                                          "fma_pipe": 0.334, "alu_pipe": 0.557, "fp64_pipe": 0.037,
-                                          "issue_active": 0.712, "warps_per_sm": 22.2}, _EOS_OTHER),
+                                          "fma_pipe": 0.333, "alu_pipe": 0.556, "fp64_pipe": 0.037,
+                                          "issue_active": 0.711, "warps_per_sm": 22.2}, _EOS_OTHER),
 }
 
 

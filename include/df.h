@@ -54,8 +54,13 @@ typedef int32_t df_status;
 #define DF_CELL_NO_ROOT 2         /* the PR cubic has no real root above B */
 #define DF_CELL_NONFINITE 4       /* non-finite T, p or Y, p <= 0, or non-finite result */
 
-/* Arithmetic of the network layers (a5-a7). The equation of state, Box-Cox, renormalisation
- * and Newton steps are FP64 in every mode (Sec. 3.3.1 keeps all non-network work double). */
+/* Arithmetic of the network layers (a5-a7). Everything else is the same in every mode. Sec. 3.3.1
+ * keeps all non-network work double; here the fields are FP64 and the equation of state, the
+ * renormalisation and the Newton solve are double-float, pairs of FP32 numbers: about 48 bits
+ * (2^-46 an operation) with FP32's exponent range. FP64 are the cubic, its root and the density of
+ * df_real_fluid_props and the state of df_transport_props; FP32 are the Box-Cox inputs and the
+ * increment that scales Y' - Y. A mass fraction below 1.4e-45 counts as zero in the step. Where
+ * the cubic has three roots, the one of least Gibbs energy is told for p >= 1 kPa. */
 typedef enum {
   DF_FP32 = 0,      /* FP32 layers: tcgen05 GEMMs on three exact BF16 planes per operand (six
                        products, FP32 sums renewed every 64 terms), or chains of FP32 FMAs for the
@@ -214,8 +219,10 @@ df_status df_chem_source(df_state* s, int64_t n_cells, double dt, const double* 
  * Forward-mode tangents through the network (Sec. 2's chemistry network; GELU of Sec. 3.3.2)
  * -- FP32 on the CUDA cores for a DF_FP32 state, BF16 tcgen05 GEMMs otherwise -- then the
  * chain through de-normalisation, renormalisation and the implicit function
- * h(T', p, Y') = h0(T, p, Y). The Box-Cox slope is taken at max(Y_j, 1e-12). Cells whose step
- * would be flagged get NaN entries. Allocates its buffers at the first call on a state: it runs
+ * h(T', p, Y') = h0(T, p, Y), in double-float (dT' to about 2e-13 of its terms besides the
+ * network's error, and that divided by the cubic's slope near critical points). The Box-Cox slope
+ * is taken at max(Y_j, 1e-12), its root at any Y_j > 0. Cells whose step would be flagged get NaN
+ * entries; so do cells whose Y' before renormalisation leaves FP32's range (3e38), as in the step. Allocates its buffers at the first call on a state: it runs
  * in batches of min(batch_cells, 65,536) cells, whose tangent activations take about
  * 2 x batch x (n + 1) x (widest hidden layer) elements (13 GB in BF16 for 30 species and a
  * 1600-wide layer). Uses the state's scratch, so it must not overlap other calls on the same
@@ -343,7 +350,8 @@ void df_graph_destroy(df_graph* g);
  * df_get_tiles reports the tile of each layer (0 for the layers of DF_FP32 states) in bn[0..max_layers): its
  * width, | DF_TILE_PAIR when the layer runs on CTA pairs (two CTAs of a cluster share one
  * 256-row tile through cta_group::2 MMAs, each holding half of the tile's weight rows), and
- * the number of layers in *n_layers.
+ * the number of layers in *n_layers. A layer on CTA pairs that no df_autotune has tiled runs
+ * launches so short that they cost less with it on 160-column pair tiles instead.
  * Paper: Sec. 3.3.3 (the network's matrix products tiled for the memory hierarchy of the
  * target processor); the timing-based choice of tiles has no counterpart in the paper. */
 #define DF_TILE_PAIR 0x1000

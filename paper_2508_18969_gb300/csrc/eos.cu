@@ -17,8 +17,10 @@
 //     is FP32 (it only scales Y' - Y);
 //   * finiteness and threshold tests look at the bits of the FP64 values, and the FP32 <-> FP64
 //     conversions are integer operations (ddfloat.cuh);
-//   * the cubic root, departure enthalpy, c_p and the Newton update are FP64; reciprocals and
-//     square roots start from FP32 values and take FP64 Newton refinements;
+//   * the state -- cubic, root, departure enthalpy, c_p, the Newton solve for T -- is double-float in
+//     the step and Jacobian kernels; the property kernel takes the cubic, its root and the density
+//     in FP64, the transport kernel its whole state; reciprocals and square roots start from FP32
+//     values and take one or two Newton refinements;
 //   * the Box-Cox features that feed the network are FP32 (they are quantised anyway).
 #include "dfgb_internal.cuh"
 #include "ddfloat.cuh"
@@ -46,7 +48,7 @@ constexpr int kPostBlocks = 3;
 // four times the blocks, so that no SM is idle while another has eight warps, and room for the compiler
 // to overlap a thread's chains (rule in small_blocks).
 constexpr int kSmallThreads = 64;
-constexpr int kPropThreads = 128;  // the property and transport kernels
+constexpr int kPropThreads = 128;  // the transport and Jacobian state kernels
 constexpr int kPropBlocks = 5;
 constexpr int kCellNotConverged = 1;
 constexpr int kCellNoRoot = 2;
@@ -1623,7 +1625,9 @@ __global__ void __launch_bounds__(256) jac_tangent0_kernel(int64_t ncell, int nt
 // at (T, Y) and (T', Y'), T' by Newton; it leaves in the cell's scratch row, as double-float pairs,
 //   [dZ_k/du_k / S (n), Y'_k (n), c_p(T, Y), c_p(T', Y'), HGrad at (T, Y), HGrad at (T', Y')];
 // jac_columns_kernel, a warp per cell, takes the rest: lane k the sums over species of dh/dY_k at both
-// states, then lane t the column of direction t. 119 and 184 us for those cells (issue-bound, FP32 pipes).
+// states, then lane t the column of direction t. 114 and 188 us for those cells. The first is bound by
+// the chains of its four warps an SM; the second by L1: lane t reads its direction's tangents one float
+// at a time from a row of its own, 25 sectors a request (L1 data pipe 77 %, FP32 pipes 33 %).
 constexpr int kJacRow = 2 + 2 * 6;   // scalars per cell after the two columns
 
 template <int NM>

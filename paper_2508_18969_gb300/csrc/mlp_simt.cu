@@ -1,7 +1,8 @@
-// Network layers as chains of FP32 FMAs on the CUDA cores, for the FP32 passes whose results leave in
-// FP64 and are held to 1e-9 of earlier versions' values, which no other order of summation keeps: the
-// Jacobian of the step and property-network inference (every other FP32 pass runs on the tensor cores,
-// mlp_split.cu). Register-tiled SGEMM, 128x128 block tile, BK = 8, 256 threads each owning an 8x8
+// Network layers as chains of FP32 FMAs on the CUDA cores, for the two FP32 passes that have not moved to
+// the tensor cores (mlp_split.cu, which is faster and closer to FP64): the Jacobian of the step and
+// property-network inference. Their FP64 results would change by some 1e-6 with the order of summation,
+// like the FP32 sums behind them; until they move, df_mlp_forward and df_propnet_infer of one FP32
+// network differ by as much. Register-tiled SGEMM, 128x128 block tile, BK = 8, 256 threads each owning an 8x8
 // sub-tile, double-buffered shared memory, persistent over the tiles of the (device-counted) valid
 // rows, with bias + tanh-GELU (Sec. 3.3.2, the accurate tanhf) fused into the epilogue.
 #include "dfgb_internal.cuh"

@@ -180,9 +180,7 @@ int prof_family(df_state* s, const char* name) {
   return (int)s->prof_names.size() - 1;
 }
 
-// The layers of an FP32 property network (df_propnet_infer) as chains of FP32 FMAs: its outputs leave in
-// FP64, and callers hold them to 1e-9 of the values of earlier versions, which a sum in another order
-// would not keep.
+// The layers of an FP32 property network (df_propnet_infer) as chains of FP32 FMAs (why: mlp_simt.cu).
 static df_status run_propnet_fp32(df_state* s, const RowMap& rm, cudaStream_t st) {
   static const char* kLayer[8] = {"layer0", "layer1", "layer2", "layer3",
                                   "layer4", "layer5", "layer6", "layer7"};

@@ -101,8 +101,9 @@ __global__ void loss_grad_kernel(int64_t B, int n, const float* __restrict__ O, 
 // part[y * C + c] = sum over the rows y, y + gridDim.y, ... of column c of a matrix of NP BF16 planes
 // (value = sum of the planes), FP32, in a fixed order: the bias gradient. Block x takes 256 columns, a
 // warp one row at a time (512 contiguous bytes a plane), eight columns a lane.
-// Bound by the reads of the gradients: eight rows in flight a warp, up to eight blocks an SM (65,536 rows
-// of 1600 columns 61 -> 43 us, 4.8 TB/s, of 800 columns 32 -> 26 us, with four rows and four blocks before).
+// Bound by the reads of the gradients: eight rows in flight a warp, up to eight blocks an SM, of which the
+// scratch for the partial sums leaves 64 a strip: under three for 1600 columns (65,536 rows of 1600 columns
+// 61 -> 43 us, 4.8 TB/s, of 800 columns 32 -> 26 us, with four rows in flight and at most four blocks before).
 template <int NP>
 __global__ void __launch_bounds__(256) colsum_kernel(int64_t R, int64_t C,
                                                      const __nv_bfloat16* __restrict__ in, int64_t ld,
