@@ -149,3 +149,34 @@ def test_step_and_jacobian_next_to_saturation():
     j = Y.argmax(0)   # (Box-Cox slopes are floored for trace species)
     off = np.abs(dT[np.arange(len(T)), 1 + j] - s["h"] / s["cp"]) * np.abs(s["cp"]) / scale
     assert off.max() <= 1e-6, off.max()
+
+
+@pytest.mark.parametrize("kind", ["critical", "dilute"])
+def test_jacobian_of_the_unchanged_cell(kind):
+    """dT'/dT = 1 and dT'/dY_j = h / c_p (above) where c_p is ill conditioned: its bound of test_properties at both
+    ends of the step, and its change over the error of T', 2^-40 of h's terms over c_p."""
+    import torch
+    import __graft_entry__ as g
+    g.build()
+    import paper_2508_18969_gb300 as df
+    T, p, Y = _states(kind)
+    net = synth.network.make_network([11, 32, 9], 9, seed=1)
+    for W, b in zip(net.W, net.b):
+        W[:], b[:] = 0, 0
+    net.out_mean[:] = 0
+    st = df.State(MECH, net, T_react=0.0, batch_cells=512)
+    J, dT = (t.cpu().numpy() for t in st.chem_jacobian(*(torch.tensor(a, device="cuda") for a in (T, p, Y))))
+    st.close()
+    s = o.state(MECH, T, p, Y)
+    A, B, Z, cp = s["A"], s["B"], s["Z"], np.abs(s["cp"])
+    terms = Z ** 3 + (1 + B) * Z ** 2 + (A + 3 * B ** 2 + 2 * B) * Z + A * B + B ** 2 + B ** 3
+    slope = np.abs(3 * Z ** 2 - 2 * (1 - B) * Z + A - 3 * B ** 2 - 2 * B)
+    dZ = 2.0 ** -41 * terms / slope
+    scale = np.sum(np.abs(Y * species_h_molar(MECH.nasa, T)) / MECH.W[:, None], axis=0) + np.abs(s["h_dep"] / s["W_mix"])
+    bend = np.abs(o.state(MECH, T * (1 + 1e-7), p, Y)["cp"] - o.state(MECH, T * (1 - 1e-7), p, Y)["cp"]) / (2e-7 * T)
+    rel = 2.0 ** -39 + 2 * (np.abs(6 * Z - 2 * (1 - B)) + 2 * (1 + B)) * dZ / slope + 2 * dZ / (Z - B)
+    rel = 2 * rel * (1 + 10 * o.R / s["W_mix"] / cp) + 2.0 ** -40 * scale / cp * bend / cp
+    assert np.all(np.abs(dT[:, 0] - 1) <= rel), np.max(np.abs(dT[:, 0] - 1) / rel)
+    j = Y.argmax(0)
+    off = np.abs(dT[np.arange(len(T)), 1 + j] - s["h"] / s["cp"])
+    assert np.all(off <= (2.0 ** -39 + rel) * scale / cp), np.max(off / ((2.0 ** -39 + rel) * scale / cp))
