@@ -195,9 +195,9 @@ MEASURED_TRAFFIC = {
     ("layer1", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 4757.3),
     ("layer2", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 2348.9),
     ("layer3", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/mlp_tc.cu", "c4fb256c1fe777e1", 1067.6),
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88", 293.2,
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "06214f7d71e8a595", 293.9,
                                         _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88", 582.0,
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "06214f7d71e8a595", 582.6,
                                          _EOS_OTHER),
     # one block Gauss-Seidel sweep (gs_rhs_kernel + gs_sweep_kernel), per cell, FP64, 512 cells
     # per block row (profiles/solver_kernels_mesh-2m.md)
@@ -411,14 +411,14 @@ def measure_peaks_live(torch, dev):
 # MEASURED_TRAFFIC).
 MEASURED_PIPES = {
     # profiles/eos_kernels_layer1d-30sp-512k_bf16.md (full capture, 512K rows, first step)
-    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88",
+    ("eos_pre", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "06214f7d71e8a595",
                                         {"binding": "issue (FP32 double-float arithmetic)",
-                                         "fma_pipe": 0.524, "alu_pipe": 0.308, "fp64_pipe": 0.013,
+                                         "fma_pipe": 0.522, "alu_pipe": 0.306, "fp64_pipe": 0.013,
                                          "issue_active": 0.612, "warps_per_sm": 21.1}, _EOS_OTHER),
-    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "13634c0b74fd6e88",
+    ("eos_post", "32-1600-800-400-30"): ("paper_2508_18969_gb300/csrc/eos.cu", "06214f7d71e8a595",
                                          {"binding": "issue (FP32 double-float arithmetic)",
-                                          "fma_pipe": 0.333, "alu_pipe": 0.556, "fp64_pipe": 0.037,
-                                          "issue_active": 0.711, "warps_per_sm": 22.2}, _EOS_OTHER),
+                                          "fma_pipe": 0.334, "alu_pipe": 0.557, "fp64_pipe": 0.038,
+                                          "issue_active": 0.712, "warps_per_sm": 22.2}, _EOS_OTHER),
 }
 
 

@@ -57,8 +57,8 @@ typedef int32_t df_status;
 /* Arithmetic of the network layers (a5-a7). Everything else is the same in every mode. Sec. 3.3.1
  * keeps all non-network work double; here the fields are FP64 and the equation of state, the
  * renormalisation and the Newton solve are double-float, pairs of FP32 numbers: about 48 bits
- * (2^-46 an operation) with FP32's exponent range. FP64 are the cubic, its root and the density of
- * df_real_fluid_props and the state of df_transport_props; FP32 are the Box-Cox inputs and the
+ * (2^-46 an operation) with FP32's exponent range. FP64 are the cubic's coefficients, the last step of
+ * its root and the density in df_real_fluid_props and the state of df_transport_props; FP32 are the Box-Cox inputs and the
  * increment that scales Y' - Y. A mass fraction below 1.4e-45 counts as zero in the step. Where
  * the cubic has three roots, the one of least Gibbs energy is told for p >= 1 kPa. */
 typedef enum {
@@ -162,8 +162,8 @@ df_status df_chem_step_host(df_state* s, int64_t n_cells, double dt, double* T, 
  * Paper: Sec. 2 (supercritical mixture properties from the Peng-Robinson EoS; the equations are
  * Peng & Robinson 1976 with van der Waals one-fluid mixing, which the paper names but does not
  * print). The sums over species and the departure functions are double-float (pairs of FP32 numbers: about
- * 48 bits, FP32's exponent range), the cubic, its root and the density FP64: about 1e-13 relative to the
- * terms on ordinary states, and that divided by the cubic's slope at the root near critical points and
+ * 48 bits, FP32's exponent range), the cubic's coefficients, the last Newton step of its root and the
+ * density FP64: about 1e-13 relative to the terms on ordinary states, and that divided by the cubic's slope at the root near critical points and
  * where two roots merge. Next to a saturation line the root of least Gibbs energy is told for p >= 1 kPa. */
 df_status df_real_fluid_props(df_state* s, int64_t n_cells, const double* T, const double* p,
                               const double* Y, int64_t ldY, double* rho, double* h, double* cp,

@@ -18,9 +18,9 @@
 //   * finiteness and threshold tests look at the bits of the FP64 values, and the FP32 <-> FP64
 //     conversions are integer operations (ddfloat.cuh);
 //   * the state -- cubic, root, departure enthalpy, c_p, the Newton solve for T -- is double-float in
-//     the step and Jacobian kernels; the property kernel takes the cubic, its root and the density
-//     in FP64, the transport kernel its whole state; reciprocals and square roots start from FP32
-//     values and take one or two Newton refinements;
+//     the step and Jacobian kernels; the property kernel takes the cubic's coefficients, the last
+//     step of its root and the density in FP64, the transport kernel its whole state; reciprocals and
+//     square roots start from FP32 values and take one or two Newton refinements;
 //   * the Box-Cox features that feed the network are FP32 (they are quantised anyway).
 #include "dfgb_internal.cuh"
 #include "ddfloat.cuh"
@@ -476,20 +476,6 @@ __device__ __forceinline__ double cubic_polish(double Z, double c2, double c1, d
   return cubic_step(cubic_step(Z, c2, c1, c0), c2, c1, c0);
 }
 
-// Departure Gibbs energy in FP32 (for choosing among the three roots when the choice is clear).
-__device__ __forceinline__ float g_dep_f(float Z, float A, float B) {
-  const float s2 = 1.41421356f;
-  return Z - 1.0f - __logf(Z - B) -
-         __fdividef(A, 2.0f * s2 * B) * __logf(__fdividef(Z + (1.0f + s2) * B, Z + (1.0f - s2) * B));
-}
-
-// The distance from B beyond which the Gibbs energy at an FP32 seed ranks its root: a hundred times the
-// seed's error (3e-7, and 2e-7 over the sine of phi, which goes to 0 at a double root). The roots are
-// stationary points of the Gibbs energy, so that error enters as (error / (Z - B))^2 / 2 = 5e-5.
-__device__ __forceinline__ float seed_distance(float cphi) {
-  return fmaf(2e-5f, rsqrtf(fmaxf(fmaf(-cphi, cphi, 1.0f), 1e-6f)), 3e-5f);
-}
-
 __device__ __forceinline__ double g_dep(double Z, double A, double B, const double* lnt) {
   return Z - 1.0 - dlog_tab(Z - B, lnt) -
          A * drcp(2.0 * kSQ2 * B) * dlog_tab((Z + (1.0 + kSQ2) * B) * drcp(Z + (1.0 - kSQ2) * B), lnt);
@@ -533,33 +519,6 @@ __device__ __noinline__ double select_Z3(double A, double B, double c2, double c
   float cphi = (pf < 0.0f) ? (3.0f * d_to_f_trunc(Q) / (2.0f * pf)) * sqrtf(-3.0f / pf) : 0.0f;
   cphi = fminf(fmaxf(cphi, -1.0f), 1.0f);
   const float phi = acosf(cphi) * (1.0f / 3.0f);
-  // A root whose Gibbs energy is clearly the least by the FP32 seeds is the only one polished (2^18 states
-  // of which a third have three roots: 211 -> 180 us): by more than 1e-4, which covers the seeds' error
-  // (seed_distance) and the FP32 energies' own (2e-5).
-  {
-    const float Bf = d_to_f_trunc(B), Af = d_to_f_trunc(A), c23 = d_to_f_trunc(c2) * (1.0f / 3.0f);
-    float tbest = 0.0f, g1 = __int_as_float(0x7f800000), g2 = g1;
-    bool clear = true;
-#pragma unroll 1
-    for (int k = 0; k < 3; ++k) {
-      const float tk = m * cosf(phi - 2.0943951023931955f * (float)k);
-      const float zk = tk - c23;
-      if (fabsf(zk - Bf) < seed_distance(cphi)) clear = false;
-      if (zk > Bf) {
-        const float g = g_dep_f(zk, Af, Bf);
-        if (!(g == g)) clear = false;
-        if (g < g1) {
-          g2 = g1;
-          g1 = g;
-          tbest = tk;
-        } else if (g < g2) {
-          g2 = g;
-        }
-      }
-    }
-    if (clear && g1 < g2 - 1e-4f)
-      return cubic_polish(cubic_polish(f_to_d(tbest) - c2 * (1.0 / 3.0), c2, c1, c0), c2, c1, c0);
-  }
   double best = __longlong_as_double(0x7ff8000000000000LL);
   double gbest = __longlong_as_double(0x7ff0000000000000LL);
 #pragma unroll
@@ -675,9 +634,26 @@ __device__ __forceinline__ f2 g_dep_df(f2 Z, f2 A, f2 B, const f2* lt) {
   return f2_sub(f2_sub(f2_addf(Z, -1.0f), f2_log_tab(f2_sub(Z, B), lt)), f2_mul(a, L));
 }
 
+// Departure Gibbs energy in FP32 (for choosing among the three roots when the choice is clear).
+__device__ __forceinline__ float g_dep_f(float Z, float A, float B) {
+  const float s2 = 1.41421356f;
+  return Z - 1.0f - __logf(Z - B) -
+         __fdividef(A, 2.0f * s2 * B) * __logf(__fdividef(Z + (1.0f + s2) * B, Z + (1.0f - s2) * B));
+}
+
+// The distance from B beyond which the Gibbs energy at an FP32 seed ranks its root: a hundred times the
+// seed's error (3e-7, and 2e-7 over the sine of phi, which goes to 0 at a double root). The roots are
+// stationary points of the Gibbs energy, so that error enters as (error / (Z - B))^2 / 2 = 5e-5.
+__device__ __forceinline__ float seed_distance(float cphi) {
+  return fmaf(2e-5f, rsqrtf(fmaxf(fmaf(-cphi, cphi, 1.0f), 1e-6f)), 3e-5f);
+}
+
 // Three real roots (select_Z3 in double-float). Out of line, as there. The roots above B are
 // first ranked by their FP32 seeds and FP32 departure Gibbs energies; when one root is lower
-// by more than 1e-4 and no seed is too close to B (as in select_Z3), only that root is polished. Otherwise every root is polished and compared in double-float.
+// by more than 1e-4 (the FP32 energies are good to 2e-5) and no seed is too close to B
+// (seed_distance), only that root is polished. Otherwise every root is polished and compared in
+// double-float: next to a saturation line, where the energies nearly agree, or at low pressure, where
+// a liquid's root lies as near to B as its FP32 seed is off.
 __device__ __noinline__ f2 select_Z3_df(f2 A, f2 B, f2 c2, f2 c1, f2 c0, f2 c23, float Pf,
                                         float Qf, const f2* lt, int& status) {
   const float m = (Pf < 0.0f) ? 2.0f * sqrtf(-Pf / 3.0f) : 0.0f;
@@ -1174,21 +1150,22 @@ __global__ void __launch_bounds__(TH, TH == kThreads ? kPostBlocks : 1) eos_post
   }
 }
 
-// Compressibility, the cubic's slope there and the density from the mixing sums in FP64, for the properties:
-// near the critical point and where roots merge the slope goes to zero and a root is off by the error of
-// the cubic's coefficients divided by it; a liquid's root at low pressure lies within 1e-4 of B, so that
-// only FP64 tells which root has the least Gibbs energy; a dilute gas's Z is 1 less a small number.
+// Compressibility, the cubic's slope there and the density from the mixing sums, for the properties: the
+// root is told and found in double-float, then takes a Newton step on the cubic in FP64, whose coefficients
+// are FP64 from the sums on. Near critical points and where roots merge the slope goes to zero and a root
+// is off by the coefficients' error divided by it; a dilute gas's Z is 1 less a small number.
 struct Root64 {
   double Z, slope, rho;
 };
-__device__ __forceinline__ Root64 root64(const MixSums& s, double T, double p, const double* lnt, int& status) {
+__device__ __forceinline__ Root64 root64(const MixSums& s, double T, double p, const f2* lt, int& status) {
   const double Wm = drcp(f2_to(s.inv)), W2 = Wm * Wm, iT = drcp(T), t = dsqrt_pos(T);
   const double am = W2 * fma(-2.0 * f2_to(s.F1), t, fma(f2_to(s.F2), T, f2_to(s.F0)));
   const double iRT = iT * kInvR, pRT = p * iRT;
   const double A = am * pRT * iRT, B = Wm * f2_to(s.bs) * pRT;
+  const double c2 = B - 1.0, c1 = fma(B, fma(-3.0, B, -2.0), A), c0 = B * (fma(B, B, B) - A);
   Root64 r;
-  r.Z = select_Z(A, B, lnt, status);
-  r.slope = fma(3.0 * r.Z, r.Z, -2.0 * (1.0 - B) * r.Z) + (A - 3.0 * B * B - 2.0 * B);
+  r.Z = cubic_step(f2_to(select_Z_df<false>(f2_from(A), f2_from(B), lt, status)), c2, c1, c0);
+  r.slope = fma(fma(3.0, r.Z, 2.0 * c2), r.Z, c1);
   r.rho = pRT * Wm * drcp(r.Z);
   return r;
 }
@@ -1271,13 +1248,11 @@ __device__ __noinline__ void state_grad(const MixDF& m, f2 T, f2 p, PRPointDF& q
   g.c0 = f2_sub(c0, f2_mul(m.bm, ga));
 }
 
-// Density, enthalpy, c_p and compressibility of every cell (outputs may be NULL): the mixing sums in
-// double-float, the cubic, its root and the density in FP64 (Root64), the departure enthalpy and c_p in
-// double-float. 2^18 cells of 30 species: 195 us with all of the state in FP64 (its pipe busy half of the
-// time) and mass fractions loaded two at a time, 165 us so. With the cubic in double-float as well it was
-// 147 us, but took the other phase's root next to saturation lines below 20 kPa, and its roots near
-// critical points were twice as far off. Errors against FP64 on ordinary states: 1.7e-13 in density and
-// 1.4e-13 in c_p, set by the mixing sums.
+// Density, enthalpy, c_p and compressibility of every cell (outputs may be NULL), in double-float but for
+// the cubic's coefficients, the last step of its root and the density (Root64). 2^18 cells of 30 species:
+// 195 us with all of the state in FP64 (its pipe busy half of the time) and mass fractions loaded two at a
+// time, 153 us so, 147 us without FP64, whose roots near critical points were twice as far off. Errors
+// against FP64 on ordinary states: 1.7e-13 in density and 1.4e-13 in c_p, set by the mixing sums.
 template <int NM>
 __global__ void __launch_bounds__(kThreads, kPreBlocks) props_kernel(EosParams P, int64_t ncell,
     const double* __restrict__ T, const double* __restrict__ p, const double* __restrict__ Y,
@@ -1301,7 +1276,7 @@ __global__ void __launch_bounds__(kThreads, kPreBlocks) props_kernel(EosParams P
     MixSums ms;
     mixture_sums<kThreads>(ycol, n, c, ms);
     int st = 0;
-    const Root64 z = root64(ms, T[i], p[i], P.lntab, st);
+    const Root64 z = root64(ms, T[i], p[i], c.lt2, st);
     if (rho) rho[i] = z.rho;
     if (Zo) Zo[i] = z.Z;
     if (!h && !cp) continue;
